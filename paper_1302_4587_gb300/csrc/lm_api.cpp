@@ -165,6 +165,8 @@ void engine_free(Engine& e) {
     destroy_job_graph(e.egraph);
     if (e.staged) cudaEventDestroy(e.staged);
     if (e.cblock) cudaFree(e.cblock);
+    if (e.lw.block) cudaFree(e.lw.block);
+    for (void* g : e.lgraph) destroy_job_graph(g);
     cudaGetLastError();
     e = Engine();
 }
@@ -571,13 +573,180 @@ int match_edges(lm_ctx* ctx, Engine& e, const lm_graph* g, uint64_t seed, uint32
     return LM_OK;
 }
 
+// Scratch of the list path for nv vertices, nc chunks of long rows, ng graphs, nb blocks
+// of k_top and np parts (grow-only).
+static int ensure_list(lm_ctx* ctx, Engine& e, size_t nv, size_t nc, size_t ng, size_t nb, size_t np) {
+    ListWs& w = e.lw;
+    if (w.block && nv <= w.cap_v && nc <= w.cap_c && ng <= w.cap_g && nb <= w.cap_b && np <= w.cap_p) return LM_OK;
+    LM_CK(ctx, cudaStreamSynchronize(e.stream));
+    ListWs nw;
+    nw.cap_v = std::max(nv, w.cap_v);
+    nw.cap_c = std::max(nc, w.cap_c);
+    nw.cap_g = std::max(std::max(ng, w.cap_g), (size_t)1);
+    nw.cap_b = std::max(nb, w.cap_b);
+    nw.cap_p = std::max(np, w.cap_p);
+    Carver c;
+    c.add(&nw.cur, nw.cap_v);
+    c.add(&nw.lst, nw.cap_v);
+    for (int k = 0; k < 2; k++) c.add(&nw.list[k], nw.cap_v);
+    for (int k = 0; k < 3; k++) c.add(&nw.queue[k], nw.cap_v);
+    c.add(&nw.mate, nw.cap_v);
+    c.add(&nw.part, 4 * nw.cap_c);
+    c.add(&nw.pcnt, nw.cap_c);
+    c.add(&nw.segs, nw.cap_g);
+    c.add(&nw.bmap, nw.cap_b);
+    c.add(&nw.pmap, nw.cap_p);
+    c.add(&nw.pcount, nw.cap_p);
+    c.add(&nw.grounds, nw.cap_g);
+    c.add(&nw.gmatched, nw.cap_g);
+    if (w.block) {
+        cudaFree(w.block);
+        w.block = nullptr;
+    }
+    void* p = nullptr;
+    const cudaError_t err = fault_alloc(ctx) ? cudaErrorMemoryAllocation : cudaMalloc(&p, c.total);
+    if (err != cudaSuccess) {
+        cudaGetLastError();
+        e.lw = ListWs();
+        return fail(ctx, LM_ENOMEM, "workspace of %zu bytes: %s", c.total, cudaGetErrorString(err));
+    }
+    c.assign(p);
+    nw.block = p;
+    e.lw = nw;
+    LM_CK(ctx, cudaMemsetAsync(e.lw.pcnt, 0, std::max<size_t>(nw.cap_c, 1) * sizeof(uint32_t), e.stream));
+    return LM_OK;
+}
+
+// The list path needs the top bit of a vertex id and an order that holds for the
+// whole job; a renewed order keys every round anew (run_job).
+static bool list_path(const Engine& e, const lm_graph* g) { return !e.cfg.renew && g->n < 0x80000000u; }
+
+// parts of a graph in a job of `total` rows: about four a multiprocessor, within the limits
+static uint32_t list_parts(const lm_ctx* ctx, uint32_t rows, uint64_t total) {
+    const uint64_t want = total / ((uint64_t)device_sm_count(ctx->device) * 4) + 1;
+    const uint32_t per = (uint32_t)std::min<uint64_t>(LIST_PART_MAX, std::max<uint64_t>(LIST_PART_MIN, want));
+    return (rows + per - 1) / per;
+}
+
+static ListSeg list_seg(const lm_graph* g, uint64_t seed, uint32_t* dst) {
+    ListSeg d;
+    memset(&d, 0, sizeof d);
+    const uint64_t z = splitmix64_first(seed);
+    d.pk = g->pk;
+    d.nbr = g->nbr;
+    d.off = g->off;
+    d.vid = g->vid;
+    d.roff = g->roff;
+    d.task = g->task;
+    d.edges = g->edges;
+    d.dst = dst;
+    d.n = g->n;
+    d.m = g->m;
+    d.nrows = g->nrows;
+    memcpy(d.ntask, g->ntask, sizeof d.ntask);
+    d.nblk = list_blocks(g->ntask, g->nrows);
+    d.k0 = (uint32_t)z;
+    d.k1 = (uint32_t)(z >> 32);
+    return d;
+}
+
+static void list_args(ListArgs& A, Engine& e) {
+    memset(&A, 0, sizeof A);
+    const ListWs& w = e.lw;
+    A.cur = w.cur;
+    for (int k = 0; k < 2; k++) A.list[k] = w.list[k];
+    for (int k = 0; k < 3; k++) A.queue[k] = w.queue[k];
+    A.lst = w.lst;
+    A.pcount = w.pcount;
+    A.part = w.part;
+    A.pcnt = w.pcnt;
+    A.st = e.st;
+}
+
+// the list path's arguments of a job sit in the last quarter of the argument area
+constexpr size_t LIST_ARGS_OFF = ARG_AREA / 4 * 3;
+struct ListJobArgs {
+    ListArgs a;
+    ListSeg seg;
+};
+
+// The live pass of a queued job, until no row is left: k_live as often as it gives rows
+// back (once, as a rule), the state copied to the host after each.
+static int run_live(lm_ctx* ctx, Engine& e, const ListArgs* D, uint32_t nparts, bool rounds, Prof& prof) {
+    for (;;) {
+        prof.begin(LM_K_SWEEP);
+        LM_CK(ctx, launch_live(e.stream, D, nparts, rounds));
+        prof.end();
+        LM_CK(ctx, cudaMemcpyAsync(e.st_host, e.st, sizeof(DevState), cudaMemcpyDeviceToHost, e.stream));
+        LM_CK(ctx, cudaStreamSynchronize(e.stream));
+        if (e.st_host->err || e.st_host->done) return check_err(ctx, e);
+    }
+}
+
+// One graph by the list path (see lm_list.cu).  rounds: the round count is wanted
+// (64-bit words); counts: the live edges and vertices of every round too.
+static int match_list(lm_ctx* ctx, Engine& e, const lm_graph* g, uint64_t seed, uint32_t* mate, bool dev_out,
+                      Prof& prof, bool async, bool rounds, bool counts) {
+    cudaStream_t s = e.stream;
+    const uint32_t nparts = list_parts(ctx, g->nrows, g->nrows);
+    int rc = ensure_list(ctx, e, g->n, g->ntask[0], 1, 0, nparts);
+    if (rc) return rc;
+    uint32_t* mate_d = dev_out ? mate : e.lw.mate;
+    static_assert(EDGE_ARGS_OFF + sizeof(EdgeJobArgs) <= LIST_ARGS_OFF &&
+                  LIST_ARGS_OFF + sizeof(ListJobArgs) <= ARG_AREA, "argument area too small");
+    ListJobArgs& J = *reinterpret_cast<ListJobArgs*>(e.hargs + LIST_ARGS_OFF);
+    ListJobArgs* D = reinterpret_cast<ListJobArgs*>(e.dargs + LIST_ARGS_OFF);
+    list_args(J.a, e);
+    J.a.segs = &D->seg;
+    J.a.nsegs = 1;
+    J.a.nparts = nparts;
+    job_limits(ctx, g->m, &J.a.max_rounds, &J.a.limit_ns);
+    if (ctx->lim_rounds) rounds = true;   // a cap on the rounds: they have to be known
+    J.seg = list_seg(g, seed, mate_d);
+    J.seg.nparts = nparts;
+    LM_CK(ctx, cudaMemcpyAsync(D, &J, sizeof J, cudaMemcpyHostToDevice, s));
+    if (async) {
+        // the next job may rewrite the staging only after this upload ran
+        if (!e.staged) LM_CK(ctx, cudaEventCreateWithFlags(&e.staged, cudaEventDisableTiming));
+        LM_CK(ctx, cudaEventRecord(e.staged, s));
+        e.staged_pending = true;
+    }
+    prof.begin(LM_K_CAND);
+    LM_CK(ctx, launch_top(s, &D->a, J.seg.nblk, rounds));
+    prof.end();
+    if (async) {  // queued; lm_sync reports device errors
+        void*& graph = e.lgraph[rounds ? 1 : 0];
+        if (!graph) LM_CK(ctx, build_list_graph(&D->a, rounds, &graph));
+        LM_CK(ctx, launch_job_graph(graph, s));
+        return LM_OK;
+    }
+    rc = run_live(ctx, e, &D->a, nparts, rounds, prof);
+    if (rc) return rc;
+    if (counts) {
+        prof.begin(LM_K_OTHER);
+        LM_CK(ctx, launch_round_counts(s, &D->a, e.lw.queue[0]));
+        prof.end();
+        LM_CK(ctx, cudaMemcpyAsync(e.st_host, e.st, sizeof(DevState), cudaMemcpyDeviceToHost, s));
+    }
+    if (!dev_out) LM_CK(ctx, cudaMemcpyAsync(mate, mate_d, (size_t)g->n * 4, cudaMemcpyDeviceToHost, s));
+    if (counts || !dev_out) LM_CK(ctx, cudaStreamSynchronize(s));
+    if (counts)  // counted by their last live round -> live at the start of round r
+        for (int r = LM_STATS_ROUNDS - 2; r >= 0; r--) {
+            e.st_host->ring_m[r] += e.st_host->ring_m[r + 1];
+            e.st_host->ring_n[r] += e.st_host->ring_n[r + 1];
+        }
+    return LM_OK;
+}
+
 // One graph on engine e, results to mate (device memory when dev_out, else host
 // memory staged through the workspace); the engine's DevState holds its statistics.
 int match_one(lm_ctx* ctx, Engine& e, const lm_graph* g, uint64_t seed, uint32_t* mate, bool dev_out, Prof& prof,
-              bool async) {
+              bool async, bool rounds, bool counts) {
     cudaStream_t s = e.stream;
     int rc = staging_ready(ctx, e);
     if (rc) return rc;
+    if (g->nent && list_path(e, g))
+        return match_list(ctx, e, g, seed, mate, dev_out, prof, async && dev_out && !prof.on, rounds, counts);
     rc = ensure_ws(ctx, e, g->n, g->nent, 1);
     if (rc) return rc;
     rc = ensure_pinned(ctx, e, sizeof(SegIn));
@@ -611,7 +780,86 @@ int match_one(lm_ctx* ctx, Engine& e, const lm_graph* g, uint64_t seed, uint32_t
 // served requests): their vertex and entry ranges are laid side by side in one
 // union id space, each graph keeping its own seed and edge ids.  mates[i] is
 // device or host memory; rounds[i] and matched2[i] receive graph i's round count
-// and matched vertices.
+// and matched vertices (either may be NULL).
+static int batch_list(lm_ctx* ctx, Engine& e, const lm_graph* const* gs, uint32_t count, const uint64_t* seeds,
+                      uint32_t* const* mates, uint32_t* rounds, unsigned long long* matched2, Prof& prof) {
+    cudaStream_t s = e.stream;
+    size_t nv = 0, nc = 0, nb = 0, np = 0;
+    uint64_t ne = 0, nr = 0;
+    for (uint32_t i = 0; i < count; i++) nr += gs[i]->nrows;
+    for (uint32_t i = 0; i < count; i++) {
+        nv += gs[i]->n;
+        ne += gs[i]->nent;
+        nc += gs[i]->ntask[0];
+        nb += list_blocks(gs[i]->ntask, gs[i]->nrows);
+        np += list_parts(ctx, gs[i]->nrows, nr);
+    }
+    const bool want = rounds || ctx->lim_rounds;
+    int rc = staging_ready(ctx, e);
+    if (!rc) rc = ensure_list(ctx, e, nv, nc, count, nb, np);
+    if (!rc) rc = ensure_pinned(ctx, e, count * sizeof(ListSeg));
+    if (rc) return rc;
+    ListWs& w = e.lw;
+    ListSeg* segs = static_cast<ListSeg*>(e.pinned);
+    std::vector<char> host_dst(count);
+    bool any_host = false;
+    uint32_t vb = 0, cb = 0, bb = 0, pb = 0;
+    for (uint32_t i = 0; i < count; i++) {
+        host_dst[i] = !is_device_ptr(mates[i]);
+        any_host |= host_dst[i] != 0;
+        ListSeg& sg = segs[i];
+        sg = list_seg(gs[i], seeds[i], host_dst[i] ? w.mate + vb : mates[i]);
+        sg.vbase = vb;
+        sg.lbase = cb;
+        sg.blk0 = bb;
+        sg.part0 = pb;
+        sg.nparts = list_parts(ctx, gs[i]->nrows, nr);
+        vb += gs[i]->n;
+        cb += gs[i]->ntask[0];
+        bb += sg.nblk;
+        pb += sg.nparts;
+    }
+    ListArgs& A = reinterpret_cast<ListJobArgs*>(e.hargs + LIST_ARGS_OFF)->a;
+    ListArgs* D = &reinterpret_cast<ListJobArgs*>(e.dargs + LIST_ARGS_OFF)->a;
+    list_args(A, e);
+    A.segs = w.segs;
+    A.nsegs = count;
+    A.nparts = pb;
+    A.bmap = w.bmap;
+    A.pmap = w.pmap;
+    A.grounds = w.grounds;
+    A.gmatched = w.gmatched;
+    job_limits(ctx, (uint32_t)(ne / 2), &A.max_rounds, &A.limit_ns);
+    LM_CK(ctx, cudaMemcpyAsync(w.segs, segs, count * sizeof(ListSeg), cudaMemcpyHostToDevice, s));
+    LM_CK(ctx, cudaMemcpyAsync(D, &A, sizeof A, cudaMemcpyHostToDevice, s));
+    LM_CK(ctx, cudaMemsetAsync(w.gmatched, 0, count * sizeof(unsigned long long), s));
+    LM_CK(ctx, cudaMemsetAsync(w.grounds, 0, count * sizeof(uint32_t), s));
+    prof.begin(LM_K_OTHER);
+    LM_CK(ctx, launch_list_map(s, D, count, w.bmap, w.pmap));
+    prof.end();
+    prof.begin(LM_K_CAND);
+    LM_CK(ctx, launch_top(s, D, bb, want));
+    prof.end();
+    if (pb) {
+        rc = run_live(ctx, e, D, pb, want, prof);
+        if (rc) return rc;
+    }
+    std::vector<uint32_t> hmate;
+    if (any_host) {
+        hmate.resize(nv);
+        LM_CK(ctx, cudaMemcpyAsync(hmate.data(), w.mate, nv * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+    }
+    if (rounds) LM_CK(ctx, cudaMemcpyAsync(rounds, w.grounds, count * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+    if (matched2)
+        LM_CK(ctx, cudaMemcpyAsync(matched2, w.gmatched, count * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
+    if (any_host || rounds || matched2 || !pb) LM_CK(ctx, cudaStreamSynchronize(s));
+    if (any_host)
+        for (uint32_t i = 0; i < count; i++)
+            if (host_dst[i] && gs[i]->n)
+                memcpy(mates[i], hmate.data() + segs[i].vbase, (size_t)gs[i]->n * sizeof(uint32_t));
+    return LM_OK;
+}
+
 int match_batch(lm_ctx* ctx, Engine& e, const lm_graph* const* gs, uint32_t count, const uint64_t* seeds,
                 uint32_t* const* mates, uint32_t* rounds, unsigned long long* matched2, Prof& prof) {
     uint64_t nv = 0, ne = 0;
@@ -620,6 +868,9 @@ int match_batch(lm_ctx* ctx, Engine& e, const lm_graph* const* gs, uint32_t coun
         ne += gs[i]->nent;
     }
     if (nv > 0xFFFFFFF0ull || ne > 0xFFFFFFF0ull) return fail(ctx, LM_EINVAL, "batch too large for 32-bit union ids");
+    bool listed = true;
+    for (uint32_t i = 0; i < count; i++) listed = listed && list_path(e, gs[i]);
+    if (listed) return batch_list(ctx, e, gs, count, seeds, mates, rounds, matched2, prof);
     cudaStream_t s = e.stream;
     int rc = ensure_ws(ctx, e, (uint32_t)nv, (uint32_t)ne, count);
     if (rc) return rc;
@@ -689,8 +940,9 @@ int match_batch(lm_ctx* ctx, Engine& e, const lm_graph* const* gs, uint32_t coun
         hmate.resize(nv);
         LM_CK(ctx, cudaMemcpyAsync(hmate.data(), w.cnbr, nv * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
     }
-    LM_CK(ctx, cudaMemcpyAsync(rounds, w.grounds, count * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-    LM_CK(ctx, cudaMemcpyAsync(matched2, w.gmatched, count * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
+    if (rounds) LM_CK(ctx, cudaMemcpyAsync(rounds, w.grounds, count * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+    if (matched2)
+        LM_CK(ctx, cudaMemcpyAsync(matched2, w.gmatched, count * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
     LM_CK(ctx, cudaStreamSynchronize(s));
     if (any_host)
         for (uint32_t i = 0; i < count; i++)
@@ -846,7 +1098,7 @@ int lm_graph_create(lm_ctx* ctx, uint32_t n, uint32_t m, const uint32_t* eu, con
     tc.add(&flags, nn);
     tc.add(&rowidx, nn);
     tc.add(&scan_tmp, scan_words);
-    tc.add(&err, 4);
+    tc.add(&err, 12);  // error bits, -, -, -, tasks of each kind (4), their cursors (4)
     if (m > 0) tc.add(&fill_tmp, build_fill_tmp_words(n, m));
     void* tmp = nullptr;
     cudaError_t ce = fault_alloc(ctx) ? cudaErrorMemoryAllocation : cudaMallocFromPoolAsync(&tmp, tc.total, ctx->pool, s);
@@ -858,7 +1110,7 @@ int lm_graph_create(lm_ctx* ctx, uint32_t n, uint32_t m, const uint32_t* eu, con
         ~TmpFree() { if (p) cudaFreeAsync(p, s); }
     } tf{tmp, s};
     LM_CK(ctx, cudaMemsetAsync(deg, 0, nn * 4, s));
-    LM_CK(ctx, cudaMemsetAsync(err, 0, 16, s));
+    LM_CK(ctx, cudaMemsetAsync(err, 0, 48, s));
     // validation rides on the degree count: endpoint < n, no self loop, no NaN
     if (mem == LM_HOST && m > 0) {
         // chunks of the host arrays go up on the upload stream; the context's stream
@@ -886,16 +1138,17 @@ int lm_graph_create(lm_ctx* ctx, uint32_t n, uint32_t m, const uint32_t* eu, con
     } else if (m > 0) {
         LM_CK(ctx, launch_build_degrees(s, d_eu, d_ev, d_w, n, m, deg, err));
     }
-    int rc = ensure_pinned(ctx, e, 64);
+    int rc = ensure_pinned(ctx, e, 64);  // 16 words
     if (rc) return rc;
     uint32_t* hp = static_cast<uint32_t*>(e.pinned);
-    LM_CK(ctx, cudaMemcpyAsync(&hp[1], err, 4, cudaMemcpyDeviceToHost, s));
-    LM_CK(ctx, launch_nonzero_flags(s, deg, n + 1, flags));
+    LM_CK(ctx, launch_nonzero_flags(s, deg, n + 1, flags, err + 4));
+    LM_CK(ctx, cudaMemcpyAsync(&hp[4], err, 32, cudaMemcpyDeviceToHost, s));
     LM_CK(ctx, launch_exclusive_scan(s, flags, rowidx, n + 1, scan_tmp, scan_words));
     LM_CK(ctx, cudaMemcpyAsync(&hp[0], rowidx + n, 4, cudaMemcpyDeviceToHost, s));
     LM_CK(ctx, cudaStreamSynchronize(s));
-    if (hp[1]) return fail(ctx, LM_EINVAL, "edge list: endpoint >= n, self loop or NaN weight");
+    if (hp[4]) return fail(ctx, LM_EINVAL, "edge list: endpoint >= n, self loop or NaN weight");
     g->nrows = hp[0];
+    for (int k = 0; k < 4; k++) g->ntask[k] = hp[8 + k] + (k ? g->ntask[k - 1] : 0u);
 
     Carver gc;
     gc.add(&g->off, nn);
@@ -907,6 +1160,7 @@ int lm_graph_create(lm_ctx* ctx, uint32_t n, uint32_t m, const uint32_t* eu, con
     gc.add(&g->tmap, (size_t)g->ntiles + 1);
     gc.add(&g->rbits, (size_t)g->ntiles * (TILE0 / 32) + 8);
     gc.add(&g->tdesc, (size_t)g->ntiles + 1);
+    gc.add(&g->task, g->ntask[3]);
     gc.add(&g->nbr, (size_t)g->nent + 4);
     gc.add(&g->pk, (size_t)g->nent + 4);
     gc.add(&g->edges, (size_t)g->m + 2);
@@ -928,7 +1182,12 @@ int lm_graph_create(lm_ctx* ctx, uint32_t n, uint32_t m, const uint32_t* eu, con
                                      scan_tmp, scan_words, err));
         LM_CK(ctx, cudaMemcpyAsync(&hp[2], err, 4, cudaMemcpyDeviceToHost, s));
     }
-    LM_CK(ctx, launch_build_rows(s, deg, rowidx, g->off, n, g->nrows, g->nent, g->vid, g->rdeg, g->roff));
+    // each kind's tasks follow the previous one's
+    hp[12] = 0;
+    for (int k = 1; k < 4; k++) hp[12 + k] = g->ntask[k - 1];
+    LM_CK(ctx, cudaMemcpyAsync(err + 8, &hp[12], 16, cudaMemcpyHostToDevice, s));
+    LM_CK(ctx, launch_build_rows(s, deg, rowidx, g->off, n, g->nrows, g->nent, g->vid, g->rdeg, g->roff, g->task,
+                                 g->ntask[3], err + 8));
     if (g->nrows) {
         LM_CK(ctx, cudaMemsetAsync(g->rbits, 0, ((size_t)g->ntiles * (TILE0 / 32) + 8) * 4, s));
         LM_CK(ctx, launch_build_tilemap(s, g->roff, g->nrows, g->nent, g->tmap, g->rbits, g->tdesc));
@@ -973,7 +1232,8 @@ int lm_match(lm_ctx* ctx, const lm_graph* g, uint64_t seed, uint32_t* mate, lm_s
     if (async && (!dev_out || stats))
         return fail(ctx, LM_EINVAL, "an asynchronous match writes device memory and returns no statistics");
     const int rc = (ctx->flags & LM_F_EDGE_CENTRIC) ? match_edges(ctx, ctx->eng, g, seed, mate, dev_out, prof)
-                                                    : match_one(ctx, ctx->eng, g, seed, mate, dev_out, prof, async);
+                                                    : match_one(ctx, ctx->eng, g, seed, mate, dev_out, prof, async,
+                                                                stats != nullptr, stats != nullptr);
     if (rc) return rc;
     if (stats) {
         fill_round_stats(*ctx->eng.st_host, stats);
@@ -1111,9 +1371,10 @@ int lm_batch_match(lm_ctx* ctx, const lm_graph* const* gs, uint32_t count, const
     if (!dg.ok) return fail(ctx, LM_ECUDA, "cudaSetDevice failed");
     if (stats) memset(stats, 0, sizeof(lm_stats) * count);
     Prof prof(ctx, ctx->eng.stream);
-    std::vector<uint32_t> grounds(count);
-    std::vector<unsigned long long> gm(count);
-    const int rc = match_batch(ctx, ctx->eng, gs, count, seeds, mates, grounds.data(), gm.data(), prof);
+    std::vector<uint32_t> grounds(stats ? count : 0);
+    std::vector<unsigned long long> gm(stats ? count : 0);
+    const int rc = match_batch(ctx, ctx->eng, gs, count, seeds, mates, stats ? grounds.data() : nullptr,
+                               stats ? gm.data() : nullptr, prof);
     if (rc) return rc;
     if (stats) {
         // per graph: rounds, |M|, initial sizes; per call (copied into every entry): launches and timings

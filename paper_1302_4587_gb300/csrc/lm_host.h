@@ -48,6 +48,25 @@ struct Workspace {
     unsigned long long* gmatched = nullptr;  // [cap_g] matched vertices per graph
 };
 
+// Scratch arrays of the list path (one allocation, carved).
+struct ListWs {
+    void* block = nullptr;
+    size_t cap_v = 0, cap_c = 0, cap_g = 0, cap_b = 0, cap_p = 0;
+    uint64_t* cur = nullptr;                      // [cap_v] words (see ListArgs)
+    uint4* lst = nullptr;                         // [cap_v]
+    uint32_t* list[2] = {nullptr, nullptr};       // [cap_v]
+    uint32_t* queue[3] = {nullptr, nullptr, nullptr};  // [cap_v]
+    uint32_t* mate = nullptr;                     // [cap_v] staging of results for the host
+    uint4* part = nullptr;                        // [4 cap_c]
+    uint32_t* pcnt = nullptr;                     // [cap_c]
+    ListSeg* segs = nullptr;                      // [cap_g]
+    uint32_t* bmap = nullptr;                     // [cap_b]
+    uint32_t* pmap = nullptr;                     // [cap_p]
+    uint32_t* pcount = nullptr;                   // [cap_p]
+    uint32_t* grounds = nullptr;                  // [cap_g]
+    unsigned long long* gmatched = nullptr;       // [cap_g]
+};
+
 // Device state + workspace + the stream they are used on.
 constexpr size_t ARG_AREA = 1 << 16;  // bytes of kernel arguments uploaded per call / step
 struct Engine {
@@ -68,6 +87,8 @@ struct Engine {
     LaunchCfg cfg;                   // launch parameters of the next jobs
     LaunchCfg graph_cfg;             // the ones `graph` was built with
     Workspace ws;
+    ListWs lw;
+    void* lgraph[2] = {nullptr, nullptr};  // executable graphs of the list path's live pass (32, 64-bit words)
     int sweep_grid = 0, vertex_grid = 0;
 };
 
@@ -125,6 +146,8 @@ struct lm_graph {
     uint64_t* pk = nullptr;          // [2m] ord(weight) << 32 | edge index, per entry
     uint64_t* edges = nullptr;       // [m] edge records eu | ev << 32
     uint32_t* eword = nullptr;       // [m] ord(weight) of each edge (edge-centric path)
+    uint4* task = nullptr;           // [ntask] long rows of the list path (see ListSeg)
+    uint32_t ntask[4] = {0, 0, 0, 0};  // ends of its kinds
 };
 
 namespace lm {
@@ -185,7 +208,7 @@ int run_job(lm_ctx* ctx, Engine& e, Job& job, Prof& prof);
 int match_batch(lm_ctx* ctx, Engine& e, const lm_graph* const* gs, uint32_t count, const uint64_t* seeds,
                 uint32_t* const* mates, uint32_t* rounds, unsigned long long* matched2, Prof& prof);
 int match_one(lm_ctx* ctx, Engine& e, const lm_graph* g, uint64_t seed, uint32_t* mate, bool dev_out, Prof& prof,
-              bool async = false);
+              bool async = false, bool rounds = true, bool counts = false);
 // the pinned staging (arguments, tables) is free again: the copies a queued
 // (asynchronous) job made from it have run
 int staging_ready(lm_ctx* ctx, Engine& e);

@@ -97,6 +97,8 @@ struct DevState {
     unsigned long long last_ent;   // live entries the last vertex pass saw (its round's)
     uint32_t tail;            // 1: the remaining rounds run in the one-CTA tail kernel
     uint32_t tail_round;      // the round the tail kernel took over at
+    uint32_t left;            // list path: live rows the running launch has given back
+    uint32_t pad_;
     uint64_t ring_m[64];      // live edges at the start of round r
     uint64_t ring_n[64];      // live vertices at the start of round r
 };
@@ -247,6 +249,52 @@ struct EdgeArgs {
     DevState* st;
 };
 
+// ---------------------------------------------------------------- list path (lm_list.cu)
+// rows of at most LIST_SHORT entries take a thread each, up to LIST_GROUP eight lanes,
+// up to LIST_WARP a warp with eight entries a lane, longer ones a warp's loop; rows of
+// more than LIST_CHUNK entries are cut into chunks of that many, a warp each
+constexpr uint32_t LIST_SHORT = 16, LIST_GROUP = 64, LIST_WARP = 256, LIST_CHUNK = 2048;
+constexpr uint32_t LIST_PART_MIN = 256, LIST_PART_MAX = 8192;  // rows a block of the live pass takes at a time
+
+// One graph of a list-path job (local vertex ids throughout).
+struct ListSeg {
+    const uint64_t* pk;       // [2m] ord(weight) << 32 | edge index, per adjacency entry
+    const uint32_t* nbr;      // [2m] neighbour of each entry
+    const uint32_t* off;      // [n + 1] row offsets of all vertices
+    const uint32_t* vid;      // [nrows] vertices with edges
+    const uint32_t* roff;     // [nrows + 1] their row offsets
+    const uint4* task;        // rows of more than LIST_SHORT entries: vertex, row offset, length, chunk
+    const uint64_t* edges;    // [m] edge records
+    uint32_t* dst;            // [n] result
+    uint32_t n, m, nrows;
+    uint32_t ntask[4];        // ends of the kinds of task: chunks of rows longer than LIST_CHUNK (a row's
+                              // are consecutive), rows of more than LIST_WARP, than LIST_GROUP, than LIST_SHORT
+    uint32_t vbase;           // first slot of the graph's vertices in the job's arrays
+    uint32_t lbase;           // first slot of its chunks in part / pcnt
+    uint32_t blk0, nblk;      // its blocks of k_top
+    uint32_t part0, nparts;   // its parts
+    uint32_t k0, k1;          // perm_seed keys of its seed
+};
+// Arguments of a list-path job in device memory.
+struct ListArgs {
+    const ListSeg* segs;
+    uint32_t nsegs, nparts;   // graphs, parts of all graphs
+    const uint32_t* bmap;     // [blocks of k_top] graph of each block (NULL: one graph)
+    const uint32_t* pmap;     // [nparts] graph of each part (NULL: one graph)
+    void* cur;                // [vertices] word of every vertex, 32 or 64 bits (rounds wanted)
+    uint4* lst;               // the next three neighbours of each row's list, and whether its row holds more
+    uint32_t* list[2];        // live rows, each part's in its own range
+    uint32_t* queue[3];       // rows to refill, likewise: short, long, the block's
+    uint32_t* pcount;         // [nparts] live rows a part was given back with, times two, plus their buffer
+    uint4* part;              // [4 per chunk] a chunk's four heaviest: key low, key high, neighbour
+    uint32_t* pcnt;           // chunks done per long row, at its first chunk's slot (zero between jobs)
+    uint32_t* grounds;        // [nsegs] rounds per graph (NULL: one graph, DevState::rounds)
+    unsigned long long* gmatched;  // [nsegs] matched vertices per graph (NULL: DevState::matched2)
+    uint32_t max_rounds;
+    unsigned long long limit_ns;
+    DevState* st;
+};
+
 constexpr unsigned long long LOOP_LIMIT_NS = 120000000000ull;  // 120 s: the default time limit of a job
 // once a round starts with fewer live entries than this, the rounds that remain
 // run in one kernel of one CTA (no launch per round)
@@ -309,6 +357,14 @@ size_t contract_sort_words(uint32_t m);  // words of shist
 // are read back once, to size the sort); returns a cudaError_t value
 int launch_contract(void* stream, const ContractArgs& c, uint32_t* mc_host_slot);
 int launch_job_graph(void* exec, void* stream);
+// list path (lm_list.cu): blocks of k_top for one graph, the maps for several, and the launches
+// (rounds: 64-bit words)
+uint32_t list_blocks(const uint32_t task[4], uint32_t nrows);
+int launch_list_map(void* stream, const ListArgs* d, uint32_t nsegs, uint32_t* bmap, uint32_t* pmap);
+int launch_top(void* stream, const ListArgs* d, uint32_t blocks, bool rounds);
+int launch_live(void* stream, const ListArgs* d, uint32_t nparts, bool rounds);
+int launch_round_counts(void* stream, const ListArgs* d, void* bytes);  // bytes: one a vertex, scratch
+int build_list_graph(const ListArgs* d, bool rounds, void** exec_out);
 // edge-centric path: the job graph (init, then a conditional loop of rounds) and the
 // per-round launches of the profiled path
 int build_edge_graph(const InitArgs* init, const EdgeArgs* dargs, DevState* st, void** exec_out);
@@ -328,11 +384,14 @@ uint32_t build_fill_scan_count(uint32_t n, uint32_t m);
 int launch_build_fill(void* stream, const uint32_t* eu, const uint32_t* ev, const float* w, uint32_t n, uint32_t m,
                       uint32_t* cursor, uint32_t* nbr, uint64_t* pk, uint64_t* edges, uint32_t* eword, uint32_t* tmp,
                       uint32_t* scan_tmp, size_t scan_words, uint32_t* err);  // err |= 2 when a fill slot falls outside 2m
+// cursors: the next place in task of each kind
 int launch_build_rows(void* stream, const uint32_t* deg, const uint32_t* rowidx_excl, const uint32_t* off,
-                      uint32_t n, uint32_t nrows, uint32_t nent, uint32_t* vid0, uint32_t* rdeg0, uint32_t* roff);
+                      uint32_t n, uint32_t nrows, uint32_t nent, uint32_t* vid0, uint32_t* rdeg0, uint32_t* roff,
+                      uint4* task, uint32_t ntask, uint32_t* cursors);
 int launch_build_tilemap(void* stream, const uint32_t* roff, uint32_t nrows, uint32_t nent, uint32_t* tmap,
                          uint32_t* rbits, uint4* tdesc);
-int launch_nonzero_flags(void* stream, const uint32_t* deg, uint32_t n, uint32_t* flags);
+// flags[v] = deg[v] != 0; counts[0 .. 3] += the tasks of each kind (see ListSeg::ntask)
+int launch_nonzero_flags(void* stream, const uint32_t* deg, uint32_t n, uint32_t* flags, uint32_t* counts);
 // union set-up of a batch: for every graph g (vertices [gvbase[g], gvbase[g+1])):
 // start[v] = ebase[g] + off_g[v - gvbase[g]], gid[v] = g, len0[v] = degree
 int launch_union_setup(void* stream, const uint32_t* gvbase, const uint32_t* ebase, const uint32_t* const* offs,

@@ -30,77 +30,11 @@
 #include <mutex>
 
 #include "../../include/lm.h"
+#include "lm_device.cuh"
 #include "lm_internal.h"
 
 namespace lm {
 
-#define FULL 0xFFFFFFFFu
-
-// ---------------------------------------------------------------- order
-// MurmurHash3 32-bit finaliser (Appleby, public domain).
-__device__ __forceinline__ uint32_t fmix32(uint32_t h) {
-    h ^= h >> 16;
-    h *= 0x85EBCA6Bu;
-    h ^= h >> 13;
-    h *= 0xC2B2AE35u;
-    h ^= h >> 16;
-    return h;
-}
-__device__ __forceinline__ uint32_t perm_seed(uint32_t e, uint32_t k0, uint32_t k1) {
-    return fmix32(fmix32(e ^ k0) ^ k1);
-}
-// inverse of x -> x * a (mod 2^32) for odd a, by Newton's iteration
-__host__ __device__ constexpr uint32_t inv_mul(uint32_t a) {
-    uint32_t x = a;  // correct to 3 bits for odd a
-    x *= 2u - a * x;
-    x *= 2u - a * x;
-    x *= 2u - a * x;
-    x *= 2u - a * x;
-    x *= 2u - a * x;
-    return x;
-}
-constexpr uint32_t INV_M1 = inv_mul(0x85EBCA6Bu), INV_M2 = inv_mul(0xC2B2AE35u);
-static_assert(0x85EBCA6Bu * INV_M1 == 1u && 0xC2B2AE35u * INV_M2 == 1u, "modular inverses");
-__device__ __forceinline__ uint32_t fmix32_inv(uint32_t h) {
-    h ^= h >> 16;                       // h ^ (h >> 16) is its own inverse on 32 bits
-    h *= INV_M2;
-    h ^= (h >> 13) ^ (h >> 26);         // inverse of h ^= h >> 13
-    h *= INV_M1;
-    h ^= h >> 16;
-    return h;
-}
-// e = perm_seed^-1(x)
-__device__ __forceinline__ uint32_t perm_seed_inv(uint32_t x, uint32_t k0, uint32_t k1) {
-    return fmix32_inv(fmix32_inv(x) ^ k1) ^ k0;
-}
-// monotone float32 -> uint32 (-0 == +0); NaN is rejected before this runs
-__device__ __forceinline__ uint32_t ord_of_bits(uint32_t b) {
-    if (b == 0x80000000u) b = 0u;
-    return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
-
-// ---------------------------------------------------------------- utilities
-__device__ __forceinline__ uint32_t ld_volatile_u32(const uint32_t* p) {
-    return *reinterpret_cast<const volatile uint32_t*>(p);
-}
-__device__ __forceinline__ uint32_t lanemask_lt() {
-    uint32_t m;
-    asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
-    return m;
-}
-__device__ __forceinline__ uint32_t lanemask_le() {
-    uint32_t m;
-    asm("mov.u32 %0, %%lanemask_le;" : "=r"(m));
-    return m;
-}
-__device__ __forceinline__ uint32_t warp_incl_scan(uint32_t x, int lane) {
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(FULL, x, o);
-        if (lane >= o) x += y;
-    }
-    return x;
-}
 // matched bit of vertex u; the bitmap is read-only during a sweep, so it may go
 // through the non-coherent (read-only) cache
 // matched bit of u.  Between kernels the read-only cache path is safe; inside the
@@ -108,16 +42,6 @@ __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t x, int lane) {
 template <bool COH = false>
 __device__ __forceinline__ bool is_dead(const VertexArrays& va, uint32_t u) {
     return ((COH ? __ldcg(&va.dead[u >> 5]) : __ldg(&va.dead[u >> 5])) >> (u & 31)) & 1u;
-}
-// device-scope fetch-and-add with acquire-release ordering
-__device__ __forceinline__ uint32_t atom_add_acq_rel(uint32_t* p, uint32_t v) {
-    uint32_t old;
-    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
-    return old;
-}
-__device__ __forceinline__ void set_err(DevState* st, uint32_t bit, uint32_t info) {
-    if ((atomicOr(&st->err, bit) & bit) == 0) st->err_info = info;
-    atomicOr(&st->err_any, bit);  // not reset by the next job's init (asynchronous matches)
 }
 // warp-wide maximum of (key, neighbour); keys are unique among live entries of a row
 __device__ __forceinline__ void warp_kv_max(uint64_t& k, uint32_t& u) {
@@ -130,12 +54,6 @@ __device__ __forceinline__ void warp_kv_max(uint64_t& k, uint32_t& u) {
 }
 
 // ---------------------------------------------------------------- init
-__device__ __forceinline__ uint64_t globaltimer_ns() {
-    uint64_t t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
 __global__ void k_init(const InitArgs* __restrict__ pa) {
     const InitArgs& A = *pa;
     uint32_t* mate = A.mate;
@@ -1582,21 +1500,64 @@ __global__ void __launch_bounds__(BF_T) k_build_fill_v(const uint4* vrec, uint32
         }
     }
 }
-__global__ void k_nonzero_flags(const uint32_t* deg, uint32_t n, uint32_t* flags) {
-    const uint32_t stride = gridDim.x * blockDim.x;
-    for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) flags[v] = deg[v] ? 1u : 0u;
+// kind of task a row of d entries makes on the list path (4: none)
+__device__ __forceinline__ uint32_t task_kind(uint32_t d) {
+    return d > LIST_CHUNK ? 0u : d > LIST_WARP ? 1u : d > LIST_GROUP ? 2u : d > LIST_SHORT ? 3u : 4u;
+}
+__global__ void k_nonzero_flags(const uint32_t* deg, uint32_t n, uint32_t* flags, uint32_t* counts) {
+    __shared__ uint32_t s[4];
+    if (threadIdx.x < 4) s[threadIdx.x] = 0;
+    __syncthreads();
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    uint32_t c[4] = {0, 0, 0, 0};
+    for (uint64_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
+        const uint32_t d = deg[v], k = task_kind(d);
+        flags[v] = d ? 1u : 0u;
+#pragma unroll
+        for (uint32_t q = 0; q < 4; q++)
+            if (k == q) c[q] += q == 0 ? (d - 1) / LIST_CHUNK + 1 : 1u;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+        const uint32_t x = __reduce_add_sync(FULL, c[q]);
+        if ((threadIdx.x & 31) == 0 && x) atomicAdd(&s[q], x);
+    }
+    __syncthreads();
+    if (threadIdx.x < 4 && s[threadIdx.x]) atomicAdd(&counts[threadIdx.x], s[threadIdx.x]);
 }
 
-__global__ void k_build_rows(const uint32_t* deg, const uint32_t* rowidx, const uint32_t* off, uint32_t n,
-                             uint32_t nrows, uint32_t nent, uint32_t* vid0, uint32_t* rdeg0, uint32_t* roff) {
-    const uint32_t stride = gridDim.x * blockDim.x;
-    for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
-        if (deg[v]) {
+// The compact row arrays, and the list path's tasks, each kind from its cursor on; a
+// block reserves its 256 vertices' places with one atomic per kind.
+__global__ void __launch_bounds__(256) k_build_rows(const uint32_t* deg, const uint32_t* rowidx, const uint32_t* off,
+                                                    uint32_t n, uint32_t nrows, uint32_t nent, uint32_t* vid0,
+                                                    uint32_t* rdeg0, uint32_t* roff, uint4* task, uint32_t ntask,
+                                                    uint32_t* cursors) {
+    __shared__ uint32_t s[4], base[4];
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t b = (uint64_t)blockIdx.x * blockDim.x; b < n; b += stride) {
+        const uint64_t v = b + threadIdx.x;
+        const uint32_t d = v < n ? deg[v] : 0u, k = task_kind(d);
+        uint32_t o = 0;
+        if (d) {
             const uint32_t i = rowidx[v];
-            vid0[i] = v;
-            rdeg0[i] = deg[v];
-            roff[i] = off[v];
+            o = off[v];
+            vid0[i] = (uint32_t)v;
+            rdeg0[i] = d;
+            roff[i] = o;
         }
+        if (!__syncthreads_or(k < 4)) continue;
+        if (threadIdx.x < 4) s[threadIdx.x] = 0;
+        __syncthreads();
+        const uint32_t nt = k == 0 ? (d - 1) / LIST_CHUNK + 1 : 1u;
+        uint32_t at = 0;
+        if (k < 4) at = atomicAdd(&s[k], nt);
+        __syncthreads();
+        if (threadIdx.x < 4 && s[threadIdx.x]) base[threadIdx.x] = atomicAdd(&cursors[threadIdx.x], s[threadIdx.x]);
+        __syncthreads();
+        if (k < 4)
+            for (uint32_t c = 0; c < nt; c++)
+                if (base[k] + at + c < ntask) task[base[k] + at + c] = make_uint4((uint32_t)v, o, d, c);
+        __syncthreads();  // s / base reuse
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) roff[nrows] = nent;
 }
@@ -1967,14 +1928,15 @@ int launch_build_fill(void* stream, const uint32_t* eu, const uint32_t* ev, cons
     k_build_fill_v<<<grid_for(m, 256), BF_T, 0, s>>>(vrec, m, cursor, nbr, pk, err);
     return (int)cudaGetLastError();
 }
-int launch_nonzero_flags(void* stream, const uint32_t* deg, uint32_t n, uint32_t* flags) {
-    k_nonzero_flags<<<grid_for(n, 256), 256, 0, (cudaStream_t)stream>>>(deg, n, flags);
+int launch_nonzero_flags(void* stream, const uint32_t* deg, uint32_t n, uint32_t* flags, uint32_t* counts) {
+    k_nonzero_flags<<<grid_for(n, 256), 256, 0, (cudaStream_t)stream>>>(deg, n, flags, counts);
     return (int)cudaGetLastError();
 }
 int launch_build_rows(void* stream, const uint32_t* deg, const uint32_t* rowidx_excl, const uint32_t* off,
-                      uint32_t n, uint32_t nrows, uint32_t nent, uint32_t* vid0, uint32_t* rdeg0, uint32_t* roff) {
+                      uint32_t n, uint32_t nrows, uint32_t nent, uint32_t* vid0, uint32_t* rdeg0, uint32_t* roff,
+                      uint4* task, uint32_t ntask, uint32_t* cursors) {
     k_build_rows<<<grid_for(n, 256), 256, 0, (cudaStream_t)stream>>>(deg, rowidx_excl, off, n, nrows, nent, vid0,
-                                                                     rdeg0, roff);
+                                                                     rdeg0, roff, task, ntask, cursors);
     return (int)cudaGetLastError();
 }
 int launch_build_tilemap(void* stream, const uint32_t* roff, uint32_t nrows, uint32_t nent, uint32_t* tmap,
