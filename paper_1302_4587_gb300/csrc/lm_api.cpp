@@ -117,8 +117,8 @@ SegIn seg_of(const lm_graph* g, uint64_t seed, uint32_t vbase, uint32_t ebase, u
     SegIn d;
     memset(&d, 0, sizeof d);
     const uint64_t z = splitmix64_first(seed);
-    d.nbr = g->nbr;
-    d.pk = g->pk;
+    d.ent = g->ent;
+    d.eid = g->eid;
     d.edges = g->edges;
     d.roff = g->roff;
     d.rvid = g->vid;
@@ -588,10 +588,11 @@ static int ensure_list(lm_ctx* ctx, Engine& e, size_t nv, size_t nc, size_t ng, 
     Carver c;
     c.add(&nw.cur, nw.cap_v);
     c.add(&nw.lst, nw.cap_v);
+    c.add(&nw.wide, nw.cap_v);
     for (int k = 0; k < 2; k++) c.add(&nw.list[k], nw.cap_v);
-    for (int k = 0; k < 3; k++) c.add(&nw.queue[k], nw.cap_v);
+    c.add(&nw.queue, nw.cap_v);
     c.add(&nw.mate, nw.cap_v);
-    c.add(&nw.part, 4 * nw.cap_c);
+    c.add(&nw.part, LIST_KEPT * nw.cap_c);
     c.add(&nw.pcnt, nw.cap_c);
     c.add(&nw.segs, nw.cap_g);
     c.add(&nw.bmap, nw.cap_b);
@@ -621,19 +622,21 @@ static int ensure_list(lm_ctx* ctx, Engine& e, size_t nv, size_t nc, size_t ng, 
 // whole job; a renewed order keys every round anew (run_job).
 static bool list_path(const Engine& e, const lm_graph* g) { return !e.cfg.renew && g->n < 0x80000000u; }
 
-// parts of a graph in a job of `total` rows: about four a multiprocessor, within the limits
+// Parts of a graph in a job of `total` rows: one for every block of the live pass that
+// runs at once, within the limits.  A graph's own never exceed those blocks: its rows
+// wait for one another, so its parts have to be in progress together.
 static uint32_t list_parts(const lm_ctx* ctx, uint32_t rows, uint64_t total) {
-    const uint64_t want = total / ((uint64_t)device_sm_count(ctx->device) * 4) + 1;
-    const uint32_t per = (uint32_t)std::min<uint64_t>(LIST_PART_MAX, std::max<uint64_t>(LIST_PART_MIN, want));
-    return (rows + per - 1) / per;
+    const uint32_t blocks = list_live_blocks(ctx->device);
+    const uint32_t per = (uint32_t)std::min<uint64_t>(LIST_PART_MAX, std::max<uint64_t>(LIST_PART_MIN, total / blocks + 1));
+    return std::min(blocks, (rows + per - 1) / per);
 }
 
 static ListSeg list_seg(const lm_graph* g, uint64_t seed, uint32_t* dst) {
     ListSeg d;
     memset(&d, 0, sizeof d);
     const uint64_t z = splitmix64_first(seed);
-    d.pk = g->pk;
-    d.nbr = g->nbr;
+    d.ent = g->ent;
+    d.eid = g->eid;
     d.off = g->off;
     d.vid = g->vid;
     d.roff = g->roff;
@@ -655,8 +658,9 @@ static void list_args(ListArgs& A, Engine& e) {
     const ListWs& w = e.lw;
     A.cur = w.cur;
     for (int k = 0; k < 2; k++) A.list[k] = w.list[k];
-    for (int k = 0; k < 3; k++) A.queue[k] = w.queue[k];
+    A.queue = w.queue;
     A.lst = w.lst;
+    A.wide = w.wide;
     A.pcount = w.pcount;
     A.part = w.part;
     A.pcnt = w.pcnt;
@@ -724,7 +728,7 @@ static int match_list(lm_ctx* ctx, Engine& e, const lm_graph* g, uint64_t seed, 
     if (rc) return rc;
     if (counts) {
         prof.begin(LM_K_OTHER);
-        LM_CK(ctx, launch_round_counts(s, &D->a, e.lw.queue[0]));
+        LM_CK(ctx, launch_round_counts(s, &D->a, e.lw.queue));
         prof.end();
         LM_CK(ctx, cudaMemcpyAsync(e.st_host, e.st, sizeof(DevState), cudaMemcpyDeviceToHost, s));
     }
@@ -1161,8 +1165,8 @@ int lm_graph_create(lm_ctx* ctx, uint32_t n, uint32_t m, const uint32_t* eu, con
     gc.add(&g->rbits, (size_t)g->ntiles * (TILE0 / 32) + 8);
     gc.add(&g->tdesc, (size_t)g->ntiles + 1);
     gc.add(&g->task, g->ntask[3]);
-    gc.add(&g->nbr, (size_t)g->nent + 4);
-    gc.add(&g->pk, (size_t)g->nent + 4);
+    gc.add(&g->eid, (size_t)g->nent + 4);
+    gc.add(&g->ent, (size_t)g->nent + 4);
     gc.add(&g->edges, (size_t)g->m + 2);
     gc.add(&g->eword, (size_t)g->m + 4);
     ce = fault_alloc(ctx) ? cudaErrorMemoryAllocation : cudaMallocFromPoolAsync(&g->block, gc.total, ctx->pool, s);
@@ -1178,7 +1182,7 @@ int lm_graph_create(lm_ctx* ctx, uint32_t n, uint32_t m, const uint32_t* eu, con
     LM_CK(ctx, launch_exclusive_scan(s, deg, g->off, n + 1, scan_tmp, scan_words));
     if (m > 0) {
         LM_CK(ctx, cudaMemcpyAsync(cursor, g->off, nn * 4, cudaMemcpyDeviceToDevice, s));
-        LM_CK(ctx, launch_build_fill(s, d_eu, d_ev, d_w, n, m, cursor, g->nbr, g->pk, g->edges, g->eword, fill_tmp,
+        LM_CK(ctx, launch_build_fill(s, d_eu, d_ev, d_w, n, m, cursor, g->eid, g->ent, g->edges, g->eword, fill_tmp,
                                      scan_tmp, scan_words, err));
         LM_CK(ctx, cudaMemcpyAsync(&hp[2], err, 4, cudaMemcpyDeviceToHost, s));
     }

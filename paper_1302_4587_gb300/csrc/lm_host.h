@@ -53,11 +53,11 @@ struct ListWs {
     void* block = nullptr;
     size_t cap_v = 0, cap_c = 0, cap_g = 0, cap_b = 0, cap_p = 0;
     uint64_t* cur = nullptr;                      // [cap_v] words (see ListArgs)
-    uint4* lst = nullptr;                         // [cap_v]
+    uint4 *lst = nullptr, *wide = nullptr;        // [cap_v]
     uint32_t* list[2] = {nullptr, nullptr};       // [cap_v]
-    uint32_t* queue[3] = {nullptr, nullptr, nullptr};  // [cap_v]
+    uint4* queue = nullptr;                       // [cap_v]
     uint32_t* mate = nullptr;                     // [cap_v] staging of results for the host
-    uint4* part = nullptr;                        // [4 cap_c]
+    uint4* part = nullptr;                        // [LIST_KEPT cap_c]
     uint32_t* pcnt = nullptr;                     // [cap_c]
     ListSeg* segs = nullptr;                      // [cap_g]
     uint32_t* bmap = nullptr;                     // [cap_b]
@@ -142,8 +142,8 @@ struct lm_graph {
     uint32_t* tmap = nullptr;        // [ntiles + 1] row holding entry t * TILE0 (round-0 tiles)
     uint32_t* rbits = nullptr;       // [ntiles * TILE0 / 32 + 8] row-start bit per entry
     uint4* tdesc = nullptr;          // [ntiles] round-0 tile descriptors
-    uint32_t* nbr = nullptr;         // [2m] neighbour of each entry
-    uint64_t* pk = nullptr;          // [2m] ord(weight) << 32 | edge index, per entry
+    uint64_t* ent = nullptr;         // [2m] ord(weight) << 32 | neighbour, per entry
+    uint32_t* eid = nullptr;         // [2m] its edge index
     uint64_t* edges = nullptr;       // [m] edge records eu | ev << 32
     uint32_t* eword = nullptr;       // [m] ord(weight) of each edge (edge-centric path)
     uint4* task = nullptr;           // [ntask] long rows of the list path (see ListSeg)

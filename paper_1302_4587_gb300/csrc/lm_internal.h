@@ -106,8 +106,8 @@ struct DevState {
 // Arrays of one graph: round 0 reads its adjacency entries, every round
 // recovers candidate neighbours from its edge records.
 struct SegIn {
-    const uint32_t* nbr;      // [2m] neighbour (local id) of each entry of the graph's CSR
-    const uint64_t* pk;       // [2m] ord(weight) << 32 | edge index, per entry
+    const uint64_t* ent;      // [2m] ord(weight) << 32 | neighbour (local id), per entry of the graph's CSR
+    const uint32_t* eid;      // [2m] its edge index
     const uint64_t* edges;    // [m] edge records: eu | ev << 32 (local ids)
     const uint32_t* roff;     // [nrows + 1] entry offset of each row (rows = vertices with edges)
     const uint32_t* rvid;     // [nrows] local vertex id of each row
@@ -253,13 +253,20 @@ struct EdgeArgs {
 // rows of at most LIST_SHORT entries take a thread each, up to LIST_GROUP eight lanes,
 // up to LIST_WARP a warp with eight entries a lane, longer ones a warp's loop; rows of
 // more than LIST_CHUNK entries are cut into chunks of that many, a warp each
-constexpr uint32_t LIST_SHORT = 16, LIST_GROUP = 64, LIST_WARP = 256, LIST_CHUNK = 2048;
-constexpr uint32_t LIST_PART_MIN = 256, LIST_PART_MAX = 8192;  // rows a block of the live pass takes at a time
+constexpr uint32_t LIST_SHORT = 32, LIST_GROUP = 64, LIST_WARP = 256, LIST_CHUNK = 2048;
+constexpr uint32_t LIST_KEPT = 8;       // neighbours kept of a long row
+#ifndef LM_PART_MIN
+#define LM_PART_MIN 256
+#endif
+#ifndef LM_PART_MAX
+#define LM_PART_MAX 2048
+#endif
+constexpr uint32_t LIST_PART_MIN = LM_PART_MIN, LIST_PART_MAX = LM_PART_MAX;  // rows a block of the live pass takes at a time
 
 // One graph of a list-path job (local vertex ids throughout).
 struct ListSeg {
-    const uint64_t* pk;       // [2m] ord(weight) << 32 | edge index, per adjacency entry
-    const uint32_t* nbr;      // [2m] neighbour of each entry
+    const uint64_t* ent;      // [2m] ord(weight) << 32 | neighbour, per adjacency entry
+    const uint32_t* eid;      // [2m] its edge index
     const uint32_t* off;      // [n + 1] row offsets of all vertices
     const uint32_t* vid;      // [nrows] vertices with edges
     const uint32_t* roff;     // [nrows + 1] their row offsets
@@ -282,11 +289,11 @@ struct ListArgs {
     const uint32_t* bmap;     // [blocks of k_top] graph of each block (NULL: one graph)
     const uint32_t* pmap;     // [nparts] graph of each part (NULL: one graph)
     void* cur;                // [vertices] word of every vertex, 32 or 64 bits (rounds wanted)
-    uint4* lst;               // the next three neighbours of each row's list, and whether its row holds more
+    uint4 *lst, *wide;        // [vertices] the rest of each row's list, and of a long row's (see lm_list.cu)
     uint32_t* list[2];        // live rows, each part's in its own range
-    uint32_t* queue[3];       // rows to refill, likewise: short, long, the block's
+    uint4* queue;             // rows to refill, likewise: vertex, row offset, length
     uint32_t* pcount;         // [nparts] live rows a part was given back with, times two, plus their buffer
-    uint4* part;              // [4 per chunk] a chunk's four heaviest: key low, key high, neighbour
+    uint4* part;              // [LIST_KEPT per chunk] a chunk's heaviest: key low, key high, neighbour
     uint32_t* pcnt;           // chunks done per long row, at its first chunk's slot (zero between jobs)
     uint32_t* grounds;        // [nsegs] rounds per graph (NULL: one graph, DevState::rounds)
     unsigned long long* gmatched;  // [nsegs] matched vertices per graph (NULL: DevState::matched2)
@@ -359,6 +366,7 @@ int launch_contract(void* stream, const ContractArgs& c, uint32_t* mc_host_slot)
 int launch_job_graph(void* exec, void* stream);
 // list path (lm_list.cu): blocks of k_top for one graph, the maps for several, and the launches
 // (rounds: 64-bit words)
+uint32_t list_live_blocks(int device);  // blocks of k_live that run at once
 uint32_t list_blocks(const uint32_t task[4], uint32_t nrows);
 int launch_list_map(void* stream, const ListArgs* d, uint32_t nsegs, uint32_t* bmap, uint32_t* pmap);
 int launch_top(void* stream, const ListArgs* d, uint32_t blocks, bool rounds);
@@ -382,7 +390,7 @@ size_t exclusive_scan_tmp_words(uint32_t count);
 size_t build_fill_tmp_words(uint32_t n, uint32_t m);
 uint32_t build_fill_scan_count(uint32_t n, uint32_t m);
 int launch_build_fill(void* stream, const uint32_t* eu, const uint32_t* ev, const float* w, uint32_t n, uint32_t m,
-                      uint32_t* cursor, uint32_t* nbr, uint64_t* pk, uint64_t* edges, uint32_t* eword, uint32_t* tmp,
+                      uint32_t* cursor, uint32_t* eid, uint64_t* ent, uint64_t* edges, uint32_t* eword, uint32_t* tmp,
                       uint32_t* scan_tmp, size_t scan_words, uint32_t* err);  // err |= 2 when a fill slot falls outside 2m
 // cursors: the next place in task of each kind
 int launch_build_rows(void* stream, const uint32_t* deg, const uint32_t* rowidx_excl, const uint32_t* off,

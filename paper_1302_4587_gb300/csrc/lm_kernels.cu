@@ -23,7 +23,7 @@
 // candidate-only sweep over the graphs' own arrays, then the match and a
 // compacting sweep that builds the 64-bit keys
 //     K(e) = ord(w_e) << 32 | perm_seed(e)
-// from the per-entry word ord(weight) << 32 | edge id on the fly.
+// from the entries' ord(weight) and edge index on the fly.
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <string.h>
@@ -587,8 +587,8 @@ __device__ void do_rows_p(const SweepArgs& a, WarpRows<RENEW>& W, WarpStage& S, 
                 const uint32_t stg = k % PS;
                 if (INPUT) {
                     const SegIn& sg = a.segs[W.rseg[r]];
-                    cp_async8(&S.key[stg][lane], sg.pk + q);
-                    if (COMPACT) cp_async4(&S.nbr[stg][lane], sg.nbr + q);
+                    cp_async8(&S.key[stg][lane], sg.ent + q);
+                    cp_async4(&S.nbr[stg][lane], sg.eid + q);
                 } else {
                     cp_async8(&S.key[stg][lane], a.in_key + q);
                     if (COMPACT) cp_async4(&S.nbr[stg][lane], a.in_nbr + q);
@@ -609,7 +609,12 @@ __device__ void do_rows_p(const SweepArgs& a, WarpRows<RENEW>& W, WarpStage& S, 
         if (r != 32) {
             const uint32_t stg = k % PS;
             w = S.key[stg][lane];
-            if (COMPACT) u = S.nbr[stg][lane] + (INPUT ? a.segs[W.rseg[r]].vbase : 0u);
+            if (INPUT) {   // the input's entry: ord(w), neighbour; its edge index beside it
+                u = (uint32_t)w + a.segs[W.rseg[r]].vbase;
+                w = (w & 0xFFFFFFFF00000000ull) | S.nbr[stg][lane];
+            } else if (COMPACT) {
+                u = S.nbr[stg][lane];
+            }
         }
         issue(k + PD);
         row_group<INPUT, COMPACT, RENEW, COH>(a, W, r, sl, uni, w, u, lane, lt);
@@ -657,8 +662,8 @@ __device__ void do_chunk_p(const SweepArgs& a, WarpStage& S, uint32_t t, uint32_
         if (k < ng && jj < je) {
             const uint32_t stg = k % PS;
             if (INPUT) {
-                cp_async8(&S.key[stg][lane], sg.pk + off + jj);
-                if (COMPACT) cp_async4(&S.nbr[stg][lane], sg.nbr + off + jj);
+                cp_async8(&S.key[stg][lane], sg.ent + off + jj);
+                cp_async4(&S.nbr[stg][lane], sg.eid + off + jj);
             } else {
                 cp_async8(&S.key[stg][lane], a.in_key + off + jj);
                 if (COMPACT) cp_async4(&S.nbr[stg][lane], a.in_nbr + off + jj);
@@ -675,7 +680,12 @@ __device__ void do_chunk_p(const SweepArgs& a, WarpStage& S, uint32_t t, uint32_
         uint32_t u = NIL;
         if (jj < je) {
             key = S.key[stg][lane];
-            if (COMPACT) u = S.nbr[stg][lane] + vb;
+            if (INPUT) {
+                u = (uint32_t)key + vb;
+                key = (key & 0xFFFFFFFF00000000ull) | S.nbr[stg][lane];
+            } else if (COMPACT) {
+                u = S.nbr[stg][lane];
+            }
         }
         issue(k + PD);
         if (COMPACT) {
@@ -857,8 +867,8 @@ __device__ __forceinline__ bool cbar_or(bool p) {
 __device__ __forceinline__ uint32_t round16(uint32_t b) { return (b + 15u) & ~15u; }
 
 struct alignas(16) R0Stage {
-    unsigned long long pk[TILE0];     // entry words (first member: 16-byte aligned)
-    uint32_t nbr[TILE0];              // neighbours
+    unsigned long long ent[TILE0];    // entries: ord(w), neighbour (first member: 16-byte aligned)
+    uint32_t eid[TILE0];              // their edge indices
     uint32_t rvid[TILE0 + 8];         // row vertices from row (r_lo & ~3)
     uint32_t bits[R0W + 4];           // row-start bits of the tile, then of the next tile's first entries
     // written by the producer before the copies are issued
@@ -946,15 +956,15 @@ __device__ void r0_producer(R0Smem& s, const Round0Args& a) {
         S.j0 = j0;
         S.nent = nent;
         S.shift = shift;
-        const uint32_t b_pk = round16(nent * 8u);
-        const uint32_t b_nbr = round16(nent * 4u);
+        const uint32_t b_ent = round16(nent * 8u);
+        const uint32_t b_eid = round16(nent * 4u);
         const uint32_t b_vid = round16((shift + nload) * 4u);
         const uint32_t b_bits = (uint32_t)(R0W + 4) * 4u;
         // order the consumers' earlier reads of this stage before the copies' writes
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        mbar_expect_tx(&s.full[k], b_pk + b_nbr + b_vid + b_bits);
-        bulk_g2s(S.pk, g->pk + j0, b_pk, &s.full[k]);
-        bulk_g2s(S.nbr, g->nbr + j0, b_nbr, &s.full[k]);
+        mbar_expect_tx(&s.full[k], b_ent + b_eid + b_vid + b_bits);
+        bulk_g2s(S.ent, g->ent + j0, b_ent, &s.full[k]);
+        bulk_g2s(S.eid, g->eid + j0, b_eid, &s.full[k]);
         bulk_g2s(S.rvid, g->rvid + a0, b_vid, &s.full[k]);
         bulk_g2s(S.bits, g->rbits + j0 / 32, b_bits, &s.full[k]);
     }
@@ -1032,8 +1042,8 @@ __device__ void r0_consumer(R0Smem& s, const Round0Args& a, int tid) {
         // the entries' ord(w): the high words of their stored words
         uint32_t o[4];
         {
-            const uint4 qa = *reinterpret_cast<const uint4*>(&S.pk[base]);
-            const uint4 qb = *reinterpret_cast<const uint4*>(&S.pk[base + 2]);
+            const uint4 qa = *reinterpret_cast<const uint4*>(&S.ent[base]);
+            const uint4 qb = *reinterpret_cast<const uint4*>(&S.ent[base + 2]);
             o[0] = qa.y; o[1] = qa.w; o[2] = qb.y; o[3] = qb.w;
 #pragma unroll
             for (int j = 0; j < 4; j++)
@@ -1099,14 +1109,14 @@ __device__ void r0_consumer(R0Smem& s, const Round0Args& a, int tid) {
                 const uint32_t t = __popc(hb & 0xEu & ((2u << j) - 1u));
                 if (o[j] && o[j] == s.rord[R + t] && s.rwin[R + t] == R0_TIED) {
                     mine |= 1u << j;
-                    atomicMax(&s.rperm[R + t], perm_seed((uint32_t)S.pk[base + j], k0, k1));
+                    atomicMax(&s.rperm[R + t], perm_seed(S.eid[base + j], k0, k1));
                 }
             }
             cbar();
 #pragma unroll
             for (int j = 0; j < 4; j++) {
                 const uint32_t t = __popc(hb & 0xEu & ((2u << j) - 1u));
-                if (((mine >> j) & 1u) && perm_seed((uint32_t)S.pk[base + j], k0, k1) == s.rperm[R + t])
+                if (((mine >> j) & 1u) && perm_seed(S.eid[base + j], k0, k1) == s.rperm[R + t])
                     s.rwin[R + t] = base + (uint32_t)j;
             }
             cbar();
@@ -1127,8 +1137,8 @@ __device__ void r0_consumer(R0Smem& s, const Round0Args& a, int tid) {
                     continue;
                 }
                 const bool cut = (r == 0 && cut0) || (r == nrt - 1 && cutL);
-                if (!cut) va.cnbr[v] = S.nbr[p] + vbase;
-                else atomicMax(&va.bkey[v], ((unsigned long long)ow << 32) | perm_seed((uint32_t)S.pk[p], g.k0, g.k1));
+                if (!cut) va.cnbr[v] = (uint32_t)S.ent[p] + vbase;
+                else atomicMax(&va.bkey[v], ((unsigned long long)ow << 32) | perm_seed(S.eid[p], g.k0, g.k1));
             }
         }
         cbar();
@@ -1441,8 +1451,8 @@ __global__ void __launch_bounds__(BF_T) k_build_vhist(const uint32_t* ev, uint32
 
 __global__ void __launch_bounds__(BF_T) k_build_fill_u(const uint32_t* eu, const uint32_t* ev, const float* w,
                                                        uint32_t m, uint32_t shift, uint32_t tiles,
-                                                       const uint32_t* offs, uint32_t* cursor, uint32_t* nbr,
-                                                       uint64_t* pk, uint64_t* edges, uint32_t* eword, uint4* vrec,
+                                                       const uint32_t* offs, uint32_t* cursor, uint32_t* eid,
+                                                       uint64_t* ent, uint64_t* edges, uint32_t* eword, uint4* vrec,
                                                        uint32_t* err) {
     __shared__ uint32_t gs[BF_NB], cnt[BF_NB];
     gs[threadIdx.x] = offs[threadIdx.x * tiles + blockIdx.x];
@@ -1454,12 +1464,11 @@ __global__ void __launch_bounds__(BF_T) k_build_fill_u(const uint32_t* eu, const
         const uint64_t e = t0 + j * BF_T + threadIdx.x;
         const bool ok = e < m;
         uint32_t u = 0, v = 0;
-        uint64_t word = 0;
+        uint32_t ow = 0;
         if (ok) {
             u = eu[e];
             v = ev[e];
-            const uint32_t ow = ord_of_bits(__float_as_uint(w[e]));
-            word = ((uint64_t)ow << 32) | (uint32_t)e;
+            ow = ord_of_bits(__float_as_uint(w[e]));
             edges[e] = (uint64_t)u | ((uint64_t)v << 32);
             eword[e] = ow;
         }
@@ -1470,19 +1479,19 @@ __global__ void __launch_bounds__(BF_T) k_build_fill_u(const uint32_t* eu, const
             if (pu >= 2 * m) {
                 atomicOr(err, 2u);
             } else {
-                nbr[pu] = v;
-                pk[pu] = word;
+                ent[pu] = ((uint64_t)ow << 32) | v;
+                eid[pu] = (uint32_t)e;
             }
             const uint32_t b = (v >> shift) & (BF_NB - 1);
             const uint32_t q = gs[b] + atomicAdd(&cnt[b], 1u);
-            if (q < m) vrec[q] = make_uint4(v, u, (uint32_t)word, (uint32_t)(word >> 32));
+            if (q < m) vrec[q] = make_uint4(v, u, (uint32_t)e, ow);
             else atomicOr(err, 2u);
         }
     }
 }
 
-__global__ void __launch_bounds__(BF_T) k_build_fill_v(const uint4* vrec, uint32_t m, uint32_t* cursor, uint32_t* nbr,
-                                                       uint64_t* pk, uint32_t* err) {
+__global__ void __launch_bounds__(BF_T) k_build_fill_v(const uint4* vrec, uint32_t m, uint32_t* cursor, uint32_t* eid,
+                                                       uint64_t* ent, uint32_t* err) {
     const uint32_t stride = gridDim.x * blockDim.x, lane = threadIdx.x & 31;
     const uint32_t mr = (m + 31) & ~31u;  // whole warps iterate together
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < mr; i += stride) {
@@ -1494,8 +1503,8 @@ __global__ void __launch_bounds__(BF_T) k_build_fill_v(const uint4* vrec, uint32
             if (pv >= 2 * m) {
                 atomicOr(err, 2u);
             } else {
-                nbr[pv] = r.y;
-                pk[pv] = ((uint64_t)r.w << 32) | r.z;
+                ent[pv] = ((uint64_t)r.w << 32) | r.y;
+                eid[pv] = r.z;
             }
         }
     }
@@ -1911,7 +1920,7 @@ uint32_t build_fill_scan_count(uint32_t n, uint32_t m) {
     return (uint32_t)(BF_NB * (((uint64_t)m + BF_TILE - 1) / BF_TILE));
 }
 int launch_build_fill(void* stream, const uint32_t* eu, const uint32_t* ev, const float* w, uint32_t n, uint32_t m,
-                      uint32_t* cursor, uint32_t* nbr, uint64_t* pk, uint64_t* edges, uint32_t* eword, uint32_t* tmp,
+                      uint32_t* cursor, uint32_t* eid, uint64_t* ent, uint64_t* edges, uint32_t* eword, uint32_t* tmp,
                       uint32_t* scan_tmp, size_t scan_words, uint32_t* err) {
     cudaStream_t s = (cudaStream_t)stream;
     if (m == 0) return 0;
@@ -1924,8 +1933,8 @@ int launch_build_fill(void* stream, const uint32_t* eu, const uint32_t* ev, cons
     uint32_t* offs = hist + ((BF_NB * (size_t)tiles + 4) & ~(size_t)3);
     k_build_vhist<<<tiles, BF_T, 0, s>>>(ev, m, shift, tiles, hist);
     if (int r = launch_exclusive_scan(stream, hist, offs, BF_NB * tiles, scan_tmp, scan_words)) return r;
-    k_build_fill_u<<<tiles, BF_T, 0, s>>>(eu, ev, w, m, shift, tiles, offs, cursor, nbr, pk, edges, eword, vrec, err);
-    k_build_fill_v<<<grid_for(m, 256), BF_T, 0, s>>>(vrec, m, cursor, nbr, pk, err);
+    k_build_fill_u<<<tiles, BF_T, 0, s>>>(eu, ev, w, m, shift, tiles, offs, cursor, eid, ent, edges, eword, vrec, err);
+    k_build_fill_v<<<grid_for(m, 256), BF_T, 0, s>>>(vrec, m, cursor, eid, ent, err);
     return (int)cudaGetLastError();
 }
 int launch_nonzero_flags(void* stream, const uint32_t* deg, uint32_t n, uint32_t* flags, uint32_t* counts) {

@@ -3,15 +3,16 @@
 // A vertex only ever looks at the heaviest few of its edges before it is
 // matched or runs out of live neighbours (2.3 to 2.5 entries a row on random,
 // grid and R-MAT graphs, 9% to 40% of the adjacency entries).  So one pass over
-// the adjacency arrays (k_top) keeps the four heaviest neighbours of every row,
-// in order, and no entry is read again unless those four are used up:
+// the adjacency arrays (k_top) keeps the heaviest neighbours of every row, in
+// order -- four, eight of the longer rows --, and no entry is read again unless
+// those are used up:
 //
-//   k_top   every row's candidate (Sec. 2.1, step 2) and the next three
+//   k_top   every row's candidate (Sec. 2.1, step 2) and the next of its list
 //   k_live  the live rows until none is left.  A row looks at its candidate's
 //           word: chosen back, it is matched (step 3); matched to another, the row
 //           moves on to the next of its list that is not (steps 4 to 6 without
 //           moving an edge: an edge is dead when the word of its other end says so),
-//           and scans its adjacency once more for the four heaviest live ones
+//           and scans its adjacency once more for the heaviest live ones
 //           when the list is used up; otherwise it stays as it is.
 //
 // A vertex's word is its candidate, with DEAD set once it is matched (to it).
@@ -38,7 +39,6 @@ namespace lm {
 namespace {
 
 constexpr uint32_t DEAD = 0x80000000u, VMASK = 0x7FFFFFFFu;
-constexpr uint32_t TOPN = 4;   // neighbours kept per row (its word and lst)
 
 // ---------------------------------------------------------------- words
 // W = uint32_t: candidate | DEAD.  W = uint64_t: the same in the low half; above it
@@ -61,258 +61,273 @@ __device__ __forceinline__ uint64_t look(const uint64_t* p) {
     return __ldcg(reinterpret_cast<const unsigned long long*>(p));
 }
 
-// ---------------------------------------------------------------- the four heaviest entries
-// Entries are compared by ord(w) alone where that decides: perm_seed tells equal
-// ones apart, and only rows where it matters (two of the four, or the fourth
-// and one left out, are equal) are taken again by their full keys.
+// ---------------------------------------------------------------- a row's list
+// The candidate is the row's word; the next three neighbours and the flags sit in
+// lst[v] (x, y, z, w), four more in wide[v] if WIDE is set.  MORE: the row holds
+// entries beyond its list.  An empty place is NIL.
+struct RowLists {
+    uint4 *lst, *wide;
+};
+constexpr uint32_t MORE = 1u, WIDE = 2u;
+constexpr int KS = 4, KL = LIST_KEPT;   // list lengths: rows of at most LIST_SHORT entries, longer ones
 
-// One unit's (a thread's, a group of lanes') four largest of up to 256 entries as
-// 32-bit numbers: ord(w) with its low BITS bits replaced by the entry's place in
-// the row (smaller first), so that an exchange is one minimum and one maximum.
-// Entries whose ord agrees above those bits count as equal.
+// entry i of a graph: ord(w), its neighbour, its full key
+__device__ __forceinline__ uint32_t ord_at(const ListSeg& g, uint32_t i) {
+    return __ldg(reinterpret_cast<const uint32_t*>(g.ent) + 2 * (size_t)i + 1);
+}
+__device__ __forceinline__ uint32_t nbr_at(const ListSeg& g, uint32_t i) {
+    return __ldg(reinterpret_cast<const uint32_t*>(g.ent) + 2 * (size_t)i);
+}
+__device__ __forceinline__ uint64_t key_of(const ListSeg& g, uint32_t ord, uint32_t i) {
+    return ((uint64_t)ord << 32) | perm_seed(__ldg(g.eid + i), g.k0, g.k1);
+}
+
+// Entries are compared by ord(w) alone where that decides: perm_seed tells equal
+// ones apart, and only rows where it matters (two of the list, or its last and one
+// left out, are equal) are taken again by their full keys.
+//
+// Up to 256 entries are compared as 32-bit numbers: ord(w) with its low bits
+// replaced by the entry's place in the row (smaller first), so that an exchange is
+// one minimum and one maximum and no two are equal.  Entries whose ord agrees above
+// those bits count as equal.
 __device__ __forceinline__ uint32_t packed(uint32_t ord, uint32_t idx, uint32_t mask) {
     return (ord & ~mask) | (mask - idx);
 }
-struct TopP {
+__device__ __forceinline__ void order2(uint32_t& a, uint32_t& b) {
+    const uint32_t hi = max(a, b);
+    b = min(a, b);
+    a = hi;
+}
+template <int E>
+__device__ __forceinline__ void order(uint32_t x[E]);
+template <>
+__device__ __forceinline__ void order<4>(uint32_t x[4]) {
+    order2(x[0], x[1]); order2(x[2], x[3]);
+    order2(x[0], x[2]); order2(x[1], x[3]);
+    order2(x[1], x[2]);
+}
+template <>
+__device__ __forceinline__ void order<8>(uint32_t x[8]) {   // Batcher's odd-even merge sort
+    order<4>(x);
+    order<4>(x + 4);
+    order2(x[0], x[4]); order2(x[1], x[5]); order2(x[2], x[6]); order2(x[3], x[7]);
+    order2(x[2], x[4]); order2(x[3], x[5]);
+    order2(x[1], x[2]); order2(x[3], x[4]); order2(x[5], x[6]);
+}
+
+// a thread's four largest of any number of such entries, taken four at a time
+struct Top4 {
     uint32_t k[4] = {0, 0, 0, 0};
     uint32_t out = 0;                 // largest one left out
-    __device__ __forceinline__ void add(uint32_t x) {
+    // the larger of each pair taken head to tail from two ordered fours is one of the
+    // four largest (a bitonic four), then put in order
+    __device__ __forceinline__ void take(uint32_t x[4]) {
+        order<4>(x);
+        out = max(out, max(max(min(k[0], x[3]), min(k[1], x[2])), max(min(k[2], x[1]), min(k[3], x[0]))));
 #pragma unroll
-        for (int i = 0; i < 4; i++) {
-            const uint32_t hi = max(k[i], x);
-            x = min(k[i], x);
-            k[i] = hi;
+        for (int i = 0; i < 4; i++) k[i] = max(k[i], x[3 - i]);
+        order2(k[0], k[2]); order2(k[1], k[3]);
+        order2(k[0], k[1]); order2(k[2], k[3]);
+    }
+};
+// equal neighbours in an ordered list r of K, the last against the largest left out (a
+// place without an entry packs to a number of at most `mask`, below every entry's)
+template <int K>
+__device__ __forceinline__ bool any_tie(const uint32_t r[K], uint32_t out, uint32_t mask) {
+    bool t = out > mask && (r[K - 1] ^ out) <= mask;
+#pragma unroll
+    for (int i = 1; i < K; i++) t |= r[i] > mask && (r[i - 1] ^ r[i]) <= mask;
+    return t;
+}
+// maximum over an aligned group of G lanes
+template <int G>
+__device__ __forceinline__ uint32_t group_max(uint32_t x) {
+    if constexpr (G == 32) {
+        return __reduce_max_sync(FULL, x);
+    } else {
+#pragma unroll
+        for (int d = 1; d < G; d <<= 1) x = max(x, __shfl_xor_sync(FULL, x, d));
+        return x;
+    }
+}
+template <int G>
+__device__ __forceinline__ uint64_t group_max64(uint64_t x) {
+#pragma unroll
+    for (int d = 1; d < G; d <<= 1) {
+        const uint64_t o = __shfl_xor_sync(FULL, x, d);
+        x = o > x ? o : x;
+    }
+    return x;
+}
+// The K largest of a group's entries, E packed ones a lane: every lane in order, then
+// the largest head K times.  r: the same for all lanes; returns the largest left out.
+template <int G, int E, int K>
+__device__ __forceinline__ uint32_t group_top(uint32_t x[E], uint32_t r[K]) {
+    order<E>(x);
+#pragma unroll
+    for (int i = 0; i < K; i++) {
+        const uint32_t h = group_max<G>(x[0]);
+        r[i] = h;
+        const bool mine = x[0] == h;
+#pragma unroll
+        for (int e = 0; e + 1 < E; e++) x[e] = mine ? x[e + 1] : x[e];
+        x[E - 1] = mine ? 0u : x[E - 1];
+    }
+    return group_max<G>(x[0]);
+}
+// the same by full key among the entries in `live` (bit e; entry e * G + the lane's
+// place): positions (NIL: none) and keys; returns whether others are left
+template <int G, int E, int K>
+__device__ __forceinline__ bool group_top_keyed(const uint64_t key[E], uint32_t live, uint32_t sub, uint32_t p[K],
+                                                uint64_t k[K]) {
+    uint32_t left = live;
+#pragma unroll
+    for (int i = 0; i < K; i++) {
+        uint64_t m = 0;
+        uint32_t at = NIL;
+#pragma unroll
+        for (int e = 0; e < E; e++)
+            if (((left >> e) & 1u) && key[e] > m) { m = key[e]; at = e; }
+        const uint64_t b = group_max64<G>(m);
+        const bool own = b && b == m;
+        p[i] = ~group_max<G>(own ? ~(at * G + sub) : 0u);   // (the owner's position; NIL without one)
+        if (own) left &= ~(1u << at);
+        k[i] = b;
+    }
+    return group_max<G>(left) != 0;
+}
+
+// A warp's KL largest of any number of entries, in order, one to a lane (lane i < KL
+// has the i-th): by ord(w) with the position, or by full key with the neighbour.  The
+// other lanes hold 0.
+struct LaneTop32 {
+    uint32_t o = 0, p = NIL;
+    __device__ __forceinline__ uint32_t last() const { return __shfl_sync(FULL, o, KL - 1); }
+    __device__ __forceinline__ void put(uint32_t h, uint32_t hp) {   // h differs from all of the list
+        const uint32_t lane = threadIdx.x & 31;
+        const uint32_t at = __popc(__ballot_sync(FULL, o > h));
+        const uint32_t uo = __shfl_up_sync(FULL, o, 1), up = __shfl_up_sync(FULL, p, 1);
+        if (lane >= at && lane < KL) {
+            o = lane == at ? h : uo;
+            p = lane == at ? hp : up;
         }
-        out = max(out, x);
     }
-    // the four largest of two ordered fours: the larger of each pair taken head to tail
-    // is one of them (a bitonic four), then put in order
-    __device__ __forceinline__ void merge(const uint32_t o[4], uint32_t oout) {
-        out = max(out, oout);
-#pragma unroll
-        for (int i = 0; i < 4; i++) out = max(out, min(k[i], o[3 - i]));
-#pragma unroll
-        for (int i = 0; i < 4; i++) k[i] = max(k[i], o[3 - i]);
-        order(0, 2);
-        order(1, 3);
-        order(0, 1);
-        order(2, 3);
-    }
-    __device__ __forceinline__ void order(int a, int b) {
-        const uint32_t hi = max(k[a], k[b]);
-        k[b] = min(k[a], k[b]);
-        k[a] = hi;
-    }
-    // over the lanes of aligned groups of G, each lane's four in order on entry
-    template <int G>
-    __device__ __forceinline__ void across() {
-#pragma unroll
-        for (int d = 1; d < G; d <<= 1) {
-            uint32_t o[4];
-#pragma unroll
-            for (int i = 0; i < 4; i++) o[i] = __shfl_xor_sync(FULL, k[i], d);
-            const uint32_t oo = __shfl_xor_sync(FULL, out, d);
-            merge(o, oo);
+};
+struct LaneTop64 {
+    uint64_t k = 0;
+    uint32_t n = NIL;
+    __device__ __forceinline__ uint64_t last() const { return __shfl_sync(FULL, k, KL - 1); }
+    __device__ __forceinline__ void put(uint64_t h, uint32_t hn) {
+        const uint32_t lane = threadIdx.x & 31;
+        const uint32_t at = __popc(__ballot_sync(FULL, k > h));
+        const uint64_t uk = __shfl_up_sync(FULL, k, 1);
+        const uint32_t un = __shfl_up_sync(FULL, n, 1);
+        if (lane >= at && lane < KL) {
+            k = lane == at ? h : uk;
+            n = lane == at ? hn : un;
         }
     }
-    __device__ __forceinline__ bool tied(uint32_t mask) const {
-        return (k[1] && (k[0] ^ k[1]) <= mask) || (k[2] && (k[1] ^ k[2]) <= mask) ||
-               (k[3] && ((k[2] ^ k[3]) <= mask || (out && (k[3] ^ out) <= mask)));
+    // every lane offers (key, neighbour), 0 for none: those above the last go in
+    __device__ __forceinline__ void offer(uint64_t key, uint32_t nb) {
+        for (uint64_t bar = last(); __any_sync(FULL, key > bar); bar = last()) {
+            const uint32_t hi = __reduce_max_sync(FULL, (uint32_t)(key >> 32));
+            const uint32_t lw = __reduce_max_sync(FULL, ((uint32_t)(key >> 32) == hi) ? (uint32_t)key : 0u);
+            const uint64_t best = ((uint64_t)hi << 32) | lw;
+            const int L = __ffs(__ballot_sync(FULL, key == best)) - 1;
+            put(best, __shfl_sync(FULL, nb, L));
+            if ((int)(threadIdx.x & 31) == L) key = 0;
+        }
     }
 };
 
-// A warp's four largest (uniform over its lanes) of any number of entries, by
-// ord(w), with their positions; an equal one is for the caller to notice (has()).
-struct Top32 {
-    uint32_t o0 = 0, o1 = 0, o2 = 0, o3 = 0;
-    uint32_t p0 = 0, p1 = 0, p2 = 0, p3 = 0;
-    __device__ __forceinline__ void swap_in(uint32_t& o, uint32_t& p, uint32_t& x, uint32_t& px) {
-        const bool g = x > o;
-        const uint32_t hi = max(o, x), lw = min(o, x), ph = g ? px : p, pl = g ? p : px;
-        o = hi; p = ph; x = lw; px = pl;
-    }
-    __device__ __forceinline__ void add(uint32_t x, uint32_t px) {
-        swap_in(o0, p0, x, px);
-        swap_in(o1, p1, x, px);
-        swap_in(o2, p2, x, px);
-        swap_in(o3, p3, x, px);
-    }
-    __device__ __forceinline__ bool has(uint32_t x) const { return x == o0 || x == o1 || x == o2 || x == o3; }
-};
-struct Top64 {
-    uint64_t k0 = 0, k1 = 0, k2 = 0, k3 = 0;
-    uint32_t p0 = NIL, p1 = NIL, p2 = NIL, p3 = NIL;
-    __device__ __forceinline__ void swap_in(uint64_t& k, uint32_t& p, uint64_t& x, uint32_t& px) {
-        if (x > k) {
-            const uint64_t t = k; k = x; x = t;
-            const uint32_t q = p; p = px; px = q;
-        }
-    }
-    __device__ __forceinline__ void add(uint64_t x, uint32_t px) {
-        swap_in(k0, p0, x, px);
-        swap_in(k1, p1, x, px);
-        swap_in(k2, p2, x, px);
-        swap_in(k3, p3, x, px);
-    }
-};
-
-__device__ __forceinline__ uint32_t hi32(const uint64_t* pk, uint32_t i) {
-    return __ldg(reinterpret_cast<const uint32_t*>(pk) + 2 * (size_t)i + 1);
-}
-__device__ __forceinline__ uint64_t full_key(uint64_t w, uint32_t k0, uint32_t k1) {
-    return (w & 0xFFFFFFFF00000000ull) | perm_seed((uint32_t)w, k0, k1);
-}
-
-// every lane offers (key, p), 0 for none: the warp's keys above t.k3 go in, largest first
-__device__ __forceinline__ void warp_add(Top64& t, uint64_t key, uint32_t p) {
-    while (__any_sync(FULL, key > t.k3)) {
-        const uint32_t hi = __reduce_max_sync(FULL, (uint32_t)(key >> 32));
-        const uint32_t lo = __reduce_max_sync(FULL, ((uint32_t)(key >> 32) == hi) ? (uint32_t)key : 0u);
-        const uint64_t best = ((uint64_t)hi << 32) | lo;
-        const uint32_t own = __ballot_sync(FULL, key == best);
-        const int L = __ffs(own) - 1;
-        t.add(best, __shfl_sync(FULL, p, L));
-        if ((int)(threadIdx.x & 31) == L) key = 0;
-    }
-}
-
-// the four heaviest entries [s, e) by full key, the warp together; p: positions
-__device__ __noinline__ void warp_top_keyed(const ListSeg& g, uint32_t s, uint32_t e, Top64& t) {
-    const uint32_t lane = threadIdx.x & 31;
-    uint64_t nx = s + lane < e ? __ldg(g.pk + s + lane) : 0ull;
-    for (uint32_t b = s; b < e; b += 32) {
-        const uint64_t w = nx;
-        const uint32_t i = b + lane, j = i + 32;
-        nx = (j < e && j > i) ? __ldg(g.pk + j) : 0ull;
-        warp_add(t, i < e ? full_key(w, g.k0, g.k1) : 0ull, i);
-    }
-}
-
-// row v's list: four neighbours (NIL: none), more = entries beyond them were left out
+// a list held by lanes 0 .. KL - 1 (NIL: none) into row `at`'s places
 template <class W>
-__device__ __forceinline__ void put_row(const ListArgs& a, size_t at, uint32_t c0, uint32_t c1, uint32_t c2,
-                                        uint32_t c3, bool more) {
-    words<W>(a)[at] = word<W>(c0, 0);
-    a.lst[at] = make_uint4(c1, c2, c3, more ? 1u : 0u);
+__device__ __forceinline__ void put_lanes(W* cur, const RowLists& R, size_t at, uint32_t lane, uint32_t c,
+                                          uint32_t inf, bool more) {
+    if (lane == 0) cur[at] = word<W>(c, inf);
+    else if (lane < 4) reinterpret_cast<uint32_t*>(R.lst + at)[lane - 1] = c;
+    else if (lane < KL) reinterpret_cast<uint32_t*>(R.wide + at)[lane - 4] = c;
+    else if (lane == KL) R.lst[at].w = WIDE | (more ? MORE : 0u);
+}
+// the same for a group's lanes, each with its place's neighbour; the flags go with the third
+template <class W, int K>
+__device__ __forceinline__ void put_group(W* cur, const RowLists& R, size_t at, uint32_t sub, uint32_t c,
+                                          uint32_t inf, uint32_t flags) {
+    uint32_t* l = reinterpret_cast<uint32_t*>(R.lst + at);
+    if (sub == 0) cur[at] = word<W>(c, inf);
+    else if (sub < 3) l[sub - 1] = c;
+    else if (sub == 3) *reinterpret_cast<uint2*>(l + 2) = make_uint2(c, flags);
+    else if (sub < K) reinterpret_cast<uint32_t*>(R.wide + at)[sub - 4] = c;
 }
 
 // ---------------------------------------------------------------- k_top
 constexpr int TT = 256, TWARPS = TT / 32;
-constexpr uint32_t SBUF = 512;    // entries of short rows a warp stages at a time
 constexpr uint32_t MPW = 2;       // long-row tasks a warp takes,
 constexpr uint32_t WPW = 8;       // rows of LIST_GROUP + 1 .. LIST_WARP entries,
 constexpr uint32_t GPW = 16;      // and rows of LIST_SHORT + 1 .. LIST_GROUP
-static_assert(LIST_SHORT <= 32 && LIST_GROUP == 8 * 8 && LIST_WARP == 8 * 32, "eight entries a lane");
+static_assert(LIST_SHORT == 32 && LIST_GROUP == 8 * 8 && LIST_WARP == 8 * 32, "eight entries a lane");
 
-struct TopSmem {
-    uint32_t o[TWARPS][SBUF];     // ord(w) of the staged entries
-    uint32_t n[TWARPS][SBUF];     // their neighbours
-};
-
-// 32 rows of at most LIST_SHORT entries (longer ones among them are skipped), a
-// thread each.  Runs of neighbouring short rows are contiguous in the arrays:
-// the warp copies them to shared memory coalesced and each thread walks its own
-// row there, so a row costs its length in warp steps shared by 32 rows instead
-// of a segmented scan over its entries.
+// A row of at most LIST_SHORT entries by one thread, four entries at a time, the next
+// four on their way.  Neighbouring threads' rows are neighbours in the arrays, so
+// their loads share sectors through L1 (staging the entries through shared memory
+// first cost more instructions than it saved wavefronts).
 template <class W>
-__device__ void top_short(const ListArgs& a, const ListSeg& g, uint32_t r0, uint32_t* so, uint32_t* sn) {
-    const uint32_t lane = threadIdx.x & 31;
-    const uint32_t r = r0 + lane;
-    uint32_t o = 0, e = 0, v = 0;
+__device__ __forceinline__ void top_short(const ListArgs& a, const ListSeg& g, uint32_t r) {
+    uint32_t o = 0, d = 0, v = 0;
     if (r < g.nrows) {
         o = __ldg(g.roff + r);
-        e = __ldg(g.roff + r + 1);
+        d = __ldg(g.roff + r + 1) - o;
         v = __ldg(g.vid + r);
     }
-    const uint32_t d = e - o;
-    const bool mine = d > 0 && d <= LIST_SHORT;
-    uint32_t todo = __ballot_sync(FULL, mine);
-    while (todo) {
-        // stage runs of short rows until the buffer is full
-        uint32_t used = 0, my = 0, taken = 0;
-        while (todo) {
-            const int f = __ffs(todo) - 1;
-            const uint32_t run = todo >> f;
-            const int len = run == (FULL >> f) ? 32 - f : __ffs(~run) - 1;
-            const uint32_t s = __shfl_sync(FULL, o, f);
-            // rows f .. of the run that still fit
-            const bool fit = (int)lane >= f && (int)lane < f + len && e - s <= SBUF - used;
-            const uint32_t fits = __ballot_sync(FULL, fit);
-            if (!fits) break;
-            const int last = 31 - __clz(fits);
-            const uint32_t cnt = __shfl_sync(FULL, e, last) - s;
-            if (fit) my = used + (o - s);
-            for (uint32_t i = lane; i < cnt; i += 128) {
-                uint32_t x[4], y[4];
+    if (d == 0 || d > LIST_SHORT) return;
+    constexpr uint32_t MASK = LIST_SHORT - 1;
+    Top4 t;
+    uint32_t x[4], nx[4];
+    auto load = [&](uint32_t y[4], uint32_t j) {
 #pragma unroll
-                for (int q = 0; q < 4; q++)
-                    if (i + 32 * q < cnt) { x[q] = hi32(g.pk, s + i + 32 * q); y[q] = __ldg(g.nbr + s + i + 32 * q); }
+        for (uint32_t q = 0; q < 4; q++) y[q] = j + q < d ? ord_at(g, o + j + q) : 0u;
+    };
+    load(x, 0);
 #pragma unroll
-                for (int q = 0; q < 4; q++)
-                    if (i + 32 * q < cnt) { so[used + i + 32 * q] = x[q]; sn[used + i + 32 * q] = y[q]; }
-            }
-            used += cnt;
-            taken |= fits;
-            todo &= ~fits;
-            if (last < f + len - 1) break;  // the buffer is full
-        }
-        __syncwarp();
-        if ((taken >> lane) & 1u) {
-            constexpr uint32_t MASK = LIST_SHORT - 1;
-            TopP t;
-            for (uint32_t j = 0; j < d; j++) t.add(packed(so[my + j], j, MASK));
-            uint32_t p[4];
+    for (uint32_t j = 0; j < LIST_SHORT; j += 4) {   // (unrolled: the places are constants)
+        if (j >= d) break;
+        if (j + 4 < LIST_SHORT) load(nx, j + 4);
 #pragma unroll
-            for (int i = 0; i < 4; i++) p[i] = MASK - (t.k[i] & MASK);
-            if (t.tied(MASK)) {
-                Top64 k;
-                for (uint32_t j = 0; j < d; j++) k.add(full_key(__ldg(g.pk + o + j), g.k0, g.k1), j);
-                p[0] = k.p0; p[1] = k.p1; p[2] = k.p2; p[3] = k.p3;
-            }
-            put_row<W>(a, (size_t)g.vbase + v, sn[my + p[0]], d > 1 ? sn[my + p[1]] : NIL, d > 2 ? sn[my + p[2]] : NIL,
-                       d > 3 ? sn[my + p[3]] : NIL, d > TOPN);
-        }
-        __syncwarp();
+        for (uint32_t q = 0; q < 4; q++) x[q] = packed(x[q], j + q, MASK);
+        t.take(x);
+#pragma unroll
+        for (int q = 0; q < 4; q++) x[q] = nx[q];
     }
+    uint32_t p[4];
+#pragma unroll
+    for (int i = 0; i < 4; i++) p[i] = MASK - (t.k[i] & MASK);
+    if (any_tie<4>(t.k, t.out, MASK)) {
+        // by full key
+        uint64_t k[4] = {0, 0, 0, 0};
+        for (uint32_t j = 0; j < d; j++) {
+            uint64_t x64 = key_of(g, ord_at(g, o + j), o + j);
+            uint32_t px = j;
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                const bool gt = x64 > k[i];
+                const uint64_t tk = k[i];
+                const uint32_t tp = p[i];
+                k[i] = gt ? x64 : tk;
+                p[i] = gt ? px : tp;
+                x64 = gt ? tk : x64;
+                px = gt ? tp : px;
+            }
+        }
+    }
+    const size_t at = (size_t)g.vbase + v;
+    words<W>(a)[at] = word<W>(nbr_at(g, o + p[0]), 0);
+    a.lst[at] = make_uint4(d > 1 ? nbr_at(g, o + p[1]) : NIL, d > 2 ? nbr_at(g, o + p[2]) : NIL,
+                           d > 3 ? nbr_at(g, o + p[3]) : NIL, d > 4 ? MORE : 0u);
 }
 
-// The four heaviest of a row held by a group of G lanes, eight entries a lane (entry
-// 8-fold: e * G + the lane's place), among those in `live` (bit e), by full key: the
-// exact form.  Positions (NIL: none) and keys; rest: others are left.
-template <int G>
-__device__ __forceinline__ void group_keyed(const uint64_t K[8], uint32_t live, uint32_t sub, uint32_t p[4],
-                                            uint64_t k[4], bool& rest) {
-    uint32_t left = live;
-#pragma unroll
-    for (int i = 0; i < 4; i++) {
-        uint64_t m = 0;
-        uint32_t at = NIL;
-#pragma unroll
-        for (int e = 0; e < 8; e++)
-            if (((left >> e) & 1u) && K[e] > m) { m = K[e]; at = e; }
-        uint64_t b = m;
-#pragma unroll
-        for (int d = 1; d < G; d <<= 1) {
-            const uint64_t o = __shfl_xor_sync(FULL, b, d);
-            b = o > b ? o : b;
-        }
-        const bool own = b && b == m;
-        uint32_t pos = own ? at * G + sub : NIL;
-#pragma unroll
-        for (int d = 1; d < G; d <<= 1) pos = min(pos, __shfl_xor_sync(FULL, pos, d));
-        p[i] = pos;
-        if (own) left &= ~(1u << at);
-        k[i] = b;
-    }
-    uint32_t any = left;
-#pragma unroll
-    for (int d = 1; d < G; d <<= 1) any |= __shfl_xor_sync(FULL, any, d);
-    rest = any != 0;
-}
-
-// `per` rows of more than LIST_SHORT entries a warp, eight entries to each of the G
-// lanes of a group (32 / G rows at a time), straight from the arrays into registers;
-// the next rows' entries are on their way while these are compared.
+// Rows of more than LIST_SHORT entries, eight entries to each of the G lanes of a group
+// (32 / G rows at a time), straight from the arrays into registers; the next rows'
+// entries are on their way while these are compared.
 template <class W, int G>
 __device__ __forceinline__ void top_group(const ListArgs& a, const ListSeg& g, uint32_t t0, uint32_t cnt) {
     constexpr uint32_t ROWS = 32 / G, MASK = 8 * G - 1;
@@ -326,178 +341,176 @@ __device__ __forceinline__ void top_group(const ListArgs& a, const ListSeg& g, u
         d = __shfl_sync(FULL, d4.z, (i + grp) & 31u);
         if (i + grp >= cnt) d = 0;
 #pragma unroll
-        for (int e = 0; e < 8; e++) x[e] = e * G + sub < d ? hi32(g.pk, s + e * G + sub) : 0u;
+        for (int e = 0; e < 8; e++) x[e] = e * G + sub < d ? ord_at(g, s + e * G + sub) : 0u;
     };
     fetch(0);
     for (uint32_t i = 0; i < cnt; i += ROWS) {
         const uint32_t cv = v, cs = s, cd = d;
-        TopP t;
 #pragma unroll
-        for (int e = 0; e < 8; e++) t.add(x[e] ? packed(x[e], e * G + sub, MASK) : 0u);
-        t.across<G>();
-        uint32_t p[4];
+        for (int e = 0; e < 8; e++) x[e] = packed(x[e], e * G + sub, MASK);
+        uint32_t r[KL];
+        const uint32_t out = group_top<G, 8, KL>(x, r);
+        uint32_t mine = r[0];
 #pragma unroll
-        for (int q = 0; q < 4; q++) p[q] = MASK - (t.k[q] & MASK);
-        if (__any_sync(FULL, t.tied(MASK))) {
-            uint64_t K[8], kk[4];
-            uint32_t pk[4];
-            bool rest;
+        for (int q = 1; q < KL; q++) mine = (sub & 7u) == (uint32_t)q ? r[q] : mine;
+        uint32_t p = MASK - (mine & MASK);
+        if (__any_sync(FULL, any_tie<KL>(r, out, MASK))) {
+            uint64_t key[8], kk[KL];
+            uint32_t pk[KL];
 #pragma unroll
             for (int e = 0; e < 8; e++)
-                K[e] = e * G + sub < cd ? full_key(__ldg(g.pk + cs + e * G + sub), g.k0, g.k1) : 0ull;
-            group_keyed<G>(K, 0xFFu, sub, pk, kk, rest);
+                key[e] = e * G + sub < cd ? key_of(g, ord_at(g, cs + e * G + sub), cs + e * G + sub) : 0ull;
+            group_top_keyed<G, 8, KL>(key, 0xFFu, sub, pk, kk);
+            p = pk[0];
 #pragma unroll
-            for (int q = 0; q < 4; q++) p[q] = pk[q];
+            for (int q = 1; q < KL; q++) p = (sub & 7u) == (uint32_t)q ? pk[q] : p;
         }
-        const uint32_t mp = sub == 0 ? p[0] : sub == 1 ? p[1] : sub == 2 ? p[2] : p[3];
         uint32_t c = 0;
-        if (cd && sub < TOPN) c = __ldg(g.nbr + cs + mp);
+        if (cd && sub < KL) c = nbr_at(g, cs + p);
         if (i + ROWS < cnt) fetch(i + ROWS);
-        if (cd) {
-            const size_t at = (size_t)g.vbase + cv;
-            if (sub == 0) words<W>(a)[at] = word<W>(c, 0);
-            else if (sub < TOPN) reinterpret_cast<uint32_t*>(a.lst + at)[sub - 1] = c;
-            else if (sub == TOPN) reinterpret_cast<uint32_t*>(a.lst + at)[3] = 1u;
-        }
+        if (cd) put_group<W, KL>(words<W>(a), {a.lst, a.wide}, (size_t)g.vbase + cv, sub, c, 0, WIDE | MORE);
     }
 }
 
-// Up to MPW long-row tasks (a row of more than LIST_WARP entries, or a
-// LIST_CHUNK-entry chunk of one longer than that), the warp together: 128
-// entries a step, the next 128 (of the next task, if need be) on their way.  A
-// step whose entries all lie below the fourth-heaviest seen so far costs a
-// maximum and a vote; an entry that does not is put in with a warp maximum.
+// Long-row tasks (a row of more than LIST_WARP entries, or a LIST_CHUNK-entry chunk of
+// one longer than that), the warp together: 256 entries a step in 16-byte loads, the
+// next step's on their way.  An entry is compared as its ord(w) with the low three
+// bits replaced by its place among the lane's eight; equal ones above those bits
+// are a tie.  The first step's list comes from the lanes' ordered eights; a later
+// step whose entries all lie below the list costs a maximum and a vote, and one that
+// does not is put in with a warp maximum.
 template <class W>
-__device__ void top_long(const ListArgs& a, const ListSeg& g, uint32_t t0, uint32_t cnt) {
+__device__ __forceinline__ void top_long(const ListArgs& a, const ListSeg& g, uint32_t t) {
     const uint32_t lane = threadIdx.x & 31;
-    uint4 d4 = make_uint4(0, 0, 0, 0);
-    if (lane < cnt) d4 = __ldg(g.task + t0 + lane);
-    // task k: row vertex, [s, e) of the pass
-    auto bounds = [&](uint32_t k, uint32_t& v, uint32_t& s, uint32_t& e, uint32_t& len, uint32_t& c) {
-        v = __shfl_sync(FULL, d4.x, k);
-        const uint32_t rs = __shfl_sync(FULL, d4.y, k);
-        len = __shfl_sync(FULL, d4.z, k);
-        c = __shfl_sync(FULL, d4.w, k);
-        s = rs + c * LIST_CHUNK;
-        e = rs + min(len, (c + 1) * LIST_CHUNK);
-        if (len <= LIST_CHUNK) e = rs + len;
-    };
-    auto load = [&](uint32_t x[4], uint32_t pos, uint32_t e) {
+    const uint4 d4 = __ldg(g.task + t);
+    const uint32_t v = d4.x, len = d4.z, c = d4.w;
+    const bool whole = len <= LIST_CHUNK;
+    const uint32_t s = d4.y + c * LIST_CHUNK, e = whole ? d4.y + len : d4.y + min(len, (c + 1) * LIST_CHUNK);
+    LaneTop32 top;
+    // pairs start at an even entry (the array is 256-byte aligned)
+    auto load = [&](uint32_t y[8], uint64_t pos) {
+        if (pos >= s && pos + 256 <= e) {
 #pragma unroll
-        for (int q = 0; q < 4; q++) {
-            const uint32_t i = pos + 32 * q + lane;
-            x[q] = (i < e && i >= pos) ? hi32(g.pk, i) : 0u;
-        }
-    };
-    uint32_t v, s, e, len, c;
-    bounds(0, v, s, e, len, c);
-    uint32_t x[4], nx[4];
-    load(x, s, e);
-    uint32_t pos = s, k = 0;
-    Top32 t;
-    bool tie = false;
-    // the neighbours of the previous row's four are stored when the next row is done,
-    // so that their loads do not stall the steps between
-    uint32_t pend_v = NIL, pend_c = NIL;
-    auto flush = [&]() {
-        if (pend_v != NIL) {
-            const size_t at = (size_t)g.vbase + pend_v;
-            if (lane == 0) words<W>(a)[at] = word<W>(pend_c, 0);
-            else if (lane < TOPN) reinterpret_cast<uint32_t*>(a.lst + at)[lane - 1] = pend_c;
-            else if (lane == TOPN) reinterpret_cast<uint32_t*>(a.lst + at)[3] = 1u;
-            pend_v = NIL;
+            for (int q = 0; q < 4; q++) {
+                const uint4 w = __ldg(reinterpret_cast<const uint4*>(g.ent + pos + 64 * q + 2 * lane));
+                y[2 * q] = w.y;
+                y[2 * q + 1] = w.w;
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < 8; q++) {
+                const uint64_t i = pos + 64 * (q >> 1) + 2 * lane + (q & 1);
+                y[q] = i >= s && i < e ? ord_at(g, (uint32_t)i) : 0u;
+            }
         }
     };
-    for (;;) {
-        // where the next step reads
-        uint32_t nv = v, ns = s, ne = e, nlen = len, nc = c, npos = pos + 128, nk = k;
-        if (npos >= e || npos < pos) {
-            nk = k + 1;
-            if (nk < cnt) {
-                bounds(nk, nv, ns, ne, nlen, nc);
-                npos = ns;
-            }
-        }
-        if (nk < cnt) load(nx, npos, ne);
-        if (!tie) {
-            uint32_t m = max(max(x[0], x[1]), max(x[2], x[3]));
-            while (__any_sync(FULL, m && m >= t.o3)) {
-                const uint32_t h = __reduce_max_sync(FULL, m);
-                const uint32_t own = __ballot_sync(FULL, m == h);
-                const uint32_t eq = (uint32_t)(x[0] == h) + (x[1] == h) + (x[2] == h) + (x[3] == h);
-                const int L = __ffs(own) - 1;
-                if (t.has(h) || (own & (own - 1)) || __shfl_sync(FULL, eq, L) > 1) {
-                    tie = true;
-                    break;
-                }
-                const uint32_t q = x[0] == h ? 0u : x[1] == h ? 1u : x[2] == h ? 2u : 3u;
-                t.add(h, __shfl_sync(FULL, pos + 32 * q + lane, L));
-                if ((int)lane == L) {
+    // the entry a packed number of lane L stands for
+    auto place = [&](uint32_t pos, uint32_t h, uint32_t L) {
+        const uint32_t z = 7u - (h & 7u);
+        return pos + 64 * (z >> 1) + 2 * L + (z & 1);
+    };
+    uint32_t x[8], y[8];
+    uint64_t pos = s & ~1u;
+    load(x, pos);
+    load(y, pos + 256);
+    bool tie;
+    {
 #pragma unroll
-                    for (int z = 0; z < 4; z++)
-                        if (x[z] == h) x[z] = 0;
-                    m = max(max(x[0], x[1]), max(x[2], x[3]));
-                }
-            }
-        }
-        if (nk != k) {
-            // the task's four, in order, one to a lane
-            uint32_t p;
-            if (tie) {
-                Top64 kt;
-                warp_top_keyed(g, s, e, kt);
-                p = lane == 0 ? kt.p0 : lane == 1 ? kt.p1 : lane == 2 ? kt.p2 : kt.p3;
-            } else {
-                // (a row or chunk may hold fewer than four entries: a chunk's remainder)
-                const uint32_t oo = lane == 0 ? t.o0 : lane == 1 ? t.o1 : lane == 2 ? t.o2 : t.o3;
-                p = lane == 0 ? t.p0 : lane == 1 ? t.p1 : lane == 2 ? t.p2 : t.p3;
-                if (!oo) p = NIL;
-            }
-            flush();
-            if (len <= LIST_CHUNK) {
-                pend_v = v;
-                pend_c = lane < TOPN ? __ldg(g.nbr + p) : 0u;
-            } else {
-                // a chunk: its four with their full keys; the last chunk of the row to
-                // finish merges all of them
-                const uint32_t first = t0 + k - c;   // the row's chunk 0 in the task list
-                const uint32_t nch = (len + LIST_CHUNK - 1) / LIST_CHUNK;
-                if (lane < TOPN) {
-                    uint4 rec = make_uint4(0, 0, NIL, 0);
-                    if (p != NIL) {
-                        const uint64_t K = full_key(__ldg(g.pk + p), g.k0, g.k1);
-                        rec = make_uint4((uint32_t)K, (uint32_t)(K >> 32), __ldg(g.nbr + p), 0);
-                    }
-                    a.part[((size_t)g.lbase + t0 + k) * TOPN + lane] = rec;
-                }
-                __syncwarp();
-                uint32_t old = 0;
-                if (lane == 0) old = atom_add_acq_rel(&a.pcnt[(size_t)g.lbase + first], 1u);
-                old = __shfl_sync(FULL, old, 0);
-                __syncwarp();
-                if (old == nch - 1) {
-                    Top64 kt;
-                    const uint4* P = a.part + ((size_t)g.lbase + first) * TOPN;
-                    for (uint32_t b = 0; b < nch * TOPN; b += 32) {
-                        uint4 rec = make_uint4(0, 0, NIL, 0);
-                        if (b + lane < nch * TOPN) rec = __ldcg(P + b + lane);
-                        warp_add(kt, ((uint64_t)rec.y << 32) | rec.x, rec.z);
-                    }
-                    if (lane == 0) {
-                        a.pcnt[(size_t)g.lbase + first] = 0;
-                        put_row<W>(a, (size_t)g.vbase + v, kt.p0, kt.p1, kt.p2, kt.p3, true);
-                    }
-                }
-            }
-            t = Top32();
-            tie = false;
-            if (nk >= cnt) break;
-        }
+        for (uint32_t z = 0; z < 8; z++) x[z] = packed(x[z], z, 7u);
+        order<8>(x);
+        uint32_t prev = ~0u, left = 0;
+        bool same = false;
 #pragma unroll
-        for (int q = 0; q < 4; q++) x[q] = nx[q];
-        v = nv; s = ns; e = ne; len = nlen; c = nc; pos = npos; k = nk;
+        for (int i = 0; i <= KL; i++) {
+            const uint32_t h = __reduce_max_sync(FULL, x[0]);
+            const uint32_t own = __ballot_sync(FULL, x[0] == h);
+            same |= h > 7u && ((prev ^ h) <= 7u || (own & (own - 1)));
+            prev = h;
+            if (i == KL) { left = h; break; }
+            const uint32_t L = __ffs(own) - 1;
+            if (h > 7u && (int)lane == i) {
+                top.o = h & ~7u;
+                top.p = place((uint32_t)pos, h, L);
+            }
+            const bool mine = lane == L;
+#pragma unroll
+            for (int z = 0; z < 7; z++) x[z] = mine ? x[z + 1] : x[z];
+            x[7] = mine ? 0u : x[7];
+        }
+        (void)left;
+        tie = same;
     }
-    flush();
+    uint32_t bar = max(top.last(), 8u);
+    auto step = [&](uint32_t w[8]) {
+        uint32_t m = max(max(max(w[0], w[1]), max(w[2], w[3])), max(max(w[4], w[5]), max(w[6], w[7])));
+        if (!__any_sync(FULL, m >= bar)) return;
+#pragma unroll
+        for (uint32_t z = 0; z < 8; z++) w[z] = packed(w[z], z, 7u);
+        for (;;) {
+            m = max(max(max(w[0], w[1]), max(w[2], w[3])), max(max(w[4], w[5]), max(w[6], w[7])));
+            const uint32_t h = __reduce_max_sync(FULL, m);
+            if (h < bar) return;
+            const uint32_t own = __ballot_sync(FULL, m == h);
+            if (__any_sync(FULL, top.o == (h & ~7u)) || (own & (own - 1))) {
+                tie = true;
+                return;
+            }
+            top.put(h & ~7u, place((uint32_t)pos, h, __ffs(own) - 1));
+#pragma unroll
+            for (int z = 0; z < 8; z++) w[z] = m == h && w[z] == h ? 0u : w[z];
+            bar = max(top.last(), 8u);
+        }
+    };
+    pos += 256;
+    while (pos < e && !tie) {
+        load(x, pos + 256);
+        step(y);
+        pos += 256;
+        if (pos >= e || tie) break;
+        load(y, pos + 256);
+        step(x);
+        pos += 256;
+    }
+    uint32_t p = top.p;
+    if (tie) {
+        LaneTop64 kt;
+        for (uint32_t b = s; b < e; b += 32) {
+            const uint32_t i = b + lane;
+            kt.offer(i < e && i >= b ? key_of(g, ord_at(g, i), i) : 0ull, i);
+        }
+        p = kt.n;
+    }
+    if (lane >= KL) p = NIL;
+    if (whole) {
+        put_lanes<W>(words<W>(a), {a.lst, a.wide}, (size_t)g.vbase + v, lane, p != NIL ? nbr_at(g, p) : NIL, 0, true);
+        return;
+    }
+    // a chunk: its list with the full keys; the last chunk of the row to finish merges all
+    const uint32_t first = t - c;   // the row's chunk 0 in the task list
+    const uint32_t nch = (len + LIST_CHUNK - 1) / LIST_CHUNK;
+    if (lane < KL) {
+        uint4 rec = make_uint4(0, 0, NIL, 0);
+        if (p != NIL) {
+            const uint64_t K = key_of(g, ord_at(g, p), p);
+            rec = make_uint4((uint32_t)K, (uint32_t)(K >> 32), nbr_at(g, p), 0);
+        }
+        a.part[((size_t)g.lbase + t) * KL + lane] = rec;
+    }
+    __syncwarp();
+    uint32_t old = 0;
+    if (lane == 0) old = atom_add_acq_rel(&a.pcnt[(size_t)g.lbase + first], 1u);
+    old = __shfl_sync(FULL, old, 0);
+    __syncwarp();
+    if (old != nch - 1) return;
+    LaneTop64 kt;
+    const uint4* P = a.part + ((size_t)g.lbase + first) * KL;
+    for (uint32_t b = 0; b < nch * KL; b += 32) {
+        uint4 rec = make_uint4(0, 0, NIL, 0);
+        if (b + lane < nch * KL) rec = __ldcg(P + b + lane);
+        kt.offer(((uint64_t)rec.y << 32) | rec.x, rec.z);
+    }
+    if (lane == 0) a.pcnt[(size_t)g.lbase + first] = 0;
+    put_lanes<W>(words<W>(a), {a.lst, a.wide}, (size_t)g.vbase + v, lane, kt.n, 0, true);
 }
 
 // Blocks of k_top for one graph, in this order: long tasks, rows of a warp, rows of a
@@ -514,11 +527,12 @@ __host__ __device__ __forceinline__ TopBlocks top_blocks(const uint32_t task[4],
     return b;
 }
 
+#ifndef LM_TMINB
+#define LM_TMINB 6
+#endif
 // Every block also clears its share of the result, and block 0 resets the job's state.
 template <class W>
-__global__ void __launch_bounds__(TT) k_top(const ListArgs* __restrict__ pa) {
-    extern __shared__ __align__(16) unsigned char top_raw[];
-    TopSmem& S = *reinterpret_cast<TopSmem*>(top_raw);
+__global__ void __launch_bounds__(TT, LM_TMINB) k_top(const ListArgs* __restrict__ pa) {
     const ListArgs& a = *pa;
     const uint32_t tid = threadIdx.x, warp = tid >> 5;
     if (blockIdx.x == 0) {
@@ -545,7 +559,7 @@ __global__ void __launch_bounds__(TT) k_top(const ListArgs* __restrict__ pa) {
     const TopBlocks nb = top_blocks(g.ntask, g.nrows);
     if (b < nb.l) {
         const uint32_t t0 = (b * TWARPS + warp) * MPW;
-        if (t0 < g.ntask[1]) top_long<W>(a, g, t0, min(MPW, g.ntask[1] - t0));
+        for (uint32_t t = t0; t < min(t0 + MPW, g.ntask[1]); t++) top_long<W>(a, g, t);
     } else if ((b -= nb.l) < nb.w) {
         const uint32_t t0 = g.ntask[1] + (b * TWARPS + warp) * WPW;
         if (t0 < g.ntask[2]) top_group<W, 32>(a, g, t0, min(WPW, g.ntask[2] - t0));
@@ -553,72 +567,69 @@ __global__ void __launch_bounds__(TT) k_top(const ListArgs* __restrict__ pa) {
         const uint32_t t0 = g.ntask[2] + (b * TWARPS + warp) * GPW;
         if (t0 < g.ntask[3]) top_group<W, 8>(a, g, t0, min(GPW, g.ntask[3] - t0));
     } else {
-        const uint32_t r0 = (b - nb.g) * TT + warp * 32;
-        if (r0 < g.nrows) top_short<W>(a, g, r0, S.o[warp], S.n[warp]);
+        top_short<W>(a, g, (b - nb.g) * TT + tid);
     }
 }
 
 // ---------------------------------------------------------------- refills
-// The four heaviest live entries of rows of at most 8 G entries, a group of G lanes
+// The K heaviest live entries of rows of at most G E entries, a group of G lanes
 // each; d = 0: no row.  Returns whether one is left (uniform over the group).
-template <class W, int G>
-__device__ __forceinline__ bool refill_group(const ListArgs& a, const ListSeg& g, uint32_t v, uint32_t s, uint32_t d) {
-    constexpr uint32_t MASK = 8 * G - 1;
+template <class W, int G, int E, int K>
+__device__ __forceinline__ bool refill_group(const ListSeg& g, W* cur, const RowLists& R, uint32_t v, uint32_t s,
+                                             uint32_t d) {
+    static_assert(G >= 4 && (K == KS || G >= 8), "a lane for every place");
+    constexpr uint32_t MASK = G * E - 1;
     constexpr bool ROUNDS = sizeof(W) == 8;
     const uint32_t sub = threadIdx.x & (G - 1);
-    W* cur = words<W>(a) + g.vbase;
-    uint4* lst = a.lst + g.vbase;
-    uint32_t x[8], n[8], live = 0;
-    W t[8];
+    uint32_t x[E], live = 0;
+    W t[E];
+    {
+        uint32_t n[E];
 #pragma unroll
-    for (int e = 0; e < 8; e++) {
-        const bool in = e * G + sub < d;
-        x[e] = in ? hi32(g.pk, s + e * G + sub) : 0u;
-        n[e] = in ? __ldg(g.nbr + s + e * G + sub) : 0u;
+        for (int e = 0; e < E; e++) {
+            const uint64_t w = e * G + sub < d ? __ldg(g.ent + s + e * G + sub) : 0ull;
+            x[e] = (uint32_t)(w >> 32);
+            n[e] = (uint32_t)w;
+        }
+#pragma unroll
+        for (int e = 0; e < E; e++) t[e] = e * G + sub < d ? look(cur + n[e]) : (W)DEAD;
     }
 #pragma unroll
-    for (int e = 0; e < 8; e++) t[e] = e * G + sub < d ? look(cur + n[e]) : (W)DEAD;
-#pragma unroll
-    for (int e = 0; e < 8; e++)
+    for (int e = 0; e < E; e++)
         if (!(lo(t[e]) & DEAD)) live |= 1u << e;
-    uint32_t p[4];
+    uint32_t p[K];
     bool rest = false, exact = ROUNDS;
     uint32_t passed = 0;
     if (!ROUNDS) {
-        TopP q;
+        uint32_t y[E], r[K];
 #pragma unroll
-        for (int e = 0; e < 8; e++) q.add(((live >> e) & 1u) ? packed(x[e], e * G + sub, MASK) : 0u);
-        q.across<G>();
+        for (int e = 0; e < E; e++) y[e] = packed(((live >> e) & 1u) ? x[e] : 0u, e * G + sub, MASK);
+        const uint32_t out = group_top<G, E, K>(y, r);
 #pragma unroll
-        for (int i = 0; i < 4; i++) p[i] = q.k[i] ? MASK - (q.k[i] & MASK) : NIL;
-        rest = q.out != 0;
-        exact = __any_sync(FULL, q.tied(MASK));
+        for (int i = 0; i < K; i++) p[i] = r[i] > MASK ? MASK - (r[i] & MASK) : NIL;
+        rest = out > MASK;
+        exact = __any_sync(FULL, any_tie<K>(r, out, MASK));
     }
     if (exact) {
-        uint64_t K[8], k[4];
+        uint64_t key[E], k[K];
 #pragma unroll
-        for (int e = 0; e < 8; e++)
-            K[e] = e * G + sub < d ? full_key(__ldg(g.pk + s + e * G + sub), g.k0, g.k1) : 0ull;
-        group_keyed<G>(K, live, sub, p, k, rest);
+        for (int e = 0; e < E; e++) key[e] = e * G + sub < d ? key_of(g, x[e], s + e * G + sub) : 0ull;
+        rest = group_top_keyed<G, E, K>(key, live, sub, p, k);
         if (ROUNDS) {
             // the latest round among the matched neighbours above the new candidate; the
             // list ends at the heaviest matched one below it, whose round counts for
             // every candidate after that
             uint64_t cut = 0;
 #pragma unroll
-            for (int e = 0; e < 8; e++) {
+            for (int e = 0; e < E; e++) {
                 if (e * G + sub >= d || ((live >> e) & 1u)) continue;
-                if (K[e] > k[0]) passed = max(passed, info(t[e]));
-                else cut = K[e] > cut ? K[e] : cut;
+                if (key[e] > k[0]) passed = max(passed, info(t[e]));
+                else cut = key[e] > cut ? key[e] : cut;
             }
+            passed = group_max<G>(passed);
+            cut = group_max64<G>(cut);
 #pragma unroll
-            for (int z = 1; z < G; z <<= 1) {
-                passed = max(passed, __shfl_xor_sync(FULL, passed, z));
-                const uint64_t o = __shfl_xor_sync(FULL, cut, z);
-                cut = o > cut ? o : cut;
-            }
-#pragma unroll
-            for (int i = 1; i < 4; i++)
+            for (int i = 1; i < K; i++)
                 if (p[i] != NIL && k[i] < cut) {
                     p[i] = NIL;
                     rest = true;
@@ -626,52 +637,46 @@ __device__ __forceinline__ bool refill_group(const ListArgs& a, const ListSeg& g
         }
     }
     if (d && p[0] != NIL) {
-        const uint32_t mp = sub == 0 ? p[0] : sub == 1 ? p[1] : sub == 2 ? p[2] : p[3];
+        uint32_t mp = p[0];
+#pragma unroll
+        for (int i = 1; i < K; i++) mp = sub == (uint32_t)i ? p[i] : mp;
         uint32_t c = NIL;
-        if (sub < TOPN && mp != NIL) c = __ldg(g.nbr + s + mp);
-        if (sub == 0) {
-            cur[v] = word<W>(c, ROUNDS ? max(passed, info(look(cur + v))) : 0u);
-            lst[v].w = rest ? 1u : 0u;
-        } else if (sub < TOPN) {
-            reinterpret_cast<uint32_t*>(lst + v)[sub - 1] = c;
-        }
+        if (sub < K && mp != NIL) c = nbr_at(g, s + mp);
+        put_group<W, K>(cur, R, v, sub, c, ROUNDS && sub == 0 ? max(passed, info(look(cur + v))) : 0u,
+                        (K == KL ? WIDE : 0u) | (rest ? MORE : 0u));
         return true;
     }
     return false;
 }
 
 // The same for longer rows: part `q` of `parts` of the row's 128-entry steps by this
-// warp.  Only entries at or above the fourth-heaviest live one so far have their end
-// looked up.
+// warp.  Only entries at or above the last of the list so far have their end looked up.
 template <class W>
 __device__ __forceinline__ void refill_scan(const ListSeg& g, const W* cur, uint32_t s, uint32_t d, uint32_t q,
-                                            uint32_t parts, Top64& t) {
+                                            uint32_t parts, LaneTop64& t) {
     const uint32_t lane = threadIdx.x & 31;
     const uint64_t stride = 128ull * parts;
-    uint32_t x[4], nx[4];
-    auto load = [&](uint32_t y[4], uint64_t b) {
+    uint64_t x[4], nx[4];
+    auto load = [&](uint64_t y[4], uint64_t b) {
 #pragma unroll
-        for (int i = 0; i < 4; i++) y[i] = b + 32 * i + lane < d ? hi32(g.pk, s + (uint32_t)b + 32 * i + lane) : 0u;
+        for (int i = 0; i < 4; i++) y[i] = b + 32 * i + lane < d ? __ldg(g.ent + s + (uint32_t)b + 32 * i + lane) : 0ull;
     };
     load(x, 128ull * q);
+    uint32_t bar = 1;
     for (uint64_t b = 128ull * q; b < d; b += stride) {
         load(nx, b + stride);
-        const uint32_t bar = (uint32_t)(t.k3 >> 32);
-        uint32_t m = max(max(x[0], x[1]), max(x[2], x[3]));
-        if (__any_sync(FULL, m && m >= bar)) {
-            uint32_t n[4];
+        const uint64_t m01 = x[0] > x[1] ? x[0] : x[1], m23 = x[2] > x[3] ? x[2] : x[3];
+        if (__any_sync(FULL, (uint32_t)((m01 > m23 ? m01 : m23) >> 32) >= bar)) {
             W y[4];
-            uint64_t key[4];
 #pragma unroll
-            for (int i = 0; i < 4; i++) n[i] = x[i] && x[i] >= bar ? __ldg(g.nbr + s + (uint32_t)b + 32 * i + lane) : NIL;
+            for (int i = 0; i < 4; i++) y[i] = (uint32_t)(x[i] >> 32) >= bar ? look(cur + (uint32_t)x[i]) : (W)DEAD;
 #pragma unroll
             for (int i = 0; i < 4; i++) {
-                y[i] = n[i] != NIL ? look(cur + n[i]) : (W)DEAD;
-                key[i] = n[i] != NIL ? __ldg(g.pk + s + (uint32_t)b + 32 * i + lane) : 0ull;
+                const bool on = !(lo(y[i]) & DEAD) && (uint32_t)(x[i] >> 32) >= bar;
+                if (!__any_sync(FULL, on)) continue;
+                t.offer(on ? key_of(g, (uint32_t)(x[i] >> 32), s + (uint32_t)b + 32 * i + lane) : 0ull, (uint32_t)x[i]);
+                bar = max((uint32_t)(t.last() >> 32), 1u);
             }
-#pragma unroll
-            for (int i = 0; i < 4; i++)
-                warp_add(t, !(lo(y[i]) & DEAD) ? full_key(key[i], g.k0, g.k1) : 0ull, n[i]);
         }
 #pragma unroll
         for (int i = 0; i < 4; i++) x[i] = nx[i];
@@ -688,59 +693,353 @@ __device__ __forceinline__ Passed refill_passed(const ListSeg& g, const uint64_t
     uint32_t r = 0;
     uint64_t cut = 0;
     for (uint64_t i = 32ull * q + (threadIdx.x & 31); i < d; i += 32ull * parts) {
-        const uint64_t w = __ldg(g.pk + s + (uint32_t)i);
+        const uint64_t w = __ldg(g.ent + s + (uint32_t)i);
         if ((uint32_t)(w >> 32) < (uint32_t)(low >> 32)) continue;
-        const uint64_t y = look(cur + __ldg(g.nbr + s + (uint32_t)i));
+        const uint64_t y = look(cur + (uint32_t)w);
         if (!(lo(y) & DEAD)) continue;
-        const uint64_t key = full_key(w, g.k0, g.k1);
+        const uint64_t key = key_of(g, (uint32_t)(w >> 32), s + (uint32_t)i);
         if (key > k0) r = max(r, info(y));
         else if (key > cut) cut = key;
     }
     r = __reduce_max_sync(FULL, r);
-    const uint32_t hi = __reduce_max_sync(FULL, (uint32_t)(cut >> 32));
-    const uint32_t l = __reduce_max_sync(FULL, ((uint32_t)(cut >> 32) == hi) ? (uint32_t)cut : 0u);
-    return {r, ((uint64_t)hi << 32) | l};
+    return {r, group_max64<32>(cut)};
 }
+// t: lanes 0 .. KL - 1; the list ends at ps.cut
 template <class W>
-__device__ __forceinline__ void refill_put(W* cur, uint4* lst, uint32_t v, const Top64& t, const Passed& ps) {
-    cur[v] = word<W>(t.p0, sizeof(W) == 8 ? max(ps.round, info(look(cur + v))) : 0u);
-    // (with four live ones there may be more of them; the list ends at ps.cut)
-    lst[v] = make_uint4(t.k1 > ps.cut ? t.p1 : NIL, t.k2 > ps.cut ? t.p2 : NIL, t.k3 > ps.cut ? t.p3 : NIL,
-                        t.k3 || (t.k1 && t.k1 <= ps.cut) || (t.k2 && t.k2 <= ps.cut) ? 1u : 0u);
+__device__ __forceinline__ void refill_put(W* cur, const RowLists& R, uint32_t v, const LaneTop64& t, const Passed& ps) {
+    const uint32_t lane = threadIdx.x & 31;
+    const bool in = lane < KL && t.k && (lane == 0 || t.k > ps.cut);
+    // (with a full list, or a cut one, there may be more)
+    const bool more = __any_sync(FULL, lane < KL && t.k && (lane == KL - 1 || !in));
+    uint32_t inf = 0;
+    if (sizeof(W) == 8 && lane == 0) inf = max(ps.round, info(look(cur + v)));
+    put_lanes<W>(cur, R, v, lane, in ? t.n : NIL, inf, more);
 }
 
 // ---------------------------------------------------------------- k_live
-constexpr int LT = 256, LV = 2;
+#ifndef LM_LT
+#define LM_LT 128
+#endif
+#ifndef LM_LV
+#define LM_LV 1
+#endif
+#ifndef LM_LMINB
+#define LM_LMINB 10
+#endif
+constexpr int LT = LM_LT, LV = LM_LV, LW = LT / 32;
 constexpr uint32_t BLOCK_ROW = 1024;  // longer rows are refilled by the whole block
 constexpr uint32_t IDLE_MAX = 48;     // passes without a change before a block gives its rows back
 
-struct LiveSmem {
-    Top64 top[LT / 32];
-    uint64_t cut[LT / 32];
-    uint32_t passed[LT / 32];
-    uint32_t part, nlive, nq0, nq1, nq2, changed, stop;
-    uint32_t red[LT / 32];
-};
-
-// append the warp's rows (one a lane where on)
-__device__ __forceinline__ void warp_append(uint32_t* ctr, uint32_t* out, bool on, uint32_t v) {
+// places for the lanes that are on, from a counter
+__device__ __forceinline__ uint32_t warp_slot(uint32_t* ctr, bool on) {
     const uint32_t b = __ballot_sync(FULL, on);
-    if (!b) return;
+    if (!b) return 0;
     uint32_t base = 0;
     if ((threadIdx.x & 31) == 0) base = atomicAdd(ctr, (uint32_t)__popc(b));
-    base = __shfl_sync(FULL, base, 0);
-    if (on) out[base + __popc(b & lanemask_lt())] = v;
+    return __shfl_sync(FULL, base, 0) + __popc(b & lanemask_lt());
+}
+__device__ __forceinline__ void warp_append(uint32_t* ctr, uint32_t* out, bool on, uint32_t v) {
+    const uint32_t q = warp_slot(ctr, on);
+    if (on) out[q] = v;
 }
 
-// Blocks take parts (consecutive rows of one graph) from a counter and pass over a
-// part's live rows, compacted after every pass in the part's own range of the list
-// buffers, until none is left.  A part may wait for words that another block writes,
-// but no block waits for good: after IDLE_MAX passes without a change it puts
-// the part's rows back for the next launch, which the last block to leave asks for.
+// A part: consecutive rows of one graph, its live rows compacted in its own range of
+// the list buffers, its rows to refill in its range of the queue (vertex, row
+// offset, length; rows of at most LIST_SHORT entries from the front, longer ones from
+// the back).
 template <class W>
-__global__ void __launch_bounds__(LT, 4) k_live(const ListArgs* __restrict__ pa, cudaGraphConditionalHandle h,
-                                                uint32_t in_graph) {
+struct Part {
+    const ListSeg& g;
+    W* cur;
+    RowLists R;
+    uint4* queue;
+    uint32_t from, rows;  // its rows of the graph
+    size_t home;          // first slot of the part
+    __device__ __forceinline__ Part(const ListArgs& a, const ListSeg& seg, uint32_t part) : g(seg) {
+        const uint32_t per = (g.nrows + g.nparts - 1) / g.nparts;
+        from = min(g.nrows, (part - g.part0) * per);
+        rows = min(g.nrows, from + per) - from;
+        home = (size_t)g.vbase + from;
+        cur = words<W>(a) + g.vbase;
+        R = {a.lst + g.vbase, a.wide + g.vbase};
+        queue = a.queue + home;
+    }
+};
+struct PartCounts {
+    uint32_t live, nshort, nlong;
+};
+struct Tally {
+    uint32_t matched = 0, last = 0;   // rows matched; 1 + their latest round
+    bool changed = false;
+};
+
+// One pass over `cnt` live rows by the block, LV to a thread and step: a row that is
+// chosen back is matched, one whose candidate is matched to another moves on in its
+// list; live rows go to `out`, rows with a used-up list to the queue.
+template <class W>
+__device__ __forceinline__ void poll_rows(const ListArgs& a, const Part<W>& P, const uint32_t* list, uint32_t cnt,
+                                          uint32_t* out, PartCounts& S, Tally& T) {
     constexpr bool ROUNDS = sizeof(W) == 8;
+    const ListSeg& g = P.g;
+    W* cur = P.cur;
+    uint32_t v[LV], nv[LV];
+    W w[LV], nw[LV], t[LV];
+    uint4 l[LV], nl[LV];
+    // the next rows' words and lists are on their way while these are decided
+    auto fetch = [&](uint32_t base) {
+#pragma unroll
+        for (int i = 0; i < LV; i++) {
+            const uint32_t at = base + i * LT + threadIdx.x;
+            nv[i] = at < cnt ? list[at] : NIL;
+        }
+    };
+    auto fetch_words = [&]() {
+#pragma unroll
+        for (int i = 0; i < LV; i++) {
+            nw[i] = nv[i] != NIL ? look(cur + nv[i]) : (W)0;
+            nl[i] = nv[i] != NIL ? P.R.lst[nv[i]] : make_uint4(NIL, NIL, NIL, 0);
+        }
+    };
+    fetch(0);
+    fetch_words();
+    for (uint32_t base = 0; base < cnt; base += LT * LV) {
+        bool gone[LV];
+#pragma unroll
+        for (int i = 0; i < LV; i++) {
+            v[i] = nv[i];
+            w[i] = nw[i];
+            l[i] = nl[i];
+        }
+#pragma unroll
+        for (int i = 0; i < LV; i++) {
+            if (v[i] != NIL && lo(w[i]) >= g.n) { set_err(a.st, ERR_BOUNDS, lo(w[i])); v[i] = NIL; }
+            t[i] = v[i] != NIL ? look(cur + lo(w[i])) : (W)0;
+        }
+        fetch(base + LT * LV);
+#pragma unroll
+        for (int i = 0; i < LV; i++)
+            gone[i] = v[i] != NIL && (lo(t[i]) & DEAD) && (lo(t[i]) & VMASK) != v[i];
+        W n[LV][3];
+#pragma unroll
+        for (int i = 0; i < LV; i++) {
+            n[i][0] = gone[i] && l[i].x != NIL ? look(cur + l[i].x) : (W)DEAD;
+            n[i][1] = gone[i] && l[i].y != NIL ? look(cur + l[i].y) : (W)DEAD;
+            n[i][2] = gone[i] && l[i].z != NIL ? look(cur + l[i].z) : (W)DEAD;
+        }
+        fetch_words();
+#pragma unroll
+        for (int i = 0; i < LV; i++) {
+            bool live = v[i] != NIL, refill = false;
+            uint32_t s = 0, d = 0;
+            if (live) {
+                uint32_t u = lo(w[i]), passed = info(w[i]);
+                W y = t[i];
+                if (gone[i]) {
+                    T.changed = true;
+                    // the first of the list that is not matched (an empty place: DEAD, no round)
+                    const bool d0 = lo(n[i][0]) & DEAD, d1 = lo(n[i][1]) & DEAD, d2 = lo(n[i][2]) & DEAD;
+                    if (ROUNDS) {
+                        passed = max(passed, info(y));
+                        if (d0) passed = max(passed, info(n[i][0]));
+                        if (d0 && d1) passed = max(passed, info(n[i][1]));
+                        if (d0 && d1 && d2) passed = max(passed, info(n[i][2]));
+                    }
+                    const uint32_t at = v[i];
+                    if (!(d0 && d1 && d2)) {
+                        u = !d0 ? l[i].x : !d1 ? l[i].y : l[i].z;
+                        y = !d0 ? n[i][0] : !d1 ? n[i][1] : n[i][2];
+                        cur[v[i]] = word<W>(u, passed);
+                        P.R.lst[at] = make_uint4(!d0 ? l[i].y : !d1 ? l[i].z : NIL, !d0 ? l[i].z : NIL, NIL, l[i].w);
+                    } else {
+                        live = false;
+                        if (l[i].w & WIDE) {
+                            // the second half of a long row's list takes the first's place
+                            const uint4 l2 = P.R.wide[at];
+                            const W m0 = l2.x != NIL ? look(cur + l2.x) : (W)DEAD;
+                            const W m1 = l2.y != NIL ? look(cur + l2.y) : (W)DEAD;
+                            const W m2 = l2.z != NIL ? look(cur + l2.z) : (W)DEAD;
+                            const W m3 = l2.w != NIL ? look(cur + l2.w) : (W)DEAD;
+                            const bool e0 = lo(m0) & DEAD, e1 = e0 && (lo(m1) & DEAD), e2 = e1 && (lo(m2) & DEAD),
+                                       e3 = e2 && (lo(m3) & DEAD);
+                            if (ROUNDS) {
+                                if (e0) passed = max(passed, info(m0));
+                                if (e1) passed = max(passed, info(m1));
+                                if (e2) passed = max(passed, info(m2));
+                                if (e3) passed = max(passed, info(m3));
+                            }
+                            l[i].w &= ~WIDE;
+                            if (!e3) {
+                                live = true;
+                                u = !e0 ? l2.x : !e1 ? l2.y : !e2 ? l2.z : l2.w;
+                                y = !e0 ? m0 : !e1 ? m1 : !e2 ? m2 : m3;
+                                cur[v[i]] = word<W>(u, passed);
+                                P.R.lst[at] = make_uint4(!e0 ? l2.y : !e1 ? l2.z : !e2 ? l2.w : NIL,
+                                                       !e0 ? l2.z : !e1 ? l2.w : NIL, !e0 ? l2.w : NIL, l[i].w);
+                            }
+                        }
+                        refill = !live && (l[i].w & MORE);
+                        if (refill) {
+                            s = __ldg(g.off + v[i]);
+                            d = __ldg(g.off + v[i] + 1) - s;
+                            if (ROUNDS) cur[v[i]] = word<W>(u, passed);
+                        }
+                    }
+                }
+                if (live && (lo(y) & VMASK) == v[i]) {
+                    // chosen back
+                    uint32_t r = 0;
+                    if (ROUNDS) {
+                        // its word, if matched already, has the round; else both ends' passed ones give it
+                        r = (lo(y) & DEAD) ? info(y) : max(passed, info(y)) + 1u;
+                        T.last = max(T.last, r);
+                    }
+                    cur[v[i]] = word<W>(u | DEAD, r);
+                    g.dst[v[i]] = u;
+                    T.matched++;
+                    live = false;
+                    T.changed = true;
+                }
+            }
+            warp_append(&S.live, out, live, v[i]);
+            if (__any_sync(FULL, refill)) {
+                const bool few = refill && d <= LIST_SHORT, many = refill && d > LIST_SHORT;
+                const uint32_t q0 = warp_slot(&S.nshort, few), q1 = warp_slot(&S.nlong, many);
+                if (refill) P.queue[few ? q0 : P.rows - 1 - q1] = make_uint4(v[i], s, d, 0);
+            }
+        }
+    }
+}
+
+// the queued rows of a part by the block, its warps taking them from two counters; the
+// live ones join `out`
+struct RefillSmem {
+    uint64_t k[LW][KL];
+    uint32_t n[LW][KL];
+    uint64_t cut[LW];
+    uint32_t passed[LW];
+};
+template <class W>
+__device__ __forceinline__ void refill_rows(const ListArgs& a, const Part<W>& P, uint32_t k0, uint32_t k1,
+                                            uint32_t* out, uint32_t* nlive, uint32_t next[2], RefillSmem& S) {
+    constexpr bool ROUNDS = sizeof(W) == 8;
+    const ListSeg& g = P.g;
+    W* cur = P.cur;
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint4 none = make_uint4(0, 0, 0, 0);
+    auto take = [&](uint32_t* ctr, uint32_t k) {
+        uint32_t b = 0;
+        if (lane == 0) b = atomicAdd(ctr, k);
+        return __shfl_sync(FULL, b, 0);
+    };
+    bool huge = false;
+    // longer rows first
+    for (uint32_t b = take(&next[1], 2); b < k1; b = take(&next[1], 2)) {
+        // two rows by half a warp each if both are of at most 64 entries, else one by one
+        const uint32_t i = b + lane / 16;
+        const uint4 q2 = i < k1 ? P.queue[P.rows - 1 - i] : none;
+        if (__all_sync(FULL, q2.z <= 64)) {
+            const bool live = refill_group<W, 16, 4, KL>(g, cur, P.R, q2.x, q2.y, q2.z);
+            warp_append(nlive, out, live && (lane & 15) == 0, q2.x);
+            continue;
+        }
+        for (int k = 0; k < 2; k++) {
+            const uint32_t v = __shfl_sync(FULL, q2.x, 16 * k), s = __shfl_sync(FULL, q2.y, 16 * k),
+                           d = __shfl_sync(FULL, q2.z, 16 * k);
+            if (d == 0) continue;
+            if (d > BLOCK_ROW) {
+                huge = true;
+                continue;
+            }
+            bool live;
+            if (d <= 128) {
+                live = refill_group<W, 32, 4, KL>(g, cur, P.R, v, s, d);
+            } else {
+                LaneTop64 t;
+                refill_scan<W>(g, cur, s, d, 0, 1, t);
+                const uint64_t first = __shfl_sync(FULL, t.k, 0), last = t.last();
+                live = first != 0;
+                Passed ps = {0, 0};
+                if (ROUNDS && live)
+                    ps = refill_passed(g, reinterpret_cast<const uint64_t*>(cur), s, d, 0, 1, first, last);
+                if (live) refill_put<W>(cur, P.R, v, t, ps);
+            }
+            warp_append(nlive, out, live && lane == 0, v);
+        }
+    }
+    // rows of at most LIST_SHORT: eight at a time by four lanes each if they are of at
+    // most 16 entries, else four by eight lanes
+    for (uint32_t b = take(&next[0], 8); b < k0; b = take(&next[0], 8)) {
+        const uint32_t i = b + lane / 4;
+        const uint4 q = i < k0 ? P.queue[i] : none;
+        if (__all_sync(FULL, q.z <= 16)) {
+            const bool live = refill_group<W, 4, 4, KS>(g, cur, P.R, q.x, q.y, q.z);
+            warp_append(nlive, out, live && (lane & 3) == 0, q.x);
+            continue;
+        }
+        for (int h = 0; h < 2; h++) {
+            const int from = 16 * h + 4 * (lane / 8);
+            const uint32_t v = __shfl_sync(FULL, q.x, from), s = __shfl_sync(FULL, q.y, from),
+                           d = __shfl_sync(FULL, q.z, from);
+            const bool live = refill_group<W, 8, 4, KS>(g, cur, P.R, v, s, d);
+            warp_append(nlive, out, live && (lane & 7) == 0, v);
+        }
+    }
+    if (!__syncthreads_or(huge)) return;
+    for (uint32_t i = 0; i < k1; i++) {
+        const uint4 q4 = P.queue[P.rows - 1 - i];
+        const uint32_t v = q4.x, s = q4.y, d = q4.z;
+        if (d <= BLOCK_ROW) continue;
+        {
+            LaneTop64 t;
+            refill_scan<W>(g, cur, s, d, warp, LW, t);
+            if (lane < KL) {
+                S.k[warp][lane] = t.k;
+                S.n[warp][lane] = t.n;
+            }
+        }
+        __syncthreads();
+        LaneTop64 r;   // every warp merges all
+        for (uint32_t z = lane; z < LW * KL; z += 32) r.offer(S.k[z / KL][z % KL], S.n[z / KL][z % KL]);
+        static_assert(LW * KL % 32 == 0, "whole warps offer");
+        const uint64_t first = __shfl_sync(FULL, r.k, 0), last = r.last();
+        if (ROUNDS) {
+            if (first) {
+                const Passed x = refill_passed(g, reinterpret_cast<const uint64_t*>(cur), s, d, warp, LW, first, last);
+                if (lane == 0) {
+                    S.passed[warp] = x.round;
+                    S.cut[warp] = x.cut;
+                }
+            }
+            __syncthreads();
+        }
+        if (warp == 0) {
+            Passed ps = {0, 0};
+            if (ROUNDS && first)
+                for (int w = 0; w < LW; w++) {
+                    ps.round = max(ps.round, S.passed[w]);
+                    ps.cut = S.cut[w] > ps.cut ? S.cut[w] : ps.cut;
+                }
+            if (first) refill_put<W>(cur, P.R, v, r, ps);
+            warp_append(nlive, out, first && lane == 0, v);
+        }
+        __syncthreads();
+    }
+}
+
+struct LiveSmem {
+    RefillSmem r;
+    PartCounts c;
+    uint32_t part, changed, stop, next[2];
+    uint32_t red[2][LW];
+};
+
+// Blocks take parts from a counter and pass over a part's live rows until none is
+// left.  A part may wait for words that another block writes, but no block waits for
+// good: after IDLE_MAX passes without a change it puts the part's rows back for the
+// next launch, which the last block to leave asks for.
+template <class W>
+__global__ void __launch_bounds__(LT, LM_LMINB) k_live(const ListArgs* __restrict__ pa, cudaGraphConditionalHandle h,
+                                                       uint32_t in_graph) {
     __shared__ LiveSmem S;
     const ListArgs& a = *pa;
     DevState* st = a.st;
@@ -753,27 +1052,17 @@ __global__ void __launch_bounds__(LT, 4) k_live(const ListArgs* __restrict__ pa,
         const uint32_t part = S.part;
         if (part >= a.nparts) break;
         const uint32_t si = a.pmap ? a.pmap[part] : 0u;
-        const ListSeg& g = a.segs[si];
-        const uint32_t per = (g.nrows + g.nparts - 1) / g.nparts;
-        const uint32_t from = min(g.nrows, (part - g.part0) * per);
-        uint32_t cnt = min(g.nrows, from + per) - from, buf = 0;
-        const uint32_t* list = g.vid + from;
-        const size_t home = (size_t)g.vbase + from;   // the part's range of the buffers
-        if (launch) {
-            cnt = a.pcount[part] >> 1;
-            buf = a.pcount[part] & 1u;
-            list = a.list[buf] + home;
-        }
-        W* cur = words<W>(a) + g.vbase;
-        uint4* lst = a.lst + g.vbase;
-        uint32_t matched = 0, last = 0, idle = 0;
+        const Part<W> P(a, a.segs[si], part);
+        const uint32_t pc = launch ? a.pcount[part] : P.rows << 1;
+        uint32_t cnt = pc >> 1, buf = pc & 1u;
+        const uint32_t* list = launch ? a.list[buf] + P.home : P.g.vid + P.from;
+        Tally T;
+        uint32_t idle = 0;
         for (uint32_t pass = 0; cnt; pass++) {
-            uint32_t* out = a.list[buf ^ 1u] + home;
-            uint32_t* q0 = a.queue[0] + home;     // rows to refill: short ones,
-            uint32_t* q1 = a.queue[1] + home;     // a warp's,
-            uint32_t* q2 = a.queue[2] + home;     // the block's
+            uint32_t* out = a.list[buf ^ 1u] + P.home;
             if (tid == 0) {
-                S.nlive = S.nq0 = S.nq1 = S.nq2 = 0;
+                S.c.live = S.c.nshort = S.c.nlong = 0;
+                S.next[0] = S.next[1] = 0;
                 S.changed = 0;
                 S.stop = 0;
                 if (globaltimer_ns() - st->t0_ns > a.limit_ns) {
@@ -784,160 +1073,16 @@ __global__ void __launch_bounds__(LT, 4) k_live(const ListArgs* __restrict__ pa,
                 }
             }
             __syncthreads();
-            bool changed = false;
-            for (uint32_t base = 0; base < cnt; base += LT * LV) {
-                uint32_t v[LV];
-                W w[LV], t[LV];
-                uint4 l[LV];
-#pragma unroll
-                for (int i = 0; i < LV; i++) {
-                    const uint32_t at = base + i * LT + tid;
-                    v[i] = at < cnt ? list[at] : NIL;
-                }
-#pragma unroll
-                for (int i = 0; i < LV; i++) {
-                    w[i] = v[i] != NIL ? look(cur + v[i]) : (W)0;
-                    l[i] = v[i] != NIL ? lst[v[i]] : make_uint4(NIL, NIL, NIL, 0);
-                }
-#pragma unroll
-                for (int i = 0; i < LV; i++) {
-                    if (v[i] != NIL && lo(w[i]) >= g.n) { set_err(st, ERR_BOUNDS, lo(w[i])); v[i] = NIL; }
-                    t[i] = v[i] != NIL ? look(cur + lo(w[i])) : (W)0;
-                }
-                W n[LV][3];
-#pragma unroll
-                for (int i = 0; i < LV; i++) {
-                    const bool gone = v[i] != NIL && (lo(t[i]) & DEAD) && (lo(t[i]) & VMASK) != v[i];
-                    n[i][0] = gone && l[i].x != NIL ? look(cur + l[i].x) : (W)DEAD;
-                    n[i][1] = gone && l[i].y != NIL ? look(cur + l[i].y) : (W)DEAD;
-                    n[i][2] = gone && l[i].z != NIL ? look(cur + l[i].z) : (W)DEAD;
-                }
-#pragma unroll
-                for (int i = 0; i < LV; i++) {
-                    bool live = false, refill = false;
-                    uint32_t d = 0;
-                    if (v[i] != NIL) {
-                        uint32_t u = lo(w[i]), passed = info(w[i]);
-                        W y = t[i];
-                        live = true;
-                        if ((lo(y) & DEAD) && (lo(y) & VMASK) != v[i]) {
-                            changed = true;
-                            const uint32_t c[3] = {l[i].x, l[i].y, l[i].z};
-                            passed = max(passed, info(y));
-                            int k = 0;
-                            for (; k < 3; k++) {
-                                if (c[k] == NIL) { k = 3; break; }
-                                if (!(lo(n[i][k]) & DEAD)) break;
-                                passed = max(passed, info(n[i][k]));
-                            }
-                            if (k < 3) {
-                                u = c[k];
-                                y = n[i][k];
-                                cur[v[i]] = word<W>(u, passed);
-                                lst[v[i]] = k == 0 ? make_uint4(c[1], c[2], NIL, l[i].w)
-                                          : k == 1 ? make_uint4(c[2], NIL, NIL, l[i].w)
-                                                   : make_uint4(NIL, NIL, NIL, l[i].w);
-                            } else {
-                                live = false;
-                                refill = l[i].w != 0;
-                                if (refill) {
-                                    d = __ldg(g.off + v[i] + 1) - __ldg(g.off + v[i]);
-                                    if (ROUNDS) cur[v[i]] = word<W>(u, passed);
-                                }
-                            }
-                        }
-                        if (live && (lo(y) & VMASK) == v[i]) {
-                            // chosen back
-                            uint32_t r = 0;
-                            if (ROUNDS) {
-                                // its word, if matched already, has the round; else both ends' passed ones give it
-                                r = (lo(y) & DEAD) ? info(y) : max(passed, info(y)) + 1u;
-                                last = max(last, r);
-                            }
-                            cur[v[i]] = word<W>(u | DEAD, r);
-                            g.dst[v[i]] = u;
-                            matched++;
-                            live = false;
-                            changed = true;
-                        }
-                    }
-                    warp_append(&S.nlive, out, live, v[i]);
-                    warp_append(&S.nq0, q0, refill && d <= 32, v[i]);
-                    warp_append(&S.nq1, q1, refill && d > 32 && d <= BLOCK_ROW, v[i]);
-                    warp_append(&S.nq2, q2, refill && d > BLOCK_ROW, v[i]);
-                }
-            }
-            if (changed) S.changed = 1;
+            T.changed = false;
+            poll_rows<W>(a, P, list, cnt, out, S.c, T);
+            if (T.changed) S.changed = 1;
             __syncthreads();
-            // rows whose list is used up
-            const uint32_t k0 = S.nq0, k1 = S.nq1, k2 = S.nq2;
-            for (uint32_t b = warp * 8; b < k0; b += LT / 4) {
-                const uint32_t i = b + lane / 4;
-                uint32_t v = 0, s = 0, d = 0;
-                if (i < k0) {
-                    v = q0[i];
-                    s = __ldg(g.off + v);
-                    d = __ldg(g.off + v + 1) - s;
-                }
-                const bool live = refill_group<W, 4>(a, g, v, s, d);
-                warp_append(&S.nlive, out, live && (lane & 3) == 0, v);
-            }
-            for (uint32_t i = warp; i < k1; i += LT / 32) {
-                const uint32_t v = q1[i], s = __ldg(g.off + v), d = __ldg(g.off + v + 1) - s;
-                bool live;
-                if (d <= 256) {
-                    live = refill_group<W, 32>(a, g, v, s, d);
-                } else {
-                    Top64 t;
-                    refill_scan<W>(g, cur, s, d, 0, 1, t);
-                    live = t.k0 != 0;
-                    Passed ps = {0, 0};
-                    if (ROUNDS && live)
-                        ps = refill_passed(g, reinterpret_cast<const uint64_t*>(cur), s, d, 0, 1, t.k0, t.k3);
-                    if (live && lane == 0) refill_put<W>(cur, lst, v, t, ps);
-                }
-                warp_append(&S.nlive, out, live && lane == 0, v);
-            }
-            for (uint32_t i = 0; i < k2; i++) {
-                const uint32_t v = q2[i], s = __ldg(g.off + v), d = __ldg(g.off + v + 1) - s;
-                {
-                    Top64 t;
-                    refill_scan<W>(g, cur, s, d, warp, LT / 32, t);
-                    if (lane == 0) S.top[warp] = t;
-                }
-                __syncthreads();
-                Top64 r;
-                {
-                    const Top64& q = S.top[lane >> 2];   // 8 warps x 4: every warp merges all
-                    const uint32_t z = lane & 3;
-                    warp_add(r, z == 0 ? q.k0 : z == 1 ? q.k1 : z == 2 ? q.k2 : q.k3,
-                             z == 0 ? q.p0 : z == 1 ? q.p1 : z == 2 ? q.p2 : q.p3);
-                }
-                if (ROUNDS) {
-                    if (r.k0) {
-                        const Passed x = refill_passed(g, reinterpret_cast<const uint64_t*>(cur), s, d, warp,
-                                                       LT / 32, r.k0, r.k3);
-                        if (lane == 0) {
-                            S.passed[warp] = x.round;
-                            S.cut[warp] = x.cut;
-                        }
-                    }
-                    __syncthreads();
-                }
-                if (warp == 0) {
-                    Passed ps = {0, 0};
-                    if (ROUNDS && r.k0)
-                        for (int w = 0; w < LT / 32; w++) {
-                            ps.round = max(ps.round, S.passed[w]);
-                            ps.cut = S.cut[w] > ps.cut ? S.cut[w] : ps.cut;
-                        }
-                    if (r.k0 && lane == 0) refill_put<W>(cur, lst, v, r, ps);
-                    warp_append(&S.nlive, out, r.k0 && lane == 0, v);
-                }
+            const uint32_t k0 = S.c.nshort, k1 = S.c.nlong;
+            if (k0 | k1) {
+                refill_rows<W>(a, P, k0, k1, out, &S.c.live, S.next, S.r);
                 __syncthreads();
             }
-            __syncthreads();
-            cnt = S.nlive;
+            cnt = S.c.live;
             const uint32_t ch = S.changed, stop = S.stop;
             list = out;
             buf ^= 1u;
@@ -945,27 +1090,27 @@ __global__ void __launch_bounds__(LT, 4) k_live(const ListArgs* __restrict__ pa,
             idle = ch ? 0u : idle + 1u;
             if (stop || idle > IDLE_MAX) break;
         }
-        if (tid == 0) a.pcount[part] = cnt << 1 | buf;
-        matched = __reduce_add_sync(FULL, matched);
-        if (lane == 0) S.red[warp] = matched;
-        if (ROUNDS) {
-            last = __reduce_max_sync(FULL, last);
-            if (lane == 0) S.passed[warp] = last;
+        // the part's matched rows and their latest round
+        const uint32_t m = __reduce_add_sync(FULL, T.matched), r = __reduce_max_sync(FULL, T.last);
+        if (lane == 0) {
+            S.red[0][warp] = m;
+            S.red[1][warp] = r;
         }
         __syncthreads();
         if (tid == 0) {
-            left += cnt;
             unsigned long long t = 0;
-            uint32_t r = 0;
-            for (int i = 0; i < LT / 32; i++) {
-                t += S.red[i];
-                if (ROUNDS) r = max(r, S.passed[i]);
+            uint32_t l = 0;
+            for (int i = 0; i < LW; i++) {
+                t += S.red[0][i];
+                l = max(l, S.red[1][i]);
             }
             if (t) atomicAdd(a.gmatched ? &a.gmatched[si] : &st->matched2, t);
-            if (ROUNDS && r) {
-                atomicMax(a.grounds ? &a.grounds[si] : &st->rounds, r);
-                if (r > a.max_rounds) set_err(st, ERR_TIMEOUT, r);
+            if (sizeof(W) == 8 && l) {
+                atomicMax(a.grounds ? &a.grounds[si] : &st->rounds, l);
+                if (l > a.max_rounds) set_err(st, ERR_TIMEOUT, l);
             }
+            a.pcount[part] = cnt << 1 | buf;
+            left += cnt;
         }
     }
     if (tid == 0) {
@@ -1031,7 +1176,7 @@ __global__ void __launch_bounds__(256) k_round_counts(const ListArgs* __restrict
                         if (own == 255) {
                             own = 0;
                             for (uint64_t j = (uint64_t)g.roff[row] + (i & 7); j < g.roff[row + 1]; j += 8)
-                                own = max(own, (uint32_t)__ldg(mr + g.nbr[j]));
+                                own = max(own, (uint32_t)__ldg(mr + nbr_at(g, (uint32_t)j)));
                         }
                     }
                     own = max(own, __shfl_xor_sync(FULL, own, 1));
@@ -1069,10 +1214,11 @@ int sms() {
     cudaGetDevice(&dev);
     return device_sm_count(dev);
 }
-uint32_t live_grid() { return (uint32_t)sms() * 4; }
+uint32_t live_grid() { return (uint32_t)sms() * LM_LMINB; }   // every block resident
 
 }  // namespace
 
+uint32_t list_live_blocks(int device) { return (uint32_t)device_sm_count(device) * LM_LMINB; }
 uint32_t list_blocks(const uint32_t task[4], uint32_t nrows) {
     const TopBlocks b = top_blocks(task, nrows);
     const uint32_t t = b.l + b.w + b.g + b.s;
@@ -1083,8 +1229,8 @@ int launch_list_map(void* stream, const ListArgs* d, uint32_t nsegs, uint32_t* b
     return (int)cudaGetLastError();
 }
 int launch_top(void* stream, const ListArgs* d, uint32_t blocks, bool rounds) {
-    if (rounds) k_top<uint64_t><<<blocks, TT, sizeof(TopSmem), (cudaStream_t)stream>>>(d);
-    else k_top<uint32_t><<<blocks, TT, sizeof(TopSmem), (cudaStream_t)stream>>>(d);
+    if (rounds) k_top<uint64_t><<<blocks, TT, 0, (cudaStream_t)stream>>>(d);
+    else k_top<uint32_t><<<blocks, TT, 0, (cudaStream_t)stream>>>(d);
     return (int)cudaGetLastError();
 }
 // (more blocks than parts would only come and go)
