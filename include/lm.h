@@ -278,7 +278,7 @@ int  lm_autotune(lm_ctx* ctx, const lm_graph* const* g, uint32_t count, const ui
  * index >= 64), LM_ECUDA (the address lookup or the launch failed). */
 #define LM_NOALLOC_MAX_N 65536u
 #define LM_NOALLOC_MAX_M 262144u
-#define LM_NOALLOC_SCRATCH_BYTES (9ull * LM_NOALLOC_MAX_N + 8ull * LM_NOALLOC_MAX_M)
+#define LM_NOALLOC_SCRATCH_BYTES (8ull * LM_NOALLOC_MAX_M)
 int  lm_match_small_noalloc(uint32_t n, uint32_t m, const uint32_t* eu, const uint32_t* ev, const float* w,
                             uint64_t seed, uint32_t* mate, uint32_t* status, void* stream);
 

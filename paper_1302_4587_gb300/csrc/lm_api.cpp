@@ -574,10 +574,12 @@ int match_edges(lm_ctx* ctx, Engine& e, const lm_graph* g, uint64_t seed, uint32
 }
 
 // Scratch of the list path for nv vertices, nc chunks of long rows, ng graphs, nb blocks
-// of k_top and np parts (grow-only).
-static int ensure_list(lm_ctx* ctx, Engine& e, size_t nv, size_t nc, size_t ng, size_t nb, size_t np) {
+// of k_top and np parts, with or without the rounds' (grow-only).
+static int ensure_list(lm_ctx* ctx, Engine& e, size_t nv, size_t nc, size_t ng, size_t nb, size_t np, bool rounds) {
     ListWs& w = e.lw;
-    if (w.block && nv <= w.cap_v && nc <= w.cap_c && ng <= w.cap_g && nb <= w.cap_b && np <= w.cap_p) return LM_OK;
+    if (w.block && nv <= w.cap_v && nc <= w.cap_c && ng <= w.cap_g && nb <= w.cap_b && np <= w.cap_p &&
+        (w.rounds || !rounds))
+        return LM_OK;
     LM_CK(ctx, cudaStreamSynchronize(e.stream));
     ListWs nw;
     nw.cap_v = std::max(nv, w.cap_v);
@@ -589,6 +591,11 @@ static int ensure_list(lm_ctx* ctx, Engine& e, size_t nv, size_t nc, size_t ng, 
     c.add(&nw.cur, nw.cap_v);
     c.add(&nw.lst, nw.cap_v);
     c.add(&nw.wide, nw.cap_v);
+    nw.rounds = w.rounds || rounds;
+    if (nw.rounds) {
+        c.add(&nw.rl, nw.cap_v);
+        c.add(&nw.rw, nw.cap_v);
+    }
     for (int k = 0; k < 2; k++) c.add(&nw.list[k], nw.cap_v);
     c.add(&nw.queue, nw.cap_v);
     c.add(&nw.mate, nw.cap_v);
@@ -661,6 +668,8 @@ static void list_args(ListArgs& A, Engine& e) {
     A.queue = w.queue;
     A.lst = w.lst;
     A.wide = w.wide;
+    A.rl = w.rl;
+    A.rw = w.rw;
     A.pcount = w.pcount;
     A.part = w.part;
     A.pcnt = w.pcnt;
@@ -693,7 +702,8 @@ static int match_list(lm_ctx* ctx, Engine& e, const lm_graph* g, uint64_t seed, 
                       Prof& prof, bool async, bool rounds, bool counts) {
     cudaStream_t s = e.stream;
     const uint32_t nparts = list_parts(ctx, g->nrows, g->nrows);
-    int rc = ensure_list(ctx, e, g->n, g->ntask[0], 1, 0, nparts);
+    if (ctx->lim_rounds) rounds = true;   // a cap on the rounds: they have to be known
+    int rc = ensure_list(ctx, e, g->n, g->ntask[0], 1, 0, nparts, rounds);
     if (rc) return rc;
     uint32_t* mate_d = dev_out ? mate : e.lw.mate;
     static_assert(EDGE_ARGS_OFF + sizeof(EdgeJobArgs) <= LIST_ARGS_OFF &&
@@ -705,7 +715,6 @@ static int match_list(lm_ctx* ctx, Engine& e, const lm_graph* g, uint64_t seed, 
     J.a.nsegs = 1;
     J.a.nparts = nparts;
     job_limits(ctx, g->m, &J.a.max_rounds, &J.a.limit_ns);
-    if (ctx->lim_rounds) rounds = true;   // a cap on the rounds: they have to be known
     J.seg = list_seg(g, seed, mate_d);
     J.seg.nparts = nparts;
     LM_CK(ctx, cudaMemcpyAsync(D, &J, sizeof J, cudaMemcpyHostToDevice, s));
@@ -800,7 +809,7 @@ static int batch_list(lm_ctx* ctx, Engine& e, const lm_graph* const* gs, uint32_
     }
     const bool want = rounds || ctx->lim_rounds;
     int rc = staging_ready(ctx, e);
-    if (!rc) rc = ensure_list(ctx, e, nv, nc, count, nb, np);
+    if (!rc) rc = ensure_list(ctx, e, nv, nc, count, nb, np, want);
     if (!rc) rc = ensure_pinned(ctx, e, count * sizeof(ListSeg));
     if (rc) return rc;
     ListWs& w = e.lw;

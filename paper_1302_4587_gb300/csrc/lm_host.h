@@ -54,6 +54,8 @@ struct ListWs {
     size_t cap_v = 0, cap_c = 0, cap_g = 0, cap_b = 0, cap_p = 0;
     uint64_t* cur = nullptr;                      // [cap_v] words (see ListArgs)
     uint4 *lst = nullptr, *wide = nullptr;        // [cap_v]
+    uint4 *rl = nullptr, *rw = nullptr;           // [cap_v] once rounds were wanted
+    bool rounds = false;
     uint32_t* list[2] = {nullptr, nullptr};       // [cap_v]
     uint4* queue = nullptr;                       // [cap_v]
     uint32_t* mate = nullptr;                     // [cap_v] staging of results for the host

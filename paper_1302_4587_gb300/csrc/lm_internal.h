@@ -290,6 +290,7 @@ struct ListArgs {
     const uint32_t* pmap;     // [nparts] graph of each part (NULL: one graph)
     void* cur;                // [vertices] word of every vertex, 32 or 64 bits (rounds wanted)
     uint4 *lst, *wide;        // [vertices] the rest of each row's list, and of a long row's (see lm_list.cu)
+    uint4 *rl, *rw;           // [vertices] the rounds that go with their places (64-bit words only)
     uint32_t* list[2];        // live rows, each part's in its own range
     uint4* queue;             // rows to refill, likewise: vertex, row offset, length
     uint32_t* pcount;         // [nparts] live rows a part was given back with, times two, plus their buffer

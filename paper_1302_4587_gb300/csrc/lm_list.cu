@@ -64,11 +64,17 @@ __device__ __forceinline__ uint64_t look(const uint64_t* p) {
 // ---------------------------------------------------------------- a row's list
 // The candidate is the row's word; the next three neighbours and the flags sit in
 // lst[v] (x, y, z, w), four more in wide[v] if WIDE is set.  MORE: the row holds
-// entries beyond its list.  An empty place is NIL.
+// entries beyond its list.  An empty place is NIL.  Where rounds are wanted and the
+// list comes from a refill (HASR), rl[v] and rw[v] hold beside every place the latest
+// round (plus one) among the neighbours above it that were matched by then: the row
+// passes over them with that place.
 struct RowLists {
-    uint4 *lst, *wide;
+    uint4 *lst, *wide, *rl, *rw;
 };
-constexpr uint32_t MORE = 1u, WIDE = 2u;
+__device__ __forceinline__ RowLists row_lists(const ListArgs& a, uint32_t vbase) {
+    return {a.lst + vbase, a.wide + vbase, a.rl ? a.rl + vbase : nullptr, a.rw ? a.rw + vbase : nullptr};
+}
+constexpr uint32_t MORE = 1u, WIDE = 2u, HASR = 4u;
 constexpr int KS = 4, KL = LIST_KEPT;   // list lengths: rows of at most LIST_SHORT entries, longer ones
 
 // entry i of a graph: ord(w), its neighbour, its full key
@@ -240,24 +246,20 @@ struct LaneTop64 {
     }
 };
 
-// a list held by lanes 0 .. KL - 1 (NIL: none) into row `at`'s places
-template <class W>
-__device__ __forceinline__ void put_lanes(W* cur, const RowLists& R, size_t at, uint32_t lane, uint32_t c,
-                                          uint32_t inf, bool more) {
-    if (lane == 0) cur[at] = word<W>(c, inf);
-    else if (lane < 4) reinterpret_cast<uint32_t*>(R.lst + at)[lane - 1] = c;
-    else if (lane < KL) reinterpret_cast<uint32_t*>(R.wide + at)[lane - 4] = c;
-    else if (lane == KL) R.lst[at].w = WIDE | (more ? MORE : 0u);
-}
-// the same for a group's lanes, each with its place's neighbour; the flags go with the third
+// A list into row `at`'s places: lane (or group lane) i has the i-th neighbour c (NIL:
+// none) and, with rounds, the r that goes with it; lane 0's r joins the word.
 template <class W, int K>
-__device__ __forceinline__ void put_group(W* cur, const RowLists& R, size_t at, uint32_t sub, uint32_t c,
-                                          uint32_t inf, uint32_t flags) {
+__device__ __forceinline__ void put_list(W* cur, const RowLists& R, size_t at, uint32_t sub, uint32_t c, uint32_t r,
+                                         uint32_t flags) {
     uint32_t* l = reinterpret_cast<uint32_t*>(R.lst + at);
-    if (sub == 0) cur[at] = word<W>(c, inf);
+    if (sub == 0) cur[at] = word<W>(c, r);
     else if (sub < 3) l[sub - 1] = c;
     else if (sub == 3) *reinterpret_cast<uint2*>(l + 2) = make_uint2(c, flags);
     else if (sub < K) reinterpret_cast<uint32_t*>(R.wide + at)[sub - 4] = c;
+    if (sizeof(W) == 8 && (flags & HASR)) {
+        if (sub > 0 && sub < 4) reinterpret_cast<uint32_t*>(R.rl + at)[sub - 1] = r;
+        else if (sub >= 4 && sub < K) reinterpret_cast<uint32_t*>(R.rw + at)[sub - 4] = r;
+    }
 }
 
 // ---------------------------------------------------------------- k_top
@@ -368,7 +370,7 @@ __device__ __forceinline__ void top_group(const ListArgs& a, const ListSeg& g, u
         uint32_t c = 0;
         if (cd && sub < KL) c = nbr_at(g, cs + p);
         if (i + ROWS < cnt) fetch(i + ROWS);
-        if (cd) put_group<W, KL>(words<W>(a), {a.lst, a.wide}, (size_t)g.vbase + cv, sub, c, 0, WIDE | MORE);
+        if (cd) put_list<W, KL>(words<W>(a) + g.vbase, row_lists(a, g.vbase), cv, sub, c, 0, WIDE | MORE);
     }
 }
 
@@ -482,7 +484,8 @@ __device__ __forceinline__ void top_long(const ListArgs& a, const ListSeg& g, ui
     }
     if (lane >= KL) p = NIL;
     if (whole) {
-        put_lanes<W>(words<W>(a), {a.lst, a.wide}, (size_t)g.vbase + v, lane, p != NIL ? nbr_at(g, p) : NIL, 0, true);
+        put_list<W, KL>(words<W>(a) + g.vbase, row_lists(a, g.vbase), v, lane, p != NIL ? nbr_at(g, p) : NIL, 0,
+                        WIDE | MORE);
         return;
     }
     // a chunk: its list with the full keys; the last chunk of the row to finish merges all
@@ -510,7 +513,7 @@ __device__ __forceinline__ void top_long(const ListArgs& a, const ListSeg& g, ui
         kt.offer(((uint64_t)rec.y << 32) | rec.x, rec.z);
     }
     if (lane == 0) a.pcnt[(size_t)g.lbase + first] = 0;
-    put_lanes<W>(words<W>(a), {a.lst, a.wide}, (size_t)g.vbase + v, lane, kt.n, 0, true);
+    put_list<W, KL>(words<W>(a) + g.vbase, row_lists(a, g.vbase), v, lane, kt.n, 0, WIDE | MORE);
 }
 
 // Blocks of k_top for one graph, in this order: long tasks, rows of a warp, rows of a
@@ -599,7 +602,7 @@ __device__ __forceinline__ bool refill_group(const ListSeg& g, W* cur, const Row
         if (!(lo(t[e]) & DEAD)) live |= 1u << e;
     uint32_t p[K];
     bool rest = false, exact = ROUNDS;
-    uint32_t passed = 0;
+    uint32_t mr = 0;   // with rounds: the place's r
     if (!ROUNDS) {
         uint32_t y[E], r[K];
 #pragma unroll
@@ -616,24 +619,15 @@ __device__ __forceinline__ bool refill_group(const ListSeg& g, W* cur, const Row
         for (int e = 0; e < E; e++) key[e] = e * G + sub < d ? key_of(g, x[e], s + e * G + sub) : 0ull;
         rest = group_top_keyed<G, E, K>(key, live, sub, p, k);
         if (ROUNDS) {
-            // the latest round among the matched neighbours above the new candidate; the
-            // list ends at the heaviest matched one below it, whose round counts for
-            // every candidate after that
-            uint64_t cut = 0;
 #pragma unroll
-            for (int e = 0; e < E; e++) {
-                if (e * G + sub >= d || ((live >> e) & 1u)) continue;
-                if (key[e] > k[0]) passed = max(passed, info(t[e]));
-                else cut = key[e] > cut ? key[e] : cut;
+            for (int i = 0; i < K; i++) {
+                uint32_t r = 0;
+#pragma unroll
+                for (int e = 0; e < E; e++)
+                    if (e * G + sub < d && !((live >> e) & 1u) && key[e] > k[i]) r = max(r, info(t[e]));
+                r = group_max<G>(r);
+                mr = sub == (uint32_t)i ? r : mr;
             }
-            passed = group_max<G>(passed);
-            cut = group_max64<G>(cut);
-#pragma unroll
-            for (int i = 1; i < K; i++)
-                if (p[i] != NIL && k[i] < cut) {
-                    p[i] = NIL;
-                    rest = true;
-                }
         }
     }
     if (d && p[0] != NIL) {
@@ -642,8 +636,8 @@ __device__ __forceinline__ bool refill_group(const ListSeg& g, W* cur, const Row
         for (int i = 1; i < K; i++) mp = sub == (uint32_t)i ? p[i] : mp;
         uint32_t c = NIL;
         if (sub < K && mp != NIL) c = nbr_at(g, s + mp);
-        put_group<W, K>(cur, R, v, sub, c, ROUNDS && sub == 0 ? max(passed, info(look(cur + v))) : 0u,
-                        (K == KL ? WIDE : 0u) | (rest ? MORE : 0u));
+        if (ROUNDS && sub == 0) mr = max(mr, info(look(cur + v)));
+        put_list<W, K>(cur, R, v, sub, c, mr, (K == KL ? WIDE : 0u) | (rest ? MORE : 0u) | (ROUNDS ? HASR : 0u));
         return true;
     }
     return false;
@@ -682,38 +676,44 @@ __device__ __forceinline__ void refill_scan(const ListSeg& g, const W* cur, uint
         for (int i = 0; i < 4; i++) x[i] = nx[i];
     }
 }
-// the latest round among the row's matched neighbours above key k0, and the heaviest
-// matched one's key below it (as far as it lies above `low`)
-struct Passed {
-    uint32_t round;
-    uint64_t cut;
-};
-__device__ __forceinline__ Passed refill_passed(const ListSeg& g, const uint64_t* cur, uint32_t s, uint32_t d,
-                                                uint32_t q, uint32_t parts, uint64_t k0, uint64_t low) {
-    uint32_t r = 0;
-    uint64_t cut = 0;
+// lane i < KL: the latest round (plus one) among the row's matched neighbours above the
+// list's i-th key (part `q` of `parts` of the row)
+__device__ __forceinline__ uint32_t refill_passed(const ListSeg& g, const uint64_t* cur, uint32_t s, uint32_t d,
+                                                  uint32_t q, uint32_t parts, const LaneTop64& t) {
+    uint64_t k[KL];
+    uint32_t r[KL];
+#pragma unroll
+    for (int i = 0; i < KL; i++) {
+        k[i] = __shfl_sync(FULL, t.k, i);
+        r[i] = 0;
+    }
+    const uint32_t low = (uint32_t)(k[KL - 1] >> 32);
     for (uint64_t i = 32ull * q + (threadIdx.x & 31); i < d; i += 32ull * parts) {
         const uint64_t w = __ldg(g.ent + s + (uint32_t)i);
-        if ((uint32_t)(w >> 32) < (uint32_t)(low >> 32)) continue;
+        if ((uint32_t)(w >> 32) < low) continue;
         const uint64_t y = look(cur + (uint32_t)w);
         if (!(lo(y) & DEAD)) continue;
         const uint64_t key = key_of(g, (uint32_t)(w >> 32), s + (uint32_t)i);
-        if (key > k0) r = max(r, info(y));
-        else if (key > cut) cut = key;
+#pragma unroll
+        for (int j = 0; j < KL; j++)
+            if (key > k[j]) r[j] = max(r[j], info(y));
     }
-    r = __reduce_max_sync(FULL, r);
-    return {r, group_max64<32>(cut)};
+    uint32_t mine = 0;
+#pragma unroll
+    for (int j = 0; j < KL; j++) {
+        const uint32_t x = __reduce_max_sync(FULL, r[j]);
+        mine = (threadIdx.x & 31) == (uint32_t)j ? x : mine;
+    }
+    return mine;
 }
-// t: lanes 0 .. KL - 1; the list ends at ps.cut
+// t, r: lanes 0 .. KL - 1
 template <class W>
-__device__ __forceinline__ void refill_put(W* cur, const RowLists& R, uint32_t v, const LaneTop64& t, const Passed& ps) {
+__device__ __forceinline__ void refill_put(W* cur, const RowLists& R, uint32_t v, const LaneTop64& t, uint32_t r) {
     const uint32_t lane = threadIdx.x & 31;
-    const bool in = lane < KL && t.k && (lane == 0 || t.k > ps.cut);
-    // (with a full list, or a cut one, there may be more)
-    const bool more = __any_sync(FULL, lane < KL && t.k && (lane == KL - 1 || !in));
-    uint32_t inf = 0;
-    if (sizeof(W) == 8 && lane == 0) inf = max(ps.round, info(look(cur + v)));
-    put_lanes<W>(cur, R, v, lane, in ? t.n : NIL, inf, more);
+    // (with a full list there may be more)
+    const uint32_t flags = WIDE | (__shfl_sync(FULL, t.n, KL - 1) != NIL ? MORE : 0u) | (sizeof(W) == 8 ? HASR : 0u);
+    if (sizeof(W) == 8 && lane == 0) r = max(r, info(look(cur + v)));
+    put_list<W, KL>(cur, R, v, lane, t.k ? t.n : NIL, r, flags);
 }
 
 // ---------------------------------------------------------------- k_live
@@ -724,7 +724,7 @@ __device__ __forceinline__ void refill_put(W* cur, const RowLists& R, uint32_t v
 #define LM_LV 1
 #endif
 #ifndef LM_LMINB
-#define LM_LMINB 10
+#define LM_LMINB 8
 #endif
 constexpr int LT = LM_LT, LV = LM_LV, LW = LT / 32;
 constexpr uint32_t BLOCK_ROW = 1024;  // longer rows are refilled by the whole block
@@ -761,7 +761,7 @@ struct Part {
         rows = min(g.nrows, from + per) - from;
         home = (size_t)g.vbase + from;
         cur = words<W>(a) + g.vbase;
-        R = {a.lst + g.vbase, a.wide + g.vbase};
+        R = row_lists(a, g.vbase);
         queue = a.queue + home;
     }
 };
@@ -845,9 +845,15 @@ __device__ __forceinline__ void poll_rows(const ListArgs& a, const Part<W>& P, c
                         if (d0 && d1 && d2) passed = max(passed, info(n[i][2]));
                     }
                     const uint32_t at = v[i];
+                    const bool hasr = ROUNDS && (l[i].w & HASR);
                     if (!(d0 && d1 && d2)) {
                         u = !d0 ? l[i].x : !d1 ? l[i].y : l[i].z;
                         y = !d0 ? n[i][0] : !d1 ? n[i][1] : n[i][2];
+                        if (hasr) {
+                            const uint4 r = P.R.rl[at];
+                            passed = max(passed, !d0 ? r.x : !d1 ? r.y : r.z);
+                            P.R.rl[at] = make_uint4(!d0 ? r.y : r.z, r.z, 0, 0);
+                        }
                         cur[v[i]] = word<W>(u, passed);
                         P.R.lst[at] = make_uint4(!d0 ? l[i].y : !d1 ? l[i].z : NIL, !d0 ? l[i].z : NIL, NIL, l[i].w);
                     } else {
@@ -872,6 +878,11 @@ __device__ __forceinline__ void poll_rows(const ListArgs& a, const Part<W>& P, c
                                 live = true;
                                 u = !e0 ? l2.x : !e1 ? l2.y : !e2 ? l2.z : l2.w;
                                 y = !e0 ? m0 : !e1 ? m1 : !e2 ? m2 : m3;
+                                if (hasr) {
+                                    const uint4 r = P.R.rw[at];
+                                    passed = max(passed, !e0 ? r.x : !e1 ? r.y : !e2 ? r.z : r.w);
+                                    P.R.rl[at] = make_uint4(!e0 ? r.y : !e1 ? r.z : r.w, !e0 ? r.z : r.w, r.w, 0);
+                                }
                                 cur[v[i]] = word<W>(u, passed);
                                 P.R.lst[at] = make_uint4(!e0 ? l2.y : !e1 ? l2.z : !e2 ? l2.w : NIL,
                                                        !e0 ? l2.z : !e1 ? l2.w : NIL, !e0 ? l2.w : NIL, l[i].w);
@@ -915,8 +926,6 @@ __device__ __forceinline__ void poll_rows(const ListArgs& a, const Part<W>& P, c
 struct RefillSmem {
     uint64_t k[LW][KL];
     uint32_t n[LW][KL];
-    uint64_t cut[LW];
-    uint32_t passed[LW];
 };
 template <class W>
 __device__ __forceinline__ void refill_rows(const ListArgs& a, const Part<W>& P, uint32_t k0, uint32_t k1,
@@ -956,12 +965,10 @@ __device__ __forceinline__ void refill_rows(const ListArgs& a, const Part<W>& P,
             } else {
                 LaneTop64 t;
                 refill_scan<W>(g, cur, s, d, 0, 1, t);
-                const uint64_t first = __shfl_sync(FULL, t.k, 0), last = t.last();
-                live = first != 0;
-                Passed ps = {0, 0};
-                if (ROUNDS && live)
-                    ps = refill_passed(g, reinterpret_cast<const uint64_t*>(cur), s, d, 0, 1, first, last);
-                if (live) refill_put<W>(cur, P.R, v, t, ps);
+                live = __shfl_sync(FULL, t.k, 0) != 0;
+                uint32_t r = 0;
+                if (ROUNDS && live) r = refill_passed(g, reinterpret_cast<const uint64_t*>(cur), s, d, 0, 1, t);
+                if (live) refill_put<W>(cur, P.R, v, t, r);
             }
             warp_append(nlive, out, live && lane == 0, v);
         }
@@ -1001,26 +1008,21 @@ __device__ __forceinline__ void refill_rows(const ListArgs& a, const Part<W>& P,
         LaneTop64 r;   // every warp merges all
         for (uint32_t z = lane; z < LW * KL; z += 32) r.offer(S.k[z / KL][z % KL], S.n[z / KL][z % KL]);
         static_assert(LW * KL % 32 == 0, "whole warps offer");
-        const uint64_t first = __shfl_sync(FULL, r.k, 0), last = r.last();
+        const bool live = __shfl_sync(FULL, r.k, 0) != 0;
         if (ROUNDS) {
-            if (first) {
-                const Passed x = refill_passed(g, reinterpret_cast<const uint64_t*>(cur), s, d, warp, LW, first, last);
-                if (lane == 0) {
-                    S.passed[warp] = x.round;
-                    S.cut[warp] = x.cut;
-                }
+            __syncthreads();   // every warp has read the lists
+            if (live) {
+                const uint32_t x = refill_passed(g, reinterpret_cast<const uint64_t*>(cur), s, d, warp, LW, r);
+                if (lane < KL) S.n[warp][lane] = x;
             }
             __syncthreads();
         }
         if (warp == 0) {
-            Passed ps = {0, 0};
-            if (ROUNDS && first)
-                for (int w = 0; w < LW; w++) {
-                    ps.round = max(ps.round, S.passed[w]);
-                    ps.cut = S.cut[w] > ps.cut ? S.cut[w] : ps.cut;
-                }
-            if (first) refill_put<W>(cur, P.R, v, r, ps);
-            warp_append(nlive, out, first && lane == 0, v);
+            uint32_t x = 0;
+            if (ROUNDS && live && lane < KL)
+                for (int w = 0; w < LW; w++) x = max(x, S.n[w][lane]);
+            if (live) refill_put<W>(cur, P.R, v, r, x);
+            warp_append(nlive, out, live && lane == 0, v);
         }
         __syncthreads();
     }
@@ -1163,10 +1165,17 @@ __global__ void __launch_bounds__(256) k_round_counts(const ListArgs* __restrict
             for (uint64_t i = base + blockIdx.x * blockDim.x + tid; i < ((end + 31) & ~31ull); i += stride) {
                 uint32_t r = NIL;
                 if (kind == 0) {
-                    if (i < end) {
-                        const uint64_t rec = __ldg(g.edges + i);
-                        r = min((uint32_t)__ldg(mr + (uint32_t)rec), (uint32_t)__ldg(mr + (uint32_t)(rec >> 32)));
-                    }
+                    // four edges a step: their gathers in flight together
+                    uint64_t rec[4];
+                    uint32_t q[4];
+#pragma unroll
+                    for (int z = 0; z < 4; z++) rec[z] = i + z * stride < end ? __ldg(g.edges + i + z * stride) : 0ull;
+#pragma unroll
+                    for (int z = 0; z < 4; z++) q[z] = min((uint32_t)__ldg(mr + (uint32_t)rec[z]), (uint32_t)__ldg(mr + (uint32_t)(rec[z] >> 32)));
+#pragma unroll
+                    for (int z = 0; z < 4; z++)
+                        if (i + z * stride < end && q[z] < 64) col[q[z] * 256]++;
+                    i += 3 * stride;
                 } else {
                     // eight lanes a row
                     uint32_t own = 0;
