@@ -161,13 +161,13 @@ int  lm_match(lm_ctx* ctx, const lm_graph* g, uint64_t seed, uint32_t* mate, lm_
 int  lm_batch_match(lm_ctx* ctx, const lm_graph* const* g, uint32_t count, const uint64_t* seeds,
                     uint32_t* const* mates, lm_stats* stats);
 
-/* Serving: queue a matching request and return at once with a ticket.  A
- * scheduler thread of the context admits requests while their device
- * footprint fits the HBM budget and a slot is free, and runs rounds of all
- * admitted requests together (a request joins between rounds).  mate
- * (uint32[n], host or device) must stay valid until the request completes;
- * the graph must outlive it.  Errors: LM_EINVAL, LM_EAGAIN (queue full),
- * LM_ENOMEM (the request alone exceeds the budget), LM_ECUDA. */
+/* Serving: queue a matching request and return at once with a ticket.  The
+ * context's serving threads take the waiting requests in arrival order, as long as
+ * they fit the HBM budget and the slots beside those in flight, and run those taken
+ * together in shared launches; requests that arrive meanwhile are taken by the next
+ * free thread and run beside them.  mate (uint32[n], host or device) must stay valid
+ * until the request completes; the graph must outlive it.  Errors: LM_EINVAL,
+ * LM_EAGAIN (queue full), LM_ENOMEM (the request alone exceeds the budget), LM_ECUDA. */
 int  lm_submit(lm_ctx* ctx, const lm_graph* g, uint64_t seed, uint32_t* mate, uint64_t* ticket);
 
 /* *done = 1 once the request's mate is complete (then stats, if non-NULL, is
@@ -218,7 +218,9 @@ int  lm_set_limits(lm_ctx* ctx, uint32_t max_rounds, uint32_t time_limit_ms);
  *                      size (as few bytes as leave about 2048 edges to a bucket)
  *   ms                 lm_autotune only: median time of one call with these parameters
  * Defaults: rmax 1024, chunk 1024, sweep 0, vertex 4, batch 512, contract_bits 0.
- * The serving thread takes the context's parameters when it starts (first lm_submit). */
+ * The serving threads take the context's parameters when they start (first lm_submit).
+ * rmax, chunk, batch and the CTAs per SM shape the round-by-round path, which the
+ * renewed order takes (LM_F_RENEW); other matches do not use them. */
 typedef struct lm_tuning {
     uint32_t rmax;
     uint32_t chunk;

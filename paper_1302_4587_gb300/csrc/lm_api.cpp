@@ -206,7 +206,6 @@ int ensure_ws(lm_ctx* ctx, Engine& e, uint32_t nv, uint32_t ne, uint32_t ng) {
     c.add(&nw.gebase, G);
     c.add(&nw.goff, G);
     c.add(&nw.grounds, G);
-    c.add(&nw.glive, G);
     c.add(&nw.gdst, G);
     c.add(&nw.gmatched, G);
     if (w.block) {

@@ -43,7 +43,6 @@ struct Workspace {
     uint32_t* gebase = nullptr;      // [cap_g] first union entry of each graph
     const uint32_t** goff = nullptr; // [cap_g] each graph's row offsets
     uint32_t* grounds = nullptr;     // [cap_g] rounds per graph
-    uint32_t* glive = nullptr;       // [cap_g] live rows per graph
     uint32_t** gdst = nullptr;       // [cap_g] result destination per graph
     unsigned long long* gmatched = nullptr;  // [cap_g] matched vertices per graph
 };

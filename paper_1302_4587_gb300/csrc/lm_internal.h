@@ -165,7 +165,6 @@ struct VertexArgs {
     uint32_t in_set;          // DevState::lcnt index of `in` (zeroed when the pass ends; 4 = none)
     const uint32_t* vlist;    // explicit rows (round 0): vertex ids
     uint32_t nvlist;
-    uint32_t vlist_base;      // added to vlist entries (union id of the list's graph)
     const uint32_t* deg0;     // explicit rows: row length source (indexed like vlist), NULL = len_cur
     Lists out;
     uint32_t out_set;
@@ -174,7 +173,6 @@ struct VertexArgs {
     uint32_t match;           // 0 = classification only (before the candidate sweep)
     uint32_t round_from_state; // 1: the round index is DevState::round (advanced by this pass)
     uint32_t* grounds;        // per-graph rounds: max(round + 1) over graphs with a live row, NULL = none
-    uint32_t* glive;          // live unmatched rows per graph seen by this pass, NULL = none
     uint32_t rmax;            // rows of at most this many live entries go to R, longer ones to C
     uint32_t chunk_shift;     // chunks of a long row hold 1 << chunk_shift entries
     uint32_t batch_shift;     // a batch of R ends where its entries cross a multiple of
@@ -317,7 +315,6 @@ constexpr unsigned long long TAIL_ENT = LM_TAIL_ENT;
 // kernel arguments are passed as pointers to device memory
 int launch_init(void* stream, const InitArgs* dargs);
 int launch_vertex(void* stream, const VertexArgs* dargs, const struct LaunchCfg& cfg);
-int launch_sweep_cand(void* stream, const SweepArgs* dargs, const struct LaunchCfg& cfg);   // round 0, candidates only
 int launch_sweep_input(void* stream, const SweepArgs* dargs, const struct LaunchCfg& cfg);  // round-0 compaction
 int launch_sweep_live(void* stream, const SweepArgs* dargs, const struct LaunchCfg& cfg);   // rounds >= 1
 int launch_round0(void* stream, const Round0Args* dargs);      // round-0 candidates in TMA-fed tiles
@@ -405,12 +402,6 @@ int launch_nonzero_flags(void* stream, const uint32_t* deg, uint32_t n, uint32_t
 // start[v] = ebase[g] + off_g[v - gvbase[g]], gid[v] = g, len0[v] = degree
 int launch_union_setup(void* stream, const uint32_t* gvbase, const uint32_t* ebase, const uint32_t* const* offs,
                        uint32_t ngraphs, uint32_t nvert, uint32_t* start, uint32_t* gid, uint32_t* len0);
-// serving: start[vbase + i] = ebase + off[i], gid[vbase + i] = slot for i < n
-int launch_req_setup(void* stream, const uint32_t* off, uint32_t n, uint32_t vbase, uint32_t ebase, uint32_t slot,
-                     uint32_t* start, uint32_t* gid);
-// out[v] = local id of mate_global[vbase + v] (v < n); *matched2 += matched vertices (if non-null)
-int launch_to_local(void* stream, const uint32_t* mate_global, uint32_t vbase, uint32_t n, uint32_t* out,
-                    unsigned long long* matched2);
 // union results -> per-graph local ids into dst[g] (device pointers; NULL = skip); matched2[g] += matched vertices
 int launch_to_local_batch(void* stream, const uint32_t* mate_union, const uint32_t* gvbase, const uint32_t* gid,
                           uint32_t ngraphs, uint32_t* const* dst, unsigned long long* matched2, uint32_t nvert);

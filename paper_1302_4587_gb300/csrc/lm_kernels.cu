@@ -1,4 +1,6 @@
-// sm_103a kernels of the local-max matching path.
+// sm_103a kernels: the round-by-round matching path (the renewed order, whose keys
+// change every round, and graphs of 2^31 vertices and more; lm_list.cu has the path
+// of all others), the edge-centric path, graph construction, prefix sums.
 //
 // One round of local max (the phase of Sec. 2: every live vertex picks its
 // heaviest live edge, edges picked by both ends join M, edges touching M are
@@ -19,9 +21,8 @@
 //             one row).  The candidate's neighbour is recovered from the key:
 //             its low half is perm_seed(e), inverted to the edge index e.
 //
-// Round 0 first files every row (k_vertex without matching), runs a
-// candidate-only sweep over the graphs' own arrays, then the match and a
-// compacting sweep that builds the 64-bit keys
+// Round 0 takes its candidates from the graphs' own arrays in tiles (k_round0); the
+// sweep after its match builds the 64-bit keys
 //     K(e) = ord(w_e) << 32 | perm_seed(e)
 // from the entries' ord(weight) and edge index on the fly.
 #include <cuda_runtime.h>
@@ -183,7 +184,7 @@ __device__ __forceinline__ void vertex_pass(const VertexArgs& a, uint32_t cta, u
             uint32_t v = NIL, L = 0;
             if (idx < total) {
                 if (a.vlist) {
-                    v = a.vlist[idx] + a.vlist_base;
+                    v = a.vlist[idx];
                     if (a.deg0) L = a.deg0[idx];
                 } else if (!a.in.cnt) {
                     v = idx;  // dense range of vertices
@@ -221,7 +222,6 @@ __device__ __forceinline__ void vertex_pass(const VertexArgs& a, uint32_t cta, u
             if (uu[i] != NIL && uu[i] >= va.nvert) { set_err(st, ERR_BOUNDS, uu[i]); uu[i] = NIL; }
             const uint32_t back = (uu[i] != NIL) ? va.cnbr[uu[i]] : NIL;
             const uint32_t v = vv[i], L = LL[i];
-            bool open_row = false;
             if (v != NIL && L > 0) {
                 my_rows++;
                 my_ent += L;
@@ -231,7 +231,6 @@ __device__ __forceinline__ void vertex_pass(const VertexArgs& a, uint32_t cta, u
                     atomicOr(&va.dead[v >> 5], 1u << (v & 31));
                     my_match++;
                 } else {
-                    open_row = true;
                     if (L <= a.rmax) { cls[i] = 1; cR++; eR += L; }
                     else {
                         cls[i] = 2;
@@ -245,11 +244,6 @@ __device__ __forceinline__ void vertex_pass(const VertexArgs& a, uint32_t cta, u
                 const uint32_t g = (v != NIL && L > 0) ? (va.gid ? va.gid[v] : 0u) : NIL;
                 const uint32_t same = __match_any_sync(FULL, g);
                 if (g != NIL && lane == __ffs(same) - 1) atomicMax(&a.grounds[g], round + 1);
-            }
-            if (a.glive) {
-                const uint32_t g = open_row ? (va.gid ? va.gid[v] : 0u) : NIL;
-                const uint32_t same = __match_any_sync(FULL, g);
-                if (g != NIL && lane == __ffs(same) - 1) atomicAdd(&a.glive[g], (uint32_t)__popc(same));
             }
         }
         // block-aggregated appends to the task lists
@@ -449,21 +443,17 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // One 32-entry group of a row batch: r = the entry's row in the batch (32: no
 // entry), sl = the group lane where that row starts, uni = one row for the whole
 // group; w = the stored word, u = the neighbour (compaction sweeps).
-template <bool INPUT, bool COMPACT, bool RENEW, bool COH>
+template <bool INPUT, bool RENEW, bool COH>
 __device__ __forceinline__ void row_group(const SweepArgs& a, WarpRows<RENEW>& W, uint32_t r, uint32_t sl, bool uni,
                                           uint64_t w, uint32_t u, int lane, uint32_t lt) {
     const VertexArrays& va = a.va;
     uint64_t key = 0;
-    if (COMPACT) {
-        bool keep = r != 32;
-        if (keep) {
-            if (u >= va.nvert) { set_err(a.st, ERR_BOUNDS, u); keep = false; }
-            else keep = !is_dead<COH>(va, u);
-        }
-        if (keep) key = row_word_key<INPUT, RENEW>(a, W, r, w);
-    } else if (r != 32) {
-        key = row_word_key<INPUT, RENEW>(a, W, r, w);
+    bool keep = r != 32;
+    if (keep) {
+        if (u >= va.nvert) { set_err(a.st, ERR_BOUNDS, u); keep = false; }
+        else keep = !is_dead<COH>(va, u);
     }
+    if (keep) key = row_word_key<INPUT, RENEW>(a, W, r, w);
     const bool surv = key != 0;
     const uint32_t ball = __ballot_sync(FULL, surv);
     if (!ball) return;
@@ -472,22 +462,18 @@ __device__ __forceinline__ void row_group(const SweepArgs& a, WarpRows<RENEW>& W
         const uint32_t hi = __reduce_max_sync(FULL, (uint32_t)(key >> 32));
         const uint32_t lo = __reduce_max_sync(FULL, ((uint32_t)(key >> 32) == hi) ? (uint32_t)key : 0u);
         const uint64_t K = ((uint64_t)hi << 32) | lo;
-        if (COMPACT) {
-            uint32_t base = 0;
-            if (surv) base = W.rcnt[r];
-            __syncwarp();
-            if (surv) {
-                const uint32_t pos = W.rstart[r] + base + __popc(ball & lt);
-                a.out_key[pos] = RENEW ? stored_word<RENEW>(W.rk0[r], W.rk1[r], key) : key;
-                a.out_nbr[pos] = u;
-            }
-            // keys are distinct: exactly one lane (a survivor) holds the maximum
-            if (key == K) {
-                W.rcnt[r] = base + __popc(ball);
-                if (K > W.rkey[r]) { W.rkey[r] = K; W.ru[r] = u; }
-            }
-        } else if (key == K && K > W.rkey[r]) {
-            W.rkey[r] = K;
+        uint32_t base = 0;
+        if (surv) base = W.rcnt[r];
+        __syncwarp();
+        if (surv) {
+            const uint32_t pos = W.rstart[r] + base + __popc(ball & lt);
+            a.out_key[pos] = RENEW ? stored_word<RENEW>(W.rk0[r], W.rk1[r], key) : key;
+            a.out_nbr[pos] = u;
+        }
+        // keys are distinct: exactly one lane (a survivor) holds the maximum
+        if (key == K) {
+            W.rcnt[r] = base + __popc(ball);
+            if (K > W.rkey[r]) { W.rkey[r] = K; W.ru[r] = u; }
         }
         __syncwarp();
         return;
@@ -498,30 +484,28 @@ __device__ __forceinline__ void row_group(const SweepArgs& a, WarpRows<RENEW>& W
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
         const uint64_t o = __shfl_up_sync(FULL, mx, d);
-        const uint32_t ou = COMPACT ? __shfl_up_sync(FULL, mu, d) : 0u;
+        const uint32_t ou = __shfl_up_sync(FULL, mu, d);
         if ((uint32_t)lane >= sl + d && o > mx) { mx = o; mu = ou; }
     }
     const uint32_t rn = __shfl_down_sync(FULL, r, 1);
     const bool last = r != 32 && (lane == 31 || rn != r);
-    if (COMPACT) {
-        const uint32_t run = FULL << sl;
-        const uint32_t base = r != 32 ? W.rcnt[r] : 0u;
-        __syncwarp();
-        if (last) W.rcnt[r] = base + __popc(ball & run & lanemask_le());
-        if (surv) {
-            const uint32_t pos = W.rstart[r] + base + __popc(ball & run & lt);
-            a.out_key[pos] = RENEW ? stored_word<RENEW>(W.rk0[r], W.rk1[r], key) : key;
-            a.out_nbr[pos] = u;
-        }
+    const uint32_t run = FULL << sl;
+    const uint32_t base = r != 32 ? W.rcnt[r] : 0u;
+    __syncwarp();
+    if (last) W.rcnt[r] = base + __popc(ball & run & lanemask_le());
+    if (surv) {
+        const uint32_t pos = W.rstart[r] + base + __popc(ball & run & lt);
+        a.out_key[pos] = RENEW ? stored_word<RENEW>(W.rk0[r], W.rk1[r], key) : key;
+        a.out_nbr[pos] = u;
     }
     if (last && mx > W.rkey[r]) {
         W.rkey[r] = mx;
-        if (COMPACT) W.ru[r] = mu;
+        W.ru[r] = mu;
     }
     __syncwarp();
 }
 
-template <bool INPUT, bool COMPACT, bool RENEW, bool COH>
+template <bool INPUT, bool RENEW, bool COH>
 __device__ void do_rows_p(const SweepArgs& a, WarpRows<RENEW>& W, WarpStage& S, uint32_t b, uint32_t nR, uint32_t nr,
                           int lane) {
     const VertexArrays& va = a.va;
@@ -590,7 +574,7 @@ __device__ void do_rows_p(const SweepArgs& a, WarpRows<RENEW>& W, WarpStage& S, 
                     cp_async4(&S.nbr[stg][lane], sg.eid + q);
                 } else {
                     cp_async8(&S.key[stg][lane], a.in_key + q);
-                    if (COMPACT) cp_async4(&S.nbr[stg][lane], a.in_nbr + q);
+                    cp_async4(&S.nbr[stg][lane], a.in_nbr + q);
                 }
             }
         }
@@ -611,31 +595,27 @@ __device__ void do_rows_p(const SweepArgs& a, WarpRows<RENEW>& W, WarpStage& S, 
             if (INPUT) {   // the input's entry: ord(w), neighbour; its edge index beside it
                 u = (uint32_t)w + a.segs[W.rseg[r]].vbase;
                 w = (w & 0xFFFFFFFF00000000ull) | S.nbr[stg][lane];
-            } else if (COMPACT) {
+            } else {
                 u = S.nbr[stg][lane];
             }
         }
         issue(k + PD);
-        row_group<INPUT, COMPACT, RENEW, COH>(a, W, r, sl, uni, w, u, lane, lt);
+        row_group<INPUT, RENEW, COH>(a, W, r, sl, uni, w, u, lane, lt);
     }
     cp_async_wait<0>();
     __syncwarp();
     if (v != NIL) {
         // the survivor count goes into the row's own task-list entry (read there by
         // the next vertex pass; the batch-start bit stays for the other warps' scans)
-        if (COMPACT) a.in.R[idx].y = W.rcnt[lane] | (rv.y & BATCH_START);
+        a.in.R[idx].y = W.rcnt[lane] | (rv.y & BATCH_START);
         const uint64_t K = W.rkey[lane];
-        // compaction sweeps carried the neighbour along; the candidate-only sweep
-        // recovers it from the key's edge id
-        if (K) va.cnbr[v] = COMPACT ? W.ru[lane]
-                                    : RENEW ? recover_nbr_keys(a.segs[g], a.st, v, K, rk0, rk1)
-                                            : recover_nbr_seg(a.segs[g], a.st, v, K);
+        if (K) va.cnbr[v] = W.ru[lane];
     }
     __syncwarp();
 }
 
 // One chunk of a long row, pipelined like the row batches.
-template <bool INPUT, bool COMPACT, bool RENEW, bool COH>
+template <bool INPUT, bool RENEW, bool COH>
 __device__ void do_chunk_p(const SweepArgs& a, WarpStage& S, uint32_t t, uint32_t nr, int lane) {
     const VertexArrays& va = a.va;
     const uint2 c = a.in.C[t];
@@ -665,7 +645,7 @@ __device__ void do_chunk_p(const SweepArgs& a, WarpStage& S, uint32_t t, uint32_
                 cp_async4(&S.nbr[stg][lane], sg.eid + off + jj);
             } else {
                 cp_async8(&S.key[stg][lane], a.in_key + off + jj);
-                if (COMPACT) cp_async4(&S.nbr[stg][lane], a.in_nbr + off + jj);
+                cp_async4(&S.nbr[stg][lane], a.in_nbr + off + jj);
             }
         }
         cp_async_commit();
@@ -682,24 +662,20 @@ __device__ void do_chunk_p(const SweepArgs& a, WarpStage& S, uint32_t t, uint32_
             if (INPUT) {
                 u = (uint32_t)key + vb;
                 key = (key & 0xFFFFFFFF00000000ull) | S.nbr[stg][lane];
-            } else if (COMPACT) {
+            } else {
                 u = S.nbr[stg][lane];
             }
         }
         issue(k + PD);
-        if (COMPACT) {
-            bool keep = jj < je;
-            if (keep) {
-                if (u >= va.nvert) { set_err(a.st, ERR_BOUNDS, u); keep = false; }
-                else keep = !is_dead<COH>(va, u);
-            }
-            key = keep ? word_key<INPUT, RENEW>(ck0, ck1, key) : 0ull;
-        } else if (jj < je) {
-            key = word_key<INPUT, RENEW>(ck0, ck1, key);
+        bool keep = jj < je;
+        if (keep) {
+            if (u >= va.nvert) { set_err(a.st, ERR_BOUNDS, u); keep = false; }
+            else keep = !is_dead<COH>(va, u);
         }
+        key = keep ? word_key<INPUT, RENEW>(ck0, ck1, key) : 0ull;
         const uint32_t ball = __ballot_sync(FULL, key != 0);
         if (key > bk) bk = key;
-        if (COMPACT && ball) {
+        if (ball) {
             uint32_t base = 0;
             if (lane == 0) base = atomicAdd(&len_next[v], (uint32_t)__popc(ball));
             base = __shfl_sync(FULL, base, 0);
@@ -738,7 +714,7 @@ __device__ void do_chunk_p(const SweepArgs& a, WarpStage& S, uint32_t t, uint32_
 
 // The sweep as CTA `cta` of `ncta` (k_sweep: the grid; the tail kernel: one CTA);
 // W and S are the calling warp's shared row state and copy stages.
-template <bool INPUT, bool COMPACT, bool RENEW, bool COH>
+template <bool INPUT, bool RENEW, bool COH>
 __device__ __forceinline__ void sweep_pass(const SweepArgs& a, WarpRows<RENEW>& W, WarpStage& S, uint32_t cta,
                                            uint32_t ncta) {
     const int lane = threadIdx.x & 31;
@@ -762,12 +738,12 @@ __device__ __forceinline__ void sweep_pass(const SweepArgs& a, WarpRows<RENEW>& 
     for (;; t = __shfl_sync(FULL, t_next, 0)) {
         if (t >= total) break;
         if (lane == 0) t_next = nw + atomicAdd(a.task_ctr, 1u);
-        if (t < nC) do_chunk_p<INPUT, COMPACT, RENEW, COH>(a, S, t, nr, lane);
-        else do_rows_p<INPUT, COMPACT, RENEW, COH>(a, W, S, t - nC, nR, nr, lane);
+        if (t < nC) do_chunk_p<INPUT, RENEW, COH>(a, S, t, nr, lane);
+        else do_rows_p<INPUT, RENEW, COH>(a, W, S, t - nC, nR, nr, lane);
     }
 }
 
-template <bool INPUT, bool COMPACT, bool RENEW>
+template <bool INPUT, bool RENEW>
 __global__ void __launch_bounds__(ST, LM_SWEEP_MINB) k_sweep(const SweepArgs* __restrict__ pav) {
     __shared__ WarpRows<RENEW> s_rows[ST / 32];
     __shared__ WarpStage s_stage[ST / 32];
@@ -778,7 +754,7 @@ __global__ void __launch_bounds__(ST, LM_SWEEP_MINB) k_sweep(const SweepArgs* __
     for (uint32_t i = threadIdx.x; i < sizeof(SweepArgs) / 4; i += ST)
         reinterpret_cast<uint32_t*>(s_args_raw)[i] = reinterpret_cast<const uint32_t*>(pav)[i];
     __syncthreads();
-    sweep_pass<INPUT, COMPACT, RENEW, false>(*reinterpret_cast<const SweepArgs*>(s_args_raw), s_rows[threadIdx.x >> 5],
+    sweep_pass<INPUT, RENEW, false>(*reinterpret_cast<const SweepArgs*>(s_args_raw), s_rows[threadIdx.x >> 5],
                                       s_stage[threadIdx.x >> 5], blockIdx.x, gridDim.x);
 }
 
@@ -1635,32 +1611,6 @@ __global__ void k_union_setup(const uint32_t* gvbase, const uint32_t* ebase, con
         len0[v] = o1 - o0;
     }
 }
-// serving: vertices [vbase, vbase + n) of one request get their row starts and slot
-__global__ void k_req_setup(const uint32_t* off, uint32_t n, uint32_t vbase, uint32_t ebase, uint32_t slot,
-                            uint32_t* start, uint32_t* gid) {
-    const uint32_t stride = gridDim.x * blockDim.x;
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        start[vbase + i] = ebase + off[i];
-        gid[vbase + i] = slot;
-    }
-}
-
-__global__ void k_to_local(const uint32_t* mate_g, uint32_t vbase, uint32_t n, uint32_t* out,
-                           unsigned long long* matched2) {
-    const uint32_t stride = gridDim.x * blockDim.x;
-    for (uint32_t base = blockIdx.x * blockDim.x; base < n; base += stride) {
-        const uint32_t v = base + threadIdx.x;
-        bool m = false;
-        if (v < n) {
-            const uint32_t x = mate_g[vbase + v];
-            out[v] = (x == NIL) ? NIL : x - vbase;
-            m = x != NIL;
-        }
-        const uint32_t b = __ballot_sync(FULL, m);
-        if (matched2 && (threadIdx.x & 31) == 0 && b) atomicAdd(matched2, (unsigned long long)__popc(b));
-    }
-}
-
 __global__ void k_to_local_batch(const uint32_t* mate_u, const uint32_t* gvbase, const uint32_t* gid,
                                  uint32_t* const* dst, unsigned long long* matched2, uint32_t nvert) {
     const uint32_t stride = gridDim.x * blockDim.x;
@@ -1847,12 +1797,12 @@ int launch_vertex(void* stream, const VertexArgs* dargs, const LaunchCfg& cfg) {
     return (int)cudaGetLastError();
 }
 
-template <bool I, bool C, bool RN>
+template <bool I, bool RN>
 static uint32_t sweep_grid(const LaunchCfg& cfg) {
     static int blocks_per_sm = 0;
     if (!blocks_per_sm) {
         int per = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_sweep<I, C, RN>, ST, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_sweep<I, RN>, ST, 0);
         blocks_per_sm = per > 0 ? per : 1;
     }
     int per = blocks_per_sm;
@@ -1860,10 +1810,10 @@ static uint32_t sweep_grid(const LaunchCfg& cfg) {
     return (uint32_t)(current_sms() * per);
 }
 
-template <bool I, bool C>
+template <bool I>
 static int launch_sweep_t(void* stream, const SweepArgs* dargs, const LaunchCfg& cfg) {
-    if (cfg.renew) k_sweep<I, C, true><<<sweep_grid<I, C, true>(cfg), ST, 0, (cudaStream_t)stream>>>(dargs);
-    else k_sweep<I, C, false><<<sweep_grid<I, C, false>(cfg), ST, 0, (cudaStream_t)stream>>>(dargs);
+    if (cfg.renew) k_sweep<I, true><<<sweep_grid<I, true>(cfg), ST, 0, (cudaStream_t)stream>>>(dargs);
+    else k_sweep<I, false><<<sweep_grid<I, false>(cfg), ST, 0, (cudaStream_t)stream>>>(dargs);
     return (int)cudaGetLastError();
 }
 static int round0_blocks_per_sm() {
@@ -1897,12 +1847,8 @@ int launch_round0_cut(void* stream, const Round0Args* d) {
     k_round0_cut<<<round0_cut_grid(), 256, 0, (cudaStream_t)stream>>>(d);
     return (int)cudaGetLastError();
 }
-int launch_sweep_cand(void* stream, const SweepArgs* d, const LaunchCfg& c) {
-    if (c.renew) return (int)cudaErrorInvalidValue;  // round 0 keeps the default order: never needed
-    return launch_sweep_t<true, false>(stream, d, c);
-}
-int launch_sweep_input(void* stream, const SweepArgs* d, const LaunchCfg& c) { return launch_sweep_t<true, true>(stream, d, c); }
-int launch_sweep_live(void* stream, const SweepArgs* d, const LaunchCfg& c) { return launch_sweep_t<false, true>(stream, d, c); }
+int launch_sweep_input(void* stream, const SweepArgs* d, const LaunchCfg& c) { return launch_sweep_t<true>(stream, d, c); }
+int launch_sweep_live(void* stream, const SweepArgs* d, const LaunchCfg& c) { return launch_sweep_t<false>(stream, d, c); }
 
 int launch_build_degrees(void* stream, const uint32_t* eu, const uint32_t* ev, const float* w, uint32_t n,
                          uint32_t m, uint32_t* deg, uint32_t* err) {
@@ -1962,18 +1908,6 @@ int launch_union_setup(void* stream, const uint32_t* gvbase, const uint32_t* eba
                                                                           gid, len0);
     return (int)cudaGetLastError();
 }
-int launch_req_setup(void* stream, const uint32_t* off, uint32_t n, uint32_t vbase, uint32_t ebase, uint32_t slot,
-                     uint32_t* start, uint32_t* gid) {
-    if (n == 0) return 0;
-    k_req_setup<<<grid_for(n, 256), 256, 0, (cudaStream_t)stream>>>(off, n, vbase, ebase, slot, start, gid);
-    return (int)cudaGetLastError();
-}
-int launch_to_local(void* stream, const uint32_t* mate_global, uint32_t vbase, uint32_t n, uint32_t* out,
-                    unsigned long long* matched2) {
-    if (n == 0) return 0;
-    k_to_local<<<grid_for(n, 256), 256, 0, (cudaStream_t)stream>>>(mate_global, vbase, n, out, matched2);
-    return (int)cudaGetLastError();
-}
 int launch_to_local_batch(void* stream, const uint32_t* mate_union, const uint32_t* gvbase, const uint32_t* gid,
                           uint32_t ngraphs, uint32_t* const* dst, unsigned long long* matched2, uint32_t nvert) {
     if (nvert == 0 || ngraphs == 0) return 0;
@@ -2029,7 +1963,7 @@ __global__ void __launch_bounds__(ST, 1) k_tail(const JobArgs* __restrict__ A, u
         for (int k = 2; k < 4; k++) {
             vertex_pass(A->v[k], 0, 1);
             __syncthreads();
-            sweep_pass<false, true, RENEW, true>(A->s[k], W, S, 0, 1);
+            sweep_pass<false, RENEW, true>(A->s[k], W, S, 0, 1);
             __syncthreads();
         }
         if (threadIdx.x == 0) {
@@ -2087,10 +2021,10 @@ int build_job_graph(const JobArgs* dargs, DevState* st, const LaunchCfg& cfg, vo
     }
     const dim3 vgrid(vertex_grid(cfg)), vblock(VT), sblock(ST), rblock(R0T), cgrid(round0_cut_grid());
     const bool rn = cfg.renew;
-    const dim3 lgrid(rn ? sweep_grid<false, true, true>(cfg) : sweep_grid<false, true, false>(cfg));
-    const dim3 igrid(rn ? sweep_grid<true, true, true>(cfg) : sweep_grid<true, true, false>(cfg));
-    void* const k_input = rn ? (void*)k_sweep<true, true, true> : (void*)k_sweep<true, true, false>;
-    void* const k_live = rn ? (void*)k_sweep<false, true, true> : (void*)k_sweep<false, true, false>;
+    const dim3 lgrid(rn ? sweep_grid<false, true>(cfg) : sweep_grid<false, false>(cfg));
+    const dim3 igrid(rn ? sweep_grid<true, true>(cfg) : sweep_grid<true, false>(cfg));
+    void* const k_input = rn ? (void*)k_sweep<true, true> : (void*)k_sweep<true, false>;
+    void* const k_live = rn ? (void*)k_sweep<false, true> : (void*)k_sweep<false, false>;
     do {
         if ((e = add_kernel(g, &node, prev, (void*)k_init, dim3(current_sms() * 16), dim3(256), init_params))) break;
         prev = node;

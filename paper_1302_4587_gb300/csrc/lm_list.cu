@@ -1157,7 +1157,7 @@ __global__ void __launch_bounds__(256) k_round_counts(const ListArgs* __restrict
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (int kind = 0; kind < 2; kind++) {
         unsigned long long* ring = reinterpret_cast<unsigned long long*>(kind ? a.st->ring_n : a.st->ring_m);
-        const uint64_t total = kind ? (uint64_t)g.nrows * 8 : g.m;
+        const uint64_t total = kind ? g.nrows : g.m;
         // (steps of at most 32768 counts a thread, so that 16 bits hold them)
         for (uint64_t base = 0; base < total; base += stride * 32768) {
             for (int i = 0; i < 64; i++) col[i * 256] = 0;
@@ -1177,21 +1177,33 @@ __global__ void __launch_bounds__(256) k_round_counts(const ListArgs* __restrict
                         if (i + z * stride < end && q[z] < 64) col[q[z] * 256]++;
                     i += 3 * stride;
                 } else {
-                    // eight lanes a row
-                    uint32_t own = 0;
+                    // a thread a row: a matched one has its round, a short unmatched one looks at
+                    // its neighbours, longer ones are done by the warp one after the other
+                    uint32_t s0 = 0, d = 0;
                     if (i < end) {
-                        const uint32_t row = (uint32_t)(i >> 3), v = g.vid[row];
-                        own = mr[v];
-                        if (own == 255) {
-                            own = 0;
-                            for (uint64_t j = (uint64_t)g.roff[row] + (i & 7); j < g.roff[row + 1]; j += 8)
-                                own = max(own, (uint32_t)__ldg(mr + nbr_at(g, (uint32_t)j)));
+                        r = mr[g.vid[i]];
+                        if (r == 255) {
+                            s0 = g.roff[i];
+                            d = g.roff[i + 1] - s0;
+                            r = 0;
+                            if (d <= 16)
+                                for (uint32_t j = 0; j < d; j += 4) {
+                                    uint32_t x[4];
+#pragma unroll
+                                    for (uint32_t z = 0; z < 4; z++) x[z] = nbr_at(g, s0 + min(j + z, d - 1));
+#pragma unroll
+                                    for (uint32_t z = 0; z < 4; z++) r = max(r, (uint32_t)__ldg(mr + x[z]));
+                                }
                         }
                     }
-                    own = max(own, __shfl_xor_sync(FULL, own, 1));
-                    own = max(own, __shfl_xor_sync(FULL, own, 2));
-                    own = max(own, __shfl_xor_sync(FULL, own, 4));
-                    if (i < end && (i & 7) == 0) r = own;
+                    for (uint32_t todo = __ballot_sync(FULL, d > 16); todo; todo &= todo - 1) {
+                        const int L = __ffs(todo) - 1;
+                        const uint32_t sl = __shfl_sync(FULL, s0, L), dl = __shfl_sync(FULL, d, L);
+                        uint32_t x = 0;
+                        for (uint64_t j = tid & 31; j < dl; j += 32) x = max(x, (uint32_t)__ldg(mr + nbr_at(g, sl + (uint32_t)j)));
+                        x = __reduce_max_sync(FULL, x);
+                        if ((int)(tid & 31) == L) r = x;
+                    }
                 }
                 if (r < 64) col[r * 256]++;
             }
