@@ -1091,27 +1091,27 @@ int lm_graph_create(lm_ctx* ctx, uint32_t n, uint32_t m, const uint32_t* eu, con
     g->m = m;
     g->nent = 2 * m;
 
-    const uint32_t* d_eu = eu;
-    const uint32_t* d_ev = ev;
-    const float* d_w = w;
     const size_t nn = (size_t)n + 1;
-    const size_t scan_words = std::max(exclusive_scan_tmp_words(n + 1), exclusive_scan_tmp_words(build_fill_scan_count(n, m)));
+    const size_t scan_words = std::max(exclusive_scan_tmp_words(n + 1), exclusive_scan_tmp_words(build_scan_count(m)));
     Carver tc;
-    uint32_t *t_eu = nullptr, *t_ev = nullptr, *deg = nullptr, *cursor = nullptr;
-    uint32_t *flags = nullptr, *rowidx = nullptr, *scan_tmp = nullptr, *err = nullptr, *fill_tmp = nullptr;
+    uint32_t *t_eu = nullptr, *t_ev = nullptr;
+    uint32_t *flags = nullptr, *rowidx = nullptr, *scan_tmp = nullptr;
+    BuildTmp bt{};
     float* t_w = nullptr;
     if (mem == LM_HOST && m > 0) {
         tc.add(&t_eu, m);
         tc.add(&t_ev, m);
         tc.add(&t_w, m);
     }
-    tc.add(&deg, nn);
-    tc.add(&cursor, nn);
+    tc.add(&bt.deg, nn);
     tc.add(&flags, nn);
     tc.add(&rowidx, nn);
     tc.add(&scan_tmp, scan_words);
-    tc.add(&err, 12);  // error bits, -, -, -, tasks of each kind (4), their cursors (4)
-    if (m > 0) tc.add(&fill_tmp, build_fill_tmp_words(n, m));
+    tc.add(&bt.err, 12);  // error bits, -, -, -, tasks of each kind (4), their cursors (4)
+    tc.add(&bt.rank, m);
+    tc.add(&bt.vrec, m);
+    tc.add(&bt.hist, build_scan_count(m));
+    tc.add(&bt.offs, build_scan_count(m));
     void* tmp = nullptr;
     cudaError_t ce = fault_alloc(ctx) ? cudaErrorMemoryAllocation : cudaMallocFromPoolAsync(&tmp, tc.total, ctx->pool, s);
     if (ce != cudaSuccess) return cuda_fail(ctx, ce, "graph staging");
@@ -1121,12 +1121,33 @@ int lm_graph_create(lm_ctx* ctx, uint32_t n, uint32_t m, const uint32_t* eu, con
         cudaStream_t s;
         ~TmpFree() { if (p) cudaFreeAsync(p, s); }
     } tf{tmp, s};
-    LM_CK(ctx, cudaMemsetAsync(deg, 0, nn * 4, s));
-    LM_CK(ctx, cudaMemsetAsync(err, 0, 48, s));
+    // the arrays whose size is known now, then (below) those of the rows
+    Carver ec;
+    ec.add(&g->off, nn);
+    ec.add(&g->eid, (size_t)g->nent + 4);
+    ec.add(&g->ent, (size_t)g->nent + 4);
+    ec.add(&g->edges, (size_t)g->m + 2);
+    ec.add(&g->eword, (size_t)g->m + 4);
+    ce = fault_alloc(ctx) ? cudaErrorMemoryAllocation : cudaMallocFromPoolAsync(&g->block[0], ec.total, ctx->pool, s);
+    if (ce != cudaSuccess) return cuda_fail(ctx, ce, "graph arrays");
+    // every return before the graph is handed out gives the blocks back
+    struct BlockFree {
+        std::unique_ptr<lm_graph>& g;
+        cudaStream_t s;
+        ~BlockFree() {
+            for (int k = 0; g && k < 2; k++)
+                if (g->block[k]) cudaFreeAsync(g->block[k], s);
+        }
+    } bf{g, s};
+    ec.assign(g->block[0]);
+    bt.edges = g->edges;
+    bt.eword = g->eword;
+    LM_CK(ctx, cudaMemsetAsync(bt.deg, 0, nn * 4, s));
+    LM_CK(ctx, cudaMemsetAsync(bt.err, 0, 48, s));
     // validation rides on the degree count: endpoint < n, no self loop, no NaN
     if (mem == LM_HOST && m > 0) {
         // chunks of the host arrays go up on the upload stream; the context's stream
-        // counts a chunk's degrees while the next chunk is copied
+        // runs a chunk's degree pass while the next chunk is copied
         if (!ctx->up) {
             LM_CK(ctx, cudaStreamCreateWithFlags(&ctx->up, cudaStreamNonBlocking));
             LM_CK(ctx, cudaEventCreateWithFlags(&ctx->up_ev, cudaEventDisableTiming));
@@ -1134,27 +1155,24 @@ int lm_graph_create(lm_ctx* ctx, uint32_t n, uint32_t m, const uint32_t* eu, con
         LM_CK(ctx, cudaEventRecord(ctx->up_ev, s));  // after the memsets (and earlier work)
         LM_CK(ctx, cudaStreamWaitEvent(ctx->up, ctx->up_ev, 0));
         constexpr uint32_t NCHUNK = 8;
-        const uint32_t step = ((m + NCHUNK - 1) / NCHUNK + 31) & ~31u;
-        for (uint32_t off = 0; off < m; off += step) {
-            const uint32_t cnt = std::min(step, m - off);
+        const uint32_t step = build_step(m, NCHUNK);
+        for (uint32_t off = 0, cnt; off < m; off += cnt) {
+            cnt = std::min(step, m - off);
             LM_CK(ctx, cudaMemcpyAsync(t_eu + off, eu + off, (size_t)cnt * 4, cudaMemcpyHostToDevice, ctx->up));
             LM_CK(ctx, cudaMemcpyAsync(t_ev + off, ev + off, (size_t)cnt * 4, cudaMemcpyHostToDevice, ctx->up));
             LM_CK(ctx, cudaMemcpyAsync(t_w + off, w + off, (size_t)cnt * 4, cudaMemcpyHostToDevice, ctx->up));
             LM_CK(ctx, cudaEventRecord(ctx->up_ev, ctx->up));
             LM_CK(ctx, cudaStreamWaitEvent(s, ctx->up_ev, 0));
-            LM_CK(ctx, launch_build_degrees(s, t_eu + off, t_ev + off, t_w + off, n, cnt, deg, err));
+            LM_CK(ctx, launch_build_degrees(s, t_eu, t_ev, t_w, n, m, off, cnt, bt));
         }
-        d_eu = t_eu;
-        d_ev = t_ev;
-        d_w = t_w;
     } else if (m > 0) {
-        LM_CK(ctx, launch_build_degrees(s, d_eu, d_ev, d_w, n, m, deg, err));
+        LM_CK(ctx, launch_build_degrees(s, eu, ev, w, n, m, 0, m, bt));
     }
     int rc = ensure_pinned(ctx, e, 64);  // 16 words
     if (rc) return rc;
     uint32_t* hp = static_cast<uint32_t*>(e.pinned);
-    LM_CK(ctx, launch_nonzero_flags(s, deg, n + 1, flags, err + 4));
-    LM_CK(ctx, cudaMemcpyAsync(&hp[4], err, 32, cudaMemcpyDeviceToHost, s));
+    LM_CK(ctx, launch_nonzero_flags(s, bt.deg, n + 1, flags, bt.err + 4));
+    LM_CK(ctx, cudaMemcpyAsync(&hp[4], bt.err, 32, cudaMemcpyDeviceToHost, s));
     LM_CK(ctx, launch_exclusive_scan(s, flags, rowidx, n + 1, scan_tmp, scan_words));
     LM_CK(ctx, cudaMemcpyAsync(&hp[0], rowidx + n, 4, cudaMemcpyDeviceToHost, s));
     LM_CK(ctx, cudaStreamSynchronize(s));
@@ -1162,10 +1180,9 @@ int lm_graph_create(lm_ctx* ctx, uint32_t n, uint32_t m, const uint32_t* eu, con
     g->nrows = hp[0];
     for (int k = 0; k < 4; k++) g->ntask[k] = hp[8 + k] + (k ? g->ntask[k - 1] : 0u);
 
-    Carver gc;
-    gc.add(&g->off, nn);
     // round-0 tiles copy rows [r & ~3, ...) of vid / roff in whole 16-byte words: pad both
     g->ntiles = (g->nent + TILE0 - 1) / TILE0;
+    Carver gc;
     gc.add(&g->vid, (size_t)g->nrows + 8);
     gc.add(&g->rdeg, (size_t)g->nrows + 1);
     gc.add(&g->roff, (size_t)g->nrows + 8);
@@ -1173,33 +1190,21 @@ int lm_graph_create(lm_ctx* ctx, uint32_t n, uint32_t m, const uint32_t* eu, con
     gc.add(&g->rbits, (size_t)g->ntiles * (TILE0 / 32) + 8);
     gc.add(&g->tdesc, (size_t)g->ntiles + 1);
     gc.add(&g->task, g->ntask[3]);
-    gc.add(&g->eid, (size_t)g->nent + 4);
-    gc.add(&g->ent, (size_t)g->nent + 4);
-    gc.add(&g->edges, (size_t)g->m + 2);
-    gc.add(&g->eword, (size_t)g->m + 4);
-    ce = fault_alloc(ctx) ? cudaErrorMemoryAllocation : cudaMallocFromPoolAsync(&g->block, gc.total, ctx->pool, s);
-    if (ce != cudaSuccess) return cuda_fail(ctx, ce, "graph arrays");
-    // every return before the graph is handed out gives the block back
-    struct BlockFree {
-        std::unique_ptr<lm_graph>& g;
-        cudaStream_t s;
-        ~BlockFree() { if (g && g->block) cudaFreeAsync(g->block, s); }
-    } bf{g, s};
-    gc.assign(g->block);
-    g->bytes = gc.total;
-    LM_CK(ctx, launch_exclusive_scan(s, deg, g->off, n + 1, scan_tmp, scan_words));
+    ce = fault_alloc(ctx) ? cudaErrorMemoryAllocation : cudaMallocFromPoolAsync(&g->block[1], gc.total, ctx->pool, s);
+    if (ce != cudaSuccess) return cuda_fail(ctx, ce, "graph rows");
+    gc.assign(g->block[1]);
+    g->bytes = ec.total + gc.total;
+    LM_CK(ctx, launch_exclusive_scan(s, bt.deg, g->off, n + 1, scan_tmp, scan_words));
     if (m > 0) {
-        LM_CK(ctx, cudaMemcpyAsync(cursor, g->off, nn * 4, cudaMemcpyDeviceToDevice, s));
-        LM_CK(ctx, launch_build_fill(s, d_eu, d_ev, d_w, n, m, cursor, g->eid, g->ent, g->edges, g->eword, fill_tmp,
-                                     scan_tmp, scan_words, err));
-        LM_CK(ctx, cudaMemcpyAsync(&hp[2], err, 4, cudaMemcpyDeviceToHost, s));
+        LM_CK(ctx, launch_build_fill(s, n, m, g->off, g->eid, g->ent, bt, scan_tmp, scan_words));
+        LM_CK(ctx, cudaMemcpyAsync(&hp[2], bt.err, 4, cudaMemcpyDeviceToHost, s));
     }
     // each kind's tasks follow the previous one's
     hp[12] = 0;
     for (int k = 1; k < 4; k++) hp[12 + k] = g->ntask[k - 1];
-    LM_CK(ctx, cudaMemcpyAsync(err + 8, &hp[12], 16, cudaMemcpyHostToDevice, s));
-    LM_CK(ctx, launch_build_rows(s, deg, rowidx, g->off, n, g->nrows, g->nent, g->vid, g->rdeg, g->roff, g->task,
-                                 g->ntask[3], err + 8));
+    LM_CK(ctx, cudaMemcpyAsync(bt.err + 8, &hp[12], 16, cudaMemcpyHostToDevice, s));
+    LM_CK(ctx, launch_build_rows(s, bt.deg, rowidx, g->off, n, g->nrows, g->nent, g->vid, g->rdeg, g->roff, g->task,
+                                 g->ntask[3], bt.err + 8));
     if (g->nrows) {
         LM_CK(ctx, cudaMemsetAsync(g->rbits, 0, ((size_t)g->ntiles * (TILE0 / 32) + 8) * 4, s));
         LM_CK(ctx, launch_build_tilemap(s, g->roff, g->nrows, g->nent, g->tmap, g->rbits, g->tdesc));
@@ -1216,7 +1221,8 @@ void lm_graph_destroy(lm_graph* g) {
     // the graph may still be read by work on the context's stream or the serving
     // engine's: wait for the device, then return the block to the context's pool
     cudaDeviceSynchronize();
-    if (g->block) cudaFreeAsync(g->block, g->ctx->eng.stream);
+    for (void* b : g->block)
+        if (b) cudaFreeAsync(b, g->ctx->eng.stream);
     cudaGetLastError();
     delete g;
 }

@@ -134,7 +134,7 @@ struct lm_ctx {
 struct lm_graph {
     lm_ctx* ctx = nullptr;
     uint32_t n = 0, m = 0, nrows = 0, nent = 0, ntiles = 0;
-    void* block = nullptr;
+    void* block[2] = {nullptr, nullptr};  // off, eid, ent, edges, eword; the rest
     size_t bytes = 0;
     uint32_t* off = nullptr;         // [n + 1] row offsets of all vertices
     uint32_t* vid = nullptr;         // [nrows] vertices with at least one edge (the rows)

@@ -378,18 +378,26 @@ int launch_edge_round(void* stream, const EdgeArgs* dargs, int phase);  // phase
 void destroy_job_graph(void* exec);
 
 // graph construction
-int launch_build_degrees(void* stream, const uint32_t* eu, const uint32_t* ev, const float* w, uint32_t n,
-                         uint32_t m, uint32_t* deg, uint32_t* err);
+// scratch and outputs of the build's passes (see k_build_degrees): deg is zero before them
+struct BuildTmp {
+    uint32_t* deg;            // [n + 1] degrees
+    uint32_t* err;            // bit 0: invalid input, 1: a place outside 2m
+    uint2* rank;              // [m] rank of either end among its vertex's entries
+    uint32_t *hist, *offs;    // [build_scan_count(m)] second ends per bucket and tile, their prefix
+    uint4* vrec;              // [m] second-end records in bucket order
+    uint64_t* edges;          // [m] edge records (the graph's own)
+    uint32_t* eword;          // [m] ord(weight) (the graph's own)
+};
+uint32_t build_scan_count(uint32_t m);
+uint32_t build_step(uint32_t m, uint32_t chunks);  // edges a chunk of the degree pass (whole tiles)
+// degrees, ranks, records and bucket counts of edges first .. first + count - 1 (first: whole tiles)
+int launch_build_degrees(void* stream, const uint32_t* eu, const uint32_t* ev, const float* w, uint32_t n, uint32_t m,
+                         uint32_t first, uint32_t count, const BuildTmp& t);
 int launch_exclusive_scan(void* stream, const uint32_t* in, uint32_t* out, uint32_t count, uint32_t* tmp,
                           size_t tmp_words);
 size_t exclusive_scan_tmp_words(uint32_t count);
-// fill: tmp = build_fill_tmp_words(n, m) words of 16-byte aligned scratch; scan_tmp sized for
-// exclusive scans of build_fill_scan_count(n, m) words
-size_t build_fill_tmp_words(uint32_t n, uint32_t m);
-uint32_t build_fill_scan_count(uint32_t n, uint32_t m);
-int launch_build_fill(void* stream, const uint32_t* eu, const uint32_t* ev, const float* w, uint32_t n, uint32_t m,
-                      uint32_t* cursor, uint32_t* eid, uint64_t* ent, uint64_t* edges, uint32_t* eword, uint32_t* tmp,
-                      uint32_t* scan_tmp, size_t scan_words, uint32_t* err);  // err |= 2 when a fill slot falls outside 2m
+int launch_build_fill(void* stream, uint32_t n, uint32_t m, const uint32_t* off, uint32_t* eid, uint64_t* ent,
+                      const BuildTmp& t, uint32_t* scan_tmp, size_t scan_words);
 // cursors: the next place in task of each kind
 int launch_build_rows(void* stream, const uint32_t* deg, const uint32_t* rowidx_excl, const uint32_t* off,
                       uint32_t n, uint32_t nrows, uint32_t nent, uint32_t* vid0, uint32_t* rdeg0, uint32_t* roff,

@@ -1377,112 +1377,140 @@ __device__ __forceinline__ uint32_t warp_add(uint32_t* ctr, uint32_t key, bool a
     return active ? base + __popc(peers & ((1u << lane) - 1u)) : 0u;
 }
 
-__global__ void k_build_degrees(const uint32_t* eu, const uint32_t* ev, const float* w, uint32_t n, uint32_t m,
-                                uint32_t* deg, uint32_t* err) {
-    const uint32_t stride = gridDim.x * blockDim.x, lane = threadIdx.x & 31;
-    const uint32_t mr = (m + 31) & ~31u;  // whole warps iterate together
-    for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < mr; e += stride) {
-        bool ok = e < m;
-        uint32_t u = 0, v = 0;
-        if (ok) {
-            u = eu[e];
-            v = ev[e];
-            const uint32_t wb = __float_as_uint(w[e]);
-            const bool nan = ((wb & 0x7F800000u) == 0x7F800000u) && (wb & 0x007FFFFFu);
-            if (u >= n || v >= n || u == v || nan) {
-                atomicOr(err, 1u);
-                ok = false;
-            }
-        }
-        warp_add(&deg[ok ? u : 0], u, ok, lane);
-        warp_add(&deg[ok ? v : 0], v, ok, lane);
-    }
-}
+// A graph is built in passes over tiles of BF_TILE edges.  k_build_degrees counts
+// the degrees and keeps each end's rank among its vertex's entries (what the counting
+// atomic returned), so that the fill needs no atomics of its own: an entry's place
+// is its row's offset plus its rank.  It also writes the edge records and, per tile, the
+// second ends' counts by bucket; of a host edge list, all of this runs chunk by
+// chunk while the next chunk is on its way.
 // The fill writes every edge's two adjacency entries.  Entries of the first end
 // follow the input's order (inputs listed by source vertex write them in runs);
 // the second end's would land at random rows, each a partial sector anywhere in
-// the arrays.  So they go through 256 buckets of vertex ranges first:
-// k_build_vhist counts each tile of BF_TILE edges per bucket, a scan places every
-// (bucket, tile) run, k_build_fill_u writes the first ends and appends each
-// second-end record (row, neighbour, entry word) to its run, and k_build_fill_v
-// walks the records in bucket order, so that the rows it writes at any time lie in
-// a window of the arrays that L2 holds.
-constexpr uint32_t BF_TILE = 4096, BF_T = 256, BF_NB = 256;
+// the arrays.  So they go through 256 buckets of vertex ranges first: a scan of the
+// counts places every (bucket, tile) run, k_build_fill_u writes the first ends and
+// appends each second-end record (place, neighbour, edge, ord) to its run, and
+// k_build_fill_v walks the records in bucket order, so that the rows it writes at
+// any time lie in a window of the arrays that L2 holds.
+// Bound by scattered stores of single entries (two sectors each).  R-MAT scale 21,
+// 31.8M edges: with a second round of atomics in the fill, degrees 330, buckets' counts
+// 61, fill 511 + 632 us; with ranks 523 (under the upload of a host list) and 470 + 520.
+constexpr uint32_t BF_TILE = 4096, BF_T = 256, BF_NB = 256, BF_U = 4;  // BF_U edges a thread and step
+static_assert(BF_TILE % (BF_T * BF_U) == 0 && BF_T == BF_NB, "whole steps, a thread per bucket");
 
-__global__ void __launch_bounds__(BF_T) k_build_vhist(const uint32_t* ev, uint32_t m, uint32_t shift, uint32_t tiles,
-                                                      uint32_t* hist) {
+__global__ void __launch_bounds__(BF_T) k_build_degrees(const uint32_t* __restrict__ eu, const uint32_t* __restrict__ ev,
+                                                        const float* __restrict__ w, uint32_t n, uint32_t m,
+                                                        uint32_t first, uint32_t shift, uint32_t tiles, uint32_t* deg,
+                                                        uint32_t* err, uint2* __restrict__ rank,
+                                                        uint64_t* __restrict__ edges, uint32_t* __restrict__ eword,
+                                                        uint32_t* __restrict__ hist) {
     __shared__ uint32_t h[BF_NB];
     h[threadIdx.x] = 0;
     __syncthreads();
-    const uint64_t t0 = (uint64_t)blockIdx.x * BF_TILE;
-#pragma unroll 4
-    for (uint32_t j = 0; j < BF_TILE / BF_T; j++) {
-        const uint64_t e = t0 + j * BF_T + threadIdx.x;
-        if (e < m) atomicAdd(&h[(ev[e] >> shift) & (BF_NB - 1)], 1u);
+    const uint32_t lane = threadIdx.x & 31, tile = first / BF_TILE + blockIdx.x;
+    const uint64_t t0 = (uint64_t)tile * BF_TILE;   // whole warps iterate together
+    for (uint32_t j = 0; j < BF_TILE / BF_T; j += BF_U) {
+        uint32_t u[BF_U], v[BF_U], wb[BF_U];
+        bool ok[BF_U];
+#pragma unroll
+        for (uint32_t q = 0; q < BF_U; q++) {
+            const uint64_t e = t0 + (j + q) * BF_T + threadIdx.x;
+            ok[q] = e < m;
+            u[q] = ok[q] ? __ldg(eu + e) : 0u;
+            v[q] = ok[q] ? __ldg(ev + e) : 0u;
+            wb[q] = ok[q] ? __float_as_uint(__ldg(w + e)) : 0u;
+        }
+#pragma unroll
+        for (uint32_t q = 0; q < BF_U; q++) {
+            const uint64_t e = t0 + (j + q) * BF_T + threadIdx.x;
+            const bool nan = ((wb[q] & 0x7F800000u) == 0x7F800000u) && (wb[q] & 0x007FFFFFu);
+            if (ok[q] && (u[q] >= n || v[q] >= n || u[q] == v[q] || nan)) {
+                atomicOr(err, 1u);
+                ok[q] = false;
+            }
+            if (ok[q]) {
+                edges[e] = (uint64_t)u[q] | ((uint64_t)v[q] << 32);
+                eword[e] = ord_of_bits(wb[q]);
+                atomicAdd(&h[(v[q] >> shift) & (BF_NB - 1)], 1u);
+            }
+        }
+        uint32_t ru[BF_U], rv[BF_U];
+#pragma unroll
+        for (uint32_t q = 0; q < BF_U; q++) {
+            ru[q] = warp_add(&deg[ok[q] ? u[q] : 0], u[q], ok[q], lane);
+            rv[q] = warp_add(&deg[ok[q] ? v[q] : 0], v[q], ok[q], lane);
+        }
+#pragma unroll
+        for (uint32_t q = 0; q < BF_U; q++) {
+            const uint64_t e = t0 + (j + q) * BF_T + threadIdx.x;
+            if (ok[q]) rank[e] = make_uint2(ru[q], rv[q]);
+        }
     }
     __syncthreads();
-    hist[threadIdx.x * tiles + blockIdx.x] = h[threadIdx.x];  // bucket-major, for the scan
+    hist[threadIdx.x * tiles + tile] = h[threadIdx.x];  // bucket-major, for the scan
 }
 
-__global__ void __launch_bounds__(BF_T) k_build_fill_u(const uint32_t* eu, const uint32_t* ev, const float* w,
+__global__ void __launch_bounds__(BF_T) k_build_fill_u(const uint64_t* __restrict__ edges,
+                                                       const uint32_t* __restrict__ eword,
+                                                       const uint2* __restrict__ rank, const uint32_t* __restrict__ off,
                                                        uint32_t m, uint32_t shift, uint32_t tiles,
-                                                       const uint32_t* offs, uint32_t* cursor, uint32_t* eid,
-                                                       uint64_t* ent, uint64_t* edges, uint32_t* eword, uint4* vrec,
+                                                       const uint32_t* __restrict__ offs, uint32_t* __restrict__ eid,
+                                                       uint64_t* __restrict__ ent, uint4* __restrict__ vrec,
                                                        uint32_t* err) {
     __shared__ uint32_t gs[BF_NB], cnt[BF_NB];
     gs[threadIdx.x] = offs[threadIdx.x * tiles + blockIdx.x];
     cnt[threadIdx.x] = 0;
     __syncthreads();
-    const uint32_t lane = threadIdx.x & 31;
     const uint64_t t0 = (uint64_t)blockIdx.x * BF_TILE;
-    for (uint32_t j = 0; j < BF_TILE / BF_T; j++) {  // whole warps iterate together
-        const uint64_t e = t0 + j * BF_T + threadIdx.x;
-        const bool ok = e < m;
-        uint32_t u = 0, v = 0;
-        uint32_t ow = 0;
-        if (ok) {
-            u = eu[e];
-            v = ev[e];
-            ow = ord_of_bits(__float_as_uint(w[e]));
-            edges[e] = (uint64_t)u | ((uint64_t)v << 32);
-            eword[e] = ow;
+    for (uint32_t j = 0; j < BF_TILE / BF_T; j += BF_U) {
+        uint64_t rec[BF_U];
+        uint32_t ow[BF_U], pu[BF_U], pv[BF_U];
+        uint2 r[BF_U];
+#pragma unroll
+        for (uint32_t q = 0; q < BF_U; q++) {
+            const uint64_t e = t0 + (j + q) * BF_T + threadIdx.x;
+            rec[q] = e < m ? __ldg(edges + e) : 0ull;
+            ow[q] = e < m ? __ldg(eword + e) : 0u;
+            r[q] = e < m ? __ldg(rank + e) : make_uint2(0, 0);
         }
-        const uint32_t pu = warp_add(&cursor[u], u, ok, lane);
-        if (ok) {
-            // the cursors start at the row offsets and the degrees were counted from the
-            // same edges, so every slot is below 2m; a stale cursor is reported, not written
-            if (pu >= 2 * m) {
+#pragma unroll
+        for (uint32_t q = 0; q < BF_U; q++) {
+            pu[q] = __ldg(off + (uint32_t)rec[q]) + r[q].x;
+            pv[q] = __ldg(off + (uint32_t)(rec[q] >> 32)) + r[q].y;
+        }
+#pragma unroll
+        for (uint32_t q = 0; q < BF_U; q++) {
+            const uint64_t e = t0 + (j + q) * BF_T + threadIdx.x;
+            if (e >= m) continue;
+            const uint32_t u = (uint32_t)rec[q], v = (uint32_t)(rec[q] >> 32);
+            // offsets and ranks come from the same counts, so every place is below 2m; one
+            // that is not is reported, not written
+            if (pu[q] >= 2 * m || pv[q] >= 2 * m) {
                 atomicOr(err, 2u);
-            } else {
-                ent[pu] = ((uint64_t)ow << 32) | v;
-                eid[pu] = (uint32_t)e;
+                continue;
             }
+            ent[pu[q]] = ((uint64_t)ow[q] << 32) | v;
+            eid[pu[q]] = (uint32_t)e;
             const uint32_t b = (v >> shift) & (BF_NB - 1);
-            const uint32_t q = gs[b] + atomicAdd(&cnt[b], 1u);
-            if (q < m) vrec[q] = make_uint4(v, u, (uint32_t)e, ow);
+            const uint32_t p = gs[b] + atomicAdd(&cnt[b], 1u);
+            if (p < m) vrec[p] = make_uint4(pv[q], u, (uint32_t)e, ow[q]);
             else atomicOr(err, 2u);
         }
     }
 }
 
-__global__ void __launch_bounds__(BF_T) k_build_fill_v(const uint4* vrec, uint32_t m, uint32_t* cursor, uint32_t* eid,
-                                                       uint64_t* ent, uint32_t* err) {
-    const uint32_t stride = gridDim.x * blockDim.x, lane = threadIdx.x & 31;
-    const uint32_t mr = (m + 31) & ~31u;  // whole warps iterate together
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < mr; i += stride) {
-        const bool ok = i < m;
-        uint4 r = make_uint4(0, 0, 0, 0);
-        if (ok) r = vrec[i];
-        const uint32_t pv = warp_add(&cursor[r.x], r.x, ok, lane);
-        if (ok) {
-            if (pv >= 2 * m) {
-                atomicOr(err, 2u);
-            } else {
-                ent[pv] = ((uint64_t)r.w << 32) | r.y;
-                eid[pv] = r.z;
-            }
+__global__ void __launch_bounds__(BF_T) k_build_fill_v(const uint4* __restrict__ vrec, uint32_t m,
+                                                       uint32_t* __restrict__ eid, uint64_t* __restrict__ ent) {
+    const uint64_t i = (uint64_t)blockIdx.x * (BF_T * BF_U) + threadIdx.x;
+    uint4 r[BF_U];
+#pragma unroll
+    for (uint32_t q = 0; q < BF_U; q++)
+        if (i + q * BF_T < m) r[q] = __ldcs(vrec + i + q * BF_T);
+#pragma unroll
+    for (uint32_t q = 0; q < BF_U; q++)
+        if (i + q * BF_T < m && r[q].x < 2 * m) {
+            ent[r[q].x] = ((uint64_t)r[q].w << 32) | r[q].y;
+            eid[r[q].x] = r[q].z;
         }
-    }
 }
 // kind of task a row of d entries makes on the list path (4: none)
 __device__ __forceinline__ uint32_t task_kind(uint32_t d) {
@@ -1850,36 +1878,34 @@ int launch_round0_cut(void* stream, const Round0Args* d) {
 int launch_sweep_input(void* stream, const SweepArgs* d, const LaunchCfg& c) { return launch_sweep_t<true>(stream, d, c); }
 int launch_sweep_live(void* stream, const SweepArgs* d, const LaunchCfg& c) { return launch_sweep_t<false>(stream, d, c); }
 
-int launch_build_degrees(void* stream, const uint32_t* eu, const uint32_t* ev, const float* w, uint32_t n,
-                         uint32_t m, uint32_t* deg, uint32_t* err) {
-    k_build_degrees<<<grid_for(m, 256), 256, 0, (cudaStream_t)stream>>>(eu, ev, w, n, m, deg, err);
+static uint32_t build_shift(uint32_t n) {  // bucket = v >> shift, below 256
+    uint32_t shift = 0;
+    while (((uint64_t)(n - 1) >> shift) > BF_NB - 1) shift++;
+    return shift;
+}
+static uint32_t build_tiles(uint32_t m) { return (uint32_t)(((uint64_t)m + BF_TILE - 1) / BF_TILE); }
+uint32_t build_scan_count(uint32_t m) { return BF_NB * build_tiles(m); }
+uint32_t build_step(uint32_t m, uint32_t chunks) {
+    return build_tiles((uint32_t)(((uint64_t)m + chunks - 1) / chunks)) * BF_TILE;
+}
+int launch_build_degrees(void* stream, const uint32_t* eu, const uint32_t* ev, const float* w, uint32_t n, uint32_t m,
+                         uint32_t first, uint32_t count, const BuildTmp& t) {
+    if (count == 0) return 0;
+    if (first % BF_TILE) return (int)cudaErrorInvalidValue;
+    // (the arrays are those of the whole list; edges first .. first + count - 1 are there)
+    k_build_degrees<<<build_tiles(count), BF_T, 0, (cudaStream_t)stream>>>(
+        eu, ev, w, n, first + count, first, build_shift(n), build_tiles(m), t.deg, t.err, t.rank, t.edges, t.eword, t.hist);
     return (int)cudaGetLastError();
 }
-size_t build_fill_tmp_words(uint32_t n, uint32_t m) {
-    (void)n;
-    const uint64_t tiles = ((uint64_t)m + BF_TILE - 1) / BF_TILE;
-    return (size_t)4 * m + 2 * (BF_NB * tiles + 4) + 8;  // the records (16 B each), counts, their prefix
-}
-uint32_t build_fill_scan_count(uint32_t n, uint32_t m) {
-    (void)n;
-    return (uint32_t)(BF_NB * (((uint64_t)m + BF_TILE - 1) / BF_TILE));
-}
-int launch_build_fill(void* stream, const uint32_t* eu, const uint32_t* ev, const float* w, uint32_t n, uint32_t m,
-                      uint32_t* cursor, uint32_t* eid, uint64_t* ent, uint64_t* edges, uint32_t* eword, uint32_t* tmp,
-                      uint32_t* scan_tmp, size_t scan_words, uint32_t* err) {
+int launch_build_fill(void* stream, uint32_t n, uint32_t m, const uint32_t* off, uint32_t* eid, uint64_t* ent,
+                      const BuildTmp& t, uint32_t* scan_tmp, size_t scan_words) {
     cudaStream_t s = (cudaStream_t)stream;
     if (m == 0) return 0;
-    if (!tmp) return (int)cudaErrorInvalidValue;
-    uint32_t shift = 0;  // bucket = v >> shift, below 256
-    while (((uint64_t)(n - 1) >> shift) > BF_NB - 1) shift++;
-    const uint32_t tiles = (uint32_t)(((uint64_t)m + BF_TILE - 1) / BF_TILE);
-    uint4* vrec = reinterpret_cast<uint4*>(tmp);           // 16-byte aligned (the caller's carve)
-    uint32_t* hist = tmp + 4 * (size_t)m;
-    uint32_t* offs = hist + ((BF_NB * (size_t)tiles + 4) & ~(size_t)3);
-    k_build_vhist<<<tiles, BF_T, 0, s>>>(ev, m, shift, tiles, hist);
-    if (int r = launch_exclusive_scan(stream, hist, offs, BF_NB * tiles, scan_tmp, scan_words)) return r;
-    k_build_fill_u<<<tiles, BF_T, 0, s>>>(eu, ev, w, m, shift, tiles, offs, cursor, eid, ent, edges, eword, vrec, err);
-    k_build_fill_v<<<grid_for(m, 256), BF_T, 0, s>>>(vrec, m, cursor, eid, ent, err);
+    const uint32_t tiles = build_tiles(m);
+    if (int r = launch_exclusive_scan(stream, t.hist, t.offs, BF_NB * tiles, scan_tmp, scan_words)) return r;
+    k_build_fill_u<<<tiles, BF_T, 0, s>>>(t.edges, t.eword, t.rank, off, m, build_shift(n), tiles, t.offs, eid, ent,
+                                          t.vrec, t.err);
+    k_build_fill_v<<<(uint32_t)(((uint64_t)m + BF_T * BF_U - 1) / (BF_T * BF_U)), BF_T, 0, s>>>(t.vrec, m, eid, ent);
     return (int)cudaGetLastError();
 }
 int launch_nonzero_flags(void* stream, const uint32_t* deg, uint32_t n, uint32_t* flags, uint32_t* counts) {
