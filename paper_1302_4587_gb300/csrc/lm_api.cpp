@@ -1337,7 +1337,7 @@ int lm_contract(lm_ctx* ctx, uint32_t n, uint32_t m, const uint32_t* eu, const u
     }
     cv.assign(e.cblock);
     int rc = staging_ready(ctx, e);
-    if (!rc) rc = ensure_pinned(ctx, e, 32);
+    if (!rc) rc = ensure_pinned(ctx, e, 64);
     if (rc) return rc;
     uint32_t* hp = static_cast<uint32_t*>(e.pinned);
     cudaError_t ce = (cudaError_t)launch_contract(s, c, &hp[4]);

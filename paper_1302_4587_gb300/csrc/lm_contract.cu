@@ -9,21 +9,26 @@
 // is their sum (accumulated in double in input order, rounded once to float32).
 //
 // Device steps (all of them here): representatives and their prefix ranks;
-// the coarse map and vertex weights; every edge, in input order, gets a 32-bit
-// hash of its unordered coarse pair as a key (edges inside a pair the key
-// 0xFFFFFFFF; no pair's hash ends in the byte 0xFF, so that they end up last),
-// and its coarse endpoints are stored.  A stable LSD radix sort by the low B
-// bits of the hash (8-bit passes, as few as leave about 2048 edges to a
-// bucket of equal low bits) brings each pair's edges into one bucket, still in
-// input order.  Inside each bucket a shared-memory hash table finds the items
-// whose full hash repeats; each such run (a group of several edges, or pairs
-// whose hashes collide) is put in input order and walked: its groups' first
-// edges lead, every later member loses its crossing bit, and a leader of
-// several edges records the group's weight summed over its edges in order.
-// An edge alone with its hash is alone in its group and leads it.  Buckets,
-// runs too long or too mixed for that walk are taken out and sorted again by
-// the pair itself.  Prefix counts of the remaining bits (the leaders) give
-// each coarse edge its place, and the leaders write the coarse edges.
+// the coarse map and vertex weights; every edge gets a 32-bit hash of its unordered
+// coarse pair, and its coarse endpoints are stored.  The crossing edges go to
+// partitions by the hash's top bits (k_c_part); in each partition a bitmap in shared
+// memory finds the edges that share their slot of the hash with another (most pairs
+// have one edge, which then is done), and a hash table the ones whose full hash repeats
+// (k_c_groups).  Each such run (a group of several edges, or pairs whose hashes collide)
+// is put in input order and walked (k_c_walk): its groups' first edges lead, every later
+// member loses its crossing bit, and a leader of several edges records the group's
+// weight summed over its edges in order.  An edge alone with its hash is alone in its
+// group and leads it.  Runs too long or too mixed for that walk are taken out in input
+// order and sorted by the pair itself.  Prefix counts of the remaining bits (the leaders)
+// give each coarse edge its place, and the leaders write the coarse edges.
+// Lists that partitions don't suit (see contract_part_bits, and one with a partition of
+// more than twice the average) are sorted instead: a stable LSD radix sort by the low B
+// bits of the hash (8-bit passes, as few as leave about 2048 edges to a bucket of equal
+// low bits; edges inside a pair have the key 0xFFFFFFFF, and no pair's hash ends in the
+// byte 0xFF, so that they end up last) brings each pair's edges into one bucket, still in
+// input order, and k_c_buckets finds the runs.
+// R-MAT scale 22 (64M edges): sort 2.18 ms, partitions 1.42 (part 525, groups 327, walk
+// 125, emit 266 us, the rest map, scans and a host round trip).
 #include <cstdint>
 #include <type_traits>
 #include <cuda_runtime.h>
@@ -187,6 +192,139 @@ __global__ void __launch_bounds__(CT) k_c_keys(const uint32_t* __restrict__ eu, 
     hist[threadIdx.x * gridDim.x + blockIdx.x] = h[threadIdx.x];  // digit-major, as the sort's counts
 }
 
+// ---- partitions --------------------------------------------------------------
+// The crossing edges go to 2^pb partitions by the top bits of their hash, as (hash, edge)
+// items in no particular order, each partition in a room of cap items of its own
+// (gcur: its items; more than cap: the count goes on, the items are not kept).  A block
+// maps and keys a tile of PT_TILE edges, counts them by partition in shared memory
+// (each item's rank is what the count returned), takes a run of every partition's room with
+// one atomic, and writes the tile out in partition order, so that runs of 8 items and
+// more are written together.  Also writes cpair, cross and counts[0], as k_c_keys.
+// R-MAT scale 21, 31.8M edges: 268 us, of which the gathers of cmap 92, the items' stores
+// 26, cpair 33, the rest the phases in shared memory.  Three blocks an SM (spills), 8 or
+// 24 edges a thread, 256 or 1024 threads: 3 to 15% slower over all.
+constexpr uint32_t PT_T = 512, PT_E = 16, PT_TILE = PT_E * PT_T, PT_MAX = 1024, PT_D = PT_MAX / PT_T;
+struct PtSmem {
+    uint32_t key[PT_TILE];
+    uint16_t edge[PT_TILE];  // its place in the tile
+    uint32_t cnt[PT_MAX];   // items of each partition, then where its run starts in it
+    uint32_t gofs[PT_MAX];  // the run's place in the partition's room, minus that
+    uint32_t ws[PT_T / 32];
+};
+static_assert(PT_MAX % PT_T == 0 && PT_E % 8 == 0 && PT_TILE <= 65536, "PT_D partitions and PT_E edges a thread, 16-bit places");
+
+template <bool VEC>
+__global__ void __launch_bounds__(PT_T, 2)
+    k_c_part(const uint32_t* __restrict__ eu, const uint32_t* __restrict__ ev, uint32_t m, uint32_t n,
+             const uint32_t* __restrict__ cmap, uint32_t pb, uint32_t cap, uint32_t* __restrict__ gcur,
+             uint2* __restrict__ items, uint32_t* __restrict__ cpair, uint32_t* __restrict__ cross,
+             uint32_t* __restrict__ counts, uint32_t* __restrict__ err) {
+    extern __shared__ __align__(16) unsigned char pt_raw[];
+    PtSmem& S = *reinterpret_cast<PtSmem*>(pt_raw);
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t dsh = 32 - pb;
+    for (uint32_t i = tid; i < PT_MAX; i += PT_T) S.cnt[i] = 0;
+    __syncthreads();
+    uint32_t mine = 0, key[PT_E], rk[PT_E / 2];
+#pragma unroll
+    for (int it = 0; it < (int)PT_E / 8; it++) {
+        uint4 a[2], b[2];
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+            const uint64_t e0 = (uint64_t)blockIdx.x * PT_TILE + 4 * ((2 * it + u) * PT_T + tid);
+            a[u] = load4<VEC>(eu, e0, m);
+            b[u] = load4<VEC>(ev, e0, m);
+        }
+        uint32_t cu[2][4], cv[2][4];
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+            const uint64_t e0 = (uint64_t)blockIdx.x * PT_TILE + 4 * ((2 * it + u) * PT_T + tid);
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                const uint32_t x = at(a[u], j), y = at(b[u], j);
+                const bool ok = e0 + j < m && x < n && y < n;
+                if (e0 + j < m && !ok) atomicOr(err, C_ERR_EDGE);
+                cu[u][j] = ok ? cmap[x] : 0u;
+                cv[u][j] = ok ? cmap[y] : 0u;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+            const uint64_t e0 = (uint64_t)blockIdx.x * PT_TILE + 4 * ((2 * it + u) * PT_T + tid);
+            uint32_t nib = 0;
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                const int i = 8 * it + 4 * u + j;
+                key[i] = 0xFFFFFFFFu;
+                uint32_t r = 0;
+                if (cu[u][j] != cv[u][j]) {  // (never past m: both are 0 there)
+                    key[i] = pair_hash(pair_word(cu[u][j], cv[u][j]));
+                    nib |= 1u << j;
+                    r = atomicAdd(&S.cnt[key[i] >> dsh], 1u);
+                }
+                if (i & 1) rk[i >> 1] |= r << 16;
+                else rk[i >> 1] = r;
+            }
+            if (e0 + 4 <= m) {
+                *reinterpret_cast<uint4*>(cpair + 2 * e0) = make_uint4(cu[u][0], cv[u][0], cu[u][1], cv[u][1]);
+                *reinterpret_cast<uint4*>(cpair + 2 * e0 + 4) = make_uint4(cu[u][2], cv[u][2], cu[u][3], cv[u][3]);
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; j++)
+                    if (e0 + j < m) {
+                        cpair[2 * (e0 + j)] = cu[u][j];
+                        cpair[2 * (e0 + j) + 1] = cv[u][j];
+                    }
+            }
+            mine += __popc(nib);
+            uint32_t w = nib << (4 * (lane & 7));
+            w |= __shfl_xor_sync(0xFFFFFFFFu, w, 1);
+            w |= __shfl_xor_sync(0xFFFFFFFFu, w, 2);
+            w |= __shfl_xor_sync(0xFFFFFFFFu, w, 4);
+            if ((lane & 7) == 0 && e0 < m) cross[e0 >> 5] = w;
+        }
+    }
+    mine = __reduce_add_sync(0xFFFFFFFFu, mine);
+    if (lane == 0 && mine) atomicAdd(&counts[0], mine);
+    __syncthreads();
+    // thread t: partitions PT_D t .. PT_D t + PT_D - 1
+    uint32_t c[PT_D], x = 0;
+#pragma unroll
+    for (uint32_t i = 0; i < PT_D; i++) x += c[i] = S.cnt[PT_D * tid + i];
+    const uint32_t sum = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+        if (lane >= (uint32_t)o) x += y;
+    }
+    if (lane == 31) S.ws[warp] = x;
+    __syncthreads();
+    uint32_t start = x - sum, total = 0;
+    for (uint32_t w = 0; w < PT_T / 32; w++) {
+        if (w < warp) start += S.ws[w];
+        total += S.ws[w];
+    }
+#pragma unroll
+    for (uint32_t i = 0; i < PT_D; i++) {
+        if (c[i]) S.gofs[PT_D * tid + i] = atomicAdd(&gcur[PT_D * tid + i], c[i]) - start;
+        S.cnt[PT_D * tid + i] = start;
+        start += c[i];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < (int)PT_E; i++) {
+        if (key[i] == 0xFFFFFFFFu) continue;
+        const uint32_t p = S.cnt[key[i] >> dsh] + ((rk[i >> 1] >> (16 * (i & 1))) & 0xFFFFu);
+        S.key[p] = key[i];
+        S.edge[p] = (uint16_t)(4 * ((i >> 2) * PT_T + tid) + (i & 3));
+    }
+    __syncthreads();
+    for (uint32_t p = tid; p < total; p += PT_T) {
+        const uint32_t x = S.key[p], d = x >> dsh, o = S.gofs[d] + p;
+        if (o < cap) items[(size_t)d * cap + o] = make_uint2(x, blockIdx.x * PT_TILE + S.edge[p]);
+    }
+}
+
 // ---- buckets of the partial hash sort --------------------------------------
 // The sort orders the items by the low B bits of their keys only, so a bucket
 // (the items sharing those bits) holds every edge of each of its pairs, in input
@@ -202,13 +340,14 @@ __global__ void __launch_bounds__(CT) k_c_keys(const uint32_t* __restrict__ eu, 
 // several edges gets its multi bit and the group's weight summed in double in
 // input order once the run is known to fit.  A bucket that runs past the window
 // is done in a second window that starts at it.  A bucket longer than a window,
-// and any run that does not fit the walk, is flagged in ofl for the general path
-// below: taken out in order with its pair as the key and sorted again by the pair
+// and any run that does not fit the walk, is flagged in ofl (a bit per edge) for the
+// general path below: taken out in order with its pair as the key and sorted by the pair
 // (which clears the same bits again).
 constexpr uint32_t GR_MAX = 64, GR_PAIRS = 4;
 constexpr uint32_t BK_T = 512, BK_J = 12, BK_W = BK_T * BK_J, BK_C = 4096, BK_TS = 8192, BK_TS_BITS = 13;
 constexpr uint32_t BK_AVG = 2048;  // the sort takes as few bytes as leave at most this many items to a bucket
 constexpr uint32_t BK_EMPTY = 0xFFFFFFFFu;
+constexpr uint32_t RUN_START = 0x80000000u, RUN_NONE = 0xFFFFFFFFu;  // (edges are below 2^31 - 1)
 static_assert(BK_TS == 1u << BK_TS_BITS && BK_TS / 16 == BK_T && BK_W < BK_TS && BK_W < 65536 && BK_C < BK_W,
               "table of at most 3/4 load, 16-bit counts and window indices, a chunk shorter than a window");
 
@@ -224,89 +363,231 @@ struct BkSmem {
     uint32_t first, lastp1, end, ndup;
 };
 
-__device__ __forceinline__ uint32_t bk_slot(uint32_t k) { return (k * 0x9E3779B1u) >> (32 - BK_TS_BITS); }
+template <uint32_t TSB>
+__device__ __forceinline__ uint32_t bk_slot(uint32_t k) {
+    return (k * 0x9E3779B1u) >> (32 - TSB);
+}
 
 __device__ __forceinline__ unsigned long long upair(const uint32_t* __restrict__ cpair, uint32_t e) {
     const uint2 p = *reinterpret_cast<const uint2*>(cpair + 2 * (size_t)e);
     return ((unsigned long long)min(p.x, p.y) << 32) | max(p.x, p.y);
 }
 
-// One run of dl[i .. i + len) (window indices in input order), items at sorted
-// positions ws + index: settled here, or flagged for the general path.
-__device__ void bk_walk(const BkSmem& S, uint32_t i, uint32_t len, uint32_t ws, const uint32_t* __restrict__ val,
-                        const uint32_t* __restrict__ cpair, const float* __restrict__ w, uint32_t* __restrict__ cross,
-                        uint32_t* __restrict__ multi, uint32_t* __restrict__ gsum, uint32_t* __restrict__ ofl,
-                        uint32_t* __restrict__ counts) {
-    unsigned long long gp[GR_PAIRS];
-    uint32_t gl[GR_PAIRS], gn[GR_PAIRS];
-    double gs[GR_PAIRS];
-    uint32_t ng = 0;
-    bool over = len > GR_MAX;
-    for (uint32_t j0 = 0; j0 < len && !over; j0 += 4) {
-        uint32_t e[4];
-        unsigned long long pj[4];
-        float wj[4];
+// The items lo <= q < hi of a window (item q: thread q % T, k[q / T]) with edges val[q]: those
+// whose key repeats, by the table in S, which is cleared (val in input order, or
+// BYVAL: in any).
+template <uint32_t T, uint32_t J, uint32_t TSB, bool BYVAL, class SM>
+__device__ __forceinline__ void bk_table(SM& S, const uint32_t (&k)[J], uint32_t lo, uint32_t hi, const uint32_t* val,
+                                         uint32_t* __restrict__ list, uint32_t* __restrict__ ofl,
+                                         uint32_t* __restrict__ counts) {
+    constexpr uint32_t TS = 1u << TSB;
+    static_assert(TS / 16 == T && T * J < TS && T * J < 65536, "16 slots a thread, a free slot always");
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // every item of [lo, hi) into the table; its slot kept in 16 bits of sp
+    uint32_t sp[(J + 1) / 2];
 #pragma unroll
-        for (uint32_t t = 0; t < 4; t++) e[t] = j0 + t < len ? val[ws + (S.dl[i + j0 + t] & 0xFFFFu)] : 0u;
-#pragma unroll
-        for (uint32_t t = 0; t < 4; t++) {
-            pj[t] = j0 + t < len ? upair(cpair, e[t]) : 0ull;
-            wj[t] = j0 + t < len ? w[e[t]] : 0.0f;
+    for (int j = 0; j < (int)J; j++) {
+        const uint32_t q = j * T + tid;
+        uint32_t sl = 0;
+        if (q >= lo && q < hi) {
+            sl = bk_slot<TSB>(k[j]);
+            // (at most the window < TS keys: a free slot or the key is always found)
+            for (uint32_t probe = 0; probe < TS; probe++) {
+                const uint32_t old = atomicCAS(&S.tab[sl], BK_EMPTY, k[j]);
+                if (old == BK_EMPTY || old == k[j]) break;
+                sl = (sl + 1) & (TS - 1);
+            }
+            atomicAdd(&S.cnt[sl >> 1], 1u << (16 * (sl & 1)));
         }
+        if (j & 1) sp[j >> 1] |= sl << 16;
+        else sp[j >> 1] = sl;
+    }
+    __syncthreads();
+    // slots of two or more items, and where each one's run starts in dl (thread t:
+    // slots 16 t .. 16 t + 15, cnt words 8 t .. 8 t + 7)
+    {
+        uint4* cq = reinterpret_cast<uint4*>(S.cnt) + 2 * tid;
+        uint32_t tot = 0, bits = 0;
 #pragma unroll
-        for (uint32_t t = 0; t < 4; t++) {
-            if (j0 + t >= len || over) continue;
-            bool found = false;
+        for (int v = 0; v < 2; v++) {
+            const uint4 x = cq[v];
+            const uint32_t wv[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-            for (uint32_t g = 0; g < GR_PAIRS; g++)
-                if (!found && g < ng && gp[g] == pj[t]) {
-                    gs[g] += (double)wj[t];
-                    gn[g]++;
-                    found = true;
-                }
-            // a later member of a group: not a leader, whatever the rest of the run
-            // holds (a run left to the general path has the same bits cleared there)
-            if (found) atomicAnd(&cross[e[t] >> 5], ~(1u << (e[t] & 31)));
-            if (!found) {
-                if (ng == GR_PAIRS) {
-                    over = true;
-                } else {
-#pragma unroll
-                    for (uint32_t g = 0; g < GR_PAIRS; g++)
-                        if (g == ng) {
-                            gp[g] = pj[t];
-                            gl[g] = e[t];
-                            gn[g] = 1;
-                            gs[g] = (double)wj[t];
-                        }
-                    ng++;
+            for (int h = 0; h < 8; h++) {
+                const uint32_t c = (wv[h >> 1] >> (16 * (h & 1))) & 0xFFFFu;
+                if (c >= 2) {
+                    tot += c;
+                    bits |= 1u << (8 * v + h);
                 }
             }
         }
-    }
-    if (over) {
-        for (uint32_t a = 0; a < len; a++) {
-            const uint32_t p = ws + (S.dl[i + a] & 0xFFFFu);
-            atomicOr(&ofl[p >> 5], 1u << (p & 31));
-        }
-        atomicAdd(&counts[1], len);
-        return;
-    }
+        uint32_t x = tot;
 #pragma unroll
-    for (uint32_t g = 0; g < GR_PAIRS; g++)
-        if (g < ng && gn[g] > 1) {
-            atomicOr(&multi[gl[g] >> 5], 1u << (gl[g] & 31));
-            gsum[gl[g]] = __float_as_uint((float)gs[g]);
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+            if (lane >= (uint32_t)o) x += y;
         }
+        if (lane == 31) S.wsum[warp] = x;
+        __syncthreads();
+        uint32_t run = x - tot;
+        for (uint32_t v = 0; v < warp; v++) run += S.wsum[v];
+#pragma unroll
+        for (int v = 0; v < 2; v++) {
+            if (!((bits >> (8 * v)) & 0xFFu)) continue;
+            const uint4 x4 = cq[v];
+            uint32_t wv[4] = {x4.x, x4.y, x4.z, x4.w};
+#pragma unroll
+            for (int h = 0; h < 8; h++) {
+                if (!((bits >> (8 * v + h)) & 1u)) continue;
+                const uint32_t sh = 16 * (h & 1);
+                const uint32_t c = (wv[h >> 1] >> sh) & 0xFFFFu;
+                wv[h >> 1] = (wv[h >> 1] & ~(0xFFFFu << sh)) | (run << sh);
+                run += c;
+            }
+            cq[v] = make_uint4(wv[0], wv[1], wv[2], wv[3]);
+        }
+        reinterpret_cast<uint16_t*>(S.dupb)[tid] = (uint16_t)bits;  // bit 16 t + h: slot 16 t + h
+        if (tid == T - 1) S.ndup = run;
+    }
+    __syncthreads();
+    // the items of repeated keys into dl, grouped by slot
+#pragma unroll
+    for (int j = 0; j < (int)J; j++) {
+        const uint32_t q = j * T + tid;
+        if (q >= lo && q < hi) {
+            const uint32_t sl = (sp[j >> 1] >> (16 * (j & 1))) & 0xFFFFu;
+            if ((S.dupb[sl >> 5] >> (sl & 31)) & 1u) {
+                const uint32_t sh = 16 * (sl & 1);
+                const uint32_t pos = (atomicAdd(&S.cnt[sl >> 1], 1u << sh) >> sh) & 0xFFFFu;
+                S.dl[pos] = (sl << 16) | q;
+            }
+        }
+    }
+    __syncthreads();
+    // each run by the thread that holds its first entry: back in input order
+    // (insertion sort on the window index, or on the edge; its entries share their slot
+    // bits, which is all that other threads read of them); a long one is flagged
+    const uint32_t nd = S.ndup;
+    for (uint32_t i = tid; i < nd; i += T) {
+        const uint32_t sl = S.dl[i] >> 16;
+        if (i > 0 && (S.dl[i - 1] >> 16) == sl) continue;
+        uint32_t len = 1;
+        while (i + len < nd && (S.dl[i + len] >> 16) == sl) len++;
+        if (len > GR_MAX) {
+            for (uint32_t a = 0; a < len; a++) {
+                const uint32_t p = val[S.dl[i + a] & 0xFFFFu];
+                atomicOr(&ofl[p >> 5], 1u << (p & 31));
+                S.dl[i + a] |= 0xFFFFu;  // (no window index)
+            }
+            atomicAdd(&counts[1], len);
+            continue;
+        }
+        for (uint32_t a = 1; a < len; a++) {
+            const uint32_t y = S.dl[i + a], vy = BYVAL ? val[y & 0xFFFFu] : y;
+            uint32_t b = a;
+            for (; b > 0; b--) {
+                const uint32_t z = S.dl[i + b - 1];
+                if ((BYVAL ? val[z & 0xFFFFu] : z) < vy) break;
+                S.dl[i + b] = z;
+            }
+            S.dl[i + b] = y;
+        }
+    }
+    if (tid == 0 && nd) S.wsum[0] = atomicAdd(&counts[5], nd);
+    __syncthreads();
+    const uint32_t lbase = S.wsum[0];
+    for (uint32_t i = tid; i < nd; i += T) {
+        const uint32_t x = S.dl[i];
+        const bool start = i == 0 || (S.dl[i - 1] >> 16) != (x >> 16);
+        list[lbase + i] = (x & 0xFFFFu) == 0xFFFFu ? RUN_NONE : val[x & 0xFFFFu] | (start ? RUN_START : 0u);
+    }
+}
+
+// The runs of list (counts[5] entries: edges in input order, RUN_START on a run's first; runs
+// of at most GR_MAX), a thread each: settled here, or flagged for the general path.  A
+// kernel of its own: the gathers of pairs and weights are all that it does, with every
+// warp that an SM holds to cover them (as the last phase of the table's block, which
+// has 32 warps an SM, they took 84 us on R-MAT scale 21, here 54).
+__global__ void __launch_bounds__(CT) k_c_walk(const uint32_t* __restrict__ list,
+                                               const uint32_t* __restrict__ cpair, const float* __restrict__ w,
+                                               uint32_t* __restrict__ cross, uint32_t* __restrict__ multi,
+                                               uint32_t* __restrict__ gsum, uint32_t* __restrict__ ofl,
+                                               uint32_t* __restrict__ counts) {
+    const uint32_t nlist = counts[5];
+    for (uint32_t i0 = blockIdx.x * CT + threadIdx.x; i0 < nlist; i0 += gridDim.x * CT) {
+        const uint32_t first = list[i0];
+        if (!(first & RUN_START) || first == RUN_NONE) continue;
+        uint32_t len = 1;
+        while (len <= GR_MAX && i0 + len < nlist && !(list[i0 + len] & RUN_START)) len++;
+        unsigned long long gp[GR_PAIRS];
+        uint32_t gl[GR_PAIRS], gn[GR_PAIRS];
+        double gs[GR_PAIRS];
+        uint32_t ng = 0;
+        bool over = false;
+        for (uint32_t j0 = 0; j0 < len && !over; j0 += 4) {
+            uint32_t e[4];
+            unsigned long long pj[4];
+            float wj[4];
+#pragma unroll
+            for (uint32_t t = 0; t < 4; t++) e[t] = j0 + t < len ? list[i0 + j0 + t] & ~RUN_START : 0u;
+#pragma unroll
+            for (uint32_t t = 0; t < 4; t++) {
+                pj[t] = j0 + t < len ? upair(cpair, e[t]) : 0ull;
+                wj[t] = j0 + t < len ? w[e[t]] : 0.0f;
+            }
+#pragma unroll
+            for (uint32_t t = 0; t < 4; t++) {
+                if (j0 + t >= len || over) continue;
+                bool found = false;
+#pragma unroll
+                for (uint32_t g = 0; g < GR_PAIRS; g++)
+                    if (!found && g < ng && gp[g] == pj[t]) {
+                        gs[g] += (double)wj[t];
+                        gn[g]++;
+                        found = true;
+                    }
+                // a later member of a group: not a leader, whatever the rest of the run
+                // holds (a run left to the general path has the same bits cleared there)
+                if (found) atomicAnd(&cross[e[t] >> 5], ~(1u << (e[t] & 31)));
+                if (!found) {
+                    if (ng == GR_PAIRS) {
+                        over = true;
+                    } else {
+#pragma unroll
+                        for (uint32_t g = 0; g < GR_PAIRS; g++)
+                            if (g == ng) {
+                                gp[g] = pj[t];
+                                gl[g] = e[t];
+                                gn[g] = 1;
+                                gs[g] = (double)wj[t];
+                            }
+                        ng++;
+                    }
+                }
+            }
+        }
+        if (over) {
+            for (uint32_t a = 0; a < len; a++) {
+                const uint32_t p = list[i0 + a] & ~RUN_START;
+                atomicOr(&ofl[p >> 5], 1u << (p & 31));
+            }
+            atomicAdd(&counts[1], len);
+            continue;
+        }
+#pragma unroll
+        for (uint32_t g = 0; g < GR_PAIRS; g++)
+            if (g < ng && gn[g] > 1) {
+                atomicOr(&multi[gl[g] >> 5], 1u << (gl[g] & 31));
+                gsum[gl[g]] = __float_as_uint((float)gs[g]);
+            }
+    }
 }
 
 // key: the sorted keys of the cnt crossing items (sorted by the bits in mask);
 // val: their edge indices
 __global__ void __launch_bounds__(BK_T, 2)
     k_c_buckets(const uint32_t* __restrict__ key, const uint32_t* __restrict__ val, uint32_t cnt, uint32_t mask,
-                const uint32_t* __restrict__ cpair, const float* __restrict__ w, uint32_t* __restrict__ cross,
-                uint32_t* __restrict__ multi, uint32_t* __restrict__ gsum, uint32_t* __restrict__ ofl,
-                uint32_t* __restrict__ counts) {
+                uint32_t* __restrict__ list, uint32_t* __restrict__ ofl, uint32_t* __restrict__ counts) {
     extern __shared__ __align__(16) unsigned char bk_raw[];
     BkSmem& S = *reinterpret_cast<BkSmem*>(bk_raw);
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -387,7 +668,8 @@ __global__ void __launch_bounds__(BK_T, 2)
                 const bool in = p < cnt && (key[p] & mask) == bv;
                 if (!__syncthreads_or(in)) break;
                 if (in) {
-                    atomicOr(&ofl[p >> 5], 1u << (p & 31));
+                    const uint32_t x = val[p];
+                    atomicOr(&ofl[x >> 5], 1u << (x & 31));
                     mine++;
                 }
             }
@@ -395,117 +677,132 @@ __global__ void __launch_bounds__(BK_T, 2)
             if (lane == 0 && mine) atomicAdd(&counts[1], mine);
             return;
         }
-        // every item of [lo, hi) into the table; its slot kept in 16 bits of sp
-        uint32_t sp[BK_J / 2];
-#pragma unroll
-        for (int j = 0; j < (int)BK_J; j++) {
-            const uint32_t q = j * BK_T + tid;
-            uint32_t sl = 0;
-            if (q >= lo && q < hi) {
-                sl = bk_slot(k[j]);
-                // (at most BK_W < BK_TS keys: a free slot or the key is always found)
-                for (uint32_t probe = 0; probe < BK_TS; probe++) {
-                    const uint32_t old = atomicCAS(&S.tab[sl], BK_EMPTY, k[j]);
-                    if (old == BK_EMPTY || old == k[j]) break;
-                    sl = (sl + 1) & (BK_TS - 1);
-                }
-                atomicAdd(&S.cnt[sl >> 1], 1u << (16 * (sl & 1)));
-            }
-            if (j & 1) sp[j >> 1] |= sl << 16;
-            else sp[j >> 1] = sl;
-        }
-        __syncthreads();
-        // slots of two or more items, and where each one's run starts in dl (thread t:
-        // slots 16 t .. 16 t + 15, cnt words 8 t .. 8 t + 7)
-        {
-            uint4* cq = reinterpret_cast<uint4*>(S.cnt) + 2 * tid;
-            uint32_t tot = 0, bits = 0;
-#pragma unroll
-            for (int v = 0; v < 2; v++) {
-                const uint4 x = cq[v];
-                const uint32_t wv[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-                for (int h = 0; h < 8; h++) {
-                    const uint32_t c = (wv[h >> 1] >> (16 * (h & 1))) & 0xFFFFu;
-                    if (c >= 2) {
-                        tot += c;
-                        bits |= 1u << (8 * v + h);
-                    }
-                }
-            }
-            uint32_t x = tot;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-                if (lane >= (uint32_t)o) x += y;
-            }
-            if (lane == 31) S.wsum[warp] = x;
-            __syncthreads();
-            uint32_t run = x - tot;
-            for (uint32_t v = 0; v < warp; v++) run += S.wsum[v];
-#pragma unroll
-            for (int v = 0; v < 2; v++) {
-                if (!((bits >> (8 * v)) & 0xFFu)) continue;
-                const uint4 x4 = cq[v];
-                uint32_t wv[4] = {x4.x, x4.y, x4.z, x4.w};
-#pragma unroll
-                for (int h = 0; h < 8; h++) {
-                    if (!((bits >> (8 * v + h)) & 1u)) continue;
-                    const uint32_t sh = 16 * (h & 1);
-                    const uint32_t c = (wv[h >> 1] >> sh) & 0xFFFFu;
-                    wv[h >> 1] = (wv[h >> 1] & ~(0xFFFFu << sh)) | (run << sh);
-                    run += c;
-                }
-                cq[v] = make_uint4(wv[0], wv[1], wv[2], wv[3]);
-            }
-            reinterpret_cast<uint16_t*>(S.dupb)[tid] = (uint16_t)bits;  // bit 16 t + h: slot 16 t + h
-            if (tid == BK_T - 1) S.ndup = run;
-        }
-        __syncthreads();
-        // the items of repeated keys into dl, grouped by slot
-#pragma unroll
-        for (int j = 0; j < (int)BK_J; j++) {
-            const uint32_t q = j * BK_T + tid;
-            if (q >= lo && q < hi) {
-                const uint32_t sl = (sp[j >> 1] >> (16 * (j & 1))) & 0xFFFFu;
-                if ((S.dupb[sl >> 5] >> (sl & 31)) & 1u) {
-                    const uint32_t sh = 16 * (sl & 1);
-                    const uint32_t pos = (atomicAdd(&S.cnt[sl >> 1], 1u << sh) >> sh) & 0xFFFFu;
-                    S.dl[pos] = (sl << 16) | q;
-                }
-            }
-        }
-        __syncthreads();
-        // each run by the thread that holds its first entry: back in input order
-        // (insertion sort on the window index; its entries share their slot bits, which
-        // is all that other threads read of them), then walked
-        const uint32_t nd = S.ndup;
-        for (uint32_t i = tid; i < nd; i += BK_T) {
-            const uint32_t sl = S.dl[i] >> 16;
-            if (i > 0 && (S.dl[i - 1] >> 16) == sl) continue;
-            uint32_t len = 1;
-            while (i + len < nd && (S.dl[i + len] >> 16) == sl) len++;
-            if (len <= GR_MAX)
-                for (uint32_t a = 1; a < len; a++) {
-                    const uint32_t y = S.dl[i + a];
-                    uint32_t b = a;
-                    for (; b > 0 && S.dl[i + b - 1] > y; b--) S.dl[i + b] = S.dl[i + b - 1];
-                    S.dl[i + b] = y;
-                }
-            bk_walk(S, i, len, ws, val, cpair, w, cross, multi, gsum, ofl, counts);
-        }
+        bk_table<BK_T, BK_J, BK_TS_BITS, false>(S, k, lo, hi, val + ws, list, ofl, counts);
         if (!again) return;
         __syncthreads();  // (dl and the table are free again)
         ws += hi > s ? hi : s;
     }
 }
 
-// The general path: the flagged items, a tile of 4096 per block, thread t holding
-// chunks c = 0..3 of four items at tile offset 1024 c + 4 t.  One launch counts
+// One partition a block: all edges of each of its pairs.  Most pairs have one edge; a
+// bitmap over slots of the hash (seen, and rep: seen again) finds the items that share
+// their slot (about an eighth by chance, at 8 slots an item, and the groups), and only
+// these go through the table, GP_CAP of them at a time: when there are more, those
+// of one residue of the hash at a time, each a pass over the partition (from L2).  A
+// residue with more than GP_CAP is left to the general path.
+// Two blocks of 512 threads an SM; one of 1024 with bitmaps, table and lists twice as
+// large where a partition has more than 32768 items (scale 21, 31K items: 763 and 800 us
+// over all; scale 22, 62K items: 2150 and 1424).  R-MAT scale 21: 154 us, of which both
+// passes over the items 120 (a bitmap in L2 instead, by atomics of the keys' kernel, cost
+// it 240 us: 130 G atomics/s).
+// counts[4]: a partition outgrew its room (nothing of this is used then).
+constexpr uint32_t GP_J = 12;
+template <int B>  // 512 << B threads
+struct GpSmem {
+    static constexpr uint32_t GP_T = 512u << B, GP_CAP = GP_T * GP_J, GP_TSB = 13 + B, GP_BITS = 18 + B;
+    uint32_t rep[1u << (GP_BITS - 5)];
+    union {
+        uint32_t seen[1u << (GP_BITS - 5)];
+        uint32_t keyl[GP_CAP];
+        uint32_t tab[1u << GP_TSB];
+        uint32_t dl[GP_CAP];
+    };
+    uint32_t cnt[1u << (GP_TSB - 1)];
+    uint32_t vall[GP_CAP];
+    uint32_t dupb[(1u << GP_TSB) / 32];
+    uint32_t wsum[GP_T / 32];
+    uint32_t ndup, nc;
+};
+
+template <int B>
+__global__ void __launch_bounds__(512 << B, 2 >> B)
+    k_c_groups(const uint2* __restrict__ items, const uint32_t* __restrict__ gcur, uint32_t cap, uint32_t pb,
+               uint32_t gb, uint32_t* __restrict__ list, uint32_t* __restrict__ ofl, uint32_t* __restrict__ counts) {
+    using SM = GpSmem<B>;
+    constexpr uint32_t GP_T = SM::GP_T, GP_CAP = SM::GP_CAP, GP_TSB = SM::GP_TSB;
+    extern __shared__ __align__(16) unsigned char gp_raw[];
+    SM& S = *reinterpret_cast<SM*>(gp_raw);
+    const uint32_t tid = threadIdx.x, lane = tid & 31;
+    const uint32_t total = gcur[blockIdx.x];
+    if (total > cap) {
+        if (tid == 0) atomicOr(&counts[4], 1u);
+        return;
+    }
+    const uint2* it = items + (size_t)blockIdx.x * cap;
+    for (uint32_t i = tid; i < 1u << (gb - 5); i += GP_T) S.seen[i] = S.rep[i] = 0;
+    __syncthreads();
+    const uint32_t gsh = 32 - gb;  // a slot: the gb bits of the key below the partition's
+    for (uint32_t i0 = tid; i0 < total; i0 += 8 * GP_T) {
+        uint32_t k[8];
+#pragma unroll
+        for (int q = 0; q < 8; q++) k[q] = i0 + q * GP_T < total ? it[i0 + q * GP_T].x : 0u;
+#pragma unroll
+        for (int q = 0; q < 8; q++) {
+            const uint32_t s = (k[q] << pb) >> gsh, bit = 1u << (s & 31);
+            if (i0 + q * GP_T < total && (atomicOr(&S.seen[s >> 5], bit) & bit)) atomicOr(&S.rep[s >> 5], bit);
+        }
+    }
+    __syncthreads();
+    uint32_t rounds = 1;  // residues (a power of two)
+    for (uint32_t r = 0; r < rounds;) {
+        if (tid == 0) S.nc = 0;
+        __syncthreads();
+        for (uint32_t i0 = tid; i0 - tid < total; i0 += 8 * GP_T) {  // (whole warps)
+            uint2 v[8];
+#pragma unroll
+            for (int q = 0; q < 8; q++) v[q] = i0 + q * GP_T < total ? it[i0 + q * GP_T] : make_uint2(0, 0);
+#pragma unroll
+            for (int q = 0; q < 8; q++) {
+                const uint32_t s = (v[q].x << pb) >> gsh;
+                const bool in = i0 + q * GP_T < total && (v[q].x & (rounds - 1)) == r && ((S.rep[s >> 5] >> (s & 31)) & 1u);
+                const uint32_t b = __ballot_sync(0xFFFFFFFFu, in);
+                uint32_t p = 0;
+                if (b && lane == 0) p = atomicAdd(&S.nc, __popc(b));
+                p = __shfl_sync(0xFFFFFFFFu, p, 0) + __popc(b & ((1u << lane) - 1u));
+                if (in && p < GP_CAP) {
+                    S.keyl[p] = v[q].x;
+                    S.vall[p] = v[q].y;
+                }
+            }
+        }
+        __syncthreads();
+        const uint32_t nc = S.nc;
+        if (nc > GP_CAP) {
+            if (rounds == 1) {  // from the start, by residues that leave a margin
+                while (rounds < 4096 && nc > (rounds * GP_CAP) / 8 * 7) rounds *= 2;
+                __syncthreads();
+                continue;
+            }
+            for (uint32_t i = tid; i < total; i += GP_T) {
+                const uint2 v = it[i];
+                const uint32_t s = (v.x << pb) >> gsh;
+                if ((v.x & (rounds - 1)) == r && ((S.rep[s >> 5] >> (s & 31)) & 1u))
+                    atomicOr(&ofl[v.y >> 5], 1u << (v.y & 31));
+            }
+            if (tid == 0) atomicAdd(&counts[1], nc);
+        } else if (nc > 1) {
+            uint32_t k[GP_J];
+#pragma unroll
+            for (int j = 0; j < (int)GP_J; j++) k[j] = j * GP_T + tid < nc ? S.keyl[j * GP_T + tid] : BK_EMPTY;
+            __syncthreads();
+            for (uint32_t i = tid; i < (1u << GP_TSB) / 4; i += GP_T)
+                reinterpret_cast<uint4*>(S.tab)[i] = make_uint4(BK_EMPTY, BK_EMPTY, BK_EMPTY, BK_EMPTY);
+            for (uint32_t i = tid; i < (1u << GP_TSB) / 8; i += GP_T)
+                reinterpret_cast<uint4*>(S.cnt)[i] = make_uint4(0, 0, 0, 0);
+            __syncthreads();
+            bk_table<GP_T, GP_J, GP_TSB, true>(S, k, 0, nc, S.vall, list, ofl, counts);
+        }
+        __syncthreads();  // (the lists are free again)
+        r++;
+    }
+}
+
+// The general path: the flagged edges, a tile of 4096 per block, thread t holding
+// chunks c = 0..3 of four edges at tile offset 1024 c + 4 t.  One launch counts
 // them per tile; after a scan of the counts the second takes them out in order.
 constexpr uint32_t RN_TILE = 4096;
 
-// bit j: item i + j is flagged (i a multiple of 4)
+// bit j: edge i + j is flagged (i a multiple of 4)
 __device__ __forceinline__ uint32_t run_bits(const uint32_t* __restrict__ ofl, uint64_t i, uint32_t cnt) {
     return i < cnt ? (ofl[i >> 5] >> (i & 31)) & 0xFu : 0u;
 }
@@ -529,12 +826,12 @@ __global__ void __launch_bounds__(CT) k_c_runs_count(const uint32_t* __restrict_
     }
 }
 
-// the flagged items in sorted order (so a pair's edges keep their input order), with
+// the flagged edges in input order, with
 // (min, max) of their coarse pair as the key of a second sort; counts[3] = how many.
 // The tile's run items are listed in shared memory first, so that the gathers of
 // their pairs spread over all threads.
-__global__ void __launch_bounds__(CT) k_c_runs_take(const uint32_t* __restrict__ ofl, const uint32_t* __restrict__ val,
-                                                    uint32_t cnt, const uint32_t* __restrict__ toffs,
+__global__ void __launch_bounds__(CT) k_c_runs_take(const uint32_t* __restrict__ ofl, uint32_t cnt,
+                                                    const uint32_t* __restrict__ toffs,
                                                     const uint32_t* __restrict__ cpair, uint32_t bits,
                                                     unsigned long long* __restrict__ skey,
                                                     uint32_t* __restrict__ sval, uint32_t* __restrict__ counts) {
@@ -572,7 +869,7 @@ __global__ void __launch_bounds__(CT) k_c_runs_take(const uint32_t* __restrict__
     __syncthreads();
     const uint32_t off = toffs[blockIdx.x];
     for (uint32_t q = threadIdx.x; q < run; q += CT) {
-        const uint32_t e = val[tile0 + list[q]];
+        const uint32_t e = (uint32_t)tile0 + list[q];
         const uint2 cp = *reinterpret_cast<const uint2*>(cpair + 2 * (size_t)e);
         const uint32_t x = cp.x, y = cp.y;
         skey[off + q] = ((unsigned long long)min(x, y) << bits) | max(x, y);  // coarse ids take `bits` bits
@@ -820,6 +1117,20 @@ uint32_t bits_for(uint32_t x) {  // bits to write 0 .. x
 
 }  // namespace
 
+// log2 of the partitions, or 0: the list is sorted by the hash.  About 8192 edges to a
+// partition as long as there are at most PT_MAX (more would be written in runs of less
+// than 8 items: R-MAT scale 22 1.54 ms at 2048 partitions, 1.42 at 1024).  Partitions beat
+// the sort from the smallest lists (fewer launches: 1,000 edges 99 us against 122, 1M
+// edges 142 against 210) to the largest measured (R-MAT scale 24, 232M edges, 9.8 ms
+// against 10.0), where three quarters of the slots are shared and the gain ends; so the
+// line lies at 2^28 edges.  A caller that sets the sort's width gets the sort.
+static uint32_t contract_part_bits(uint32_t m, uint32_t sort_bits) {
+    if (sort_bits || m > 1u << 28) return 0;
+    uint32_t b = 1;
+    while ((2u << b) <= PT_MAX && (m >> b) > 8192) b++;
+    return b;
+}
+
 size_t contract_sort_words(uint32_t m) {
     const uint64_t tiles = ((uint64_t)m + RS_TILE - 1) / RS_TILE;
     return (size_t)(2 * (256 * tiles + 4));
@@ -863,78 +1174,103 @@ int launch_contract(void* stream, const ContractArgs& c, uint32_t* mc_host_slot)
         }
         return (int)cudaGetLastError();
     };
-    // 1. every edge keyed by its pair's hash in input order; the stable sort keeps input
-    //    order among equal keys and puts the edges inside pairs last, after the mc crossing edges
     uint32_t* hk[2] = {reinterpret_cast<uint32_t*>(c.key[0]), reinterpret_cast<uint32_t*>(c.key[1])};
     const uint32_t words = (uint32_t)(((uint64_t)c.m + 31) / 32);
     const uint32_t egrid = grid_for(((uint64_t)c.m + 3) / 4);
     const bool vec = ((reinterpret_cast<uintptr_t>(c.eu) | reinterpret_cast<uintptr_t>(c.ev) |
                        reinterpret_cast<uintptr_t>(c.w)) & 15u) == 0;
-    if ((e = cudaMemsetAsync(c.counts, 0, 8 * sizeof(uint32_t), s))) return (int)e;
-    static_assert(RS_TILE == 4096 && CT == 256, "k_c_keys takes one tile of the sort per block");
-    const uint32_t kgrid = (uint32_t)(((uint64_t)c.m + RS_TILE - 1) / RS_TILE);  // the sort's tiles
-    if (vec)
-        k_c_keys<true><<<kgrid, CT, 0, s>>>(c.eu, c.ev, c.m, c.n, c.cmap, hk[0], c.cpair, c.cross, c.counts, c.shist,
-                                            c.err);
-    else
-        k_c_keys<false><<<kgrid, CT, 0, s>>>(c.eu, c.ev, c.m, c.n, c.cmap, hk[0], c.cpair, c.cross, c.counts, c.shist,
-                                             c.err);
-    if ((e = cudaMemcpyAsync(mc_host_slot, c.counts, sizeof(uint32_t), cudaMemcpyDeviceToHost, s))) return (int)e;
-    if ((e = cudaMemcpyAsync(mc_host_slot + 1, c.rank + c.n, sizeof(uint32_t), cudaMemcpyDeviceToHost, s))) return (int)e;
-    if ((e = cudaStreamSynchronize(s))) return (int)e;
-    const uint32_t mc = mc_host_slot[0], nc = mc_host_slot[1];
-    // the sort's bits: as few bytes as leave at most BK_AVG crossing edges to a bucket
-    uint32_t sbits = c.sort_bits;
-    if (!sbits)
-        for (sbits = 8; sbits < 32 && (uint64_t)mc > ((uint64_t)BK_AVG << sbits); sbits += 8) {
-        }
-    const uint32_t mask = sbits >= 32 ? ~0u : (1u << sbits) - 1u;
-    int hc = 0;
-    if (mc > 1)
-        if (int r = radix(hk[0], hk[1], c.val[0], c.val[1], c.m, sbits, true, true, &hc)) return r;
-    // 2. runs of equal hash (groups of several edges, and collisions): the crossing bits
-    //    become the leader bits, every group member but the first cleared.  Runs with
-    //    few pairs are settled by k_c_buckets; the rest are taken out in sorted order
-    //    with their pair as the key, sorted again by the pair and marked.
-    if ((e = cudaMemsetAsync(c.multi, 0, ((size_t)c.m / 32 + 2) * sizeof(uint32_t), s))) return (int)e;
-    uint32_t nsub = 0;
-    const uint32_t bits = bits_for(nc ? nc - 1 : 0);
     uint32_t* ofl = c.wlead;  // (free until the leaders are counted)
-    if (mc > 1) {
-        if ((e = cudaMemsetAsync(ofl, 0, ((size_t)mc / 32 + 2) * sizeof(uint32_t), s))) return (int)e;
-        if ((e = cudaFuncSetAttribute(k_c_buckets, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BkSmem))))
+    const size_t bitmap = ((size_t)c.m / 32 + 2) * sizeof(uint32_t);
+    uint32_t mc = 0, nc = 0;  // crossing edges, coarse vertices
+    bool done = false;
+    // counts to the host: crossing edges, coarse vertices, edges left to the general path, a
+    // partition outgrew its room
+    auto read_counts = [&]() -> int {
+        cudaError_t x;
+        if ((x = cudaMemcpyAsync(mc_host_slot, c.counts, 5 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s))) return (int)x;
+        if ((x = cudaMemcpyAsync(mc_host_slot + 5, c.rank + c.n, sizeof(uint32_t), cudaMemcpyDeviceToHost, s)))
+            return (int)x;
+        if ((x = cudaStreamSynchronize(s))) return (int)x;
+        mc = mc_host_slot[0];
+        nc = mc_host_slot[5];
+        return 0;
+    };
+    // 1. partitions, where their rule holds: the crossing bits become the leader bits, every
+    //    group member but the first cleared
+    if (const uint32_t pb = contract_part_bits(c.m, c.sort_bits)) {
+        const uint32_t cap = (uint32_t)(2ull * c.m >> pb);  // twice the average: key[0] and key[1], which follows it
+        uint32_t gb = 10;
+        while (gb < GpSmem<1>::GP_BITS && (1ull << gb) < (8ull * c.m >> pb)) gb++;
+        uint2* items = reinterpret_cast<uint2*>(c.key[0]);
+        auto part = vec ? k_c_part<true> : k_c_part<false>;
+        const int big = gb > GpSmem<0>::GP_BITS;
+        auto groups = big ? k_c_groups<1> : k_c_groups<0>;
+        const size_t gsmem = big ? sizeof(GpSmem<1>) : sizeof(GpSmem<0>);
+        if ((e = cudaFuncSetAttribute(part, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PtSmem))) ||
+            (e = cudaFuncSetAttribute(groups, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsmem)) ||
+            (e = cudaMemsetAsync(c.counts, 0, 8 * sizeof(uint32_t), s)) ||
+            (e = cudaMemsetAsync(c.shist, 0, sizeof(uint32_t) << pb, s)) ||
+            (e = cudaMemsetAsync(c.multi, 0, bitmap, s)) || (e = cudaMemsetAsync(ofl, 0, bitmap, s)))
             return (int)e;
-        if ((e = cudaFuncSetAttribute(k_c_buckets, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                      (int)cudaSharedmemCarveoutMaxShared)))
-            return (int)e;
-        k_c_buckets<<<(mc + BK_C - 1) / BK_C, BK_T, sizeof(BkSmem), s>>>(hk[hc], c.val[hc], mc, mask, c.cpair, c.w,
-                                                                       c.cross, c.multi, c.gref, ofl, c.counts);
-        if ((e = cudaMemcpyAsync(mc_host_slot + 2, c.counts + 1, sizeof(uint32_t), cudaMemcpyDeviceToHost, s)))
+        part<<<(uint32_t)(((uint64_t)c.m + PT_TILE - 1) / PT_TILE), PT_T, sizeof(PtSmem), s>>>(
+            c.eu, c.ev, c.m, c.n, c.cmap, pb, cap, c.shist, items, c.cpair, c.cross, c.counts, c.err);
+        groups<<<1u << pb, 512u << big, gsmem, s>>>(items, c.shist, cap, pb, gb, c.val[0], ofl, c.counts);
+        k_c_walk<<<egrid, CT, 0, s>>>(c.val[0], c.cpair, c.w, c.cross, c.multi, c.gref, ofl, c.counts);
+        if (int r = read_counts()) return r;
+        done = mc_host_slot[4] == 0;
+    }
+    // or every edge keyed by its pair's hash in input order; the stable sort keeps input
+    // order among equal keys and puts the edges inside pairs last, after the mc crossing
+    // edges; then the buckets
+    if (!done) {
+        if ((e = cudaMemsetAsync(c.counts, 0, 8 * sizeof(uint32_t), s))) return (int)e;
+        static_assert(RS_TILE == 4096 && CT == 256, "k_c_keys takes one tile of the sort per block");
+        const uint32_t kgrid = (uint32_t)(((uint64_t)c.m + RS_TILE - 1) / RS_TILE);  // the sort's tiles
+        auto keys = vec ? k_c_keys<true> : k_c_keys<false>;
+        keys<<<kgrid, CT, 0, s>>>(c.eu, c.ev, c.m, c.n, c.cmap, hk[0], c.cpair, c.cross, c.counts, c.shist, c.err);
+        if (int r = read_counts()) return r;
+        mc_host_slot[1] = 0;
+        // the sort's bits: as few bytes as leave at most BK_AVG crossing edges to a bucket
+        uint32_t sbits = c.sort_bits;
+        if (!sbits)
+            for (sbits = 8; sbits < 32 && (uint64_t)mc > ((uint64_t)BK_AVG << sbits); sbits += 8) {
+            }
+        const uint32_t mask = sbits >= 32 ? ~0u : (1u << sbits) - 1u;
+        int hc = 0;
+        if ((e = cudaMemsetAsync(c.multi, 0, bitmap, s))) return (int)e;
+        if (mc > 1) {
+            if (int r = radix(hk[0], hk[1], c.val[0], c.val[1], c.m, sbits, true, true, &hc)) return r;
+            if ((e = cudaMemsetAsync(ofl, 0, bitmap, s)) ||
+                (e = cudaFuncSetAttribute(k_c_buckets, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BkSmem))) ||
+                (e = cudaFuncSetAttribute(k_c_buckets, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                          (int)cudaSharedmemCarveoutMaxShared)))
+                return (int)e;
+            k_c_buckets<<<(mc + BK_C - 1) / BK_C, BK_T, sizeof(BkSmem), s>>>(hk[hc], c.val[hc], mc, mask, c.val[hc ^ 1], ofl,
+                                                                           c.counts);
+            k_c_walk<<<egrid, CT, 0, s>>>(c.val[hc ^ 1], c.cpair, c.w, c.cross, c.multi, c.gref, ofl, c.counts);
+            if (int r = read_counts()) return r;
+        }
+    }
+    // 2. the flagged edges are taken out in order with their pair as the key, sorted by the
+    //    pair and marked
+    if (mc_host_slot[1]) {
+        const uint32_t bits = bits_for(nc ? nc - 1 : 0);
+        const uint32_t tiles = (c.m + RN_TILE - 1) / RN_TILE;
+        uint32_t* toffs = c.tsum + ((size_t)c.m / RN_TILE + 2);
+        k_c_runs_count<<<tiles, CT, 0, s>>>(ofl, c.m, c.tsum);
+        if (int r = launch_exclusive_scan(s, c.tsum, toffs, tiles, c.scan_tmp, c.scan_words)) return r;
+        k_c_runs_take<<<tiles, CT, 0, s>>>(ofl, c.m, toffs, c.cpair, bits, c.key[0], c.val[0], c.counts);
+        if ((e = cudaMemcpyAsync(mc_host_slot, c.counts + 3, sizeof(uint32_t), cudaMemcpyDeviceToHost, s)))
             return (int)e;
         if ((e = cudaStreamSynchronize(s))) return (int)e;
-        if (mc_host_slot[2]) {
-            const uint32_t tiles = (mc + RN_TILE - 1) / RN_TILE;
-            uint32_t* toffs = c.tsum + ((size_t)c.m / RN_TILE + 2);
-            k_c_runs_count<<<tiles, CT, 0, s>>>(ofl, mc, c.tsum);
-            if (int r = launch_exclusive_scan(s, c.tsum, toffs, tiles, c.scan_tmp, c.scan_words)) return r;
-            k_c_runs_take<<<tiles, CT, 0, s>>>(ofl, c.val[hc], mc, toffs, c.cpair, bits, c.key[hc ^ 1],
-                                               c.val[hc ^ 1], c.counts);
-            if ((e = cudaMemcpyAsync(mc_host_slot + 2, c.counts + 3, sizeof(uint32_t), cudaMemcpyDeviceToHost, s)))
-                return (int)e;
-            if ((e = cudaStreamSynchronize(s))) return (int)e;
-            nsub = mc_host_slot[2];
+        const uint32_t nsub = mc_host_slot[0];
+        int cur = 0;
+        if (nsub) {
+            if (int r = radix(c.key[0], c.key[1], c.val[0], c.val[1], nsub, 2 * bits, false, false, &cur)) return r;
+            k_c_marks<<<grid_for(nsub), CT, 0, s>>>(c.key[cur], c.val[cur], nsub, c.w, c.cross, c.multi, c.gref);
         }
     }
-    // the subset's two buffers: the ones the hash sort did not end in, and, once the
-    // subset is taken out, the ones it did
-    unsigned long long* sk[2] = {c.key[hc ^ 1], c.key[hc]};
-    uint32_t* sv[2] = {c.val[hc ^ 1], c.val[hc]};
-    int cur = 0;
-    if (nsub) {
-        if (int r = radix(sk[0], sk[1], sv[0], sv[1], nsub, 2 * bits, false, false, &cur)) return r;
-        k_c_marks<<<grid_for(nsub), CT, 0, s>>>(sk[cur], sv[cur], nsub, c.w, c.cross, c.multi, c.gref);
-    }
-    // 4. leaders ranked by words of the bitmask; the leaders write the coarse edges
+    // 3. leaders ranked by words of the bitmask; the leaders write the coarse edges
     k_c_wcount<<<grid_for((uint64_t)words + 1), CT, 0, s>>>(c.cross, words, c.wlead);
     if (int r = launch_exclusive_scan(s, c.wlead, c.wpos, words + 1, c.scan_tmp, c.scan_words)) return r;
     if ((e = cudaMemcpyAsync(c.counts + 2, c.wpos + words, sizeof(uint32_t), cudaMemcpyDeviceToDevice, s)))

@@ -340,14 +340,15 @@ struct ContractArgs {
     uint32_t* flag;           // [n + 1] representative flags
     uint32_t* rank;           // [n + 1] their exclusive prefix (rank[n] = coarse vertices)
     uint32_t* cross;          // [m / 32 + 2] bit e: edge e joins two coarse vertices, then: it leads its group
-    uint32_t* counts;         // [8] crossing edges, items of runs left to the pair sort, coarse edges,
-                              // items taken out for it
+    uint32_t* counts;         // [8] crossing edges, edges of runs left to the pair sort, coarse edges,
+                              // edges taken out for it, a partition outgrew its room
     uint32_t* cpair;          // [2 m] coarse endpoints of every edge, cmap[eu[e]] then cmap[ev[e]]
-    unsigned long long* key[2];  // [m] coarse pair of each crossing edge (radix ping-pong)
+    unsigned long long* key[2];  // [m] coarse pair of each crossing edge (radix ping-pong); key[1] follows
+                                 // key[0], together the partitions' room: 2 m (hash, edge) items
     uint32_t* val[2];         // [m] its edge index
     uint32_t* shist;          // radix pass: [256 * tiles] per-tile digit counts, then their exclusive prefix
     uint32_t* multi;          // [m / 32 + 2] bit e: edge e leads a group of several edges
-    uint32_t* wlead;          // [m / 32 + 2] flags of the sorted items left to the pair sort, then
+    uint32_t* wlead;          // [m / 32 + 2] flags of the edges left to the pair sort, then
                               // leaders per word of cross
     uint32_t* wpos;           // [m / 32 + 2] their exclusive prefix (wpos[words] = coarse edges)
     uint32_t* tsum;           // [2 * (m / 4096 + 2)] per-tile counts of run items and their prefix
@@ -358,7 +359,7 @@ struct ContractArgs {
     uint32_t sort_bits;       // low bits of the hash the sort orders by (8, 16, 24, 32; 0: by size)
 };
 size_t contract_sort_words(uint32_t m);  // words of shist
-// runs every step; mc_host_slot: 2 pinned words (crossing edges and coarse vertices
+// runs every step; mc_host_slot: 3 pinned words (crossing edges and coarse vertices
 // are read back once, to size the sort); returns a cudaError_t value
 int launch_contract(void* stream, const ContractArgs& c, uint32_t* mc_host_slot);
 int launch_job_graph(void* exec, void* stream);

@@ -1,0 +1,56 @@
+"""Contraction by partitions of the hash: sizes at the edges of its tiles and of the rule
+that counts its partitions, groups beyond what one partition takes at once (passes by
+residue), a residue beyond that (the pair sort), and a pair that outgrows a partition's
+room (the hash sort instead), each identical to the oracle's contraction."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import oracle
+from gpu_util import NIL, Lm
+from test_gpu_contract import _contract, _same
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lmc():
+    c = Lm()
+    yield c
+    c.close()
+
+
+def _edges(rng, n, m):
+    eu = rng.integers(0, n, m, dtype=np.uint32)
+    ev = ((eu + rng.integers(1, n, m, dtype=np.uint32)) % n).astype(np.uint32)
+    return eu, ev, rng.standard_normal(m).astype(np.float32)
+
+
+@pytest.mark.parametrize("m", [1, 2, 3, 31, 33, 8191, 8192, 8193, 16383, 16384, 16385, 32769, 40001, 262147])
+def test_sizes(lmc, m):
+    # about one edge in four in a group of several, orientations mixed, some pairs matched
+    rng = np.random.default_rng(m)
+    n = max(3, int(1.2 * m ** 0.5))
+    eu, ev, w = _edges(rng, n, m)
+    mate = oracle.greedy(n, eu, ev, w, 7) if m & 1 else np.full(n, NIL, np.uint32)
+    _same(_contract(lmc, n, eu, ev, w, mate), oracle.contract(n, eu, ev, w, mate))
+
+
+@pytest.mark.parametrize("kind", ["every_pair_twice", "one_pair_7000", "one_pair_40000", "pairs_of_500"])
+def test_groups_beyond_a_partition(lmc, kind):
+    # 64 partitions of about 8000 items, 16000 at most, 6144 of them at once
+    rng = np.random.default_rng(5)
+    n, m = 100_000, 512_000
+    eu, ev, w = _edges(rng, n, m)
+    if kind == "every_pair_twice":
+        eu[m // 2:], ev[m // 2:] = ev[: m // 2], eu[: m // 2]
+    elif kind == "pairs_of_500":
+        eu[:], ev[:] = eu[np.arange(m) % (m // 500)], ev[np.arange(m) % (m // 500)]
+    else:
+        k = rng.permutation(m)[: int(kind.rsplit("_", 1)[1])]
+        eu[k], ev[k] = 17, 4711
+    p = rng.permutation(m)
+    eu, ev = eu[p], ev[p]
+    mate = np.full(n, NIL, np.uint32)
+    _same(_contract(lmc, n, eu, ev, w, mate), oracle.contract(n, eu, ev, w, mate))
