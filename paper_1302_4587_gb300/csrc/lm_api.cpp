@@ -656,6 +656,7 @@ static ListSeg list_seg(const lm_graph* g, uint64_t seed, uint32_t* dst) {
     d.nblk = list_blocks(g->ntask, g->nrows);
     d.k0 = (uint32_t)z;
     d.k1 = (uint32_t)(z >> 32);
+    d.seed = seed;
     return d;
 }
 
@@ -750,6 +751,34 @@ static int match_list(lm_ctx* ctx, Engine& e, const lm_graph* g, uint64_t seed, 
     return LM_OK;
 }
 
+// One graph under a renewed order (see lm_renew.cu), in the list path's workspace.
+static int match_renewed(lm_ctx* ctx, Engine& e, const lm_graph* g, uint64_t seed, uint32_t* mate, bool dev_out,
+                         Prof& prof, bool async, bool counts) {
+    cudaStream_t s = e.stream;
+    int rc = ensure_list(ctx, e, g->n, g->ntask[0], 1, 0, RENEW_CTRS, false);
+    if (rc) return rc;
+    uint32_t* mate_d = dev_out ? mate : e.lw.mate;
+    RenewArgs A;
+    memset(&A, 0, sizeof A);
+    A.g = list_seg(g, seed, mate_d);
+    A.cur = reinterpret_cast<uint32_t*>(e.lw.cur);
+    A.dead = reinterpret_cast<uint32_t*>(e.lw.lst);
+    for (int k = 0; k < 2; k++) A.list[k] = e.lw.list[k];
+    A.part = e.lw.part;
+    A.pcnt = e.lw.pcnt;
+    A.ctr = e.lw.pcount;
+    A.st = e.st;
+    job_limits(ctx, g->m, &A.max_rounds, &A.limit_ns);
+    prof.begin(LM_K_SWEEP);
+    LM_CK(ctx, launch_renew(s, A, counts));
+    prof.end();
+    if (async) return LM_OK;  // queued; lm_sync reports device errors
+    LM_CK(ctx, cudaMemcpyAsync(e.st_host, e.st, sizeof(DevState), cudaMemcpyDeviceToHost, s));
+    if (!dev_out) LM_CK(ctx, cudaMemcpyAsync(mate, mate_d, (size_t)g->n * 4, cudaMemcpyDeviceToHost, s));
+    LM_CK(ctx, cudaStreamSynchronize(s));
+    return check_err(ctx, e);
+}
+
 // One graph on engine e, results to mate (device memory when dev_out, else host
 // memory staged through the workspace); the engine's DevState holds its statistics.
 int match_one(lm_ctx* ctx, Engine& e, const lm_graph* g, uint64_t seed, uint32_t* mate, bool dev_out, Prof& prof,
@@ -759,6 +788,8 @@ int match_one(lm_ctx* ctx, Engine& e, const lm_graph* g, uint64_t seed, uint32_t
     if (rc) return rc;
     if (g->nent && list_path(e, g))
         return match_list(ctx, e, g, seed, mate, dev_out, prof, async && dev_out && !prof.on, rounds, counts);
+    if (g->nent && g->n < 0x80000000u)
+        return match_renewed(ctx, e, g, seed, mate, dev_out, prof, async && dev_out && !prof.on, counts);
     rc = ensure_ws(ctx, e, g->n, g->nent, 1);
     if (rc) return rc;
     rc = ensure_pinned(ctx, e, sizeof(SegIn));

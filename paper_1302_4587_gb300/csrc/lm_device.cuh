@@ -47,6 +47,13 @@ __device__ __forceinline__ uint32_t fmix32_inv(uint32_t h) {
 __device__ __forceinline__ uint32_t perm_seed_inv(uint32_t x, uint32_t k0, uint32_t k1) {
     return fmix32_inv(fmix32_inv(x) ^ k1) ^ k0;
 }
+// SplitMix64 (Steele, Lea, Flood 2014): the r-th output (r >= 0) for state `seed`
+__device__ __forceinline__ uint64_t splitmix64_at(uint64_t seed, uint32_t r) {
+    uint64_t z = seed + (uint64_t)(r + 1u) * 0x9E3779B97F4A7C15ull;
+    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+    return z ^ (z >> 31);
+}
 // monotone float32 -> uint32 (-0 == +0); NaN is rejected before this runs
 __device__ __forceinline__ uint32_t ord_of_bits(uint32_t b) {
     if (b == 0x80000000u) b = 0u;

@@ -279,6 +279,7 @@ struct ListSeg {
     uint32_t blk0, nblk;      // its blocks of k_top
     uint32_t part0, nparts;   // its parts
     uint32_t k0, k1;          // perm_seed keys of its seed
+    uint64_t seed;
 };
 // Arguments of a list-path job in device memory.
 struct ListArgs {
@@ -296,6 +297,20 @@ struct ListArgs {
     uint32_t* pcnt;           // chunks done per long row, at its first chunk's slot (zero between jobs)
     uint32_t* grounds;        // [nsegs] rounds per graph (NULL: one graph, DevState::rounds)
     unsigned long long* gmatched;  // [nsegs] matched vertices per graph (NULL: DevState::matched2)
+    uint32_t max_rounds;
+    unsigned long long limit_ns;
+    DevState* st;
+};
+// Arguments of a job under a renewed order (lm_renew.cu)
+constexpr uint32_t RENEW_CTRS = 16;
+struct RenewArgs {
+    ListSeg g;
+    uint32_t* cur;            // [n] candidates
+    uint32_t* dead;           // [n / 32 + 1] bitmap of matched vertices
+    uint32_t* list[2];        // [n] live rows
+    uint4* part;              // [LIST_KEPT per chunk] its heaviest, then (second word 0, 1) the chunks' lists
+    uint32_t* pcnt;           // chunks done per long row (zero between jobs)
+    uint32_t* ctr;            // [RENEW_CTRS]
     uint32_t max_rounds;
     unsigned long long limit_ns;
     DevState* st;
@@ -370,6 +385,8 @@ uint32_t list_blocks(const uint32_t task[4], uint32_t nrows);
 int launch_list_map(void* stream, const ListArgs* d, uint32_t nsegs, uint32_t* bmap, uint32_t* pmap);
 int launch_top(void* stream, const ListArgs* d, uint32_t blocks, bool rounds);
 int launch_live(void* stream, const ListArgs* d, uint32_t nparts, bool rounds);
+// renewed order (lm_renew.cu): a graph's whole job; counts: the live edges of every round too
+int launch_renew(void* stream, const RenewArgs& a, bool counts);
 int launch_round_counts(void* stream, const ListArgs* d, void* bytes);  // bytes: one a vertex, scratch
 int build_list_graph(const ListArgs* d, bool rounds, void** exec_out);
 // edge-centric path: the job graph (init, then a conditional loop of rounds) and the

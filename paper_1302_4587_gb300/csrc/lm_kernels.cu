@@ -360,13 +360,6 @@ struct WarpRows {              // one warp's batch of rows
     uint32_t rk0[RENEW ? 32 : 1], rk1[RENEW ? 32 : 1];  // renewed order: the row's keys this round
 };
 
-// SplitMix64 (Steele, Lea, Flood 2014): the r-th output (r >= 0) for state `seed`
-__device__ __forceinline__ uint64_t splitmix64_at(uint64_t seed, uint32_t r) {
-    uint64_t z = seed + (uint64_t)(r + 1u) * 0x9E3779B97F4A7C15ull;
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
-}
 // keys ordering the entries of graph g in the round being prepared (nr): the graph's
 // own keys, or with a renewed order those of the nr-th SplitMix64 output
 template <bool RENEW>
