@@ -676,19 +676,15 @@ static void list_args(ListArgs& A, Engine& e) {
     A.st = e.st;
 }
 
-// the list path's arguments of a job sit in the last quarter of the argument area
+// an asynchronous list job's arguments sit in the last quarter of the argument area
 constexpr size_t LIST_ARGS_OFF = ARG_AREA / 4 * 3;
-struct ListJobArgs {
-    ListArgs a;
-    ListSeg seg;
-};
 
 // The live pass of a queued job, until no row is left: k_live as often as it gives rows
 // back (once, as a rule), the state copied to the host after each.
-static int run_live(lm_ctx* ctx, Engine& e, const ListArgs* D, uint32_t nparts, bool rounds, Prof& prof) {
+static int run_live(lm_ctx* ctx, Engine& e, const ListArgs& A, uint32_t nparts, bool rounds, Prof& prof) {
     for (;;) {
         prof.begin(LM_K_SWEEP);
-        LM_CK(ctx, launch_live(e.stream, D, nparts, rounds));
+        LM_CK(ctx, launch_live(e.stream, A, nparts, rounds));
         prof.end();
         LM_CK(ctx, cudaMemcpyAsync(e.st_host, e.st, sizeof(DevState), cudaMemcpyDeviceToHost, e.stream));
         LM_CK(ctx, cudaStreamSynchronize(e.stream));
@@ -706,38 +702,36 @@ static int match_list(lm_ctx* ctx, Engine& e, const lm_graph* g, uint64_t seed, 
     int rc = ensure_list(ctx, e, g->n, g->ntask[0], 1, 0, nparts, rounds);
     if (rc) return rc;
     uint32_t* mate_d = dev_out ? mate : e.lw.mate;
-    static_assert(EDGE_ARGS_OFF + sizeof(EdgeJobArgs) <= LIST_ARGS_OFF &&
-                  LIST_ARGS_OFF + sizeof(ListJobArgs) <= ARG_AREA, "argument area too small");
-    ListJobArgs& J = *reinterpret_cast<ListJobArgs*>(e.hargs + LIST_ARGS_OFF);
-    ListJobArgs* D = reinterpret_cast<ListJobArgs*>(e.dargs + LIST_ARGS_OFF);
-    list_args(J.a, e);
-    J.a.segs = &D->seg;
-    J.a.nsegs = 1;
-    J.a.nparts = nparts;
-    job_limits(ctx, g->m, &J.a.max_rounds, &J.a.limit_ns);
-    J.seg = list_seg(g, seed, mate_d);
-    J.seg.nparts = nparts;
-    LM_CK(ctx, cudaMemcpyAsync(D, &J, sizeof J, cudaMemcpyHostToDevice, s));
-    if (async) {
+    ListArgs A;
+    list_args(A, e);
+    A.nsegs = 1;
+    A.nparts = nparts;
+    job_limits(ctx, g->m, &A.max_rounds, &A.limit_ns);
+    A.one = list_seg(g, seed, mate_d);
+    A.one.nparts = nparts;
+    prof.begin(LM_K_CAND);
+    LM_CK(ctx, launch_top(s, A, A.one.nblk, rounds));
+    prof.end();
+    if (async) {  // queued, the arguments in device memory for the graph; lm_sync reports device errors
+        static_assert(EDGE_ARGS_OFF + sizeof(EdgeJobArgs) <= LIST_ARGS_OFF &&
+                      LIST_ARGS_OFF + sizeof(ListArgs) <= ARG_AREA, "argument area too small");
+        ListArgs* D = reinterpret_cast<ListArgs*>(e.dargs + LIST_ARGS_OFF);
+        memcpy(e.hargs + LIST_ARGS_OFF, &A, sizeof A);
+        LM_CK(ctx, cudaMemcpyAsync(D, e.hargs + LIST_ARGS_OFF, sizeof A, cudaMemcpyHostToDevice, s));
         // the next job may rewrite the staging only after this upload ran
         if (!e.staged) LM_CK(ctx, cudaEventCreateWithFlags(&e.staged, cudaEventDisableTiming));
         LM_CK(ctx, cudaEventRecord(e.staged, s));
         e.staged_pending = true;
-    }
-    prof.begin(LM_K_CAND);
-    LM_CK(ctx, launch_top(s, &D->a, J.seg.nblk, rounds));
-    prof.end();
-    if (async) {  // queued; lm_sync reports device errors
         void*& graph = e.lgraph[rounds ? 1 : 0];
-        if (!graph) LM_CK(ctx, build_list_graph(&D->a, rounds, &graph));
+        if (!graph) LM_CK(ctx, build_list_graph(D, rounds, &graph));
         LM_CK(ctx, launch_job_graph(graph, s));
         return LM_OK;
     }
-    rc = run_live(ctx, e, &D->a, nparts, rounds, prof);
+    rc = run_live(ctx, e, A, nparts, rounds, prof);
     if (rc) return rc;
     if (counts) {
         prof.begin(LM_K_OTHER);
-        LM_CK(ctx, launch_round_counts(s, &D->a, e.lw.queue));
+        LM_CK(ctx, launch_round_counts(s, A, e.lw.queue));
         prof.end();
         LM_CK(ctx, cudaMemcpyAsync(e.st_host, e.st, sizeof(DevState), cudaMemcpyDeviceToHost, s));
     }
@@ -862,8 +856,7 @@ static int batch_list(lm_ctx* ctx, Engine& e, const lm_graph* const* gs, uint32_
         bb += sg.nblk;
         pb += sg.nparts;
     }
-    ListArgs& A = reinterpret_cast<ListJobArgs*>(e.hargs + LIST_ARGS_OFF)->a;
-    ListArgs* D = &reinterpret_cast<ListJobArgs*>(e.dargs + LIST_ARGS_OFF)->a;
+    ListArgs A;
     list_args(A, e);
     A.segs = w.segs;
     A.nsegs = count;
@@ -874,17 +867,16 @@ static int batch_list(lm_ctx* ctx, Engine& e, const lm_graph* const* gs, uint32_
     A.gmatched = w.gmatched;
     job_limits(ctx, (uint32_t)(ne / 2), &A.max_rounds, &A.limit_ns);
     LM_CK(ctx, cudaMemcpyAsync(w.segs, segs, count * sizeof(ListSeg), cudaMemcpyHostToDevice, s));
-    LM_CK(ctx, cudaMemcpyAsync(D, &A, sizeof A, cudaMemcpyHostToDevice, s));
     LM_CK(ctx, cudaMemsetAsync(w.gmatched, 0, count * sizeof(unsigned long long), s));
     LM_CK(ctx, cudaMemsetAsync(w.grounds, 0, count * sizeof(uint32_t), s));
     prof.begin(LM_K_OTHER);
-    LM_CK(ctx, launch_list_map(s, D, count, w.bmap, w.pmap));
+    LM_CK(ctx, launch_list_map(s, A, count, w.bmap, w.pmap));
     prof.end();
     prof.begin(LM_K_CAND);
-    LM_CK(ctx, launch_top(s, D, bb, want));
+    LM_CK(ctx, launch_top(s, A, bb, want));
     prof.end();
     if (pb) {
-        rc = run_live(ctx, e, D, pb, want, prof);
+        rc = run_live(ctx, e, A, pb, want, prof);
         if (rc) return rc;
     }
     std::vector<uint32_t> hmate;

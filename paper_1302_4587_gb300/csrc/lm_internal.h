@@ -253,13 +253,7 @@ struct EdgeArgs {
 // more than LIST_CHUNK entries are cut into chunks of that many, a warp each
 constexpr uint32_t LIST_SHORT = 32, LIST_GROUP = 64, LIST_WARP = 256, LIST_CHUNK = 2048;
 constexpr uint32_t LIST_KEPT = 8;       // neighbours kept of a long row
-#ifndef LM_PART_MIN
-#define LM_PART_MIN 256
-#endif
-#ifndef LM_PART_MAX
-#define LM_PART_MAX 2048
-#endif
-constexpr uint32_t LIST_PART_MIN = LM_PART_MIN, LIST_PART_MAX = LM_PART_MAX;  // rows a block of the live pass takes at a time
+constexpr uint32_t LIST_PART_MIN = 256, LIST_PART_MAX = 2048;  // rows a block of the live pass takes at a time
 
 // One graph of a list-path job (local vertex ids throughout).
 struct ListSeg {
@@ -281,9 +275,10 @@ struct ListSeg {
     uint32_t k0, k1;          // perm_seed keys of its seed
     uint64_t seed;
 };
-// Arguments of a list-path job in device memory.
+// Arguments of a list-path job.
 struct ListArgs {
-    const ListSeg* segs;
+    ListSeg one;              // the graph of a job of one
+    const ListSeg* segs;      // several: theirs
     uint32_t nsegs, nparts;   // graphs, parts of all graphs
     const uint32_t* bmap;     // [blocks of k_top] graph of each block (NULL: one graph)
     const uint32_t* pmap;     // [nparts] graph of each part (NULL: one graph)
@@ -382,12 +377,12 @@ int launch_job_graph(void* exec, void* stream);
 // (rounds: 64-bit words)
 uint32_t list_live_blocks(int device);  // blocks of k_live that run at once
 uint32_t list_blocks(const uint32_t task[4], uint32_t nrows);
-int launch_list_map(void* stream, const ListArgs* d, uint32_t nsegs, uint32_t* bmap, uint32_t* pmap);
-int launch_top(void* stream, const ListArgs* d, uint32_t blocks, bool rounds);
-int launch_live(void* stream, const ListArgs* d, uint32_t nparts, bool rounds);
+int launch_list_map(void* stream, const ListArgs& a, uint32_t nsegs, uint32_t* bmap, uint32_t* pmap);
+int launch_top(void* stream, const ListArgs& a, uint32_t blocks, bool rounds);
+int launch_live(void* stream, const ListArgs& a, uint32_t nparts, bool rounds);
 // renewed order (lm_renew.cu): a graph's whole job; counts: the live edges of every round too
 int launch_renew(void* stream, const RenewArgs& a, bool counts);
-int launch_round_counts(void* stream, const ListArgs* d, void* bytes);  // bytes: one a vertex, scratch
+int launch_round_counts(void* stream, const ListArgs& a, void* bytes);  // bytes: one a vertex, scratch
 int build_list_graph(const ListArgs* d, bool rounds, void** exec_out);
 // edge-centric path: the job graph (init, then a conditional loop of rounds) and the
 // per-round launches of the profiled path

@@ -74,7 +74,10 @@ struct RowLists {
 __device__ __forceinline__ RowLists row_lists(const ListArgs& a, uint32_t vbase) {
     return {a.lst + vbase, a.wide + vbase, a.rl ? a.rl + vbase : nullptr, a.rw ? a.rw + vbase : nullptr};
 }
-constexpr uint32_t MORE = 1u, WIDE = 2u, HASR = 4u;
+// Above the flags: the largest ord(w) that an entry beyond the list can have (its low
+// bits lost): a scan of a long row need not look at the ends of heavier ones, which are
+// all matched (rows of at most 128 entries look at all ends at once).
+constexpr uint32_t MORE = 1u, WIDE = 2u, HASR = 4u, FLAGS = 7u;
 constexpr int KS = 4, KL = LIST_KEPT;   // list lengths: rows of at most LIST_SHORT entries, longer ones
 
 // entry i of a graph: ord(w), its neighbour, its full key
@@ -262,6 +265,16 @@ __device__ __forceinline__ void put_list(W* cur, const RowLists& R, size_t at, u
     }
 }
 
+// A job's arguments and a graph's record are read from shared memory: from global
+// memory through two pointers they were loaded again after every barrier and atomic, or
+// held in registers that the rows need.
+template <class T>
+__device__ __forceinline__ void copy_words(T* to, const T* from, uint32_t threads) {
+    static_assert(sizeof(T) % 4 == 0, "words");
+    for (uint32_t i = threadIdx.x; i < sizeof(T) / 4; i += threads)
+        reinterpret_cast<uint32_t*>(to)[i] = reinterpret_cast<const uint32_t*>(from)[i];
+}
+
 // ---------------------------------------------------------------- k_top
 constexpr int TT = 256, TWARPS = TT / 32;
 constexpr uint32_t MPW = 2;       // long-row tasks a warp takes,
@@ -324,7 +337,7 @@ __device__ __forceinline__ void top_short(const ListArgs& a, const ListSeg& g, u
     const size_t at = (size_t)g.vbase + v;
     words<W>(a)[at] = word<W>(nbr_at(g, o + p[0]), 0);
     a.lst[at] = make_uint4(d > 1 ? nbr_at(g, o + p[1]) : NIL, d > 2 ? nbr_at(g, o + p[2]) : NIL,
-                           d > 3 ? nbr_at(g, o + p[3]) : NIL, d > 4 ? MORE : 0u);
+                           d > 3 ? nbr_at(g, o + p[3]) : NIL, d > 4 ? MORE | (t.k[3] & ~FLAGS) | (MASK & ~FLAGS) : 0u);
 }
 
 // Rows of more than LIST_SHORT entries, eight entries to each of the G lanes of a group
@@ -370,7 +383,8 @@ __device__ __forceinline__ void top_group(const ListArgs& a, const ListSeg& g, u
         uint32_t c = 0;
         if (cd && sub < KL) c = nbr_at(g, cs + p);
         if (i + ROWS < cnt) fetch(i + ROWS);
-        if (cd) put_list<W, KL>(words<W>(a) + g.vbase, row_lists(a, g.vbase), cv, sub, c, 0, WIDE | MORE);
+        if (cd) put_list<W, KL>(words<W>(a) + g.vbase, row_lists(a, g.vbase), cv, sub, c, 0,
+                                WIDE | MORE | ((r[KL - 1] | MASK) & ~FLAGS));
     }
 }
 
@@ -481,11 +495,13 @@ __device__ __forceinline__ void top_long(const ListArgs& a, const ListSeg& g, ui
             kt.offer(i < e && i >= b ? key_of(g, ord_at(g, i), i) : 0ull, i);
         }
         p = kt.n;
+        top.o = (uint32_t)(kt.k >> 32);
     }
     if (lane >= KL) p = NIL;
     if (whole) {
+        const uint32_t last = top.last();
         put_list<W, KL>(words<W>(a) + g.vbase, row_lists(a, g.vbase), v, lane, p != NIL ? nbr_at(g, p) : NIL, 0,
-                        WIDE | MORE);
+                        WIDE | MORE | (last & ~FLAGS));
         return;
     }
     // a chunk: its list with the full keys; the last chunk of the row to finish merges all
@@ -513,7 +529,8 @@ __device__ __forceinline__ void top_long(const ListArgs& a, const ListSeg& g, ui
         kt.offer(((uint64_t)rec.y << 32) | rec.x, rec.z);
     }
     if (lane == 0) a.pcnt[(size_t)g.lbase + first] = 0;
-    put_list<W, KL>(words<W>(a) + g.vbase, row_lists(a, g.vbase), v, lane, kt.n, 0, WIDE | MORE);
+    put_list<W, KL>(words<W>(a) + g.vbase, row_lists(a, g.vbase), v, lane, kt.n, 0,
+                    WIDE | MORE | ((uint32_t)(kt.last() >> 32) & ~FLAGS));
 }
 
 // Blocks of k_top for one graph, in this order: long tasks, rows of a warp, rows of a
@@ -530,13 +547,11 @@ __host__ __device__ __forceinline__ TopBlocks top_blocks(const uint32_t task[4],
     return b;
 }
 
-#ifndef LM_TMINB
-#define LM_TMINB 6
-#endif
+constexpr int TMINB = 6;
 // Every block also clears its share of the result, and block 0 resets the job's state.
 template <class W>
-__global__ void __launch_bounds__(TT, LM_TMINB) k_top(const ListArgs* __restrict__ pa) {
-    const ListArgs& a = *pa;
+__global__ void __launch_bounds__(TT, TMINB) k_top(const __grid_constant__ ListArgs a) {
+    __shared__ ListSeg g;
     const uint32_t tid = threadIdx.x, warp = tid >> 5;
     if (blockIdx.x == 0) {
         DevState* st = a.st;
@@ -551,8 +566,8 @@ __global__ void __launch_bounds__(TT, LM_TMINB) k_top(const ListArgs* __restrict
             st->t0_ns = globaltimer_ns();
         }
     }
-    const uint32_t sg = a.bmap ? a.bmap[blockIdx.x] : 0u;
-    const ListSeg& g = a.segs[sg];
+    copy_words(&g, a.bmap ? a.segs + a.bmap[blockIdx.x] : &a.one, TT);
+    __syncthreads();
     uint32_t b = blockIdx.x - g.blk0;
     {
         const uint32_t per = (uint32_t)(((uint64_t)g.n + g.nblk - 1) / g.nblk);
@@ -601,6 +616,7 @@ __device__ __forceinline__ bool refill_group(const ListSeg& g, W* cur, const Row
     for (int e = 0; e < E; e++)
         if (!(lo(t[e]) & DEAD)) live |= 1u << e;
     uint32_t p[K];
+    uint32_t last = 0;   // ord(w) of the list's last place
     bool rest = false, exact = ROUNDS;
     uint32_t mr = 0;   // with rounds: the place's r
     if (!ROUNDS) {
@@ -611,6 +627,7 @@ __device__ __forceinline__ bool refill_group(const ListSeg& g, W* cur, const Row
 #pragma unroll
         for (int i = 0; i < K; i++) p[i] = r[i] > MASK ? MASK - (r[i] & MASK) : NIL;
         rest = out > MASK;
+        last = r[K - 1] | MASK;
         exact = __any_sync(FULL, any_tie<K>(r, out, MASK));
     }
     if (exact) {
@@ -637,17 +654,18 @@ __device__ __forceinline__ bool refill_group(const ListSeg& g, W* cur, const Row
         uint32_t c = NIL;
         if (sub < K && mp != NIL) c = nbr_at(g, s + mp);
         if (ROUNDS && sub == 0) mr = max(mr, info(look(cur + v)));
-        put_list<W, K>(cur, R, v, sub, c, mr, (K == KL ? WIDE : 0u) | (rest ? MORE : 0u) | (ROUNDS ? HASR : 0u));
+        put_list<W, K>(cur, R, v, sub, c, mr, 
+                       (K == KL ? WIDE : 0u) | (rest ? MORE : 0u) | (ROUNDS ? HASR : 0u) | (last & ~FLAGS));
         return true;
     }
     return false;
 }
 
 // The same for longer rows: part `q` of `parts` of the row's 128-entry steps by this
-// warp.  Only entries at or above the last of the list so far have their end looked up.
+// warp.  Only entries between the last of the list so far and ub have their end looked up.
 template <class W>
-__device__ __forceinline__ void refill_scan(const ListSeg& g, const W* cur, uint32_t s, uint32_t d, uint32_t q,
-                                            uint32_t parts, LaneTop64& t) {
+__device__ __forceinline__ void refill_scan(const ListSeg& g, const W* cur, uint32_t s, uint32_t d, uint32_t ub,
+                                            uint32_t q, uint32_t parts, LaneTop64& t) {
     const uint32_t lane = threadIdx.x & 31;
     const uint64_t stride = 128ull * parts;
     uint64_t x[4], nx[4];
@@ -659,16 +677,21 @@ __device__ __forceinline__ void refill_scan(const ListSeg& g, const W* cur, uint
     uint32_t bar = 1;
     for (uint64_t b = 128ull * q; b < d; b += stride) {
         load(nx, b + stride);
-        const uint64_t m01 = x[0] > x[1] ? x[0] : x[1], m23 = x[2] > x[3] ? x[2] : x[3];
-        if (__any_sync(FULL, (uint32_t)((m01 > m23 ? m01 : m23) >> 32) >= bar)) {
-            W y[4];
+        bool in[4];
 #pragma unroll
-            for (int i = 0; i < 4; i++) y[i] = (uint32_t)(x[i] >> 32) >= bar ? look(cur + (uint32_t)x[i]) : (W)DEAD;
+        for (int i = 0; i < 4; i++) in[i] = (uint32_t)(x[i] >> 32) >= bar && (uint32_t)(x[i] >> 32) <= ub;
+        if (__any_sync(FULL, in[0] | in[1] | in[2] | in[3])) {
+            uint32_t y[4], e[4];   // (the indices together with the words, not one by one)
 #pragma unroll
             for (int i = 0; i < 4; i++) {
-                const bool on = !(lo(y[i]) & DEAD) && (uint32_t)(x[i] >> 32) >= bar;
+                y[i] = in[i] ? lo(look(cur + (uint32_t)x[i])) : DEAD;
+                e[i] = in[i] ? __ldg(g.eid + s + (uint32_t)b + 32 * i + lane) : 0u;
+            }
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                const bool on = !(y[i] & DEAD) && (uint32_t)(x[i] >> 32) >= bar;
                 if (!__any_sync(FULL, on)) continue;
-                t.offer(on ? key_of(g, (uint32_t)(x[i] >> 32), s + (uint32_t)b + 32 * i + lane) : 0ull, (uint32_t)x[i]);
+                t.offer(on ? (x[i] & 0xFFFFFFFF00000000ull) | perm_seed(e[i], g.k0, g.k1) : 0ull, (uint32_t)x[i]);
                 bar = max((uint32_t)(t.last() >> 32), 1u);
             }
         }
@@ -711,22 +734,17 @@ template <class W>
 __device__ __forceinline__ void refill_put(W* cur, const RowLists& R, uint32_t v, const LaneTop64& t, uint32_t r) {
     const uint32_t lane = threadIdx.x & 31;
     // (with a full list there may be more)
-    const uint32_t flags = WIDE | (__shfl_sync(FULL, t.n, KL - 1) != NIL ? MORE : 0u) | (sizeof(W) == 8 ? HASR : 0u);
+    const uint32_t flags = WIDE | (__shfl_sync(FULL, t.n, KL - 1) != NIL ? MORE : 0u) | (sizeof(W) == 8 ? HASR : 0u) |
+                           ((uint32_t)(t.last() >> 32) & ~FLAGS);
     if (sizeof(W) == 8 && lane == 0) r = max(r, info(look(cur + v)));
     put_list<W, KL>(cur, R, v, lane, t.k ? t.n : NIL, r, flags);
 }
 
 // ---------------------------------------------------------------- k_live
-#ifndef LM_LT
-#define LM_LT 128
-#endif
-#ifndef LM_LV
-#define LM_LV 1
-#endif
-#ifndef LM_LMINB
-#define LM_LMINB 8
-#endif
-constexpr int LT = LM_LT, LV = LM_LV, LW = LT / 32;
+constexpr int LT = 128, LW = LT / 32;
+// blocks an SM: rounds' words apart, 8 need no spills but 10 cover more latency (R-MAT scale 23
+// 1.32 and 1.28 ms, 4096 graphs 3.88 and 3.80; 12: 1.30, 3.72, but coarsening 9.9 ms for 9.5)
+constexpr int LMINB = 10;
 constexpr uint32_t BLOCK_ROW = 1024;  // longer rows are refilled by the whole block
 constexpr uint32_t IDLE_MAX = 48;     // passes without a change before a block gives its rows back
 
@@ -743,26 +761,39 @@ __device__ __forceinline__ void warp_append(uint32_t* ctr, uint32_t* out, bool o
     if (on) out[q] = v;
 }
 
-// A part: consecutive rows of one graph, its live rows compacted in its own range of
-// the list buffers, its rows to refill in its range of the queue (vertex, row
-// offset, length; rows of at most LIST_SHORT entries from the front, longer ones from
-// the back).
+constexpr uint32_t RUN = 32;
+
+// A part: every nparts-th run of RUN consecutive rows of one graph (the long rows of a graph
+// that numbers its vertices by degree, R-MAT's, a coarsened one's, would otherwise be in a
+// few parts, which the others wait for: fifth level of R-MAT
+// scale 20, 47 rounds: 2.26 ms by consecutive rows, 0.96 by runs of 8 to 64; runs of 8 cost
+// graphs with local edges coalescing, a unit grid of 1M 115 and 138 us), its
+// live rows compacted in its own range of the list buffers, its rows to refill in its
+// range of the queue (vertex, row offset, length, heaviest entry to look at; rows of at
+// most LIST_SHORT entries from the front, longer ones from the back).
 template <class W>
 struct Part {
-    const ListSeg& g;
+    ListSeg g;
     W* cur;
     RowLists R;
     uint4* queue;
-    uint32_t from, rows;  // its rows of the graph
-    size_t home;          // first slot of the part
-    __device__ __forceinline__ Part(const ListArgs& a, const ListSeg& seg, uint32_t part) : g(seg) {
-        const uint32_t per = (g.nrows + g.nparts - 1) / g.nparts;
-        from = min(g.nrows, (part - g.part0) * per);
-        rows = min(g.nrows, from + per) - from;
-        home = (size_t)g.vbase + from;
+    uint32_t first, rows;  // its first run, and the rows it has
+    size_t home;           // first slot of the part
+    // (g is there)
+    __device__ __forceinline__ void init(const ListArgs& a, uint32_t part) {
+        const uint32_t p = part - g.part0, np = g.nparts;
+        const uint32_t runs = (g.nrows + RUN - 1) / RUN, q = runs / np, r = runs - q * np;
+        const uint32_t missing = RUN * runs - g.nrows, owner = (runs - 1) % np;   // of the last run
+        first = p;
+        rows = RUN * (q + (p < r)) - (owner == p ? missing : 0u);
+        home = (size_t)g.vbase + RUN * (p * q + min(p, r)) - (owner < p ? missing : 0u);
         cur = words<W>(a) + g.vbase;
         R = row_lists(a, g.vbase);
         queue = a.queue + home;
+    }
+    // the vertex of its row i
+    __device__ __forceinline__ uint32_t vertex(uint32_t i) const {
+        return __ldg(g.vid + (size_t)RUN * ((i / RUN) * (size_t)g.nparts + first) + (i & (RUN - 1)));
     }
 };
 struct PartCounts {
@@ -773,8 +804,8 @@ struct Tally {
     bool changed = false;
 };
 
-// One pass over `cnt` live rows by the block, LV to a thread and step: a row that is
-// chosen back is matched, one whose candidate is matched to another moves on in its
+// One pass over `cnt` live rows (list NULL: all of the part's) by the block: a row that
+// is chosen back is matched, one whose candidate is matched to another moves on in its
 // list; live rows go to `out`, rows with a used-up list to the queue.
 template <class W>
 __device__ __forceinline__ void poll_rows(const ListArgs& a, const Part<W>& P, const uint32_t* list, uint32_t cnt,
@@ -782,141 +813,118 @@ __device__ __forceinline__ void poll_rows(const ListArgs& a, const Part<W>& P, c
     constexpr bool ROUNDS = sizeof(W) == 8;
     const ListSeg& g = P.g;
     W* cur = P.cur;
-    uint32_t v[LV], nv[LV];
-    W w[LV], nw[LV], t[LV];
-    uint4 l[LV], nl[LV];
-    // the next rows' words and lists are on their way while these are decided
-    auto fetch = [&](uint32_t base) {
-#pragma unroll
-        for (int i = 0; i < LV; i++) {
-            const uint32_t at = base + i * LT + threadIdx.x;
-            nv[i] = at < cnt ? list[at] : NIL;
-        }
-    };
+    uint32_t v, nv;
+    W w, nw, t;
+    uint4 l, nl;
+    // the next row's word and list are on their way while this one is decided
+    auto fetch = [&](uint32_t at) { nv = at >= cnt ? NIL : list ? list[at] : P.vertex(at); };
     auto fetch_words = [&]() {
-#pragma unroll
-        for (int i = 0; i < LV; i++) {
-            nw[i] = nv[i] != NIL ? look(cur + nv[i]) : (W)0;
-            nl[i] = nv[i] != NIL ? P.R.lst[nv[i]] : make_uint4(NIL, NIL, NIL, 0);
-        }
+        nw = nv != NIL ? look(cur + nv) : (W)0;
+        nl = nv != NIL ? P.R.lst[nv] : make_uint4(NIL, NIL, NIL, 0);
     };
-    fetch(0);
+    fetch(threadIdx.x);
     fetch_words();
-    for (uint32_t base = 0; base < cnt; base += LT * LV) {
-        bool gone[LV];
-#pragma unroll
-        for (int i = 0; i < LV; i++) {
-            v[i] = nv[i];
-            w[i] = nw[i];
-            l[i] = nl[i];
-        }
-#pragma unroll
-        for (int i = 0; i < LV; i++) {
-            if (v[i] != NIL && lo(w[i]) >= g.n) { set_err(a.st, ERR_BOUNDS, lo(w[i])); v[i] = NIL; }
-            t[i] = v[i] != NIL ? look(cur + lo(w[i])) : (W)0;
-        }
-        fetch(base + LT * LV);
-#pragma unroll
-        for (int i = 0; i < LV; i++)
-            gone[i] = v[i] != NIL && (lo(t[i]) & DEAD) && (lo(t[i]) & VMASK) != v[i];
-        W n[LV][3];
-#pragma unroll
-        for (int i = 0; i < LV; i++) {
-            n[i][0] = gone[i] && l[i].x != NIL ? look(cur + l[i].x) : (W)DEAD;
-            n[i][1] = gone[i] && l[i].y != NIL ? look(cur + l[i].y) : (W)DEAD;
-            n[i][2] = gone[i] && l[i].z != NIL ? look(cur + l[i].z) : (W)DEAD;
-        }
+    for (uint32_t base = 0; base < cnt; base += LT) {
+        v = nv;
+        w = nw;
+        l = nl;
+        if (v != NIL && lo(w) >= g.n) { set_err(a.st, ERR_BOUNDS, lo(w)); v = NIL; }
+        t = v != NIL ? look(cur + lo(w)) : (W)0;
+        fetch(base + LT + threadIdx.x);
+        const bool gone = v != NIL && (lo(t) & DEAD) && (lo(t) & VMASK) != v;
+        W n[3];
+        n[0] = gone && l.x != NIL ? look(cur + l.x) : (W)DEAD;
+        n[1] = gone && l.y != NIL ? look(cur + l.y) : (W)DEAD;
+        n[2] = gone && l.z != NIL ? look(cur + l.z) : (W)DEAD;
         fetch_words();
-#pragma unroll
-        for (int i = 0; i < LV; i++) {
-            bool live = v[i] != NIL, refill = false;
-            uint32_t s = 0, d = 0;
-            if (live) {
-                uint32_t u = lo(w[i]), passed = info(w[i]);
-                W y = t[i];
-                if (gone[i]) {
-                    T.changed = true;
-                    // the first of the list that is not matched (an empty place: DEAD, no round)
-                    const bool d0 = lo(n[i][0]) & DEAD, d1 = lo(n[i][1]) & DEAD, d2 = lo(n[i][2]) & DEAD;
-                    if (ROUNDS) {
-                        passed = max(passed, info(y));
-                        if (d0) passed = max(passed, info(n[i][0]));
-                        if (d0 && d1) passed = max(passed, info(n[i][1]));
-                        if (d0 && d1 && d2) passed = max(passed, info(n[i][2]));
-                    }
-                    const uint32_t at = v[i];
-                    const bool hasr = ROUNDS && (l[i].w & HASR);
-                    if (!(d0 && d1 && d2)) {
-                        u = !d0 ? l[i].x : !d1 ? l[i].y : l[i].z;
-                        y = !d0 ? n[i][0] : !d1 ? n[i][1] : n[i][2];
-                        if (hasr) {
-                            const uint4 r = P.R.rl[at];
-                            passed = max(passed, !d0 ? r.x : !d1 ? r.y : r.z);
-                            P.R.rl[at] = make_uint4(!d0 ? r.y : r.z, r.z, 0, 0);
-                        }
-                        cur[v[i]] = word<W>(u, passed);
-                        P.R.lst[at] = make_uint4(!d0 ? l[i].y : !d1 ? l[i].z : NIL, !d0 ? l[i].z : NIL, NIL, l[i].w);
-                    } else {
-                        live = false;
-                        if (l[i].w & WIDE) {
-                            // the second half of a long row's list takes the first's place
-                            const uint4 l2 = P.R.wide[at];
-                            const W m0 = l2.x != NIL ? look(cur + l2.x) : (W)DEAD;
-                            const W m1 = l2.y != NIL ? look(cur + l2.y) : (W)DEAD;
-                            const W m2 = l2.z != NIL ? look(cur + l2.z) : (W)DEAD;
-                            const W m3 = l2.w != NIL ? look(cur + l2.w) : (W)DEAD;
-                            const bool e0 = lo(m0) & DEAD, e1 = e0 && (lo(m1) & DEAD), e2 = e1 && (lo(m2) & DEAD),
-                                       e3 = e2 && (lo(m3) & DEAD);
-                            if (ROUNDS) {
-                                if (e0) passed = max(passed, info(m0));
-                                if (e1) passed = max(passed, info(m1));
-                                if (e2) passed = max(passed, info(m2));
-                                if (e3) passed = max(passed, info(m3));
-                            }
-                            l[i].w &= ~WIDE;
-                            if (!e3) {
-                                live = true;
-                                u = !e0 ? l2.x : !e1 ? l2.y : !e2 ? l2.z : l2.w;
-                                y = !e0 ? m0 : !e1 ? m1 : !e2 ? m2 : m3;
-                                if (hasr) {
-                                    const uint4 r = P.R.rw[at];
-                                    passed = max(passed, !e0 ? r.x : !e1 ? r.y : !e2 ? r.z : r.w);
-                                    P.R.rl[at] = make_uint4(!e0 ? r.y : !e1 ? r.z : r.w, !e0 ? r.z : r.w, r.w, 0);
-                                }
-                                cur[v[i]] = word<W>(u, passed);
-                                P.R.lst[at] = make_uint4(!e0 ? l2.y : !e1 ? l2.z : !e2 ? l2.w : NIL,
-                                                       !e0 ? l2.z : !e1 ? l2.w : NIL, !e0 ? l2.w : NIL, l[i].w);
-                            }
-                        }
-                        refill = !live && (l[i].w & MORE);
-                        if (refill) {
-                            s = __ldg(g.off + v[i]);
-                            d = __ldg(g.off + v[i] + 1) - s;
-                            if (ROUNDS) cur[v[i]] = word<W>(u, passed);
-                        }
-                    }
+        bool live = v != NIL, refill = false;
+        uint32_t s = 0, d = 0;
+        if (live) {
+            uint32_t u = lo(w), passed = info(w);
+            W y = t;
+            if (gone) {
+                T.changed = true;
+                // the first of the list that is not matched (an empty place: DEAD, no round)
+                const bool d0 = lo(n[0]) & DEAD, d1 = lo(n[1]) & DEAD, d2 = lo(n[2]) & DEAD;
+                if (ROUNDS) {
+                    passed = max(passed, info(y));
+                    if (d0) passed = max(passed, info(n[0]));
+                    if (d0 && d1) passed = max(passed, info(n[1]));
+                    if (d0 && d1 && d2) passed = max(passed, info(n[2]));
                 }
-                if (live && (lo(y) & VMASK) == v[i]) {
-                    // chosen back
-                    uint32_t r = 0;
-                    if (ROUNDS) {
-                        // its word, if matched already, has the round; else both ends' passed ones give it
-                        r = (lo(y) & DEAD) ? info(y) : max(passed, info(y)) + 1u;
-                        T.last = max(T.last, r);
+                const uint32_t at = v;
+                const bool hasr = ROUNDS && (l.w & HASR);
+                if (!(d0 && d1 && d2)) {
+                    u = !d0 ? l.x : !d1 ? l.y : l.z;
+                    y = !d0 ? n[0] : !d1 ? n[1] : n[2];
+                    if (hasr) {
+                        const uint4 r = P.R.rl[at];
+                        passed = max(passed, !d0 ? r.x : !d1 ? r.y : r.z);
+                        P.R.rl[at] = make_uint4(!d0 ? r.y : r.z, r.z, 0, 0);
                     }
-                    cur[v[i]] = word<W>(u | DEAD, r);
-                    g.dst[v[i]] = u;
-                    T.matched++;
+                    cur[v] = word<W>(u, passed);
+                    P.R.lst[at] = make_uint4(!d0 ? l.y : !d1 ? l.z : NIL, !d0 ? l.z : NIL, NIL, l.w);
+                } else {
                     live = false;
-                    T.changed = true;
+                    if (l.w & WIDE) {
+                        // the second half of a long row's list takes the first's place
+                        const uint4 l2 = P.R.wide[at];
+                        const W m0 = l2.x != NIL ? look(cur + l2.x) : (W)DEAD;
+                        const W m1 = l2.y != NIL ? look(cur + l2.y) : (W)DEAD;
+                        const W m2 = l2.z != NIL ? look(cur + l2.z) : (W)DEAD;
+                        const W m3 = l2.w != NIL ? look(cur + l2.w) : (W)DEAD;
+                        const bool e0 = lo(m0) & DEAD, e1 = e0 && (lo(m1) & DEAD), e2 = e1 && (lo(m2) & DEAD),
+                                   e3 = e2 && (lo(m3) & DEAD);
+                        if (ROUNDS) {
+                            if (e0) passed = max(passed, info(m0));
+                            if (e1) passed = max(passed, info(m1));
+                            if (e2) passed = max(passed, info(m2));
+                            if (e3) passed = max(passed, info(m3));
+                        }
+                        l.w &= ~WIDE;
+                        if (!e3) {
+                            live = true;
+                            u = !e0 ? l2.x : !e1 ? l2.y : !e2 ? l2.z : l2.w;
+                            y = !e0 ? m0 : !e1 ? m1 : !e2 ? m2 : m3;
+                            if (hasr) {
+                                const uint4 r = P.R.rw[at];
+                                passed = max(passed, !e0 ? r.x : !e1 ? r.y : !e2 ? r.z : r.w);
+                                P.R.rl[at] = make_uint4(!e0 ? r.y : !e1 ? r.z : r.w, !e0 ? r.z : r.w, r.w, 0);
+                            }
+                            cur[v] = word<W>(u, passed);
+                            P.R.lst[at] = make_uint4(!e0 ? l2.y : !e1 ? l2.z : !e2 ? l2.w : NIL,
+                                                   !e0 ? l2.z : !e1 ? l2.w : NIL, !e0 ? l2.w : NIL, l.w);
+                        }
+                    }
+                    refill = !live && (l.w & MORE);
+                    if (refill) {
+                        s = __ldg(g.off + v);
+                        d = __ldg(g.off + v + 1) - s;
+                        if (ROUNDS) cur[v] = word<W>(u, passed);
+                    }
                 }
             }
-            warp_append(&S.live, out, live, v[i]);
-            if (__any_sync(FULL, refill)) {
-                const bool few = refill && d <= LIST_SHORT, many = refill && d > LIST_SHORT;
-                const uint32_t q0 = warp_slot(&S.nshort, few), q1 = warp_slot(&S.nlong, many);
-                if (refill) P.queue[few ? q0 : P.rows - 1 - q1] = make_uint4(v[i], s, d, 0);
+            if (live && (lo(y) & VMASK) == v) {
+                // chosen back
+                uint32_t r = 0;
+                if (ROUNDS) {
+                    // its word, if matched already, has the round; else both ends' passed ones give it
+                    r = (lo(y) & DEAD) ? info(y) : max(passed, info(y)) + 1u;
+                    T.last = max(T.last, r);
+                }
+                cur[v] = word<W>(u | DEAD, r);
+                g.dst[v] = u;
+                T.matched++;
+                live = false;
+                T.changed = true;
             }
+        }
+        warp_append(&S.live, out, live, v);
+        if (__any_sync(FULL, refill)) {
+            const bool few = refill && d <= LIST_SHORT, many = refill && d > LIST_SHORT;
+            const uint32_t q0 = warp_slot(&S.nshort, few), q1 = warp_slot(&S.nlong, many);
+            // (the rounds of matched ends are wanted again, however heavy their edges)
+            if (refill) P.queue[few ? q0 : P.rows - 1 - q1] = make_uint4(v, s, d, ROUNDS ? ~0u : l.w | FLAGS);
         }
     }
 }
@@ -953,7 +961,7 @@ __device__ __forceinline__ void refill_rows(const ListArgs& a, const Part<W>& P,
         }
         for (int k = 0; k < 2; k++) {
             const uint32_t v = __shfl_sync(FULL, q2.x, 16 * k), s = __shfl_sync(FULL, q2.y, 16 * k),
-                           d = __shfl_sync(FULL, q2.z, 16 * k);
+                           d = __shfl_sync(FULL, q2.z, 16 * k), ub = __shfl_sync(FULL, q2.w, 16 * k);
             if (d == 0) continue;
             if (d > BLOCK_ROW) {
                 huge = true;
@@ -964,7 +972,7 @@ __device__ __forceinline__ void refill_rows(const ListArgs& a, const Part<W>& P,
                 live = refill_group<W, 32, 4, KL>(g, cur, P.R, v, s, d);
             } else {
                 LaneTop64 t;
-                refill_scan<W>(g, cur, s, d, 0, 1, t);
+                refill_scan<W>(g, cur, s, d, ub, 0, 1, t);
                 live = __shfl_sync(FULL, t.k, 0) != 0;
                 uint32_t r = 0;
                 if (ROUNDS && live) r = refill_passed(g, reinterpret_cast<const uint64_t*>(cur), s, d, 0, 1, t);
@@ -998,7 +1006,7 @@ __device__ __forceinline__ void refill_rows(const ListArgs& a, const Part<W>& P,
         if (d <= BLOCK_ROW) continue;
         {
             LaneTop64 t;
-            refill_scan<W>(g, cur, s, d, warp, LW, t);
+            refill_scan<W>(g, cur, s, d, q4.w, warp, LW, t);
             if (lane < KL) {
                 S.k[warp][lane] = t.k;
                 S.n[warp][lane] = t.n;
@@ -1028,7 +1036,10 @@ __device__ __forceinline__ void refill_rows(const ListArgs& a, const Part<W>& P,
     }
 }
 
+template <class W>
 struct LiveSmem {
+    ListArgs a;
+    Part<W> p;
     RefillSmem r;
     PartCounts c;
     uint32_t part, changed, stop, next[2];
@@ -1038,12 +1049,16 @@ struct LiveSmem {
 // Blocks take parts from a counter and pass over a part's live rows until none is
 // left.  A part may wait for words that another block writes, but no block waits for
 // good: after IDLE_MAX passes without a change it puts the part's rows back for the
-// next launch, which the last block to leave asks for.
+// next launch, which the last block to leave asks for.  (pa: the arguments in device
+// memory, for a launch in a graph.)
 template <class W>
-__global__ void __launch_bounds__(LT, LM_LMINB) k_live(const ListArgs* __restrict__ pa, cudaGraphConditionalHandle h,
-                                                       uint32_t in_graph) {
-    __shared__ LiveSmem S;
-    const ListArgs& a = *pa;
+__global__ void __launch_bounds__(LT, LMINB) k_live(const __grid_constant__ ListArgs av,
+                                                       const ListArgs* __restrict__ pa, cudaGraphConditionalHandle h) {
+    __shared__ LiveSmem<W> S;
+    copy_words(&S.a, pa ? pa : &av, LT);
+    __syncthreads();
+    const ListArgs& a = S.a;
+    const Part<W>& P = S.p;
     DevState* st = a.st;
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t launch = ld_volatile_u32(&st->round);
@@ -1054,10 +1069,13 @@ __global__ void __launch_bounds__(LT, LM_LMINB) k_live(const ListArgs* __restric
         const uint32_t part = S.part;
         if (part >= a.nparts) break;
         const uint32_t si = a.pmap ? a.pmap[part] : 0u;
-        const Part<W> P(a, a.segs[si], part);
+        copy_words(&S.p.g, a.pmap ? a.segs + si : &a.one, LT);
+        __syncthreads();
+        if (tid == 0) S.p.init(a, part);
+        __syncthreads();
         const uint32_t pc = launch ? a.pcount[part] : P.rows << 1;
         uint32_t cnt = pc >> 1, buf = pc & 1u;
-        const uint32_t* list = launch ? a.list[buf] + P.home : P.g.vid + P.from;
+        const uint32_t* list = launch ? a.list[buf] + P.home : nullptr;
         Tally T;
         uint32_t idle = 0;
         for (uint32_t pass = 0; cnt; pass++) {
@@ -1126,7 +1144,7 @@ __global__ void __launch_bounds__(LT, LM_LMINB) k_live(const ListArgs* __restric
             st->left = 0;
             st->round = launch + 1;
             if (rest == 0) st->done = 1;
-            if (in_graph) cudaGraphSetConditional(h, rest && !ld_volatile_u32(&st->err) ? 1u : 0u);
+            if (pa) cudaGraphSetConditional(h, rest && !ld_volatile_u32(&st->err) ? 1u : 0u);
             __threadfence();
         }
     }
@@ -1139,19 +1157,17 @@ __global__ void __launch_bounds__(LT, LM_LMINB) k_live(const ListArgs* __restric
 // unmatched) so that the gathers of k_round_counts stay in L2; ring_m / ring_n get the
 // edges and rows by their last live round.  Counters are a thread's own columns of a
 // shared table: nearly all lanes count the same few rounds.
-__global__ void k_round_bytes(const ListArgs* __restrict__ pa, uint8_t* mr) {
-    const ListArgs& a = *pa;
-    const uint32_t n = a.segs[0].n;
+__global__ void k_round_bytes(const __grid_constant__ ListArgs a, uint8_t* mr) {
+    const uint32_t n = a.one.n;
     const uint64_t* cur = words<uint64_t>(a);
-    const uint32_t* dst = a.segs[0].dst;
+    const uint32_t* dst = a.one.dst;
     for (uint64_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (uint64_t)gridDim.x * blockDim.x)
         mr[v] = dst[v] == NIL ? 255 : (uint8_t)min(info(cur[v]) - 1u, 63u);
 }
-__global__ void __launch_bounds__(256) k_round_counts(const ListArgs* __restrict__ pa,
+__global__ void __launch_bounds__(256) k_round_counts(const __grid_constant__ ListArgs a,
                                                       const uint8_t* __restrict__ mr) {
     __shared__ uint32_t h[64][128];   // two threads a column: counts of either by halves of 16 bits
-    const ListArgs& a = *pa;
-    const ListSeg& g = a.segs[0];
+    const ListSeg& g = a.one;
     const uint32_t tid = threadIdx.x;
     uint16_t* col = reinterpret_cast<uint16_t*>(&h[0][0]) + tid;   // [round][thread]
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -1221,8 +1237,7 @@ __global__ void __launch_bounds__(256) k_round_counts(const ListArgs* __restrict
 }
 
 // graph of every block of k_top and of every part
-__global__ void k_list_map(const ListArgs* __restrict__ pa, uint32_t* bmap, uint32_t* pmap) {
-    const ListArgs& a = *pa;
+__global__ void k_list_map(const __grid_constant__ ListArgs a, uint32_t* bmap, uint32_t* pmap) {
     const uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (w >= a.nsegs) return;
     const ListSeg& g = a.segs[w];
@@ -1235,34 +1250,34 @@ int sms() {
     cudaGetDevice(&dev);
     return device_sm_count(dev);
 }
-uint32_t live_grid() { return (uint32_t)sms() * LM_LMINB; }   // every block resident
+uint32_t live_grid() { return (uint32_t)sms() * LMINB; }   // every block resident
 
 }  // namespace
 
-uint32_t list_live_blocks(int device) { return (uint32_t)device_sm_count(device) * LM_LMINB; }
+uint32_t list_live_blocks(int device) { return (uint32_t)device_sm_count(device) * LMINB; }
 uint32_t list_blocks(const uint32_t task[4], uint32_t nrows) {
     const TopBlocks b = top_blocks(task, nrows);
     const uint32_t t = b.l + b.w + b.g + b.s;
     return t ? t : 1u;
 }
-int launch_list_map(void* stream, const ListArgs* d, uint32_t nsegs, uint32_t* bmap, uint32_t* pmap) {
+int launch_list_map(void* stream, const ListArgs& d, uint32_t nsegs, uint32_t* bmap, uint32_t* pmap) {
     k_list_map<<<(nsegs + 7) / 8, 256, 0, (cudaStream_t)stream>>>(d, bmap, pmap);
     return (int)cudaGetLastError();
 }
-int launch_top(void* stream, const ListArgs* d, uint32_t blocks, bool rounds) {
+int launch_top(void* stream, const ListArgs& d, uint32_t blocks, bool rounds) {
     if (rounds) k_top<uint64_t><<<blocks, TT, 0, (cudaStream_t)stream>>>(d);
     else k_top<uint32_t><<<blocks, TT, 0, (cudaStream_t)stream>>>(d);
     return (int)cudaGetLastError();
 }
 // (more blocks than parts would only come and go)
-int launch_live(void* stream, const ListArgs* d, uint32_t nparts, bool rounds) {
+int launch_live(void* stream, const ListArgs& d, uint32_t nparts, bool rounds) {
     const uint32_t grid = nparts < live_grid() ? nparts : live_grid();
     const cudaGraphConditionalHandle none{};
-    if (rounds) k_live<uint64_t><<<grid, LT, 0, (cudaStream_t)stream>>>(d, none, 0u);
-    else k_live<uint32_t><<<grid, LT, 0, (cudaStream_t)stream>>>(d, none, 0u);
+    if (rounds) k_live<uint64_t><<<grid, LT, 0, (cudaStream_t)stream>>>(d, nullptr, none);
+    else k_live<uint32_t><<<grid, LT, 0, (cudaStream_t)stream>>>(d, nullptr, none);
     return (int)cudaGetLastError();
 }
-int launch_round_counts(void* stream, const ListArgs* d, void* bytes) {
+int launch_round_counts(void* stream, const ListArgs& d, void* bytes) {
     k_round_bytes<<<sms() * 8, 256, 0, (cudaStream_t)stream>>>(d, (uint8_t*)bytes);
     k_round_counts<<<sms() * 6, 256, 0, (cudaStream_t)stream>>>(d, (const uint8_t*)bytes);
     return (int)cudaGetLastError();
@@ -1275,8 +1290,9 @@ int build_list_graph(const ListArgs* dargs, bool rounds, void** exec_out) {
     cudaError_t e = cudaGraphCreate(&g, 0);
     if (e != cudaSuccess) return (int)e;
     cudaGraphConditionalHandle h{};
-    uint32_t yes = 1;
-    void* params[3] = {&dargs, &h, &yes};
+    ListArgs unused;
+    memset(&unused, 0, sizeof unused);
+    void* params[3] = {&unused, &dargs, &h};
     cudaKernelNodeParams kp{};
     kp.func = rounds ? (void*)k_live<uint64_t> : (void*)k_live<uint32_t>;
     kp.gridDim = dim3(live_grid());
