@@ -674,19 +674,19 @@ static void list_args(ListArgs& A, Engine& e) {
     A.part = w.part;
     A.pcnt = w.pcnt;
     A.st = e.st;
+    A.host = e.st_host;
 }
 
 // an asynchronous list job's arguments sit in the last quarter of the argument area
 constexpr size_t LIST_ARGS_OFF = ARG_AREA / 4 * 3;
 
 // The live pass of a queued job, until no row is left: k_live as often as it gives rows
-// back (once, as a rule), the state copied to the host after each.
+// back (once, as a rule), the state in the host's mirror after each.
 static int run_live(lm_ctx* ctx, Engine& e, const ListArgs& A, uint32_t nparts, bool rounds, Prof& prof) {
     for (;;) {
         prof.begin(LM_K_SWEEP);
         LM_CK(ctx, launch_live(e.stream, A, nparts, rounds));
         prof.end();
-        LM_CK(ctx, cudaMemcpyAsync(e.st_host, e.st, sizeof(DevState), cudaMemcpyDeviceToHost, e.stream));
         LM_CK(ctx, cudaStreamSynchronize(e.stream));
         if (e.st_host->err || e.st_host->done) return check_err(ctx, e);
     }
@@ -709,6 +709,7 @@ static int match_list(lm_ctx* ctx, Engine& e, const lm_graph* g, uint64_t seed, 
     job_limits(ctx, g->m, &A.max_rounds, &A.limit_ns);
     A.one = list_seg(g, seed, mate_d);
     A.one.nparts = nparts;
+    if (async) A.host = nullptr;
     prof.begin(LM_K_CAND);
     LM_CK(ctx, launch_top(s, A, A.one.nblk, rounds));
     prof.end();
@@ -762,12 +763,12 @@ static int match_renewed(lm_ctx* ctx, Engine& e, const lm_graph* g, uint64_t see
     A.pcnt = e.lw.pcnt;
     A.ctr = e.lw.pcount;
     A.st = e.st;
+    A.host = async ? nullptr : e.st_host;
     job_limits(ctx, g->m, &A.max_rounds, &A.limit_ns);
     prof.begin(LM_K_SWEEP);
     LM_CK(ctx, launch_renew(s, A, counts));
     prof.end();
     if (async) return LM_OK;  // queued; lm_sync reports device errors
-    LM_CK(ctx, cudaMemcpyAsync(e.st_host, e.st, sizeof(DevState), cudaMemcpyDeviceToHost, s));
     if (!dev_out) LM_CK(ctx, cudaMemcpyAsync(mate, mate_d, (size_t)g->n * 4, cudaMemcpyDeviceToHost, s));
     LM_CK(ctx, cudaStreamSynchronize(s));
     return check_err(ctx, e);
@@ -1088,6 +1089,8 @@ void lm_destroy(lm_ctx* ctx) {
     for (int i = 0; i < ctx->nev; i++) cudaEventDestroy(ctx->ev[i]);
     if (ctx->up) cudaStreamDestroy(ctx->up);
     if (ctx->up_ev) cudaEventDestroy(ctx->up_ev);
+    for (cudaEvent_t ev : ctx->up_w)
+        if (ev) cudaEventDestroy(ev);
     if (ctx->pool) cudaMemPoolDestroy(ctx->pool);  // released once no allocation is left
     cudaGetLastError();
     delete ctx;
@@ -1167,39 +1170,51 @@ int lm_graph_create(lm_ctx* ctx, uint32_t n, uint32_t m, const uint32_t* eu, con
     bt.eword = g->eword;
     LM_CK(ctx, cudaMemsetAsync(bt.deg, 0, nn * 4, s));
     LM_CK(ctx, cudaMemsetAsync(bt.err, 0, 48, s));
-    // validation rides on the degree count: endpoint < n, no self loop, no NaN
-    if (mem == LM_HOST && m > 0) {
-        // chunks of the host arrays go up on the upload stream; the context's stream
-        // runs a chunk's degree pass while the next chunk is copied
+    // validation rides on the passes: endpoint < n and no self loop on the degree count, no NaN on
+    // the fill
+    const bool upload = mem == LM_HOST && m > 0;
+    const uint32_t step = upload ? build_step(m, lm_ctx::UP_CHUNKS) : m;
+    // no return before the uploads have read the caller's arrays and left the staging
+    struct UpWait {
+        cudaStream_t s;
+        ~UpWait() { if (s) cudaStreamSynchronize(s); }
+    } uw{nullptr};
+    if (upload) {
+        // chunks of the host arrays go up on the upload stream, the ends first, then the
+        // weights; the context's stream runs a chunk's pass while the next chunk is copied
         if (!ctx->up) {
             LM_CK(ctx, cudaStreamCreateWithFlags(&ctx->up, cudaStreamNonBlocking));
             LM_CK(ctx, cudaEventCreateWithFlags(&ctx->up_ev, cudaEventDisableTiming));
+            for (cudaEvent_t& ev2 : ctx->up_w) LM_CK(ctx, cudaEventCreateWithFlags(&ev2, cudaEventDisableTiming));
         }
         LM_CK(ctx, cudaEventRecord(ctx->up_ev, s));  // after the memsets (and earlier work)
         LM_CK(ctx, cudaStreamWaitEvent(ctx->up, ctx->up_ev, 0));
-        constexpr uint32_t NCHUNK = 8;
-        const uint32_t step = build_step(m, NCHUNK);
-        for (uint32_t off = 0, cnt; off < m; off += cnt) {
-            cnt = std::min(step, m - off);
-            LM_CK(ctx, cudaMemcpyAsync(t_eu + off, eu + off, (size_t)cnt * 4, cudaMemcpyHostToDevice, ctx->up));
-            LM_CK(ctx, cudaMemcpyAsync(t_ev + off, ev + off, (size_t)cnt * 4, cudaMemcpyHostToDevice, ctx->up));
-            LM_CK(ctx, cudaMemcpyAsync(t_w + off, w + off, (size_t)cnt * 4, cudaMemcpyHostToDevice, ctx->up));
+        uw.s = ctx->up;
+        for (uint32_t at = 0, cnt; at < m; at += cnt) {
+            cnt = std::min(step, m - at);
+            LM_CK(ctx, cudaMemcpyAsync(t_eu + at, eu + at, (size_t)cnt * 4, cudaMemcpyHostToDevice, ctx->up));
+            LM_CK(ctx, cudaMemcpyAsync(t_ev + at, ev + at, (size_t)cnt * 4, cudaMemcpyHostToDevice, ctx->up));
             LM_CK(ctx, cudaEventRecord(ctx->up_ev, ctx->up));
             LM_CK(ctx, cudaStreamWaitEvent(s, ctx->up_ev, 0));
-            LM_CK(ctx, launch_build_degrees(s, t_eu, t_ev, t_w, n, m, off, cnt, bt));
+            LM_CK(ctx, launch_build_degrees(s, t_eu, t_ev, n, m, at, cnt, bt));
+        }
+        for (uint32_t at = 0, cnt, i = 0; at < m; at += cnt, i++) {
+            cnt = std::min(step, m - at);
+            LM_CK(ctx, cudaMemcpyAsync(t_w + at, w + at, (size_t)cnt * 4, cudaMemcpyHostToDevice, ctx->up));
+            LM_CK(ctx, cudaEventRecord(ctx->up_w[i], ctx->up));
         }
     } else if (m > 0) {
-        LM_CK(ctx, launch_build_degrees(s, eu, ev, w, n, m, 0, m, bt));
+        LM_CK(ctx, launch_build_degrees(s, eu, ev, n, m, 0, m, bt));
     }
     int rc = ensure_pinned(ctx, e, 64);  // 16 words
     if (rc) return rc;
     uint32_t* hp = static_cast<uint32_t*>(e.pinned);
     LM_CK(ctx, launch_nonzero_flags(s, bt.deg, n + 1, flags, bt.err + 4));
-    LM_CK(ctx, cudaMemcpyAsync(&hp[4], bt.err, 32, cudaMemcpyDeviceToHost, s));
     LM_CK(ctx, launch_exclusive_scan(s, flags, rowidx, n + 1, scan_tmp, scan_words));
-    LM_CK(ctx, cudaMemcpyAsync(&hp[0], rowidx + n, 4, cudaMemcpyDeviceToHost, s));
+    LM_CK(ctx, launch_build_counts(s, bt.err, rowidx + n, hp));
     LM_CK(ctx, cudaStreamSynchronize(s));
-    if (hp[4]) return fail(ctx, LM_EINVAL, "edge list: endpoint >= n, self loop or NaN weight");
+    static const char* const bad = "edge list: endpoint >= n, self loop or NaN weight";
+    if (hp[4]) return fail(ctx, LM_EINVAL, bad);
     g->nrows = hp[0];
     for (int k = 0; k < 4; k++) g->ntask[k] = hp[8 + k] + (k ? g->ntask[k - 1] : 0u);
 
@@ -1218,21 +1233,24 @@ int lm_graph_create(lm_ctx* ctx, uint32_t n, uint32_t m, const uint32_t* eu, con
     gc.assign(g->block[1]);
     g->bytes = ec.total + gc.total;
     LM_CK(ctx, launch_exclusive_scan(s, bt.deg, g->off, n + 1, scan_tmp, scan_words));
-    if (m > 0) {
-        LM_CK(ctx, launch_build_fill(s, n, m, g->off, g->eid, g->ent, bt, scan_tmp, scan_words));
-        LM_CK(ctx, cudaMemcpyAsync(&hp[2], bt.err, 4, cudaMemcpyDeviceToHost, s));
-    }
-    // each kind's tasks follow the previous one's
-    hp[12] = 0;
-    for (int k = 1; k < 4; k++) hp[12 + k] = g->ntask[k - 1];
-    LM_CK(ctx, cudaMemcpyAsync(bt.err + 8, &hp[12], 16, cudaMemcpyHostToDevice, s));
     LM_CK(ctx, launch_build_rows(s, bt.deg, rowidx, g->off, n, g->nrows, g->nent, g->vid, g->rdeg, g->roff, g->task,
                                  g->ntask[3], bt.err + 8));
     if (g->nrows) {
         LM_CK(ctx, cudaMemsetAsync(g->rbits, 0, ((size_t)g->ntiles * (TILE0 / 32) + 8) * 4, s));
         LM_CK(ctx, launch_build_tilemap(s, g->roff, g->nrows, g->nent, g->tmap, g->rbits, g->tdesc));
     }
+    if (m > 0) {
+        LM_CK(ctx, launch_exclusive_scan(s, bt.hist, bt.offs, build_scan_count(m), scan_tmp, scan_words));
+        for (uint32_t at = 0, cnt, i = 0; at < m; at += cnt, i++) {
+            cnt = std::min(step, m - at);
+            if (upload) LM_CK(ctx, cudaStreamWaitEvent(s, ctx->up_w[i], 0));
+            LM_CK(ctx, launch_build_fill_u(s, upload ? t_w : w, n, m, at, cnt, g->off, g->eid, g->ent, bt));
+        }
+        LM_CK(ctx, launch_build_fill_v(s, m, g->eid, g->ent, bt));
+        LM_CK(ctx, cudaMemcpyAsync(&hp[2], bt.err, 4, cudaMemcpyDeviceToHost, s));
+    }
     LM_CK(ctx, cudaStreamSynchronize(s));
+    if (m > 0 && (hp[2] & 1u)) return fail(ctx, LM_EINVAL, bad);
     if (m > 0 && (hp[2] & 2u)) return fail(ctx, LM_ECUDA, "graph build: a fill slot fell outside the edge arrays");
     *out = g.release();
     return LM_OK;
@@ -1363,17 +1381,13 @@ int lm_contract(lm_ctx* ctx, uint32_t n, uint32_t m, const uint32_t* eu, const u
     if (!rc) rc = ensure_pinned(ctx, e, 64);
     if (rc) return rc;
     uint32_t* hp = static_cast<uint32_t*>(e.pinned);
-    cudaError_t ce = (cudaError_t)launch_contract(s, c, &hp[4]);
-    if (ce == cudaSuccess) ce = cudaMemcpyAsync(&hp[0], c.err, 4, cudaMemcpyDeviceToHost, s);
-    if (ce == cudaSuccess) ce = cudaMemcpyAsync(&hp[1], c.rank + n, 4, cudaMemcpyDeviceToHost, s);
-    hp[2] = 0;
-    if (ce == cudaSuccess && m > 0) ce = cudaMemcpyAsync(&hp[2], c.counts + 2, 4, cudaMemcpyDeviceToHost, s);
+    cudaError_t ce = (cudaError_t)launch_contract(s, c, hp);
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
     if (ce != cudaSuccess) return fail(ctx, LM_ECUDA, "contraction: %s", cudaGetErrorString(ce));
-    if (hp[0] & 1u) return fail(ctx, LM_EINVAL, "mate is not a matching of the vertex set");
-    if (hp[0] & 2u) return fail(ctx, LM_EINVAL, "an edge endpoint is >= n");
-    *n_out = hp[1];
-    *m_out = hp[2];
+    if (hp[6] & 1u) return fail(ctx, LM_EINVAL, "mate is not a matching of the vertex set");
+    if (hp[6] & 2u) return fail(ctx, LM_EINVAL, "an edge endpoint is >= n");
+    *n_out = hp[5];
+    *m_out = hp[7];
     return LM_OK;
 }
 

@@ -1109,6 +1109,17 @@ __global__ void __launch_bounds__(CT) k_c_emit(uint32_t m, const uint32_t* __res
     }
 }
 
+// What the host waits for, written to its memory: counts[0 .. 4], the coarse vertices, the
+// error bits, the coarse edges (0 without edges).  One launch instead of a copy each.
+__global__ void k_c_report(const uint32_t* __restrict__ counts, const uint32_t* __restrict__ nc,
+                           const uint32_t* __restrict__ err, const uint32_t* __restrict__ mc,
+                           volatile uint32_t* host) {
+    for (int i = 0; i < 5; i++) host[i] = counts[i];
+    host[5] = *nc;
+    host[6] = *err;
+    host[7] = mc ? *mc : 0u;
+}
+
 uint32_t bits_for(uint32_t x) {  // bits to write 0 .. x
     uint32_t b = 1;
     while (b < 32 && (x >> b)) b++;
@@ -1136,7 +1147,7 @@ size_t contract_sort_words(uint32_t m) {
     return (size_t)(2 * (256 * tiles + 4));
 }
 
-int launch_contract(void* stream, const ContractArgs& c, uint32_t* mc_host_slot) {
+int launch_contract(void* stream, const ContractArgs& c, uint32_t* host) {
     cudaStream_t s = (cudaStream_t)stream;
     cudaError_t e;
     if ((e = cudaMemsetAsync(c.err, 0, sizeof(uint32_t), s))) return (int)e;
@@ -1145,7 +1156,12 @@ int launch_contract(void* stream, const ContractArgs& c, uint32_t* mc_host_slot)
     k_c_rep<<<grid_for(c.n), CT, 0, s>>>(c.mate, c.n, c.flag, c.err);
     if (int r = launch_exclusive_scan(s, c.flag, c.rank, c.n + 1, c.scan_tmp, c.scan_words)) return r;
     k_c_map<<<grid_for(c.n), CT, 0, s>>>(c.mate, c.n, c.rank, c.vw, c.cmap, c.cvw);
-    if (c.m == 0) return (int)cudaGetLastError();
+    const uint32_t words = (uint32_t)(((uint64_t)c.m + 31) / 32);
+    auto report = [&](bool last) -> int {
+        k_c_report<<<1, 1, 0, s>>>(c.counts, c.rank + c.n, c.err, last && c.m ? c.wpos + words : nullptr, host);
+        return (int)cudaGetLastError();
+    };
+    if (c.m == 0) return report(true);
     if ((e = cudaFuncSetAttribute(k_rs_scatter<uint32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)sizeof(RsSmem<uint32_t>)))) return (int)e;
     if ((e = cudaFuncSetAttribute(k_rs_scatter<unsigned long long>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1175,7 +1191,6 @@ int launch_contract(void* stream, const ContractArgs& c, uint32_t* mc_host_slot)
         return (int)cudaGetLastError();
     };
     uint32_t* hk[2] = {reinterpret_cast<uint32_t*>(c.key[0]), reinterpret_cast<uint32_t*>(c.key[1])};
-    const uint32_t words = (uint32_t)(((uint64_t)c.m + 31) / 32);
     const uint32_t egrid = grid_for(((uint64_t)c.m + 3) / 4);
     const bool vec = ((reinterpret_cast<uintptr_t>(c.eu) | reinterpret_cast<uintptr_t>(c.ev) |
                        reinterpret_cast<uintptr_t>(c.w)) & 15u) == 0;
@@ -1186,13 +1201,10 @@ int launch_contract(void* stream, const ContractArgs& c, uint32_t* mc_host_slot)
     // counts to the host: crossing edges, coarse vertices, edges left to the general path, a
     // partition outgrew its room
     auto read_counts = [&]() -> int {
-        cudaError_t x;
-        if ((x = cudaMemcpyAsync(mc_host_slot, c.counts, 5 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s))) return (int)x;
-        if ((x = cudaMemcpyAsync(mc_host_slot + 5, c.rank + c.n, sizeof(uint32_t), cudaMemcpyDeviceToHost, s)))
-            return (int)x;
-        if ((x = cudaStreamSynchronize(s))) return (int)x;
-        mc = mc_host_slot[0];
-        nc = mc_host_slot[5];
+        if (int r = report(false)) return r;
+        if (cudaError_t x = cudaStreamSynchronize(s)) return (int)x;
+        mc = host[0];
+        nc = host[5];
         return 0;
     };
     // 1. partitions, where their rule holds: the crossing bits become the leader bits, every
@@ -1217,7 +1229,7 @@ int launch_contract(void* stream, const ContractArgs& c, uint32_t* mc_host_slot)
         groups<<<1u << pb, 512u << big, gsmem, s>>>(items, c.shist, cap, pb, gb, c.val[0], ofl, c.counts);
         k_c_walk<<<egrid, CT, 0, s>>>(c.val[0], c.cpair, c.w, c.cross, c.multi, c.gref, ofl, c.counts);
         if (int r = read_counts()) return r;
-        done = mc_host_slot[4] == 0;
+        done = host[4] == 0;
     }
     // or every edge keyed by its pair's hash in input order; the stable sort keeps input
     // order among equal keys and puts the edges inside pairs last, after the mc crossing
@@ -1229,7 +1241,7 @@ int launch_contract(void* stream, const ContractArgs& c, uint32_t* mc_host_slot)
         auto keys = vec ? k_c_keys<true> : k_c_keys<false>;
         keys<<<kgrid, CT, 0, s>>>(c.eu, c.ev, c.m, c.n, c.cmap, hk[0], c.cpair, c.cross, c.counts, c.shist, c.err);
         if (int r = read_counts()) return r;
-        mc_host_slot[1] = 0;
+        host[1] = 0;
         // the sort's bits: as few bytes as leave at most BK_AVG crossing edges to a bucket
         uint32_t sbits = c.sort_bits;
         if (!sbits)
@@ -1253,17 +1265,15 @@ int launch_contract(void* stream, const ContractArgs& c, uint32_t* mc_host_slot)
     }
     // 2. the flagged edges are taken out in order with their pair as the key, sorted by the
     //    pair and marked
-    if (mc_host_slot[1]) {
+    if (host[1]) {
         const uint32_t bits = bits_for(nc ? nc - 1 : 0);
         const uint32_t tiles = (c.m + RN_TILE - 1) / RN_TILE;
         uint32_t* toffs = c.tsum + ((size_t)c.m / RN_TILE + 2);
         k_c_runs_count<<<tiles, CT, 0, s>>>(ofl, c.m, c.tsum);
         if (int r = launch_exclusive_scan(s, c.tsum, toffs, tiles, c.scan_tmp, c.scan_words)) return r;
         k_c_runs_take<<<tiles, CT, 0, s>>>(ofl, c.m, toffs, c.cpair, bits, c.key[0], c.val[0], c.counts);
-        if ((e = cudaMemcpyAsync(mc_host_slot, c.counts + 3, sizeof(uint32_t), cudaMemcpyDeviceToHost, s)))
-            return (int)e;
-        if ((e = cudaStreamSynchronize(s))) return (int)e;
-        const uint32_t nsub = mc_host_slot[0];
+        if (int r = read_counts()) return r;
+        const uint32_t nsub = host[3];
         int cur = 0;
         if (nsub) {
             if (int r = radix(c.key[0], c.key[1], c.val[0], c.val[1], nsub, 2 * bits, false, false, &cur)) return r;
@@ -1273,8 +1283,6 @@ int launch_contract(void* stream, const ContractArgs& c, uint32_t* mc_host_slot)
     // 3. leaders ranked by words of the bitmask; the leaders write the coarse edges
     k_c_wcount<<<grid_for((uint64_t)words + 1), CT, 0, s>>>(c.cross, words, c.wlead);
     if (int r = launch_exclusive_scan(s, c.wlead, c.wpos, words + 1, c.scan_tmp, c.scan_words)) return r;
-    if ((e = cudaMemcpyAsync(c.counts + 2, c.wpos + words, sizeof(uint32_t), cudaMemcpyDeviceToDevice, s)))
-        return (int)e;
     if (mc) {
         if (vec)
             k_c_emit<true><<<egrid, CT, 0, s>>>(c.m, c.cpair, c.w, c.cross, c.wpos, c.multi, c.gref, c.ceu, c.cev,
@@ -1283,7 +1291,7 @@ int launch_contract(void* stream, const ContractArgs& c, uint32_t* mc_host_slot)
             k_c_emit<false><<<egrid, CT, 0, s>>>(c.m, c.cpair, c.w, c.cross, c.wpos, c.multi, c.gref, c.ceu, c.cev,
                                                  c.cw);
     }
-    return (int)cudaGetLastError();
+    return report(true);
 }
 
 }  // namespace lm

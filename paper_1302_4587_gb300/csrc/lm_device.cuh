@@ -92,6 +92,13 @@ __device__ __forceinline__ void set_err(DevState* st, uint32_t bit, uint32_t inf
     if ((atomicOr(&st->err, bit) & bit) == 0) st->err_info = info;
     atomicOr(&st->err_any, bit);  // not reset by the next job's init (asynchronous matches)
 }
+// the job's state into the host's mirror by the last block to leave (`threads` threads): a
+// copy in the stream would cost a small job 5 us more
+__device__ __forceinline__ void state_to_host(DevState* host, const DevState* st, uint32_t threads) {
+    static_assert(sizeof(DevState) % 4 == 0, "words");
+    for (uint32_t i = threadIdx.x; i < sizeof(DevState) / 4; i += threads)
+        reinterpret_cast<volatile uint32_t*>(host)[i] = __ldcg(reinterpret_cast<const uint32_t*>(st) + i);
+}
 __device__ __forceinline__ uint64_t globaltimer_ns() {
     uint64_t t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));

@@ -117,7 +117,8 @@ struct lm_ctx {
     // upload of a host edge list in chunks on its own stream, each chunk's degree
     // count on the context's stream while the next chunk is in flight
     cudaStream_t up = nullptr;
-    cudaEvent_t up_ev = nullptr;
+    static constexpr uint32_t UP_CHUNKS = 8;  // chunks of an uploaded edge list
+    cudaEvent_t up_ev = nullptr, up_w[UP_CHUNKS] = {};
     // limits of every match (lm_set_limits): a round cap (0 = none beyond m + 2)
     // and a time limit in ns (0 = LOOP_LIMIT_NS)
     uint32_t lim_rounds = 0;

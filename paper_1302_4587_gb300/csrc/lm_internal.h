@@ -295,6 +295,7 @@ struct ListArgs {
     uint32_t max_rounds;
     unsigned long long limit_ns;
     DevState* st;
+    DevState* host;           // its mirror in pinned memory (NULL: nobody waits for it)
 };
 // Arguments of a job under a renewed order (lm_renew.cu)
 constexpr uint32_t RENEW_CTRS = 16;
@@ -309,6 +310,7 @@ struct RenewArgs {
     uint32_t max_rounds;
     unsigned long long limit_ns;
     DevState* st;
+    DevState* host;           // as in ListArgs
 };
 
 constexpr unsigned long long LOOP_LIMIT_NS = 120000000000ull;  // 120 s: the default time limit of a job
@@ -350,8 +352,8 @@ struct ContractArgs {
     uint32_t* flag;           // [n + 1] representative flags
     uint32_t* rank;           // [n + 1] their exclusive prefix (rank[n] = coarse vertices)
     uint32_t* cross;          // [m / 32 + 2] bit e: edge e joins two coarse vertices, then: it leads its group
-    uint32_t* counts;         // [8] crossing edges, edges of runs left to the pair sort, coarse edges,
-                              // edges taken out for it, a partition outgrew its room
+    uint32_t* counts;         // [8] crossing edges, edges of runs left to the pair sort, -,
+                              // edges taken out for it, a partition outgrew its room, items of runs
     uint32_t* cpair;          // [2 m] coarse endpoints of every edge, cmap[eu[e]] then cmap[ev[e]]
     unsigned long long* key[2];  // [m] coarse pair of each crossing edge (radix ping-pong); key[1] follows
                                  // key[0], together the partitions' room: 2 m (hash, edge) items
@@ -369,9 +371,9 @@ struct ContractArgs {
     uint32_t sort_bits;       // low bits of the hash the sort orders by (8, 16, 24, 32; 0: by size)
 };
 size_t contract_sort_words(uint32_t m);  // words of shist
-// runs every step; mc_host_slot: 3 pinned words (crossing edges and coarse vertices
-// are read back once, to size the sort); returns a cudaError_t value
-int launch_contract(void* stream, const ContractArgs& c, uint32_t* mc_host_slot);
+// runs every step; host: 8 pinned words, the last report in them once the stream is done: [5]
+// coarse vertices, [6] error bits, [7] coarse edges; returns a cudaError_t value
+int launch_contract(void* stream, const ContractArgs& c, uint32_t* host);
 int launch_job_graph(void* exec, void* stream);
 // list path (lm_list.cu): blocks of k_top for one graph, the maps for several, and the launches
 // (rounds: 64-bit words)
@@ -404,13 +406,19 @@ struct BuildTmp {
 uint32_t build_scan_count(uint32_t m);
 uint32_t build_step(uint32_t m, uint32_t chunks);  // edges a chunk of the degree pass (whole tiles)
 // degrees, ranks, records and bucket counts of edges first .. first + count - 1 (first: whole tiles)
-int launch_build_degrees(void* stream, const uint32_t* eu, const uint32_t* ev, const float* w, uint32_t n, uint32_t m,
-                         uint32_t first, uint32_t count, const BuildTmp& t);
+int launch_build_degrees(void* stream, const uint32_t* eu, const uint32_t* ev, uint32_t n, uint32_t m, uint32_t first,
+                         uint32_t count, const BuildTmp& t);
+// with the counts' prefix in t.offs: the first ends' entries of edges first .. first + count - 1
+// and their second ends' records; then, of all, the second ends' entries
+int launch_build_fill_u(void* stream, const float* w, uint32_t n, uint32_t m, uint32_t first, uint32_t count,
+                        const uint32_t* off, uint32_t* eid, uint64_t* ent, const BuildTmp& t);
+int launch_build_fill_v(void* stream, uint32_t m, uint32_t* eid, uint64_t* ent, const BuildTmp& t);
 int launch_exclusive_scan(void* stream, const uint32_t* in, uint32_t* out, uint32_t count, uint32_t* tmp,
                           size_t tmp_words);
 size_t exclusive_scan_tmp_words(uint32_t count);
-int launch_build_fill(void* stream, uint32_t n, uint32_t m, const uint32_t* off, uint32_t* eid, uint64_t* ent,
-                      const BuildTmp& t, uint32_t* scan_tmp, size_t scan_words);
+// after them and the rows' scan: host[0] = *nrows, host[4] = err[0], host[8..11] = the tasks of each kind
+// (err[4..7]), written straight to pinned memory, and their cursors to err[8..11]
+int launch_build_counts(void* stream, uint32_t* err, const uint32_t* nrows, uint32_t* host);
 // cursors: the next place in task of each kind
 int launch_build_rows(void* stream, const uint32_t* deg, const uint32_t* rowidx_excl, const uint32_t* off,
                       uint32_t n, uint32_t nrows, uint32_t nent, uint32_t* vid0, uint32_t* rdeg0, uint32_t* roff,

@@ -1374,8 +1374,9 @@ __device__ __forceinline__ uint32_t warp_add(uint32_t* ctr, uint32_t key, bool a
 // the degrees and keeps each end's rank among its vertex's entries (what the counting
 // atomic returned), so that the fill needs no atomics of its own: an entry's place
 // is its row's offset plus its rank.  It also writes the edge records and, per tile, the
-// second ends' counts by bucket; of a host edge list, all of this runs chunk by
-// chunk while the next chunk is on its way.
+// second ends' counts by bucket.  Of a host edge list it runs chunk by chunk while
+// the next chunk is on its way; the weights come last, and k_build_fill_u runs on their
+// chunks in the same way.
 // The fill writes every edge's two adjacency entries.  Entries of the first end
 // follow the input's order (inputs listed by source vertex write them in runs);
 // the second end's would land at random rows, each a partial sector anywhere in
@@ -1391,10 +1392,9 @@ constexpr uint32_t BF_TILE = 4096, BF_T = 256, BF_NB = 256, BF_U = 4;  // BF_U e
 static_assert(BF_TILE % (BF_T * BF_U) == 0 && BF_T == BF_NB, "whole steps, a thread per bucket");
 
 __global__ void __launch_bounds__(BF_T) k_build_degrees(const uint32_t* __restrict__ eu, const uint32_t* __restrict__ ev,
-                                                        const float* __restrict__ w, uint32_t n, uint32_t m,
-                                                        uint32_t first, uint32_t shift, uint32_t tiles, uint32_t* deg,
-                                                        uint32_t* err, uint2* __restrict__ rank,
-                                                        uint64_t* __restrict__ edges, uint32_t* __restrict__ eword,
+                                                        uint32_t n, uint32_t m, uint32_t first, uint32_t shift,
+                                                        uint32_t tiles, uint32_t* deg, uint32_t* err,
+                                                        uint2* __restrict__ rank, uint64_t* __restrict__ edges,
                                                         uint32_t* __restrict__ hist) {
     __shared__ uint32_t h[BF_NB];
     h[threadIdx.x] = 0;
@@ -1402,7 +1402,7 @@ __global__ void __launch_bounds__(BF_T) k_build_degrees(const uint32_t* __restri
     const uint32_t lane = threadIdx.x & 31, tile = first / BF_TILE + blockIdx.x;
     const uint64_t t0 = (uint64_t)tile * BF_TILE;   // whole warps iterate together
     for (uint32_t j = 0; j < BF_TILE / BF_T; j += BF_U) {
-        uint32_t u[BF_U], v[BF_U], wb[BF_U];
+        uint32_t u[BF_U], v[BF_U];
         bool ok[BF_U];
 #pragma unroll
         for (uint32_t q = 0; q < BF_U; q++) {
@@ -1410,19 +1410,16 @@ __global__ void __launch_bounds__(BF_T) k_build_degrees(const uint32_t* __restri
             ok[q] = e < m;
             u[q] = ok[q] ? __ldg(eu + e) : 0u;
             v[q] = ok[q] ? __ldg(ev + e) : 0u;
-            wb[q] = ok[q] ? __float_as_uint(__ldg(w + e)) : 0u;
         }
 #pragma unroll
         for (uint32_t q = 0; q < BF_U; q++) {
             const uint64_t e = t0 + (j + q) * BF_T + threadIdx.x;
-            const bool nan = ((wb[q] & 0x7F800000u) == 0x7F800000u) && (wb[q] & 0x007FFFFFu);
-            if (ok[q] && (u[q] >= n || v[q] >= n || u[q] == v[q] || nan)) {
+            if (ok[q] && (u[q] >= n || v[q] >= n || u[q] == v[q])) {
                 atomicOr(err, 1u);
                 ok[q] = false;
             }
             if (ok[q]) {
                 edges[e] = (uint64_t)u[q] | ((uint64_t)v[q] << 32);
-                eword[e] = ord_of_bits(wb[q]);
                 atomicAdd(&h[(v[q] >> shift) & (BF_NB - 1)], 1u);
             }
         }
@@ -1443,17 +1440,19 @@ __global__ void __launch_bounds__(BF_T) k_build_degrees(const uint32_t* __restri
 }
 
 __global__ void __launch_bounds__(BF_T) k_build_fill_u(const uint64_t* __restrict__ edges,
-                                                       const uint32_t* __restrict__ eword,
+                                                       const float* __restrict__ w, uint32_t* __restrict__ eword,
                                                        const uint2* __restrict__ rank, const uint32_t* __restrict__ off,
-                                                       uint32_t m, uint32_t shift, uint32_t tiles,
-                                                       const uint32_t* __restrict__ offs, uint32_t* __restrict__ eid,
+                                                       uint32_t first, uint32_t m_all, uint32_t m, uint32_t shift,
+                                                       uint32_t tiles, const uint32_t* __restrict__ offs,
+                                                       uint32_t* __restrict__ eid,
                                                        uint64_t* __restrict__ ent, uint4* __restrict__ vrec,
                                                        uint32_t* err) {
     __shared__ uint32_t gs[BF_NB], cnt[BF_NB];
-    gs[threadIdx.x] = offs[threadIdx.x * tiles + blockIdx.x];
+    const uint32_t tile = first / BF_TILE + blockIdx.x;
+    gs[threadIdx.x] = offs[threadIdx.x * tiles + tile];
     cnt[threadIdx.x] = 0;
     __syncthreads();
-    const uint64_t t0 = (uint64_t)blockIdx.x * BF_TILE;
+    const uint64_t t0 = (uint64_t)tile * BF_TILE;
     for (uint32_t j = 0; j < BF_TILE / BF_T; j += BF_U) {
         uint64_t rec[BF_U];
         uint32_t ow[BF_U], pu[BF_U], pv[BF_U];
@@ -1462,7 +1461,7 @@ __global__ void __launch_bounds__(BF_T) k_build_fill_u(const uint64_t* __restric
         for (uint32_t q = 0; q < BF_U; q++) {
             const uint64_t e = t0 + (j + q) * BF_T + threadIdx.x;
             rec[q] = e < m ? __ldg(edges + e) : 0ull;
-            ow[q] = e < m ? __ldg(eword + e) : 0u;
+            ow[q] = e < m ? __float_as_uint(__ldg(w + e)) : 0u;
             r[q] = e < m ? __ldg(rank + e) : make_uint2(0, 0);
         }
 #pragma unroll
@@ -1475,9 +1474,11 @@ __global__ void __launch_bounds__(BF_T) k_build_fill_u(const uint64_t* __restric
             const uint64_t e = t0 + (j + q) * BF_T + threadIdx.x;
             if (e >= m) continue;
             const uint32_t u = (uint32_t)rec[q], v = (uint32_t)(rec[q] >> 32);
+            if ((ow[q] & 0x7F800000u) == 0x7F800000u && (ow[q] & 0x007FFFFFu)) atomicOr(err, 1u);  // NaN
+            eword[e] = ow[q] = ord_of_bits(ow[q]);
             // offsets and ranks come from the same counts, so every place is below 2m; one
             // that is not is reported, not written
-            if (pu[q] >= 2 * m || pv[q] >= 2 * m) {
+            if (pu[q] >= 2 * m_all || pv[q] >= 2 * m_all) {
                 atomicOr(err, 2u);
                 continue;
             }
@@ -1485,7 +1486,7 @@ __global__ void __launch_bounds__(BF_T) k_build_fill_u(const uint64_t* __restric
             eid[pu[q]] = (uint32_t)e;
             const uint32_t b = (v >> shift) & (BF_NB - 1);
             const uint32_t p = gs[b] + atomicAdd(&cnt[b], 1u);
-            if (p < m) vrec[p] = make_uint4(pv[q], u, (uint32_t)e, ow[q]);
+            if (p < m_all) vrec[p] = make_uint4(pv[q], u, (uint32_t)e, ow[q]);
             else atomicOr(err, 2u);
         }
     }
@@ -1529,6 +1530,21 @@ __global__ void k_nonzero_flags(const uint32_t* deg, uint32_t n, uint32_t* flags
     }
     __syncthreads();
     if (threadIdx.x < 4 && s[threadIdx.x]) atomicAdd(&counts[threadIdx.x], s[threadIdx.x]);
+}
+
+// What the host waits for, written to its memory by the kernel: a copy would queue in the
+// copy engine behind the weights that are still being uploaded (R-MAT scale 21: 3.12 ms
+// from host arrays, with this 2.69).  Each kind's tasks follow the previous one's.
+__global__ void k_build_counts(uint32_t* err, const uint32_t* nrows, uint32_t* host) {
+    host[0] = *nrows;
+    host[4] = err[0];
+    uint32_t at = 0;
+    for (int k = 0; k < 4; k++) {
+        const uint32_t c = err[4 + k];
+        host[8 + k] = c;
+        err[8 + k] = at;
+        at += c;
+    }
 }
 
 // The compact row arrays, and the list path's tasks, each kind from its cursor on; a
@@ -1881,28 +1897,35 @@ uint32_t build_scan_count(uint32_t m) { return BF_NB * build_tiles(m); }
 uint32_t build_step(uint32_t m, uint32_t chunks) {
     return build_tiles((uint32_t)(((uint64_t)m + chunks - 1) / chunks)) * BF_TILE;
 }
-int launch_build_degrees(void* stream, const uint32_t* eu, const uint32_t* ev, const float* w, uint32_t n, uint32_t m,
-                         uint32_t first, uint32_t count, const BuildTmp& t) {
+int launch_build_degrees(void* stream, const uint32_t* eu, const uint32_t* ev, uint32_t n, uint32_t m, uint32_t first,
+                         uint32_t count, const BuildTmp& t) {
     if (count == 0) return 0;
     if (first % BF_TILE) return (int)cudaErrorInvalidValue;
     // (the arrays are those of the whole list; edges first .. first + count - 1 are there)
     k_build_degrees<<<build_tiles(count), BF_T, 0, (cudaStream_t)stream>>>(
-        eu, ev, w, n, first + count, first, build_shift(n), build_tiles(m), t.deg, t.err, t.rank, t.edges, t.eword, t.hist);
+        eu, ev, n, first + count, first, build_shift(n), build_tiles(m), t.deg, t.err, t.rank, t.edges, t.hist);
     return (int)cudaGetLastError();
 }
-int launch_build_fill(void* stream, uint32_t n, uint32_t m, const uint32_t* off, uint32_t* eid, uint64_t* ent,
-                      const BuildTmp& t, uint32_t* scan_tmp, size_t scan_words) {
-    cudaStream_t s = (cudaStream_t)stream;
-    if (m == 0) return 0;
-    const uint32_t tiles = build_tiles(m);
-    if (int r = launch_exclusive_scan(stream, t.hist, t.offs, BF_NB * tiles, scan_tmp, scan_words)) return r;
-    k_build_fill_u<<<tiles, BF_T, 0, s>>>(t.edges, t.eword, t.rank, off, m, build_shift(n), tiles, t.offs, eid, ent,
-                                          t.vrec, t.err);
-    k_build_fill_v<<<(uint32_t)(((uint64_t)m + BF_T * BF_U - 1) / (BF_T * BF_U)), BF_T, 0, s>>>(t.vrec, m, eid, ent);
+int launch_build_fill_u(void* stream, const float* w, uint32_t n, uint32_t m, uint32_t first, uint32_t count,
+                        const uint32_t* off, uint32_t* eid, uint64_t* ent, const BuildTmp& t) {
+    if (count == 0) return 0;
+    if (first % BF_TILE) return (int)cudaErrorInvalidValue;
+    k_build_fill_u<<<build_tiles(count), BF_T, 0, (cudaStream_t)stream>>>(
+        t.edges, w, t.eword, t.rank, off, first, m, first + count, build_shift(n), build_tiles(m), t.offs, eid, ent,
+        t.vrec, t.err);
+    return (int)cudaGetLastError();
+}
+int launch_build_fill_v(void* stream, uint32_t m, uint32_t* eid, uint64_t* ent, const BuildTmp& t) {
+    k_build_fill_v<<<(uint32_t)(((uint64_t)m + BF_T * BF_U - 1) / (BF_T * BF_U)), BF_T, 0, (cudaStream_t)stream>>>(
+        t.vrec, m, eid, ent);
     return (int)cudaGetLastError();
 }
 int launch_nonzero_flags(void* stream, const uint32_t* deg, uint32_t n, uint32_t* flags, uint32_t* counts) {
     k_nonzero_flags<<<grid_for(n, 256), 256, 0, (cudaStream_t)stream>>>(deg, n, flags, counts);
+    return (int)cudaGetLastError();
+}
+int launch_build_counts(void* stream, uint32_t* err, const uint32_t* nrows, uint32_t* host) {
+    k_build_counts<<<1, 1, 0, (cudaStream_t)stream>>>(err, nrows, host);
     return (int)cudaGetLastError();
 }
 int launch_build_rows(void* stream, const uint32_t* deg, const uint32_t* rowidx_excl, const uint32_t* off,

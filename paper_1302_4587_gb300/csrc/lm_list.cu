@@ -1136,7 +1136,8 @@ __global__ void __launch_bounds__(LT, LMINB) k_live(const __grid_constant__ List
     if (tid == 0) {
         if (left) atomicAdd(&st->left, left);
         __threadfence();
-        if (atomicAdd(&st->exit_v, 1u) == gridDim.x - 1) {
+        S.stop = atomicAdd(&st->exit_v, 1u) == gridDim.x - 1;
+        if (S.stop) {
             __threadfence();
             st->exit_v = 0;
             st->task[0] = 0;
@@ -1148,6 +1149,8 @@ __global__ void __launch_bounds__(LT, LMINB) k_live(const __grid_constant__ List
             __threadfence();
         }
     }
+    __syncthreads();
+    if (S.stop && a.host) state_to_host(a.host, st, LT);
 }
 
 // ---------------------------------------------------------------- per-round counts

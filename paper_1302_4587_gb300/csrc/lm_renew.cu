@@ -471,11 +471,14 @@ __global__ void __launch_bounds__(RT, RMINB) k_renew(const __grid_constant__ Ren
             blocks = 1;
         }
     }
-    if (COUNT && blockIdx.x == 0) {
-        __syncthreads();
+    if (blockIdx.x) return;
+    __syncthreads();
+    if (COUNT)
         for (uint32_t i = tid; i < 64; i += RT) st->ring_m[i] /= 2;   // both ends counted every edge
-    }
-    if (blockIdx.x == 0 && tid == 0) st->done = 1;
+    if (tid == 0) st->done = 1;
+    __threadfence();
+    __syncthreads();
+    if (a.host) state_to_host(a.host, st, RT);
 }
 
 }  // namespace
