@@ -1387,7 +1387,8 @@ __device__ __forceinline__ uint32_t warp_add(uint32_t* ctr, uint32_t key, bool a
 // any time lie in a window of the arrays that L2 holds.
 // Bound by scattered stores of single entries (two sectors each).  R-MAT scale 21,
 // 31.8M edges: with a second round of atomics in the fill, degrees 330, buckets' counts
-// 61, fill 511 + 632 us; with ranks 523 (under the upload of a host list) and 470 + 520.
+// 61, fill 511 + 632 us; with ranks 430 (under the upload of a host list's ends), 505
+// (under that of its weights) and 440.
 constexpr uint32_t BF_TILE = 4096, BF_T = 256, BF_NB = 256, BF_U = 4;  // BF_U edges a thread and step
 static_assert(BF_TILE % (BF_T * BF_U) == 0 && BF_T == BF_NB, "whole steps, a thread per bucket");
 
@@ -1492,19 +1493,18 @@ __global__ void __launch_bounds__(BF_T) k_build_fill_u(const uint64_t* __restric
     }
 }
 
+// A record a thread: what counts is that the rows written at any time lie close together
+// (31.8M records: four a thread 534 us, one 440; persistent blocks 720; blocks spread over
+// 4 or 64 places of the array 530 and 680).  Each of the two stores is a sector of its own, about
+// 120 G a second.
 __global__ void __launch_bounds__(BF_T) k_build_fill_v(const uint4* __restrict__ vrec, uint32_t m,
                                                        uint32_t* __restrict__ eid, uint64_t* __restrict__ ent) {
-    const uint64_t i = (uint64_t)blockIdx.x * (BF_T * BF_U) + threadIdx.x;
-    uint4 r[BF_U];
-#pragma unroll
-    for (uint32_t q = 0; q < BF_U; q++)
-        if (i + q * BF_T < m) r[q] = __ldcs(vrec + i + q * BF_T);
-#pragma unroll
-    for (uint32_t q = 0; q < BF_U; q++)
-        if (i + q * BF_T < m && r[q].x < 2 * m) {
-            ent[r[q].x] = ((uint64_t)r[q].w << 32) | r[q].y;
-            eid[r[q].x] = r[q].z;
-        }
+    const uint64_t i = (uint64_t)blockIdx.x * BF_T + threadIdx.x;
+    if (i >= m) return;
+    const uint4 r = __ldg(vrec + i);
+    if (r.x >= 2 * m) return;
+    ent[r.x] = ((uint64_t)r.w << 32) | r.y;
+    eid[r.x] = r.z;
 }
 // kind of task a row of d entries makes on the list path (4: none)
 __device__ __forceinline__ uint32_t task_kind(uint32_t d) {
@@ -1916,8 +1916,7 @@ int launch_build_fill_u(void* stream, const float* w, uint32_t n, uint32_t m, ui
     return (int)cudaGetLastError();
 }
 int launch_build_fill_v(void* stream, uint32_t m, uint32_t* eid, uint64_t* ent, const BuildTmp& t) {
-    k_build_fill_v<<<(uint32_t)(((uint64_t)m + BF_T * BF_U - 1) / (BF_T * BF_U)), BF_T, 0, (cudaStream_t)stream>>>(
-        t.vrec, m, eid, ent);
+    k_build_fill_v<<<(uint32_t)(((uint64_t)m + BF_T - 1) / BF_T), BF_T, 0, (cudaStream_t)stream>>>(t.vrec, m, eid, ent);
     return (int)cudaGetLastError();
 }
 int launch_nonzero_flags(void* stream, const uint32_t* deg, uint32_t n, uint32_t* flags, uint32_t* counts) {
