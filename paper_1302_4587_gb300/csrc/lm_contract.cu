@@ -27,7 +27,7 @@
 // low bits; edges inside a pair have the key 0xFFFFFFFF, and no pair's hash ends in the
 // byte 0xFF, so that they end up last) brings each pair's edges into one bucket, still in
 // input order, and k_c_buckets finds the runs.
-// R-MAT scale 22 (64M edges): sort 2.18 ms, partitions 1.42 (part 525, groups 327, walk
+// R-MAT scale 22 (64M edges): sort 2.18 ms, partitions 1.40 (part 525, groups 327, walk
 // 125, emit 266 us, the rest map, scans and a host round trip).
 #include <cstdint>
 #include <type_traits>
@@ -203,27 +203,28 @@ __global__ void __launch_bounds__(CT) k_c_keys(const uint32_t* __restrict__ eu, 
 // R-MAT scale 21, 31.8M edges: 268 us, of which the gathers of cmap 92, the items' stores
 // 26, cpair 33, the rest the phases in shared memory.  Three blocks an SM (spills), 8 or
 // 24 edges a thread, 256 or 1024 threads: 3 to 15% slower over all.
-constexpr uint32_t PT_T = 512, PT_E = 16, PT_TILE = PT_E * PT_T, PT_MAX = 1024, PT_D = PT_MAX / PT_T;
+constexpr uint32_t PT_T = 512, PT_E = 16, PT_TILE = PT_E * PT_T;
+template <uint32_t D>  // partitions a thread: at most D PT_T
 struct PtSmem {
     uint32_t key[PT_TILE];
     uint16_t edge[PT_TILE];  // its place in the tile
-    uint32_t cnt[PT_MAX];   // items of each partition, then where its run starts in it
-    uint32_t gofs[PT_MAX];  // the run's place in the partition's room, minus that
+    uint32_t cnt[D * PT_T];   // items of each partition, then where its run starts in it
+    uint32_t gofs[D * PT_T];  // the run's place in the partition's room, minus that
     uint32_t ws[PT_T / 32];
 };
-static_assert(PT_MAX % PT_T == 0 && PT_E % 8 == 0 && PT_TILE <= 65536, "PT_D partitions and PT_E edges a thread, 16-bit places");
+static_assert(PT_E % 8 == 0 && PT_TILE <= 65536, "eight edges a step, 16-bit places");
 
-template <bool VEC>
+template <bool VEC, uint32_t D>
 __global__ void __launch_bounds__(PT_T, 2)
     k_c_part(const uint32_t* __restrict__ eu, const uint32_t* __restrict__ ev, uint32_t m, uint32_t n,
              const uint32_t* __restrict__ cmap, uint32_t pb, uint32_t cap, uint32_t* __restrict__ gcur,
              uint2* __restrict__ items, uint32_t* __restrict__ cpair, uint32_t* __restrict__ cross,
              uint32_t* __restrict__ counts, uint32_t* __restrict__ err) {
     extern __shared__ __align__(16) unsigned char pt_raw[];
-    PtSmem& S = *reinterpret_cast<PtSmem*>(pt_raw);
+    PtSmem<D>& S = *reinterpret_cast<PtSmem<D>*>(pt_raw);
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t dsh = 32 - pb;
-    for (uint32_t i = tid; i < PT_MAX; i += PT_T) S.cnt[i] = 0;
+    for (uint32_t i = tid; i < D * PT_T; i += PT_T) S.cnt[i] = 0;
     __syncthreads();
     uint32_t mine = 0, key[PT_E], rk[PT_E / 2];
 #pragma unroll
@@ -287,10 +288,10 @@ __global__ void __launch_bounds__(PT_T, 2)
     mine = __reduce_add_sync(0xFFFFFFFFu, mine);
     if (lane == 0 && mine) atomicAdd(&counts[0], mine);
     __syncthreads();
-    // thread t: partitions PT_D t .. PT_D t + PT_D - 1
-    uint32_t c[PT_D], x = 0;
+    // thread t: partitions D t .. D t + D - 1
+    uint32_t c[D], x = 0;
 #pragma unroll
-    for (uint32_t i = 0; i < PT_D; i++) x += c[i] = S.cnt[PT_D * tid + i];
+    for (uint32_t i = 0; i < D; i++) x += c[i] = S.cnt[D * tid + i];
     const uint32_t sum = x;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -305,9 +306,9 @@ __global__ void __launch_bounds__(PT_T, 2)
         total += S.ws[w];
     }
 #pragma unroll
-    for (uint32_t i = 0; i < PT_D; i++) {
-        if (c[i]) S.gofs[PT_D * tid + i] = atomicAdd(&gcur[PT_D * tid + i], c[i]) - start;
-        S.cnt[PT_D * tid + i] = start;
+    for (uint32_t i = 0; i < D; i++) {
+        if (c[i]) S.gofs[D * tid + i] = atomicAdd(&gcur[D * tid + i], c[i]) - start;
+        S.cnt[D * tid + i] = start;
         start += c[i];
     }
     __syncthreads();
@@ -1129,16 +1130,19 @@ uint32_t bits_for(uint32_t x) {  // bits to write 0 .. x
 }  // namespace
 
 // log2 of the partitions, or 0: the list is sorted by the hash.  About 8192 edges to a
-// partition as long as there are at most PT_MAX (more would be written in runs of less
-// than 8 items: R-MAT scale 22 1.54 ms at 2048 partitions, 1.42 at 1024).  Partitions beat
-// the sort from the smallest lists (fewer launches: 1,000 edges 99 us against 122, 1M
-// edges 142 against 210) to the largest measured (R-MAT scale 24, 232M edges, 9.8 ms
-// against 10.0), where three quarters of the slots are shared and the gain ends; so the
-// line lies at 2^28 edges.  A caller that sets the sort's width gets the sort.
+// partition up to 1024 partitions, which are written in runs of 8 items; then as many as
+// a bitmap of 8 slots an item allows (R-MAT scale 22, 64M edges: 1.42 ms with 1024, 1.54
+// with 2048), and from there up to 4096 (scale 23, 129M: 4.34 ms with 1024, 3.19 with
+// 2048; 300M: 10.5 with 2048, 8.4 with 4096).  Partitions beat the sort from the
+// smallest lists (fewer launches: 1,000 edges 99 us against 122, 1M edges 142 against
+// 210) to the largest measured (590M edges 23.8 ms against 29.4), with a gain that shrinks
+// as the slots are shared; so the line lies at 2^30 edges.  A caller that sets the
+// sort's width gets the sort.
 static uint32_t contract_part_bits(uint32_t m, uint32_t sort_bits) {
-    if (sort_bits || m > 1u << 28) return 0;
+    if (sort_bits || m > 1u << 30) return 0;
     uint32_t b = 1;
-    while ((2u << b) <= PT_MAX && (m >> b) > 8192) b++;
+    while (b < 10 && (m >> b) > 8192) b++;
+    while (b < 12 && (m >> b) > 1u << (GpSmem<1>::GP_BITS - 3)) b++;
     return b;
 }
 
@@ -1210,21 +1214,28 @@ int launch_contract(void* stream, const ContractArgs& c, uint32_t* host) {
     // 1. partitions, where their rule holds: the crossing bits become the leader bits, every
     //    group member but the first cleared
     if (const uint32_t pb = contract_part_bits(c.m, c.sort_bits)) {
-        const uint32_t cap = (uint32_t)(2ull * c.m >> pb);  // twice the average: key[0] and key[1], which follows it
+        // twice the average (key[0] and key[1], which follows it), less what makes the rooms' distance
+        // an odd number of cache lines (R-MAT scale 22 1.42 and 1.40 ms)
+        uint32_t cap = (uint32_t)(2ull * c.m >> pb);
+        if (cap > 4096) cap = (((cap >> 4) - 1) | 1u) << 4;
         uint32_t gb = 10;
         while (gb < GpSmem<1>::GP_BITS && (1ull << gb) < (8ull * c.m >> pb)) gb++;
         uint2* items = reinterpret_cast<uint2*>(c.key[0]);
-        auto part = vec ? k_c_part<true> : k_c_part<false>;
+        const int d = pb > 10 ? pb - 9 : 1;   // (log2 of) partitions a thread
+        auto part = d == 1 ? (vec ? k_c_part<true, 2> : k_c_part<false, 2>)
+                  : d == 2 ? (vec ? k_c_part<true, 4> : k_c_part<false, 4>)
+                           : (vec ? k_c_part<true, 8> : k_c_part<false, 8>);
+        const size_t psmem = d == 1 ? sizeof(PtSmem<2>) : d == 2 ? sizeof(PtSmem<4>) : sizeof(PtSmem<8>);
         const int big = gb > GpSmem<0>::GP_BITS;
         auto groups = big ? k_c_groups<1> : k_c_groups<0>;
         const size_t gsmem = big ? sizeof(GpSmem<1>) : sizeof(GpSmem<0>);
-        if ((e = cudaFuncSetAttribute(part, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PtSmem))) ||
+        if ((e = cudaFuncSetAttribute(part, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psmem)) ||
             (e = cudaFuncSetAttribute(groups, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsmem)) ||
             (e = cudaMemsetAsync(c.counts, 0, 8 * sizeof(uint32_t), s)) ||
             (e = cudaMemsetAsync(c.shist, 0, sizeof(uint32_t) << pb, s)) ||
             (e = cudaMemsetAsync(c.multi, 0, bitmap, s)) || (e = cudaMemsetAsync(ofl, 0, bitmap, s)))
             return (int)e;
-        part<<<(uint32_t)(((uint64_t)c.m + PT_TILE - 1) / PT_TILE), PT_T, sizeof(PtSmem), s>>>(
+        part<<<(uint32_t)(((uint64_t)c.m + PT_TILE - 1) / PT_TILE), PT_T, psmem, s>>>(
             c.eu, c.ev, c.m, c.n, c.cmap, pb, cap, c.shist, items, c.cpair, c.cross, c.counts, c.err);
         groups<<<1u << pb, 512u << big, gsmem, s>>>(items, c.shist, cap, pb, gb, c.val[0], ofl, c.counts);
         k_c_walk<<<egrid, CT, 0, s>>>(c.val[0], c.cpair, c.w, c.cross, c.multi, c.gref, ofl, c.counts);

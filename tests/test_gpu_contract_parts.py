@@ -54,3 +54,29 @@ def test_groups_beyond_a_partition(lmc, kind):
     eu, ev = eu[p], ev[p]
     mate = np.full(n, NIL, np.uint32)
     _same(_contract(lmc, n, eu, ev, w, mate), oracle.contract(n, eu, ev, w, mate))
+
+
+@pytest.mark.parametrize("m", [66_000_001, 70_000_000, 135_000_003])
+def test_many_partitions(lmc, m):
+    # 1024, 2048 and 4096 partitions, against the sort (which the smaller sizes tie to the
+    # oracle); a twentieth of the edges repeated, in the other orientation
+    torch, lm = lmc.torch, lmc.lm
+    n = 3_000_000
+    gen = torch.Generator(device="cuda").manual_seed(m)
+    eu = torch.randint(0, n, (m,), generator=gen, device="cuda", dtype=torch.int32)
+    ev = torch.randint(0, n, (m,), generator=gen, device="cuda", dtype=torch.int32)
+    ev = torch.where(ev == eu, (ev + 1) % n, ev)
+    k = m // 20
+    eu[-k:], ev[-k:] = ev[:k].clone(), eu[:k].clone()
+    w = torch.rand(m, generator=gen, device="cuda")
+    mate = torch.arange(n, device="cuda", dtype=torch.int32) ^ 1   # pairs (2 i, 2 i + 1)
+    keep = lm.lm_get_tuning(lmc.ctx)
+    tune = {x: keep[x] for x in ("rmax", "chunk", "sweep_ctas_per_sm", "vertex_ctas_per_sm", "batch")}
+    got = lm.lm_contract(lmc.ctx, n, eu, ev, w, mate)
+    try:
+        lm.lm_set_tuning(lmc.ctx, **tune, contract_bits=16)
+        want = lm.lm_contract(lmc.ctx, n, eu, ev, w, mate)
+    finally:
+        lm.lm_set_tuning(lmc.ctx, **tune, contract_bits=keep["contract_bits"])
+    for a, b in zip(got, want):
+        assert torch.equal(a, b)
