@@ -40,9 +40,9 @@ METRIC_COARSEN = "input edges/s coarsened (8 levels of match + contract)"
 METRIC_SWEEP = "speedup of lm_match over the sequential local max (max over the sweep)"
 
 # dram__bytes_read.sum + dram__bytes_write.sum per match of a kernel's launches, from an ncu
-# capture on R-MAT scale 21 scaled by the entries processed (R-MAT 23 is too large to capture
-# with several metrics), keyed by (workload, kernel), for kernels whose current code was captured
-TRAFFIC = {("rmat23", "k_sweep"): 5812000000, ("rmat23", "k_round0"): 3257000000}
+# capture on R-MAT scale 21 scaled by the edges (x4.071; R-MAT 23 is too large to capture with
+# several metrics), keyed by (workload, kernel), for kernels whose current code was captured
+TRAFFIC = {("rmat23", "k_top"): 2721000000, ("rmat23", "k_live"): 933000000}
 
 
 def _peaks():
@@ -160,30 +160,26 @@ def make_workload(name: str):
     raise ValueError(name)
 
 
-def sweep_model_bytes(st: dict, nsweeps: int | None = None) -> int:
-    """Algorithmic HBM bytes of the k_sweep launches of one match (round-0
-    compaction from the input arrays and every later round up to the one-CTA
-    tail: the sweep of round r is launch r), from the per-round live counts: a
-    sweep over E_r entries / R_r rows reads 16 B per entry (12 B entry + 4 B
-    neighbour-state gather), writes 12 B per surviving entry, reads 8 B per row
-    and writes 12 B per row of the next round."""
-    rm, rn = st["round_m"], st["round_n"]
-    R = len(rm) if nsweeps is None else min(len(rm), nsweeps)
-    E = [2 * x for x in rm] + [0]
-    N = list(rn) + [0]
-    b = 0
-    for r in range(R):
-        b += 16 * E[r] + 12 * E[r + 1] + 8 * N[r] + 12 * N[r + 1]
-    return b
-
-
-def cand_model_bytes(st: dict) -> int:
-    """Algorithmic HBM bytes of the round-0 candidate kernel: 12 B per input
-    entry (8 B weight/edge word + 4 B neighbour) and 8 B per row (row vertex
-    read, candidate written)."""
+def top_model_bytes(st: dict, n: int) -> int:
+    """Algorithmic HBM bytes of k_top (every row's heaviest neighbours from one pass):
+    8 B per input entry, per row 8 B of tables read and 20 B of candidate and list
+    written, per vertex 4 B of result cleared."""
     if not st["round_m"]:
         return 0
-    return 12 * 2 * st["round_m"][0] + 8 * st["round_n"][0]
+    return 8 * 2 * st["round_m"][0] + 28 * st["round_n"][0] + 4 * n
+
+
+def live_model_bytes(st: dict) -> int:
+    """Algorithmic HBM bytes of k_live: its rows looked at once a round (the row's id,
+    word and list and its candidate's word, 28 B) and 8 B per matched vertex.  Rows polled
+    more or less often, and the entries of rows scanned again, are not modelled."""
+    return sum(28 * x for x in st["round_n"]) + 16 * st["matched"]
+
+
+def renew_model_bytes(st: dict) -> int:
+    """Algorithmic HBM bytes of k_renew: per live entry and round 12 B (entry word, edge
+    index), per live row 20 B (tables, candidate written, its candidate's read)."""
+    return sum(24 * x for x in st["round_m"]) + sum(20 * x for x in st["round_n"])
 
 
 def path_model_bytes(st: dict) -> int:
@@ -231,10 +227,8 @@ def run_lm(args, ws, rank, local):
     # launch parameters picked by the library's autotuner on this graph (untimed; the
     # edge-centric path has none)
     tuning = None if edge else lm.lm_autotune(ctx, [h], [seed], [mate])
-    launches = 0
     for _ in range(max(args.warmup, 3)):
         _, st = lm.lm_match(ctx, h, seed, mate, stats=True)
-    launches_per_step = st["launches"]
     torch.cuda.synchronize()
     _barrier(ws)
     e0 = torch.cuda.Event(enable_timing=True)
@@ -244,7 +238,6 @@ def run_lm(args, ws, rank, local):
         e0.record(stream)
         for _ in range(args.steps):
             lm.lm_match(ctx, h, seed, mate)
-            launches += launches_per_step
         e1.record(stream)
         torch.cuda.synchronize()
     _barrier(ws)
@@ -267,36 +260,45 @@ def run_lm(args, ws, rank, local):
             total_ms.append(pst["total_ms"])
     lm.lm_destroy(pctx)
     med = {k: statistics.median(v) for k, v in kms.items()}
+    # launches of the timed matches, which want no statistics: the edge-centric path's are the
+    # same with them, of the others only k_top and k_live (or k_renew)
+    per_step = (st["launches"] if edge else
+                pst["kernel_launches"][lm.LM_K_CAND] + pst["kernel_launches"][lm.LM_K_SWEEP])
+    launches = per_step * args.steps
     peak, peak_kind = _peaks()
-    bytes_sweep = sweep_model_bytes(pst, pst["kernel_launches"][lm.LM_K_SWEEP])
-    bytes_cand = cand_model_bytes(pst)
-    sw_ms, cd_ms = med[lm.LM_K_SWEEP], med[lm.LM_K_CAND]
     gbs = lambda b, ms: b / (ms * 1e-3) / 1e9 if ms > 0 else 0.0
-    names = {lm.LM_K_INIT: "k_init", lm.LM_K_SWEEP: "k_sweep", lm.LM_K_VERTEX: "k_vertex",
-             lm.LM_K_CAND: "k_round0", lm.LM_K_OTHER: "other (k_round0_cut, k_loop_check)", lm.LM_K_TAIL: "k_tail"}
+    unused = lambda kind: f"(kind {kind}, not on this path)"
     if edge:
         names = {lm.LM_K_INIT: "k_init", lm.LM_K_SWEEP: "k_ec_compact", lm.LM_K_VERTEX: "k_ec_match",
-                 lm.LM_K_CAND: "k_ec_offer", lm.LM_K_OTHER: "k_ec_close", lm.LM_K_TAIL: "(none)"}
+                 lm.LM_K_CAND: "k_ec_offer", lm.LM_K_OTHER: "k_ec_close", lm.LM_K_TAIL: unused(lm.LM_K_TAIL)}
+        models = {}
+    elif order:
+        names = {lm.LM_K_SWEEP: "k_renew"}
+        models = {"k_renew": (lm.LM_K_SWEEP, renew_model_bytes(pst))}
+    else:
+        # (the profiled matches want the rounds' counts: k_live with 64-bit words, and
+        # k_round_bytes + k_round_counts, which the timed matches do not run)
+        names = {lm.LM_K_CAND: "k_top", lm.LM_K_SWEEP: "k_live",
+                 lm.LM_K_OTHER: "k_round_bytes + k_round_counts (statistics only)"}
+        models = {"k_top": (lm.LM_K_CAND, top_model_bytes(pst, g.n)),
+                  "k_live": (lm.LM_K_SWEEP, live_model_bytes(pst))}
+    names = {k: names.get(k, unused(k)) for k in range(lm.LM_K_COUNT)}
     # per-kernel rooflines (algorithmic bytes per launch set / their CUDA-event time); the
     # line's `roofline` is the one of the kernel with the most time
-    per_kernel = {
-        "k_sweep": {"bytes_per_match": bytes_sweep, "ms_per_match": sw_ms,
-                    "launches_per_match": pst["kernel_launches"][lm.LM_K_SWEEP]},
-        "k_round0": {"bytes_per_match": bytes_cand, "ms_per_match": cd_ms, "launches_per_match": 1},
-    }
+    per_kernel = {name: {"bytes_per_match": by, "ms_per_match": med[kind],
+                         "launches_per_match": pst["kernel_launches"][kind]}
+                  for name, (kind, by) in models.items()}
     for kname, d in per_kernel.items():
         d["achieved"] = gbs(d["bytes_per_match"], d["ms_per_match"])
         d["frac"] = d["achieved"] / peak
         d["traffic"] = TRAFFIC.get((args.workload, kname)) if not order else None
-    top = max(per_kernel, key=lambda k: per_kernel[k]["ms_per_match"])
-    achieved = per_kernel[top]["achieved"]
-    cand_achieved = per_kernel["k_round0"]["achieved"]
+    top = max(per_kernel, key=lambda k: per_kernel[k]["ms_per_match"]) if per_kernel else None
+    achieved = per_kernel[top]["achieved"] if top else 0.0
     kernels = {names[k]: {"ms_per_match": med[k], "launches_per_match": pst["kernel_launches"][k]}
                for k in range(lm.LM_K_COUNT)}
     # the whole match (every kernel, the timed step) against two byte counts: the
-    # bytes this design moves (the input read twice in round 0: candidates, then
-    # compaction) and the hot-path model's (input read once per round)
-    design_bytes = bytes_cand + bytes_sweep
+    # kernels' modelled bytes and the hot-path model's (live entries read once per round)
+    design_bytes = sum(by for _, by in models.values())
     model_bytes = path_model_bytes(pst)
     whole = {"ms_per_match": ms_max, "peak": peak, "peak_kind": peak_kind, "unit": "GB/s",
              "bytes_design": design_bytes,
@@ -305,8 +307,7 @@ def run_lm(args, ws, rank, local):
              "bytes_model": model_bytes,
              "achieved_model": model_bytes / (ms_max * 1e-3) / 1e9,
              "frac_model": model_bytes / (ms_max * 1e-3) / 1e9 / peak,
-             "bytes": "design: k_round0 (12 B per input entry + 8 B per row) + every k_sweep launch "
-                      "(16 B per live entry + 12 B per surviving entry + 8 B per row + 12 B per next row); "
+             "bytes": "design: the modelled bytes of roofline_per_kernel, summed; "
                       "model: sum_r 16*2m_r + 12*2m_(r+1) + 40*n_r",
              "round_m": pst["round_m"], "round_n": pst["round_n"]} if not edge else None
     bytes_ec = edge_model_bytes(pst, g.m) if edge else 0
@@ -691,7 +692,9 @@ def run_contract(args, ws, rank, local):
             # two hash passes (16 bits for about 1900 edges a bucket) of 4 and 5 (counts but in the
             # first, scan 3, scatter), buckets 1, leader counts 1 + scan 3, emit 1 (no run here needs
             # the pair sort)
-            "clocks": clk.summary(), "gpu_launches": 21 * args.steps}
+            "clocks": clk.summary(), # (representatives, map and 3 launches of scan, partitions, groups, walk, leaders with 3 of
+            # scan, emit, 2 reports; the pair sort's, if any, not counted)
+            "gpu_launches": 15 * args.steps}
 
 
 def run_coarsen(args, ws, rank, local):

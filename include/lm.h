@@ -88,13 +88,19 @@ typedef struct {
 } lm_config;
 
 #define LM_STATS_ROUNDS 64
-/* kernel kinds (index into the per-kind arrays of lm_stats) */
-#define LM_K_INIT    0   /* reset of mate / candidate / deletion state */
-#define LM_K_SWEEP   1   /* k_sweep: deletion + compaction + next candidates over live rows */
-#define LM_K_VERTEX  2   /* k_vertex: mutual-choice match over live rows + task lists */
-#define LM_K_CAND    3   /* k_round0: round-0 candidates over the input arrays in tiles */
-#define LM_K_OTHER   4   /* cut rows of round 0, loop checks, result conversion, batch set-up */
-#define LM_K_TAIL    5   /* k_tail: the last rounds (few live entries) in one CTA, no launch per round */
+/* kernel kinds (index into the per-kind arrays of lm_stats): of lm_match and lm_batch_match by the
+ * row lists (the default; in brackets the round-by-round path, which batches under LM_F_RENEW and
+ * graphs of 2^31 vertices and more take, and the edge-centric one) */
+#define LM_K_INIT    0   /* - [k_init: reset of mate / candidate / deletion state] */
+#define LM_K_SWEEP   1   /* k_live: all live rows until none is left; one graph under LM_F_RENEW:
+                            k_renew, the whole job [k_sweep: deletion + compaction + next candidates;
+                            k_ec_compact] */
+#define LM_K_VERTEX  2   /* - [k_vertex: mutual-choice match + task lists; k_ec_match] */
+#define LM_K_CAND    3   /* k_top: every row's heaviest neighbours [k_round0: round-0 candidates in
+                            tiles; k_ec_offer] */
+#define LM_K_OTHER   4   /* per-round counts for lm_stats, batch tables [cut rows of round 0, loop
+                            checks, result conversion, batch set-up; k_ec_close] */
+#define LM_K_TAIL    5   /* - [k_tail: the last rounds in one CTA, no launch per round] */
 #define LM_K_COUNT   6
 
 typedef struct {
@@ -212,15 +218,16 @@ int  lm_set_limits(lm_ctx* ctx, uint32_t max_rounds, uint32_t time_limit_ms);
  *                      entries); a power of two, 2^6 .. 2^20, or 0 = 32 rows only
  *   sweep_ctas_per_sm  CTAs per SM of the sweep kernel (0 = as many as fit, at most 16)
  *   vertex_ctas_per_sm CTAs per SM of the vertex pass (0 = 4, at most 4)
- *   contract_bits      lm_contract: the low bits of each edge's pair hash that its
- *                      sort orders by (8, 16, 24 or 32), the buckets of equal low bits
- *                      then searched for repeated hashes in shared memory; 0 = by
- *                      size (as few bytes as leave about 2048 edges to a bucket)
+ *   contract_bits      lm_contract: sort every edge by this many low bits of its pair's
+ *                      hash (8, 16, 24 or 32), the buckets of equal low bits then
+ *                      searched for repeated hashes in shared memory; 0 = partitions
+ *                      by the hash, sorted only where those do not suit
  *   ms                 lm_autotune only: median time of one call with these parameters
  * Defaults: rmax 1024, chunk 1024, sweep 0, vertex 4, batch 512, contract_bits 0.
  * The serving threads take the context's parameters when they start (first lm_submit).
- * rmax, chunk, batch and the CTAs per SM shape the round-by-round path, which the
- * renewed order takes (LM_F_RENEW); other matches do not use them. */
+ * rmax, chunk, batch and the CTAs per SM shape the round-by-round path, which batches under a
+ * renewed order (LM_F_RENEW) and graphs of 2^31 vertices and more take; other matches do not
+ * use them. */
 typedef struct lm_tuning {
     uint32_t rmax;
     uint32_t chunk;
