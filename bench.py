@@ -688,12 +688,10 @@ def run_contract(args, ws, rank, local):
             "roofline": {"bound": "hbm", "kernel": "lm_contract (all its kernels)", "achieved": ach, "peak": peak,
                          "peak_kind": peak_kind, "unit": "GB/s", "frac": ach / peak, "traffic": None,
                          "bytes_per_step": algo},
-            # R-MAT 23, per call: coarse map 2 + scan 3, keys (with the first pass's digit counts) 1,
-            # two hash passes (16 bits for about 1900 edges a bucket) of 4 and 5 (counts but in the
-            # first, scan 3, scatter), buckets 1, leader counts 1 + scan 3, emit 1 (no run here needs
-            # the pair sort)
-            "clocks": clk.summary(), # (representatives, map and 3 launches of scan, partitions, groups, walk, leaders with 3 of
-            # scan, emit, 2 reports; the pair sort's, if any, not counted)
+            "clocks": clk.summary(),
+            # per call: representatives, map and 3 launches of scan, partitions, groups, walk,
+            # leaders with 3 of scan, emit, 2 reports (the pair sort's, where a run needs it, not
+            # counted)
             "gpu_launches": 15 * args.steps}
 
 

@@ -1,6 +1,7 @@
 // Host side of liblm: context, graphs, plain and batched matching (include/lm.h).
 //
-// Everything on the result path runs on the GPU (lm_kernels.cu); this file
+// Everything on the result path runs on the GPU (lm_list.cu, lm_renew.cu, lm_kernels.cu,
+// lm_contract.cu); this file
 // validates arguments, owns device memory, builds launch arguments, drives
 // the round loop and moves results between host and device.
 #include <cuda_runtime.h>
@@ -625,7 +626,7 @@ static int ensure_list(lm_ctx* ctx, Engine& e, size_t nv, size_t nc, size_t ng, 
 }
 
 // The list path needs the top bit of a vertex id and an order that holds for the
-// whole job; a renewed order keys every round anew (run_job).
+// whole job; a renewed order keys every round anew (match_renewed, or run_job for batches).
 static bool list_path(const Engine& e, const lm_graph* g) { return !e.cfg.renew && g->n < 0x80000000u; }
 
 // Parts of a graph in a job of `total` rows: one for every block of the live pass that

@@ -1,5 +1,6 @@
-// sm_103a kernels: the round-by-round matching path (the renewed order, whose keys
-// change every round, and graphs of 2^31 vertices and more; lm_list.cu has the path
+// sm_103a kernels: the round-by-round matching path (batches under a renewed order, whose
+// keys change every round, and graphs of 2^31 vertices and more; lm_list.cu and, for one
+// graph under a renewed order, lm_renew.cu have the paths
 // of all others), the edge-centric path, graph construction, prefix sums.
 //
 // One round of local max (the phase of Sec. 2: every live vertex picks its
