@@ -253,7 +253,7 @@ struct EdgeArgs {
 // more than LIST_CHUNK entries are cut into chunks of that many, a warp each
 constexpr uint32_t LIST_SHORT = 32, LIST_GROUP = 64, LIST_WARP = 256, LIST_CHUNK = 2048;
 constexpr uint32_t LIST_KEPT = 8;       // neighbours kept of a long row
-constexpr uint32_t LIST_PART_MIN = 256, LIST_PART_MAX = 2048;  // rows a block of the live pass takes at a time
+constexpr uint32_t LIST_PART_MIN = 256, LIST_PART_MAX = 2048, LIST_PART_ENTS = 4096;  // rows a block of the live pass takes at a time
 
 // One graph of a list-path job (local vertex ids throughout).
 struct ListSeg {
@@ -272,6 +272,7 @@ struct ListSeg {
     uint32_t lbase;           // first slot of its chunks in part / pcnt
     uint32_t blk0, nblk;      // its blocks of k_top
     uint32_t part0, nparts;   // its parts
+    uint32_t run;             // log2 of the consecutive rows a part takes at a time
     uint32_t k0, k1;          // perm_seed keys of its seed
     uint64_t seed;
 };

@@ -711,15 +711,26 @@ __device__ __forceinline__ uint32_t refill_passed(const ListSeg& g, const uint64
         r[i] = 0;
     }
     const uint32_t low = (uint32_t)(k[KL - 1] >> 32);
-    for (uint64_t i = 32ull * q + (threadIdx.x & 31); i < d; i += 32ull * parts) {
-        const uint64_t w = __ldg(g.ent + s + (uint32_t)i);
-        if ((uint32_t)(w >> 32) < low) continue;
-        const uint64_t y = look(cur + (uint32_t)w);
-        if (!(lo(y) & DEAD)) continue;
-        const uint64_t key = key_of(g, (uint32_t)(w >> 32), s + (uint32_t)i);
+    // four entries a lane and step, their words and indices side by side
+    for (uint64_t b = 128ull * q + (threadIdx.x & 31); b < d; b += 128ull * parts) {
+        uint64_t w[4], y[4];
+        uint32_t e[4];
 #pragma unroll
-        for (int j = 0; j < KL; j++)
-            if (key > k[j]) r[j] = max(r[j], info(y));
+        for (int z = 0; z < 4; z++) w[z] = b + 32 * z < d ? __ldg(g.ent + s + (uint32_t)b + 32 * z) : 0ull;
+#pragma unroll
+        for (int z = 0; z < 4; z++) {
+            const bool on = b + 32 * z < d && (uint32_t)(w[z] >> 32) >= low;
+            y[z] = on ? look(cur + (uint32_t)w[z]) : 0ull;
+            e[z] = on ? __ldg(g.eid + s + (uint32_t)b + 32 * z) : 0u;
+        }
+#pragma unroll
+        for (int z = 0; z < 4; z++) {
+            if (!(lo(y[z]) & DEAD)) continue;
+            const uint64_t key = (w[z] & 0xFFFFFFFF00000000ull) | perm_seed(e[z], g.k0, g.k1);
+#pragma unroll
+            for (int j = 0; j < KL; j++)
+                if (key > k[j]) r[j] = max(r[j], info(y[z]));
+        }
     }
     uint32_t mine = 0;
 #pragma unroll
@@ -761,9 +772,7 @@ __device__ __forceinline__ void warp_append(uint32_t* ctr, uint32_t* out, bool o
     if (on) out[q] = v;
 }
 
-constexpr uint32_t RUN = 32;
-
-// A part: every nparts-th run of RUN consecutive rows of one graph (the long rows of a graph
+// A part: every nparts-th run of 2^run consecutive rows of one graph (the long rows of a graph
 // that numbers its vertices by degree, R-MAT's, a coarsened one's, would otherwise be in a
 // few parts, which the others wait for: fifth level of R-MAT
 // scale 20, 47 rounds: 2.26 ms by consecutive rows, 0.96 by runs of 8 to 64; runs of 8 cost
@@ -782,7 +791,8 @@ struct Part {
     // (g is there)
     __device__ __forceinline__ void init(const ListArgs& a, uint32_t part) {
         const uint32_t p = part - g.part0, np = g.nparts;
-        const uint32_t runs = (g.nrows + RUN - 1) / RUN, q = runs / np, r = runs - q * np;
+        const uint32_t RUN = 1u << g.run;
+        const uint32_t runs = (g.nrows + RUN - 1) >> g.run, q = runs / np, r = runs - q * np;
         const uint32_t missing = RUN * runs - g.nrows, owner = (runs - 1) % np;   // of the last run
         first = p;
         rows = RUN * (q + (p < r)) - (owner == p ? missing : 0u);
@@ -793,7 +803,7 @@ struct Part {
     }
     // the vertex of its row i
     __device__ __forceinline__ uint32_t vertex(uint32_t i) const {
-        return __ldg(g.vid + (size_t)RUN * ((i / RUN) * (size_t)g.nparts + first) + (i & (RUN - 1)));
+        return __ldg(g.vid + ((((i >> g.run) * (size_t)g.nparts + first) << g.run) + (i & ((1u << g.run) - 1u))));
     }
 };
 struct PartCounts {

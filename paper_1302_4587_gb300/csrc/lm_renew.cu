@@ -40,7 +40,12 @@ namespace {
 
 constexpr uint32_t RT = 256, RW = RT / 32;
 constexpr uint32_t RMINB = 4;   // (3 a SM: 2 to 10% slower on large graphs, 4% faster on small ones; 5: spills, 5 to 12%)
-constexpr uint32_t TAIL_ROWS = 512;       // live rows (and chunks) that one block finishes (2048: 10 to 20% slower)
+// one block finishes the job once its warps' share of a round is short: 512 short rows, 64 of up
+// to 64 entries, 32 of up to 256, 8 longer ones or 4 chunks (2048 short rows: 10 to 20% slower;
+// any 512 rows: a complete graph of 1000 vertices 723 us, this 151)
+__device__ __forceinline__ bool tail(const uint32_t cnt[5]) {
+    return 16ull * cnt[0] + 8ull * cnt[1] + 2ull * cnt[2] + cnt[3] + cnt[4] / 8 <= 64;
+}
 constexpr uint32_t NONE = 0x7FFFFFFFu;  // (vertex ids are below it)
 constexpr unsigned long long BAR_LIMIT_NS = 20000000000ull;  // a barrier gives up after 20 s
 // kinds of rows: chunks of the longest, then the other kinds of task, then short rows
@@ -466,7 +471,7 @@ __global__ void __launch_bounds__(RT, RMINB) k_renew(const __grid_constant__ Ren
         for (int k = 0; k < KINDS; k++) total += c.cnt[k] = __ldcg(ctr + out * KINDS + k);
         c.buf = out;
         if (total == 0 || ld_volatile_u32(&st->err)) break;
-        if (total <= TAIL_ROWS && blocks > 1) {
+        if (blocks > 1 && tail(c.cnt)) {
             if (blockIdx.x) return;
             blocks = 1;
         }
