@@ -16,7 +16,7 @@
 //               the others are listed for the next round, those without a live
 //               neighbour are dropped.
 //
-// Once few rows are left one block finishes the job without grid barriers.
+// Once little work is left one block finishes the job without grid barriers.
 //
 // The line to the rounds of launches (lm_kernels.cu) lies at 2^31 vertices and at batches,
 // whose graphs that path takes side by side.  One graph is faster here at every size and
