@@ -261,9 +261,9 @@ def run_lm(args, ws, rank, local):
     lm.lm_destroy(pctx)
     med = {k: statistics.median(v) for k, v in kms.items()}
     # launches of the timed matches, which want no statistics: the edge-centric path's are the
-    # same with them, of the others only k_top and k_live (or k_renew)
+    # same with them; of the others k_top and k_live (once at least), or k_renew
     per_step = (st["launches"] if edge else
-                pst["kernel_launches"][lm.LM_K_CAND] + pst["kernel_launches"][lm.LM_K_SWEEP])
+                (1 if order else 2))
     launches = per_step * args.steps
     peak, peak_kind = _peaks()
     gbs = lambda b, ms: b / (ms * 1e-3) / 1e9 if ms > 0 else 0.0
