@@ -31,6 +31,9 @@ namespace lm {
 
 constexpr uint32_t NIL = 0xFFFFFFFFu;
 
+// x / d rounded up, for every 32-bit x (x + d - 1 may not fit: lists hold up to 2^32 - 2 entries)
+LM_HD uint32_t div_up(uint32_t x, uint32_t d) { return x / d + (x % d != 0); }
+
 // Task sizes of the sweep.  A warp walks a sweep's task list at a rate set by
 // memory latency, so the longest task bounds the sweep's tail: rows of up to
 // LM_RMAX live entries are batched (at most 32 rows, and a batch ends where

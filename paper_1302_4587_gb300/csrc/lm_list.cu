@@ -490,9 +490,11 @@ __device__ __forceinline__ void top_long(const ListArgs& a, const ListSeg& g, ui
     uint32_t p = top.p;
     if (tie) {
         LaneTop64 kt;
-        for (uint32_t b = s; b < e; b += 32) {
-            const uint32_t i = b + lane;
-            kt.offer(i < e && i >= b ? key_of(g, ord_at(g, i), i) : 0ull, i);
+        // (by places within the row: positions may end close to 2^32)
+        const uint32_t d = e - s;
+        for (uint32_t k = 0; k < div_up(d, 32); k++) {
+            const uint32_t j = 32 * k + lane, i = s + j;
+            kt.offer(j < d ? key_of(g, ord_at(g, i), i) : 0ull, i);
         }
         p = kt.n;
         top.o = (uint32_t)(kt.k >> 32);
