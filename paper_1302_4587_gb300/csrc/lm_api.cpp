@@ -1236,7 +1236,7 @@ int lm_graph_create(lm_ctx* ctx, uint32_t n, uint32_t m, const uint32_t* eu, con
     for (int k = 0; k < 4; k++) g->ntask[k] = hp[8 + k] + (k ? g->ntask[k - 1] : 0u);
 
     // round-0 tiles copy rows [r & ~3, ...) of vid / roff in whole 16-byte words: pad both
-    g->ntiles = (g->nent + TILE0 - 1) / TILE0;
+    g->ntiles = div_up(g->nent, TILE0);
     Carver gc;
     gc.add(&g->vid, (size_t)g->nrows + 8);
     gc.add(&g->rdeg, (size_t)g->nrows + 1);

@@ -1587,10 +1587,10 @@ __global__ void __launch_bounds__(256) k_build_rows(const uint32_t* deg, const u
 __global__ void k_build_tilemap(const uint32_t* roff, uint32_t nrows, uint32_t nent, uint32_t* tmap,
                                 uint32_t* rbits) {
     const uint32_t stride = gridDim.x * blockDim.x;
-    const uint32_t ntiles = (nent + TILE0 - 1) / TILE0;
+    const uint32_t ntiles = div_up(nent, TILE0);
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nrows; i += stride) {
         const uint32_t lo = roff[i], hi = roff[i + 1];
-        for (uint32_t t = (lo + TILE0 - 1) / TILE0; t < (hi + TILE0 - 1) / TILE0; t++) tmap[t] = i;
+        for (uint32_t t = div_up(lo, TILE0); t < div_up(hi, TILE0); t++) tmap[t] = i;
         atomicOr(&rbits[lo >> 5], 1u << (lo & 31));
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) tmap[ntiles] = nrows;
@@ -1938,7 +1938,7 @@ int launch_build_rows(void* stream, const uint32_t* deg, const uint32_t* rowidx_
 int launch_build_tilemap(void* stream, const uint32_t* roff, uint32_t nrows, uint32_t nent, uint32_t* tmap,
                          uint32_t* rbits, uint4* tdesc) {
     k_build_tilemap<<<grid_for(nrows + 1, 256), 256, 0, (cudaStream_t)stream>>>(roff, nrows, nent, tmap, rbits);
-    const uint32_t ntiles = (nent + TILE0 - 1) / TILE0;
+    const uint32_t ntiles = div_up(nent, TILE0);
     if (ntiles) k_build_tiledesc<<<grid_for(ntiles, 256), 256, 0, (cudaStream_t)stream>>>(roff, tmap, nrows, ntiles,
                                                                                          tdesc);
     return (int)cudaGetLastError();

@@ -23,3 +23,16 @@ def test_division_rounds_up_for_every_32_bit_number(tmp_path):
     ds = [1, 32, 1024, 4096]
     body = "\n".join(f'printf("%u\\n", div_up({x}u, {d}u));' for x in xs for d in ds)
     assert [int(t) for t in _run(tmp_path, body)] == [-(-x // d) for x in xs for d in ds]
+
+
+def test_tiles_cover_the_largest_lists(tmp_path):
+    # round-0 tiles of 2m entries: as many as allocate tmap / rbits, none missing for m >= 2^31 - 511
+    ms = [0, 1, 511, 512, 513, (1 << 31) - 513, (1 << 31) - 512, (1 << 31) - 511, (1 << 31) - 1]
+    body = "\n".join(f'printf("%u %u\\n", div_up({2 * m}u, TILE0), TILE0);' for m in ms)
+    got = [int(t) for t in _run(tmp_path, body)]
+    for m, tiles, tile in zip(ms, got[::2], got[1::2]):
+        assert (tiles - 1) * tile < max(2 * m, 1) <= max(tiles, 1) * tile, m
+    # the build and its launch count them the same way, and a row's first tile too
+    for f in ("lm_api.cpp", "lm_kernels.cu"):
+        src = open(os.path.join(CSRC, f)).read()
+        assert "div_up(" in src and "TILE0 - 1) / TILE0" not in src, f
