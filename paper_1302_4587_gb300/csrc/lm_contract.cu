@@ -50,9 +50,10 @@ uint32_t grid_for(uint64_t count) {
     return (uint32_t)(b < 1 ? 1 : (b > cap ? cap : b));
 }
 
+// (vertex numbers of a step beyond n may not fit 32 bits)
 __global__ void k_c_rep(const uint32_t* __restrict__ mate, uint32_t n, uint32_t* __restrict__ flag,
                         uint32_t* __restrict__ err) {
-    for (uint32_t v = blockIdx.x * CT + threadIdx.x; v < n; v += gridDim.x * CT) {
+    for (uint64_t v = blockIdx.x * CT + threadIdx.x; v < n; v += gridDim.x * CT) {
         const uint32_t u = mate[v];
         bool rep = true;
         if (u != NIL) {
@@ -65,7 +66,8 @@ __global__ void k_c_rep(const uint32_t* __restrict__ mate, uint32_t n, uint32_t*
 
 __global__ void k_c_map(const uint32_t* __restrict__ mate, uint32_t n, const uint32_t* __restrict__ rank,
                         const uint32_t* __restrict__ vw, uint32_t* __restrict__ cmap, uint32_t* __restrict__ cvw) {
-    for (uint32_t v = blockIdx.x * CT + threadIdx.x; v < n; v += gridDim.x * CT) {
+    for (uint64_t i = blockIdx.x * CT + threadIdx.x; i < n; i += gridDim.x * CT) {
+        const uint32_t v = (uint32_t)i;
         uint32_t u = mate[v];
         if (u >= n) u = v;  // unmatched (an invalid mate was flagged by k_c_rep)
         const uint32_t c = rank[u < v ? u : v];

@@ -64,7 +64,7 @@ __global__ void k_init(const InitArgs* __restrict__ pa) {
     const uint32_t n = A.n;
     DevState* st = A.st;
     const uint32_t stride = gridDim.x * blockDim.x;
-    for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
+    for (uint64_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
         if (mate) mate[v] = NIL;
         bcnt[v] = 0;
         bkey[v] = 0;
@@ -75,7 +75,7 @@ __global__ void k_init(const InitArgs* __restrict__ pa) {
         const uint32_t b0 = A.dbase, b1 = A.dbase + n;
         const uint32_t w0 = b0 >> 5, w1 = (b1 - 1) >> 5;
         for (uint32_t w = w0 + blockIdx.x * blockDim.x + threadIdx.x; w <= w1; w += stride) {
-            const uint32_t lo = max(b0, w * 32u), hi = min(b1, w * 32u + 32u);
+            const uint32_t lo = max(b0, w * 32u), hi = min(b1 - 1u, w * 32u + 31u) + 1u;
             if (lo == w * 32u && hi == w * 32u + 32u) {
                 dead[w] = 0;
             } else {
@@ -1588,9 +1588,9 @@ __global__ void k_build_tilemap(const uint32_t* roff, uint32_t nrows, uint32_t n
                                 uint32_t* rbits) {
     const uint32_t stride = gridDim.x * blockDim.x;
     const uint32_t ntiles = div_up(nent, TILE0);
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nrows; i += stride) {
+    for (uint64_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nrows; i += stride) {
         const uint32_t lo = roff[i], hi = roff[i + 1];
-        for (uint32_t t = div_up(lo, TILE0); t < div_up(hi, TILE0); t++) tmap[t] = i;
+        for (uint32_t t = div_up(lo, TILE0); t < div_up(hi, TILE0); t++) tmap[t] = (uint32_t)i;
         atomicOr(&rbits[lo >> 5], 1u << (lo & 31));
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) tmap[ntiles] = nrows;
@@ -1636,12 +1636,12 @@ __global__ void k_union_setup(const uint32_t* gvbase, const uint32_t* ebase, con
                               uint32_t ngraphs, uint32_t nvert, uint32_t* start, uint32_t* gid, uint32_t* len0) {
     const uint32_t stride = gridDim.x * blockDim.x;
     const int lane = threadIdx.x & 31;
-    const uint32_t nr = (nvert + 31) & ~31u;  // whole warps iterate together
-    for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < nr; v += stride) {
-        const uint32_t vv = min(v, nvert - 1);
+    const uint64_t nr = ((uint64_t)nvert + 31) & ~31ull;  // whole warps iterate together
+    for (uint64_t v = blockIdx.x * blockDim.x + threadIdx.x; v < nr; v += stride) {
+        const uint32_t vv = v < nvert ? (uint32_t)v : nvert - 1;
         const uint32_t g = graph_of_warp(gvbase, ngraphs, vv, vv, lane);  // lane 0's vertex starts the warp
         if (v >= nvert) continue;
-        const uint32_t i = v - gvbase[g];
+        const uint32_t i = vv - gvbase[g];
         const uint32_t* off = offs[g];
         const uint32_t o0 = off[i], o1 = off[i + 1];
         start[v] = ebase[g] + o0;
@@ -1653,8 +1653,8 @@ __global__ void k_to_local_batch(const uint32_t* mate_u, const uint32_t* gvbase,
                                  uint32_t* const* dst, unsigned long long* matched2, uint32_t nvert) {
     const uint32_t stride = gridDim.x * blockDim.x;
     const int lane = threadIdx.x & 31;
-    const uint32_t nr = (nvert + 31) & ~31u;  // whole warps iterate together
-    for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < nr; v += stride) {
+    const uint64_t nr = ((uint64_t)nvert + 31) & ~31ull;  // whole warps iterate together
+    for (uint64_t v = blockIdx.x * blockDim.x + threadIdx.x; v < nr; v += stride) {
         const bool live = v < nvert;
         uint32_t x = NIL, g = NIL;
         if (live) {
@@ -1772,7 +1772,7 @@ int launch_exclusive_scan(void* stream, const uint32_t* in, uint32_t* out, uint3
     cudaStream_t s = (cudaStream_t)stream;
     if (count == 0) return 0;
     const bool vec = ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15u) == 0;
-    const uint32_t blocks = (count + SCAN_TILE - 1) / SCAN_TILE;
+    const uint32_t blocks = div_up(count, SCAN_TILE);
     if (blocks == 1) {
         if (vec) k_scan_apply<true><<<1, SCAN_THREADS, 0, s>>>(in, count, nullptr, out);
         else k_scan_apply<false><<<1, SCAN_THREADS, 0, s>>>(in, count, nullptr, out);
