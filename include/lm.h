@@ -193,8 +193,10 @@ int  lm_wait(lm_ctx* ctx, uint64_t ticket, uint32_t timeout_ms);
  *   max_rounds     the match gives up with LM_ETIMEOUT once it has run more than
  *                  this many rounds without emptying the edge set (0 = no cap
  *                  beyond m + 2, which a match never reaches: every round matches
- *                  the heaviest live edge).  Checked after every second round,
- *                  so up to one round more may run.
+ *                  the heaviest live edge).  Checked after every pass over a block's
+ *                  rows (row lists, whose rounds are not steps of the whole graph: a
+ *                  few rounds more may be matched in places before all blocks stop),
+ *                  every round (one graph under LM_F_RENEW) or every second one.
  *   time_limit_ms  the match gives up with LM_ETIMEOUT once its rounds have run
  *                  longer than this (0 = 120 s).  Checked with the cap.
  * A match that gives up leaves mate undefined; the context stays usable.

@@ -812,7 +812,7 @@ struct PartCounts {
     uint32_t live, nshort, nlong;
 };
 struct Tally {
-    uint32_t matched = 0, last = 0;   // rows matched; 1 + their latest round
+    uint32_t matched = 0, last = 0;   // rows matched; 1 + their latest round (the rounds that it takes)
     bool changed = false;
 };
 
@@ -1061,8 +1061,10 @@ struct LiveSmem {
 // Blocks take parts from a counter and pass over a part's live rows until none is
 // left.  A part may wait for words that another block writes, but no block waits for
 // good: after IDLE_MAX passes without a change it puts the part's rows back for the
-// next launch, which the last block to leave asks for.  (pa: the arguments in device
-// memory, for a launch in a graph.)
+// next launch, which the last block to leave asks for.  A part's block stops after the
+// pass that matched a row beyond the round cap, the others when they see the error: with
+// rounds at their next pass, else (no cap then, only the time limit) within 16.  (pa: the
+// arguments in device memory, for a launch in a graph.)
 template <class W>
 __global__ void __launch_bounds__(LT, LMINB) k_live(const __grid_constant__ ListArgs av,
                                                        const ListArgs* __restrict__ pa, cudaGraphConditionalHandle h) {
@@ -1092,6 +1094,8 @@ __global__ void __launch_bounds__(LT, LMINB) k_live(const __grid_constant__ List
         uint32_t idle = 0;
         for (uint32_t pass = 0; cnt; pass++) {
             uint32_t* out = a.list[buf ^ 1u] + P.home;
+            // (thread 0: asked for ahead of the pass and looked at after it)
+            const uint32_t err = sizeof(W) == 8 && tid == 0 ? ld_volatile_u32(&st->err) : 0u;
             if (tid == 0) {
                 S.c.live = S.c.nshort = S.c.nlong = 0;
                 S.next[0] = S.next[1] = 0;
@@ -1100,7 +1104,7 @@ __global__ void __launch_bounds__(LT, LMINB) k_live(const __grid_constant__ List
                 if (globaltimer_ns() - st->t0_ns > a.limit_ns) {
                     set_err(st, ERR_TIMEOUT, pass);
                     S.stop = 1;
-                } else if ((pass & 15u) == 15u && ld_volatile_u32(&st->err)) {
+                } else if (sizeof(W) == 4 && (pass & 15u) == 15u && ld_volatile_u32(&st->err)) {
                     S.stop = 1;
                 }
             }
@@ -1108,6 +1112,11 @@ __global__ void __launch_bounds__(LT, LMINB) k_live(const __grid_constant__ List
             T.changed = false;
             poll_rows<W>(a, P, list, cnt, out, S.c, T);
             if (T.changed) S.changed = 1;
+            if (sizeof(W) == 8) {
+                const bool over = T.last > a.max_rounds;
+                if (over) set_err(st, ERR_TIMEOUT, T.last);
+                if (over || err) S.stop = 1;
+            }
             __syncthreads();
             const uint32_t k0 = S.c.nshort, k1 = S.c.nlong;
             if (k0 | k1) {
@@ -1137,10 +1146,7 @@ __global__ void __launch_bounds__(LT, LMINB) k_live(const __grid_constant__ List
                 l = max(l, S.red[1][i]);
             }
             if (t) atomicAdd(a.gmatched ? &a.gmatched[si] : &st->matched2, t);
-            if (sizeof(W) == 8 && l) {
-                atomicMax(a.grounds ? &a.grounds[si] : &st->rounds, l);
-                if (l > a.max_rounds) set_err(st, ERR_TIMEOUT, l);
-            }
+            if (sizeof(W) == 8 && l) atomicMax(a.grounds ? &a.grounds[si] : &st->rounds, l);
             a.pcount[part] = cnt << 1 | buf;
             left += cnt;
         }

@@ -1,8 +1,8 @@
 """The error contract of the C ABI, provoked without faulting a GPU.
 
 LM_ETIMEOUT: a round cap or time limit (lm_set_limits) that a long run
-exceeds.  The device-driven loop checks both after every second round and
-returns an error status; the profiled path checks them on the host.  A path
+exceeds.  The kernels check both after every pass over a part's rows (row
+lists) or every round or two (the other paths) and return an error status.  A path
 with monotone weights needs ceil((n - 1) / 2) rounds under the fixed order
 (Sec. 2 bounds the rounds only in expectation), so it runs past any small cap.
 
@@ -54,6 +54,38 @@ def test_round_cap_times_out_and_the_context_stays_usable(profile):
         st = _exact(L, path, 1, handle=h)
         assert st["rounds"] == math.ceil((path.n - 1) / 2)
         lm.lm_graph_destroy(h)
+    finally:
+        L.close()
+
+
+@pytest.mark.parametrize("n,most", [(250, 60), (100_000, 2000)])
+def test_round_cap_stops_the_run(n, most):
+    """A monotone path matches one edge a round.  250 vertices are one part of one block:
+    a pass is 8 steps of a warp, each good for one more round (two if its lanes part),
+    so at most cap + 1 + 16 edges are matched when the pass that passes the cap ends.
+    100,000 vertices: the chain goes through runs of 32 rows of different blocks, which
+    see the error at their next pass; without a stop all n - 1 edges' rounds are run."""
+    import paper_1302_4587_gb300 as lm
+    L = Lm()
+    try:
+        path = _mono_path(n)
+        h = L.graph(path)
+        mate = L.torch.full((n,), -1, dtype=L.torch.int32, device="cuda")
+        lm.lm_set_limits(L.ctx, 10, 0)
+        with pytest.raises(lm.LmError) as ei:
+            lm.lm_match(L.ctx, h, 1, mate)
+        assert ei.value.code == lm.LM_ETIMEOUT
+        assert 0 < int((mate != -1).sum()) <= most
+        other = [L.graph(g) for g in (synth.er(2000, 8000, 5), synth.er(500, 900, 6))]
+        mates = [L.torch.full((k,), -1, dtype=L.torch.int32, device="cuda") for k in (2000, n, 500)]
+        with pytest.raises(lm.LmError) as ei:
+            lm.lm_batch_match(L.ctx, [other[0], h, other[1]], [1, 1, 1], mates)
+        assert ei.value.code == lm.LM_ETIMEOUT
+        assert 0 < int((mates[1] != -1).sum()) <= most
+        lm.lm_set_limits(L.ctx, 0, 0)
+        _exact(L, path, 1, handle=h)
+        for g in (h, *other):
+            lm.lm_graph_destroy(g)
     finally:
         L.close()
 
