@@ -185,11 +185,11 @@ int  lm_poll(lm_ctx* ctx, uint64_t ticket, int* done, lm_stats* stats);
  * ticket stays valid).  Does not release the ticket: call lm_poll after. */
 int  lm_wait(lm_ctx* ctx, uint64_t ticket, uint32_t timeout_ms);
 
-/* Limits of every later lm_match / lm_batch_match on the context (and of served
- * requests that run alone).  Sec. 2 bounds the rounds of local max by O(log m)
- * only in expectation; with a fixed order a graph can need Theta(n) rounds (a
- * path with monotone weights), so a caller who must bound how long the GPU is
- * held sets either limit:
+/* Limits of every later lm_match / lm_batch_match on the context, and of every served
+ * request for itself (one that exceeds a limit fails alone, whatever ran beside it).
+ * Sec. 2 bounds the rounds of local max by O(log m) only in expectation; with a fixed
+ * order a graph can need Theta(n) rounds (a path with monotone weights), so a caller who
+ * must bound how long the GPU is held sets either limit:
  *   max_rounds     the match gives up with LM_ETIMEOUT once it has run more than
  *                  this many rounds without emptying the edge set (0 = no cap
  *                  beyond m + 2, which a match never reaches: every round matches

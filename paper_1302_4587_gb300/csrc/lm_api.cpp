@@ -83,9 +83,11 @@ bool fault_alloc(lm_ctx* ctx) {
 void job_limits(const lm_ctx* ctx, uint32_t nedges, uint32_t* max_rounds, unsigned long long* limit_ns) {
     // every round matches at least the heaviest live edge, so m + 2 rounds never run out
     uint32_t r = nedges + 2;
-    if (ctx && ctx->lim_rounds && ctx->lim_rounds < r) r = ctx->lim_rounds;
+    const uint32_t lim = ctx ? ctx->lim_rounds.load() : 0u;
+    const uint64_t ns = ctx ? ctx->lim_ns.load() : 0u;
+    if (lim && lim < r) r = lim;
     *max_rounds = r;
-    *limit_ns = (ctx && ctx->lim_ns) ? ctx->lim_ns : LOOP_LIMIT_NS;
+    *limit_ns = ns ? ns : LOOP_LIMIT_NS;
 }
 
 int cuda_fail(lm_ctx* ctx, cudaError_t e, const char* where) {

@@ -121,8 +121,9 @@ struct lm_ctx {
     cudaEvent_t up_ev = nullptr, up_w[UP_CHUNKS] = {};
     // limits of every match (lm_set_limits): a round cap (0 = none beyond m + 2)
     // and a time limit in ns (0 = LOOP_LIMIT_NS)
-    uint32_t lim_rounds = 0;
-    uint64_t lim_ns = 0;
+    // (read by the serving lanes while a caller may set them)
+    std::atomic<uint32_t> lim_rounds{0};
+    std::atomic<uint64_t> lim_ns{0};
     // host-side fault injection read from LM_FAULT at lm_create: the next
     // fault_alloc device allocations fail as out of memory (-1: all of them)
     std::atomic<int64_t> fault_alloc{0};

@@ -7,7 +7,8 @@
 // same launches.  Requests that arrive meanwhile are taken by the next free lane, so
 // they join the device while earlier ones are on it and leave as soon as their own
 // group is done.  Every request keeps its own seed and edge ids, so its result does not
-// depend on what else is in flight.
+// depend on what else is in flight.  When a group fails for want of memory or at a limit
+// (lm_set_limits), its requests run again one by one, so that each gets its own outcome.
 //
 // A burst of 48 requests of 1 thousand to 4 million edges takes 1.28 ms with two lanes
 // (1.36 with one, 1.32 with three); stepping all requests together round by round,
@@ -34,6 +35,7 @@ struct Request {
     uint64_t seed = 0;
     uint32_t* mate = nullptr;
     bool host_dst = false;
+    bool alone = false;     // ran in a group that failed: not in a group again
     uint32_t rounds = 0;
     int state = 0;          // 0 queued, 1 in flight, 2 done
     int rc = LM_OK;
@@ -103,6 +105,7 @@ void lane(ServeState* S, int which) {
         uint64_t gv = 0, ge = 0;
         while (!S->queue.empty() && group.size() < MAX_GROUP && (S->fatal || fits(S, S->queue.front()))) {
             Request* r = S->queue.front();
+            if (!group.empty() && (r->alone || group[0]->alone)) break;
             S->queue.pop_front();
             r->state = 1;
             gv += r->g->n;
@@ -115,36 +118,34 @@ void lane(ServeState* S, int which) {
         const size_t k = group.size();
         std::vector<uint32_t> rounds(k);
         std::vector<unsigned long long> m2(k);
-        std::vector<int> rcs(k, S->fatal);
-        if (!S->fatal) {
+        int rc = S->fatal;
+        if (!rc) {
             lk.unlock();
-            int rc = run_group(S, e, group, rounds, m2);
-            std::fill(rcs.begin(), rcs.end(), rc);
-            if (rc == LM_ENOMEM && k > 1) {
-                // no memory for all at once: one after the other
-                for (size_t i = 0; i < k; i++) {
-                    std::vector<uint32_t> r1(1);
-                    std::vector<unsigned long long> q1(1);
-                    rcs[i] = run_group(S, e, {group[i]}, r1, q1);
-                    rounds[i] = r1[0];
-                    m2[i] = q1[0];
-                }
-            }
+            rc = run_group(S, e, group, rounds, m2);
             lk.lock();
         }
+        S->used_v -= gv;
+        S->used_e -= ge;
+        S->used_slots -= (uint32_t)k;
+        if ((rc == LM_ENOMEM || rc == LM_ETIMEOUT) && k > 1) {
+            for (size_t i = k; i-- > 0;) {
+                group[i]->alone = true;
+                group[i]->state = 0;
+                S->queue.push_front(group[i]);
+            }
+            S->cv_work.notify_all();
+            continue;
+        }
+        if (rc == LM_ECUDA) S->fatal = rc;
         for (size_t i = 0; i < k; i++) {
             Request* r = group[i];
-            r->rc = rcs[i];
-            if (r->rc == LM_ECUDA) S->fatal = LM_ECUDA;
-            if (r->rc == LM_OK) {
+            r->rc = rc;
+            if (rc == LM_OK) {
                 r->rounds = rounds[i];
                 r->matched = m2[i] / 2;
             }
             r->state = 2;
         }
-        S->used_v -= gv;
-        S->used_e -= ge;
-        S->used_slots -= (uint32_t)k;
         S->cv_done.notify_all();
         if (!S->queue.empty()) S->cv_work.notify_all();  // there is room again
     }

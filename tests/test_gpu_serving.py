@@ -98,3 +98,39 @@ def test_destroy_with_requests_in_flight_returns():
     srv.close()  # stops the scheduler; must not hang on the requests in flight
     assert time.perf_counter() - t0 < 30
     # (the graph belonged to the destroyed context: its handle is abandoned, not destroyed)
+
+
+def _mono_path(n):
+    eu = np.arange(n - 1, dtype=np.uint32)
+    return synth.Graph(n, eu, eu + 1, (np.arange(n - 1) + 1).astype(np.float32), f"mono{n}")
+
+
+def test_a_request_beyond_a_limit_fails_alone():
+    # the path needs 1500 rounds, the others at most 40; all of them wait together behind
+    # two larger graphs, so that they are taken as groups
+    import paper_1302_4587_gb300 as lm
+    srv = Lm()
+    try:
+        lm.lm_set_limits(srv.ctx, 40, 0)
+        big = [synth.er(1_000_000, 4_000_000, seed=s) for s in (1, 2)]
+        small = [synth.er(300 + 10 * i, 900 + 50 * i, seed=20 + i) for i in range(12)]
+        order = big + small[:6] + [_mono_path(3001)] + small[6:]
+        hs = [srv.graph(g) for g in order]
+        want = [oracle.greedy(g.n, g.eu, g.ev, g.w, 5) for g in order]
+        for _ in range(5):
+            mates = [srv.torch.empty(g.n, dtype=srv.torch.int32, device="cuda") for g in order]
+            tickets = [lm.lm_submit(srv.ctx, h, 5, m) for h, m in zip(hs, mates)]
+            for g, t, m, x in zip(order, tickets, mates, want):
+                assert lm.lm_wait(srv.ctx, t, 60_000)
+                if g.name.startswith("mono"):
+                    with pytest.raises(lm.LmError) as ei:
+                        lm.lm_poll(srv.ctx, t)
+                    assert ei.value.code == lm.LM_ETIMEOUT
+                else:
+                    done, st = lm.lm_poll(srv.ctx, t)
+                    assert done and st["rounds"] <= 40 and st["matched"] == int((x != NIL).sum()) // 2
+                    assert np.array_equal(to_u32(m), x)
+        for h in hs:
+            lm.lm_graph_destroy(h)
+    finally:
+        srv.close()
