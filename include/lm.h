@@ -170,8 +170,10 @@ int  lm_batch_match(lm_ctx* ctx, const lm_graph* const* g, uint32_t count, const
 /* Serving: queue a matching request and return at once with a ticket.  The
  * context's serving threads take the waiting requests in arrival order, as long as
  * they fit the HBM budget and the slots beside those in flight, and run those taken
- * together in shared launches; requests that arrive meanwhile are taken by the next
- * free thread and run beside them.  mate (uint32[n], host or device) must stay valid
+ * together in shared launches, a few milliseconds at a time: a request leaves at the end of
+ * the slice in which it is done, and requests that arrive meanwhile are taken by a free
+ * thread, or between two slices by one whose requests need many rounds (up to 8 such
+ * groups a thread).  mate (uint32[n], host or device) must stay valid
  * until the request completes; the graph must outlive it.  Errors: LM_EINVAL,
  * LM_EAGAIN (queue full), LM_ENOMEM (the request alone exceeds the budget), LM_ECUDA. */
 int  lm_submit(lm_ctx* ctx, const lm_graph* g, uint64_t seed, uint32_t* mate, uint64_t* ticket);

@@ -155,6 +155,16 @@ int engine_init(lm_ctx* ctx, Engine& e, cudaStream_t stream) {
     return LM_OK;
 }
 
+// gives an engine's scratch back (nothing of it is in use)
+void engine_trim(Engine& e) {
+    cudaStreamSynchronize(e.stream);
+    if (e.ws.block) cudaFree(e.ws.block);
+    if (e.lw.block) cudaFree(e.lw.block);
+    cudaGetLastError();
+    e.ws = Workspace();
+    e.lw = ListWs();
+}
+
 void engine_free(Engine& e) {
     if (e.stream) cudaStreamSynchronize(e.stream);
     else cudaDeviceSynchronize();
@@ -629,7 +639,7 @@ static int ensure_list(lm_ctx* ctx, Engine& e, size_t nv, size_t nc, size_t ng, 
 
 // The list path needs the top bit of a vertex id and an order that holds for the
 // whole job; a renewed order keys every round anew (match_renewed, or run_job for batches).
-static bool list_path(const Engine& e, const lm_graph* g) { return !e.cfg.renew && g->n < 0x80000000u; }
+bool list_path(const Engine& e, const lm_graph* g) { return !e.cfg.renew && g->n < 0x80000000u; }
 
 // Parts of a graph in a job of `rows` rows and `ents` entries in all: one for every block of
 // the live pass that runs at once, within the limits.  A graph's own never exceed those
@@ -695,64 +705,77 @@ static void list_args(ListArgs& A, Engine& e) {
 // an asynchronous list job's arguments sit in the last quarter of the argument area
 constexpr size_t LIST_ARGS_OFF = ARG_AREA / 4 * 3;
 
-// The live pass of a queued job, until no row is left: k_live as often as it gives rows
-// back (once, as a rule), the state in the host's mirror after each.
-static int run_live(lm_ctx* ctx, Engine& e, const ListArgs& A, uint32_t nparts, bool rounds, Prof& prof) {
+// One launch of the live pass of a queued job, the state in the host's mirror after it:
+// rows may be left (st_host->done not set).
+int list_pass(lm_ctx* ctx, Engine& e, const ListRun& R, Prof& prof) {
+    prof.begin(LM_K_SWEEP);
+    LM_CK(ctx, launch_live(e.stream, R.A, R.A.nparts, R.rounds));
+    prof.end();
+    LM_CK(ctx, cudaStreamSynchronize(e.stream));
+    return e.st_host->err ? check_err(ctx, e) : LM_OK;
+}
+// The live pass until no row is left: as often as it gives rows back (once, as a rule).
+static int run_live(lm_ctx* ctx, Engine& e, const ListRun& R, Prof& prof) {
     for (;;) {
-        prof.begin(LM_K_SWEEP);
-        LM_CK(ctx, launch_live(e.stream, A, nparts, rounds));
-        prof.end();
-        LM_CK(ctx, cudaStreamSynchronize(e.stream));
-        if (e.st_host->err || e.st_host->done) return check_err(ctx, e);
+        const int rc = list_pass(ctx, e, R, prof);
+        if (rc || e.st_host->done) return rc;
     }
 }
 
-// One graph by the list path (see lm_list.cu).  rounds: the round count is wanted
-// (64-bit words); counts: the live edges and vertices of every round too.
-static int match_list(lm_ctx* ctx, Engine& e, const lm_graph* g, uint64_t seed, uint32_t* mate, bool dev_out,
-                      Prof& prof, bool async, bool rounds, bool counts) {
-    cudaStream_t s = e.stream;
+// Arguments and first kernel of one graph's job by the list path (see lm_list.cu), its
+// result at mate_d.  rounds: the round count is wanted (64-bit words).
+int list_start(lm_ctx* ctx, Engine& e, const lm_graph* g, uint64_t seed, uint32_t* mate, bool dev_out, Prof& prof,
+               bool rounds, ListRun& R) {
     const uint32_t nparts = list_parts(ctx, g, g->nrows, g->nent);
-    if (ctx->lim_rounds) rounds = true;   // a cap on the rounds: they have to be known
-    int rc = ensure_list(ctx, e, g->n, g->ntask[0], 1, 0, nparts, rounds);
-    if (rc) return rc;
-    uint32_t* mate_d = dev_out ? mate : e.lw.mate;
-    ListArgs A;
+    R.rounds = rounds || ctx->lim_rounds;   // a cap on the rounds: they have to be known
+    if (int rc = staging_ready(ctx, e)) return rc;
+    if (int rc = ensure_list(ctx, e, g->n, g->ntask[0], 1, 0, nparts, R.rounds)) return rc;
+    ListArgs& A = R.A;
     list_args(A, e);
     A.nsegs = 1;
     A.nparts = nparts;
     job_limits(ctx, g->m, &A.max_rounds, &A.limit_ns);
-    A.one = list_seg(g, seed, mate_d);
+    A.one = list_seg(g, seed, dev_out ? mate : e.lw.mate);
     A.one.nparts = nparts;
     A.one.run = list_run(g, nparts);
-    if (async) A.host = nullptr;
     prof.begin(LM_K_CAND);
-    LM_CK(ctx, launch_top(s, A, A.one.nblk, rounds));
+    LM_CK(ctx, launch_top(e.stream, A, A.one.nblk, R.rounds));
     prof.end();
+    return LM_OK;
+}
+
+// One graph by the list path.  counts: the live edges and vertices of every round too.
+static int match_list(lm_ctx* ctx, Engine& e, const lm_graph* g, uint64_t seed, uint32_t* mate, bool dev_out,
+                      Prof& prof, bool async, bool rounds, bool counts) {
+    cudaStream_t s = e.stream;
+    ListRun R;
+    int rc = list_start(ctx, e, g, seed, mate, dev_out, prof, rounds, R);
+    if (rc) return rc;
     if (async) {  // queued, the arguments in device memory for the graph; lm_sync reports device errors
         static_assert(EDGE_ARGS_OFF + sizeof(EdgeJobArgs) <= LIST_ARGS_OFF &&
                       LIST_ARGS_OFF + sizeof(ListArgs) <= ARG_AREA, "argument area too small");
+        R.A.host = nullptr;
         ListArgs* D = reinterpret_cast<ListArgs*>(e.dargs + LIST_ARGS_OFF);
-        memcpy(e.hargs + LIST_ARGS_OFF, &A, sizeof A);
-        LM_CK(ctx, cudaMemcpyAsync(D, e.hargs + LIST_ARGS_OFF, sizeof A, cudaMemcpyHostToDevice, s));
+        memcpy(e.hargs + LIST_ARGS_OFF, &R.A, sizeof R.A);
+        LM_CK(ctx, cudaMemcpyAsync(D, e.hargs + LIST_ARGS_OFF, sizeof R.A, cudaMemcpyHostToDevice, s));
         // the next job may rewrite the staging only after this upload ran
         if (!e.staged) LM_CK(ctx, cudaEventCreateWithFlags(&e.staged, cudaEventDisableTiming));
         LM_CK(ctx, cudaEventRecord(e.staged, s));
         e.staged_pending = true;
-        void*& graph = e.lgraph[rounds ? 1 : 0];
-        if (!graph) LM_CK(ctx, build_list_graph(D, rounds, &graph));
+        void*& graph = e.lgraph[R.rounds ? 1 : 0];
+        if (!graph) LM_CK(ctx, build_list_graph(D, R.rounds, &graph));
         LM_CK(ctx, launch_job_graph(graph, s));
         return LM_OK;
     }
-    rc = run_live(ctx, e, A, nparts, rounds, prof);
+    rc = run_live(ctx, e, R, prof);
     if (rc) return rc;
     if (counts) {
         prof.begin(LM_K_OTHER);
-        LM_CK(ctx, launch_round_counts(s, A, e.lw.queue));
+        LM_CK(ctx, launch_round_counts(s, R.A, e.lw.queue));
         prof.end();
         LM_CK(ctx, cudaMemcpyAsync(e.st_host, e.st, sizeof(DevState), cudaMemcpyDeviceToHost, s));
     }
-    if (!dev_out) LM_CK(ctx, cudaMemcpyAsync(mate, mate_d, (size_t)g->n * 4, cudaMemcpyDeviceToHost, s));
+    if (!dev_out) LM_CK(ctx, cudaMemcpyAsync(mate, e.lw.mate, (size_t)g->n * 4, cudaMemcpyDeviceToHost, s));
     if (counts || !dev_out) LM_CK(ctx, cudaStreamSynchronize(s));
     if (counts)  // counted by their last live round -> live at the start of round r
         for (int r = LM_STATS_ROUNDS - 2; r >= 0; r--) {
@@ -830,13 +853,11 @@ int match_one(lm_ctx* ctx, Engine& e, const lm_graph* g, uint64_t seed, uint32_t
     return LM_OK;
 }
 
-// Many graphs on engine e in the same launches (lm_batch_match, and groups of
-// served requests): their vertex and entry ranges are laid side by side in one
-// union id space, each graph keeping its own seed and edge ids.  mates[i] is
-// device or host memory; rounds[i] and matched2[i] receive graph i's round count
-// and matched vertices (either may be NULL).
-static int batch_list(lm_ctx* ctx, Engine& e, const lm_graph* const* gs, uint32_t count, const uint64_t* seeds,
-                      uint32_t* const* mates, uint32_t* rounds, unsigned long long* matched2, Prof& prof) {
+// Tables, arguments and first kernels of a batch's job by the list path: the graphs' vertices
+// side by side in one id space, each graph with its own seed and edge ids.  mates[i] is
+// device or host memory (its result then waits in the workspace).  want: round counts.
+int list_batch_start(lm_ctx* ctx, Engine& e, const lm_graph* const* gs, uint32_t count, const uint64_t* seeds,
+                     uint32_t* const* mates, bool want, Prof& prof, ListRun& R) {
     cudaStream_t s = e.stream;
     size_t nv = 0, nc = 0, nb = 0, np = 0;
     uint64_t ne = 0, nr = 0;
@@ -850,21 +871,18 @@ static int batch_list(lm_ctx* ctx, Engine& e, const lm_graph* const* gs, uint32_
         nb += list_blocks(gs[i]->ntask, gs[i]->nrows);
         np += list_parts(ctx, gs[i], nr, ne);
     }
-    const bool want = rounds || ctx->lim_rounds;
+    R.rounds = want || ctx->lim_rounds;
+    R.nv = nv;
     int rc = staging_ready(ctx, e);
-    if (!rc) rc = ensure_list(ctx, e, nv, nc, count, nb, np, want);
+    if (!rc) rc = ensure_list(ctx, e, nv, nc, count, nb, np, R.rounds);
     if (!rc) rc = ensure_pinned(ctx, e, count * sizeof(ListSeg));
     if (rc) return rc;
     ListWs& w = e.lw;
-    ListSeg* segs = static_cast<ListSeg*>(e.pinned);
-    std::vector<char> host_dst(count);
-    bool any_host = false;
+    ListSeg* segs = static_cast<ListSeg*>(e.pinned);   // (stays there until the job is done)
     uint32_t vb = 0, cb = 0, bb = 0, pb = 0;
     for (uint32_t i = 0; i < count; i++) {
-        host_dst[i] = !is_device_ptr(mates[i]);
-        any_host |= host_dst[i] != 0;
         ListSeg& sg = segs[i];
-        sg = list_seg(gs[i], seeds[i], host_dst[i] ? w.mate + vb : mates[i]);
+        sg = list_seg(gs[i], seeds[i], is_device_ptr(mates[i]) ? mates[i] : w.mate + vb);
         sg.vbase = vb;
         sg.lbase = cb;
         sg.blk0 = bb;
@@ -876,7 +894,7 @@ static int batch_list(lm_ctx* ctx, Engine& e, const lm_graph* const* gs, uint32_
         bb += sg.nblk;
         pb += sg.nparts;
     }
-    ListArgs A;
+    ListArgs& A = R.A;
     list_args(A, e);
     A.segs = w.segs;
     A.nsegs = count;
@@ -893,28 +911,77 @@ static int batch_list(lm_ctx* ctx, Engine& e, const lm_graph* const* gs, uint32_
     LM_CK(ctx, launch_list_map(s, A, count, w.bmap, w.pmap));
     prof.end();
     prof.begin(LM_K_CAND);
-    LM_CK(ctx, launch_top(s, A, bb, want));
+    LM_CK(ctx, launch_top(s, A, bb, R.rounds));
     prof.end();
-    if (pb) {
-        rc = run_live(ctx, e, A, pb, want, prof);
-        if (rc) return rc;
-    }
+    return LM_OK;
+}
+// a result that waits in the workspace for host memory
+static bool list_staged(const Engine& e, const ListSeg& sg) {
+    return sg.dst >= e.lw.mate && sg.dst < e.lw.mate + e.lw.cap_v;
+}
+// The results of a batch that is done: host results to mates, rounds and matched vertices per
+// graph (either may be NULL).
+int list_batch_finish(lm_ctx* ctx, Engine& e, const ListRun& R, uint32_t* const* mates, uint32_t* rounds,
+                      unsigned long long* matched2) {
+    cudaStream_t s = e.stream;
+    const ListWs& w = e.lw;
+    const ListSeg* segs = static_cast<const ListSeg*>(e.pinned);
+    const uint32_t count = R.A.nsegs;
+    bool any_host = false;
+    for (uint32_t i = 0; i < count; i++) any_host |= list_staged(e, segs[i]);
     std::vector<uint32_t> hmate;
     if (any_host) {
-        hmate.resize(nv);
-        LM_CK(ctx, cudaMemcpyAsync(hmate.data(), w.mate, nv * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+        hmate.resize(R.nv);
+        LM_CK(ctx, cudaMemcpyAsync(hmate.data(), w.mate, R.nv * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
     }
     if (rounds) LM_CK(ctx, cudaMemcpyAsync(rounds, w.grounds, count * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
     if (matched2)
         LM_CK(ctx, cudaMemcpyAsync(matched2, w.gmatched, count * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
-    if (any_host || rounds || matched2 || !pb) LM_CK(ctx, cudaStreamSynchronize(s));
+    if (any_host || rounds || matched2 || !R.A.nparts) LM_CK(ctx, cudaStreamSynchronize(s));
     if (any_host)
         for (uint32_t i = 0; i < count; i++)
-            if (host_dst[i] && gs[i]->n)
-                memcpy(mates[i], hmate.data() + segs[i].vbase, (size_t)gs[i]->n * sizeof(uint32_t));
+            if (mates[i] && list_staged(e, segs[i]))
+                memcpy(mates[i], hmate.data() + segs[i].vbase, (size_t)segs[i].n * sizeof(uint32_t));
+    return LM_OK;
+}
+// Which graphs of a started batch have no live row left after a pass, with their rounds and
+// matched vertices; the host results of those with mates[i] set.
+int list_batch_progress(lm_ctx* ctx, Engine& e, const ListRun& R, uint32_t* const* mates, char* done, uint32_t* rounds,
+                        unsigned long long* matched2) {
+    cudaStream_t s = e.stream;
+    const ListWs& w = e.lw;
+    const ListSeg* segs = static_cast<const ListSeg*>(e.pinned);
+    const uint32_t count = R.A.nsegs;
+    std::vector<uint32_t> left(R.A.nparts);
+    if (R.A.nparts)
+        LM_CK(ctx, cudaMemcpyAsync(left.data(), w.pcount, R.A.nparts * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+    LM_CK(ctx, cudaMemcpyAsync(rounds, w.grounds, count * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+    LM_CK(ctx, cudaMemcpyAsync(matched2, w.gmatched, count * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
+    LM_CK(ctx, cudaStreamSynchronize(s));
+    for (uint32_t i = 0; i < count; i++) {
+        done[i] = 1;
+        for (uint32_t p = 0; p < segs[i].nparts; p++) done[i] = done[i] && (left[segs[i].part0 + p] >> 1) == 0;
+        if (done[i] && mates[i] && segs[i].n && list_staged(e, segs[i]))
+            LM_CK(ctx, cudaMemcpyAsync(mates[i], w.mate + segs[i].vbase, (size_t)segs[i].n * sizeof(uint32_t),
+                                       cudaMemcpyDeviceToHost, s));
+    }
+    LM_CK(ctx, cudaStreamSynchronize(s));
     return LM_OK;
 }
 
+static int batch_list(lm_ctx* ctx, Engine& e, const lm_graph* const* gs, uint32_t count, const uint64_t* seeds,
+                      uint32_t* const* mates, uint32_t* rounds, unsigned long long* matched2, Prof& prof) {
+    ListRun R;
+    int rc = list_batch_start(ctx, e, gs, count, seeds, mates, rounds != nullptr, prof, R);
+    if (!rc && R.A.nparts) rc = run_live(ctx, e, R, prof);
+    return rc ? rc : list_batch_finish(ctx, e, R, mates, rounds, matched2);
+}
+
+// Many graphs on engine e in the same launches (lm_batch_match, and groups of
+// served requests): their vertex and entry ranges are laid side by side in one
+// union id space, each graph keeping its own seed and edge ids.  mates[i] is
+// device or host memory; rounds[i] and matched2[i] receive graph i's round count
+// and matched vertices (either may be NULL).
 int match_batch(lm_ctx* ctx, Engine& e, const lm_graph* const* gs, uint32_t count, const uint64_t* seeds,
                 uint32_t* const* mates, uint32_t* rounds, unsigned long long* matched2, Prof& prof) {
     uint64_t nv = 0, ne = 0;

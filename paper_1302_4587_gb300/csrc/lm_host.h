@@ -171,6 +171,7 @@ inline uint32_t chunks_cap(uint64_t ne, const LaunchCfg& c) {
 }
 
 int engine_init(lm_ctx* ctx, Engine& e, cudaStream_t stream);
+void engine_trim(Engine& e);
 void engine_free(Engine& e);
 int ensure_ws(lm_ctx* ctx, Engine& e, uint32_t nv, uint32_t ne, uint32_t ng);
 int ensure_pinned(lm_ctx* ctx, Engine& e, size_t bytes);
@@ -212,6 +213,23 @@ int match_batch(lm_ctx* ctx, Engine& e, const lm_graph* const* gs, uint32_t coun
                 uint32_t* const* mates, uint32_t* rounds, unsigned long long* matched2, Prof& prof);
 int match_one(lm_ctx* ctx, Engine& e, const lm_graph* g, uint64_t seed, uint32_t* mate, bool dev_out, Prof& prof,
               bool async = false, bool rounds = true, bool counts = false);
+// A job of the list path that is run in steps: started (arguments, first kernel), then passes
+// until the engine's st_host->done is set, then the results (see lm_api.cpp).
+struct ListRun {
+    ListArgs A;
+    bool rounds = false;             // 64-bit words
+    size_t nv = 0;                   // vertices of a batch
+};
+bool list_path(const Engine& e, const lm_graph* g);
+int list_start(lm_ctx* ctx, Engine& e, const lm_graph* g, uint64_t seed, uint32_t* mate, bool dev_out, Prof& prof,
+               bool rounds, ListRun& R);
+int list_batch_start(lm_ctx* ctx, Engine& e, const lm_graph* const* gs, uint32_t count, const uint64_t* seeds,
+                     uint32_t* const* mates, bool want, Prof& prof, ListRun& R);
+int list_pass(lm_ctx* ctx, Engine& e, const ListRun& R, Prof& prof);
+int list_batch_progress(lm_ctx* ctx, Engine& e, const ListRun& R, uint32_t* const* mates, char* done, uint32_t* rounds,
+                        unsigned long long* matched2);
+int list_batch_finish(lm_ctx* ctx, Engine& e, const ListRun& R, uint32_t* const* mates, uint32_t* rounds,
+                      unsigned long long* matched2);
 // the pinned staging (arguments, tables) is free again: the copies a queued
 // (asynchronous) job made from it have run
 int staging_ready(lm_ctx* ctx, Engine& e);

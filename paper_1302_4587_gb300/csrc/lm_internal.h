@@ -298,6 +298,7 @@ struct ListArgs {
     unsigned long long* gmatched;  // [nsegs] matched vertices per graph (NULL: DevState::matched2)
     uint32_t max_rounds;
     unsigned long long limit_ns;
+    unsigned long long slice_ns;  // k_live gives its rows back after this long (0: never; 64-bit words only)
     DevState* st;
     DevState* host;           // its mirror in pinned memory (NULL: nobody waits for it)
 };

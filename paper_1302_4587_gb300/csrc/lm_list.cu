@@ -1056,6 +1056,7 @@ struct LiveSmem {
     PartCounts c;
     uint32_t part, changed, stop, next[2];
     uint32_t red[2][LW];
+    uint64_t begin;   // when the block started
 };
 
 // Blocks take parts from a counter and pass over a part's live rows until none is
@@ -1063,7 +1064,9 @@ struct LiveSmem {
 // good: after IDLE_MAX passes without a change it puts the part's rows back for the
 // next launch, which the last block to leave asks for.  A part's block stops after the
 // pass that matched a row beyond the round cap, the others when they see the error: with
-// rounds at their next pass, else (no cap then, only the time limit) within 16.  (pa: the
+// rounds at their next pass, else (no cap then, only the time limit) within 16.  With a
+// slice, a block also puts back what is left of its parts once that time is over, each after
+// one pass at least, so that a host that shares the GPU among jobs gets it back.  (pa: the
 // arguments in device memory, for a launch in a graph.)
 template <class W>
 __global__ void __launch_bounds__(LT, LMINB) k_live(const __grid_constant__ ListArgs av,
@@ -1077,6 +1080,7 @@ __global__ void __launch_bounds__(LT, LMINB) k_live(const __grid_constant__ List
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t launch = ld_volatile_u32(&st->round);
     uint32_t left = 0;   // thread 0: rows given back
+    if (sizeof(W) == 8 && tid == 0) S.begin = globaltimer_ns();
     for (;;) {
         if (tid == 0) S.part = atomicAdd(&st->task[0], 1u);
         __syncthreads();
@@ -1101,8 +1105,11 @@ __global__ void __launch_bounds__(LT, LMINB) k_live(const __grid_constant__ List
                 S.next[0] = S.next[1] = 0;
                 S.changed = 0;
                 S.stop = 0;
-                if (globaltimer_ns() - st->t0_ns > a.limit_ns) {
+                const uint64_t now = globaltimer_ns();
+                if (now - st->t0_ns > a.limit_ns) {
                     set_err(st, ERR_TIMEOUT, pass);
+                    S.stop = 1;
+                } else if (sizeof(W) == 8 && a.slice_ns && now - S.begin > a.slice_ns) {
                     S.stop = 1;
                 } else if (sizeof(W) == 4 && (pass & 15u) == 15u && ld_volatile_u32(&st->err)) {
                     S.stop = 1;

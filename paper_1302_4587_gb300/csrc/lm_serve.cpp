@@ -1,14 +1,19 @@
 // Serving: lm_submit / lm_poll / lm_wait (include/lm.h).
 //
-// A few lanes (threads, each with its own engine and stream) serve one queue.  A
-// lane that is free takes the requests that wait, in arrival order, as long as they
-// fit the HBM budget and the slots beside those in flight, and runs them together to
-// completion: one by the plain path, several by the batched one, their rows in the
-// same launches.  Requests that arrive meanwhile are taken by the next free lane, so
-// they join the device while earlier ones are on it and leave as soon as their own
-// group is done.  Every request keeps its own seed and edge ids, so its result does not
-// depend on what else is in flight.  When a group fails for want of memory or at a limit
-// (lm_set_limits), its requests run again one by one, so that each gets its own outcome.
+// A few lanes (threads) serve one queue.  A lane takes the requests that wait, in
+// arrival order, as long as they fit the HBM budget and the slots beside those in
+// flight, and runs them together: one by the plain path, several by the batched one,
+// their rows in the same launches.  Requests that arrive meanwhile are taken by the next
+// free lane, so they join the device while earlier ones are on it.  Every request keeps its
+// own seed and edge ids, so its result does not depend on what else is in flight.  When a
+// group fails for want of memory or at a limit (lm_set_limits), the requests that are not
+// done run again one by one, so that each gets its own outcome.
+//
+// A graph can need many rounds (Theta(n) on a path with monotone weights).  So a lane runs a
+// group in slices: after SLICE_NS the live pass gives its rows back, the group's requests
+// that are done leave, and the lane takes what waits as a run of its own (an engine
+// each, up to MAX_RUNS), whose slices alternate with the first one's.  A group that is
+// done within a slice, as nearly all are, never notices.
 //
 // A burst of 48 requests of 1 thousand to 4 million edges takes 1.28 ms with two lanes
 // (1.36 with one, 1.32 with three); stepping all requests together round by round,
@@ -16,6 +21,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <condition_variable>
 #include <cstring>
@@ -45,15 +51,20 @@ struct Request {
 constexpr size_t MAX_QUEUE = 1u << 20;
 constexpr size_t MAX_GROUP = 256;  // requests a lane runs together
 constexpr int LANES = 2;
+constexpr int MAX_RUNS = 8;        // groups a lane has in progress at most
+// (a pass over the largest groups measured takes about 1 ms, a launch and its wait 20 us)
+constexpr unsigned long long SLICE_NS = 4000000ull;
+
+using Clock = std::chrono::steady_clock;
 
 struct ServeState {
     lm_ctx* ctx = nullptr;
-    Engine eng[LANES];
+    Engine eng[LANES][MAX_RUNS];    // the first of each lane from the start, the others when needed
     std::thread th[LANES];
     std::mutex mu;
     std::condition_variable cv_work, cv_done;
     bool stop = false;
-    int fatal = LM_OK;
+    std::atomic<int> fatal{LM_OK};
     uint64_t next_ticket = 1;
     std::deque<Request*> queue;
     std::unordered_map<uint64_t, Request*> all;
@@ -69,103 +80,247 @@ bool fits(const ServeState* S, const Request* r) {
     return S->used_v + r->g->n <= S->cap_v && S->used_e + r->g->nent <= S->cap_e && S->used_slots < S->ctx->max_slots;
 }
 
-int run_group(ServeState* S, Engine& e, const std::vector<Request*>& group, std::vector<uint32_t>& rounds,
-              std::vector<unsigned long long>& m2) {
-    Prof off(nullptr, e.stream);
-    const size_t k = group.size();
-    if (k == 1) {
-        Request* r = group[0];
-        const int rc = match_one(S->ctx, e, r->g, r->seed, r->mate, !r->host_dst, off);
-        if (rc == LM_OK) {
-            rounds[0] = e.st_host->rounds;
-            m2[0] = e.st_host->matched2;
+// A group in progress on an engine of its own.
+struct Run {
+    Engine* e = nullptr;
+    std::vector<Request*> req;       // by place in the group; NULL: has left
+    std::vector<uint32_t*> mates;    // likewise
+    ListRun list;
+    bool started = false;
+    unsigned long long limit_ns = 0; // the group's own time limit,
+    unsigned long long waited = 0;   // and how long it stood between slices, which does not count
+    Clock::time_point paused;
+};
+// What a slice settled: requests with their outcome, or to run again one by one.
+struct Settled {
+    Request* r;
+    int rc;
+    uint32_t rounds;
+    unsigned long long matched2;
+    bool again;
+};
+
+// all requests of the group that have not left, with one outcome
+void settle_all(Run& run, int rc, std::vector<Settled>& out) {
+    const bool again = (rc == LM_ENOMEM || rc == LM_ETIMEOUT) && run.req.size() > 1;
+    for (Request*& r : run.req)
+        if (r) {
+            out.push_back({r, rc, 0, 0, again});
+            r = nullptr;
         }
+}
+void settle(Run& run, size_t i, uint32_t rounds, unsigned long long matched2, std::vector<Settled>& out) {
+    if (!run.req[i]) return;
+    out.push_back({run.req[i], LM_OK, rounds, matched2, false});
+    run.req[i] = nullptr;
+    run.mates[i] = nullptr;
+}
+
+// Starts the group; what the list path does not take (no edges, 2^31 vertices) runs to its end.
+int start(ServeState* S, Run& run, Prof& off, std::vector<Settled>& out) {
+    Engine& e = *run.e;
+    const size_t k = run.req.size();
+    run.started = true;
+    if (k == 1) {
+        Request* r = run.req[0];
+        if (r->g->nent && list_path(e, r->g))
+            return list_start(S->ctx, e, r->g, r->seed, r->mate, !r->host_dst, off, true, run.list);
+        const int rc = match_one(S->ctx, e, r->g, r->seed, r->mate, !r->host_dst, off);
+        if (rc == LM_OK) settle(run, 0, e.st_host->rounds, e.st_host->matched2, out);
         return rc;
     }
     std::vector<const lm_graph*> gs(k);
     std::vector<uint64_t> seeds(k);
-    std::vector<uint32_t*> mates(k);
+    bool listed = true;
     for (size_t i = 0; i < k; i++) {
-        gs[i] = group[i]->g;
-        seeds[i] = group[i]->seed;
-        mates[i] = group[i]->mate;
+        gs[i] = run.req[i]->g;
+        seeds[i] = run.req[i]->seed;
+        listed = listed && list_path(e, gs[i]);
     }
-    return match_batch(S->ctx, e, gs.data(), (uint32_t)k, seeds.data(), mates.data(), rounds.data(), m2.data(), off);
+    if (listed)
+        return list_batch_start(S->ctx, e, gs.data(), (uint32_t)k, seeds.data(), run.mates.data(), true, off, run.list);
+    std::vector<uint32_t> rounds(k);
+    std::vector<unsigned long long> m2(k);
+    const int rc = match_batch(S->ctx, e, gs.data(), (uint32_t)k, seeds.data(), run.mates.data(), rounds.data(), m2.data(), off);
+    if (rc == LM_OK)
+        for (size_t i = 0; i < k; i++) settle(run, i, rounds[i], m2[i], out);
+    return rc;
+}
+
+// A slice of the run (the first one starts it); out: the requests that it settled.
+// Returns whether the run is over.
+bool step(ServeState* S, Run& run, std::vector<Settled>& out) {
+    lm_ctx* ctx = S->ctx;
+    Engine& e = *run.e;
+    Prof off(nullptr, e.stream);
+    const size_t k = run.req.size();
+    int rc = LM_OK;
+    if (!run.started) {
+        rc = start(S, run, off, out);
+        if (rc || !out.empty()) {
+            settle_all(run, rc, out);
+            return true;
+        }
+        run.list.A.slice_ns = SLICE_NS;
+        run.limit_ns = run.list.A.limit_ns;
+    } else {
+        run.waited += (unsigned long long)std::chrono::duration_cast<std::chrono::nanoseconds>(Clock::now() - run.paused).count();
+        run.list.A.limit_ns = run.limit_ns + run.waited;
+    }
+    bool done = run.list.A.nparts == 0;
+    // (a pass may also give rows back early, which wait for one another)
+    const auto end = Clock::now() + std::chrono::nanoseconds(SLICE_NS);
+    while (!done && rc == LM_OK) {
+        rc = list_pass(ctx, e, run.list, off);
+        done = rc == LM_OK && e.st_host->done;
+        if (Clock::now() >= end) break;
+    }
+    run.paused = Clock::now();
+    if (k == 1) {
+        Request* r = run.req[0];
+        if (rc == LM_OK && !done) return false;
+        if (rc == LM_OK && r->host_dst) {
+            cudaError_t ce = cudaMemcpyAsync(r->mate, e.lw.mate, (size_t)r->g->n * 4, cudaMemcpyDeviceToHost, e.stream);
+            if (ce == cudaSuccess) ce = cudaStreamSynchronize(e.stream);
+            if (ce != cudaSuccess) rc = cuda_fail(ctx, ce, "result of a served request");
+        }
+        if (rc == LM_OK) settle(run, 0, e.st_host->rounds, e.st_host->matched2, out);
+        settle_all(run, rc, out);
+        return true;
+    }
+    std::vector<uint32_t> rounds(k);
+    std::vector<unsigned long long> m2(k);
+    if (done) {
+        rc = list_batch_finish(ctx, e, run.list, run.mates.data(), rounds.data(), m2.data());
+        if (rc == LM_OK)
+            for (size_t i = 0; i < k; i++) settle(run, i, rounds[i], m2[i], out);
+        settle_all(run, rc, out);
+        return true;
+    }
+    if (rc == LM_OK || rc == LM_ETIMEOUT) {
+        // those that are done leave (beyond the cap: by themselves again)
+        std::vector<char> fin(k);
+        const int pc = list_batch_progress(ctx, e, run.list, run.mates.data(), fin.data(), rounds.data(), m2.data());
+        if (pc) rc = pc;
+        else
+            for (size_t i = 0; i < k; i++)
+                if (fin[i] && rounds[i] <= run.list.A.max_rounds) settle(run, i, rounds[i], m2[i], out);
+    }
+    if (rc) settle_all(run, rc, out);
+    return rc != LM_OK;
+}
+
+// an engine of the lane that no run uses (NULL: none can be had)
+Engine* free_engine(ServeState* S, int which, const std::vector<std::unique_ptr<Run>>& runs) {
+    for (Engine& e : S->eng[which]) {
+        bool used = false;
+        for (const auto& r : runs) used = used || r->e == &e;
+        if (used) continue;
+        if (e.stream) return &e;
+        cudaStream_t st = nullptr;
+        if (cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        if (engine_init(S->ctx, e, st)) {
+            engine_free(e);
+            cudaStreamDestroy(st);
+            return nullptr;
+        }
+        e.cfg = S->eng[which][0].cfg;
+        return &e;
+    }
+    return nullptr;
 }
 
 void lane(ServeState* S, int which) {
     cudaSetDevice(S->ctx->device);
-    Engine& e = S->eng[which];
+    std::vector<std::unique_ptr<Run>> runs;
+    std::vector<Settled> out;
     std::unique_lock<std::mutex> lk(S->mu);
+    // (a request that does not fit beside those in flight waits for one of them)
+    const auto ready = [&] { return !S->queue.empty() && (S->fatal || fits(S, S->queue.front())); };
     for (;;) {
-        // (a request that does not fit beside those in flight waits for one of them)
-        S->cv_work.wait(lk, [&] { return S->stop || (!S->queue.empty() && (S->fatal || fits(S, S->queue.front()))); });
+        if (runs.empty()) S->cv_work.wait(lk, [&] { return S->stop || ready(); });
         if (S->stop) return;
-        std::vector<Request*> group;
-        uint64_t gv = 0, ge = 0;
-        while (!S->queue.empty() && group.size() < MAX_GROUP && (S->fatal || fits(S, S->queue.front()))) {
-            Request* r = S->queue.front();
-            if (!group.empty() && (r->alone || group[0]->alone)) break;
-            S->queue.pop_front();
-            r->state = 1;
-            gv += r->g->n;
-            ge += r->g->nent;
-            S->used_v += r->g->n;
-            S->used_e += r->g->nent;
-            S->used_slots++;
-            group.push_back(r);
-        }
-        const size_t k = group.size();
-        std::vector<uint32_t> rounds(k);
-        std::vector<unsigned long long> m2(k);
-        int rc = S->fatal;
-        if (!rc) {
+        if (ready() && runs.size() < MAX_RUNS) {
             lk.unlock();
-            rc = run_group(S, e, group, rounds, m2);
+            Engine* e = free_engine(S, which, runs);
             lk.lock();
-        }
-        S->used_v -= gv;
-        S->used_e -= ge;
-        S->used_slots -= (uint32_t)k;
-        if ((rc == LM_ENOMEM || rc == LM_ETIMEOUT) && k > 1) {
-            for (size_t i = k; i-- > 0;) {
-                group[i]->alone = true;
-                group[i]->state = 0;
-                S->queue.push_front(group[i]);
+            auto run = std::make_unique<Run>();
+            run->e = e;
+            while (e && ready() && run->req.size() < MAX_GROUP) {
+                Request* r = S->queue.front();
+                if (!run->req.empty() && (r->alone || run->req[0]->alone)) break;
+                S->queue.pop_front();
+                r->state = 1;
+                S->used_v += r->g->n;
+                S->used_e += r->g->nent;
+                S->used_slots++;
+                run->req.push_back(r);
+                run->mates.push_back(r->mate);
             }
-            S->cv_work.notify_all();
-            continue;
+            if (!run->req.empty()) runs.push_back(std::move(run));
         }
-        if (rc == LM_ECUDA) S->fatal = rc;
-        for (size_t i = 0; i < k; i++) {
-            Request* r = group[i];
-            r->rc = rc;
-            if (rc == LM_OK) {
-                r->rounds = rounds[i];
-                r->matched = m2[i] / 2;
+        for (size_t i = 0; i < runs.size();) {
+            Run& run = *runs[i];
+            bool over = true;
+            out.clear();
+            if (S->fatal) {
+                settle_all(run, S->fatal, out);
+            } else {
+                lk.unlock();
+                over = step(S, run, out);
+                // only a lane's first engine keeps its scratch: the budget holds two of them
+                // beside what is in flight
+                if (over && run.e != &S->eng[which][0]) engine_trim(*run.e);
+                lk.lock();
             }
-            r->state = 2;
+            for (size_t j = out.size(); j-- > 0;) {
+                const Settled& o = out[j];
+                Request* r = o.r;
+                S->used_v -= r->g->n;
+                S->used_e -= r->g->nent;
+                S->used_slots--;
+                if (o.again) {
+                    r->alone = true;
+                    r->state = 0;
+                    S->queue.push_front(r);
+                    continue;
+                }
+                if (o.rc == LM_ECUDA) S->fatal = LM_ECUDA;
+                r->rc = o.rc;
+                r->rounds = o.rounds;
+                r->matched = o.matched2 / 2;
+                r->state = 2;
+            }
+            if (!out.empty()) {
+                S->cv_done.notify_all();
+                if (!S->queue.empty()) S->cv_work.notify_all();  // there is room again
+            }
+            if (over) runs.erase(runs.begin() + (long)i);
+            else i++;
         }
-        S->cv_done.notify_all();
-        if (!S->queue.empty()) S->cv_work.notify_all();  // there is room again
     }
 }
 
 // the lanes' streams and engines back (also of a start that failed half-way)
 void serve_free(ServeState* S) {
-    for (Engine& e : S->eng) {
-        const cudaStream_t st = e.stream;
-        if (!st) continue;
-        engine_free(e);
-        cudaStreamDestroy(st);
-    }
+    for (auto& lane_eng : S->eng)
+        for (Engine& e : lane_eng) {
+            const cudaStream_t st = e.stream;
+            if (!st) continue;
+            engine_free(e);
+            cudaStreamDestroy(st);
+        }
 }
 
 int serve_start(lm_ctx* ctx) {
     if (ctx->serve) return LM_OK;
     std::unique_ptr<ServeState> S(new ServeState());
     S->ctx = ctx;
-    for (Engine& e : S->eng) {
+    for (auto& lane_eng : S->eng) {
+        Engine& e = lane_eng[0];
         cudaStream_t st = nullptr;
         cudaError_t ce = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
         int rc = ce == cudaSuccess ? engine_init(ctx, e, st) : cuda_fail(ctx, ce, "serving stream");
@@ -177,7 +332,7 @@ int serve_start(lm_ctx* ctx) {
         e.cfg = ctx->eng.cfg;  // the context's launch parameters when serving starts
     }
     // what may be in flight at once, from the budget (the list path's scratch takes about
-    // 100 bytes a vertex, and nothing for an entry)
+    // 100 bytes a vertex, and nothing for an entry; the lanes' first engines keep theirs)
     const double B = (double)ctx->budget;
     const double lim = 4.0e9;
     S->cap_e = (uint32_t)std::min(lim, B * 0.80 / 25.0);

@@ -134,3 +134,84 @@ def test_a_request_beyond_a_limit_fails_alone():
             lm.lm_graph_destroy(h)
     finally:
         srv.close()
+
+
+def _serve(srv, handles, mates, seed=5):
+    import paper_1302_4587_gb300 as lm
+    return [lm.lm_submit(srv.ctx, h, seed, m) for h, m in zip(handles, mates)]
+
+
+def _finish(srv, g, ticket, mate, want):
+    import paper_1302_4587_gb300 as lm
+    assert lm.lm_wait(srv.ctx, ticket, 60_000)
+    done, st = lm.lm_poll(srv.ctx, ticket)
+    assert done and st["matched"] == int((want != NIL).sum()) // 2
+    assert np.array_equal(to_u32(mate) if not isinstance(mate, np.ndarray) else mate, want), g.name
+
+
+@pytest.mark.parametrize("host", [False, True], ids=["device", "host"])
+def test_short_requests_leave_before_a_long_one(host):
+    # the path needs 100,000 rounds (half a second), the others a handful; two larger graphs
+    # keep both lanes busy while the others arrive, so that they are taken together
+    import paper_1302_4587_gb300 as lm
+    srv = Lm()
+    try:
+        big = [synth.er(1_000_000, 4_000_000, seed=s) for s in (1, 2)]
+        path = _mono_path(200_001)
+        small = [synth.er(300 + 10 * i, 900 + 50 * i, seed=20 + i) for i in range(12)]
+        order = big + small[:6] + [path] + small[6:]
+        hs = [srv.graph(g) for g in order]
+        want = [oracle.greedy(g.n, g.eu, g.ev, g.w, 5) for g in order]
+        mates = [np.zeros(g.n, np.uint32) if host else srv.torch.empty(g.n, dtype=srv.torch.int32, device="cuda")
+                 for g in order]
+        tickets = _serve(srv, hs, mates)
+        for g, t, m, x in zip(order, tickets, mates, want):
+            if g is not path:
+                _finish(srv, g, t, m, x)
+        assert not lm.lm_poll(srv.ctx, tickets[8])[0]   # still on its way
+        _finish(srv, path, tickets[8], mates[8], want[8])
+        for h in hs:
+            lm.lm_graph_destroy(h)
+    finally:
+        srv.close()
+
+
+def test_arrivals_pass_groups_of_many_rounds():
+    # both lanes are busy with paths of half a second and more when the others arrive
+    import paper_1302_4587_gb300 as lm
+    srv = Lm()
+    try:
+        paths = [_mono_path(200_001 + 2 * i) for i in range(4)]
+        small = [synth.er(300 + 10 * i, 900 + 50 * i, seed=20 + i) for i in range(4)] + [synth.grid(300, 300, 0.05, seed=3)]
+        hp, hs = [srv.graph(g) for g in paths], [srv.graph(g) for g in small]
+        wp, ws = ([oracle.greedy(g.n, g.eu, g.ev, g.w, 5) for g in gs] for gs in (paths, small))
+        new = lambda gs: [srv.torch.empty(g.n, dtype=srv.torch.int32, device="cuda") for g in gs]
+        mp, ms = new(paths), new(small)
+        tp = []
+        for h, m in zip(hp, mp):      # one by one, so that both lanes have some
+            tp += _serve(srv, [h], [m])
+            time.sleep(0.01)
+        for _ in range(3):
+            ts = _serve(srv, hs, ms)
+            for g, t, m, x in zip(small, ts, ms, ws):
+                _finish(srv, g, t, m, x)
+        assert not any(lm.lm_poll(srv.ctx, t)[0] for t in tp)
+        for g, t, m, x in zip(paths, tp, mp, wp):
+            _finish(srv, g, t, m, x)
+        for h in hp + hs:
+            lm.lm_graph_destroy(h)
+    finally:
+        srv.close()
+
+
+def test_destroy_with_a_request_of_many_rounds_in_flight():
+    import paper_1302_4587_gb300 as lm
+    srv = Lm()
+    g = _mono_path(2_000_001)   # a million rounds
+    h = srv.graph(g)
+    mate = srv.torch.empty(g.n, dtype=srv.torch.int32, device="cuda")
+    lm.lm_submit(srv.ctx, h, 1, mate)
+    time.sleep(0.05)
+    t0 = time.perf_counter()
+    srv.close()   # at the next slice, not after all rounds
+    assert time.perf_counter() - t0 < 2
