@@ -586,54 +586,63 @@ int match_edges(lm_ctx* ctx, Engine& e, const lm_graph* g, uint64_t seed, uint32
 }
 
 // Scratch of the list path for nv vertices, nc chunks of long rows, ng graphs, nb blocks
-// of k_top and np parts, with or without the rounds' (grow-only).
+// of k_top and np parts, with or without the rounds' (grow-only).  What has to grow gets
+// room for a quarter more, since cudaFree waits for the whole device, a serving lane's
+// neighbour included; exactly the size asked for at first, and where memory is short.
 static int ensure_list(lm_ctx* ctx, Engine& e, size_t nv, size_t nc, size_t ng, size_t nb, size_t np, bool rounds) {
     ListWs& w = e.lw;
     if (w.block && nv <= w.cap_v && nc <= w.cap_c && ng <= w.cap_g && nb <= w.cap_b && np <= w.cap_p &&
         (w.rounds || !rounds))
         return LM_OK;
     LM_CK(ctx, cudaStreamSynchronize(e.stream));
-    ListWs nw;
-    nw.cap_v = std::max(nv, w.cap_v);
-    nw.cap_c = std::max(nc, w.cap_c);
-    nw.cap_g = std::max(std::max(ng, w.cap_g), (size_t)1);
-    nw.cap_b = std::max(nb, w.cap_b);
-    nw.cap_p = std::max(np, w.cap_p);
-    Carver c;
-    c.add(&nw.cur, nw.cap_v);
-    c.add(&nw.lst, nw.cap_v);
-    c.add(&nw.wide, nw.cap_v);
-    nw.rounds = w.rounds || rounds;
-    if (nw.rounds) {
-        c.add(&nw.rl, nw.cap_v);
-        c.add(&nw.rw, nw.cap_v);
+    const ListWs old = w;
+    if (w.block) cudaFree(w.block);
+    w = ListWs();
+    const bool inject = fault_alloc(ctx);
+    cudaError_t err = cudaErrorMemoryAllocation;
+    for (int room = old.block ? 1 : 0; room >= 0; room--) {
+        ListWs nw;
+        const auto cap = [&](size_t need, size_t had) {
+            return need <= had ? had : need + (room ? std::min<size_t>(need / 4, 1u << 24) : 0);
+        };
+        nw.cap_v = cap(nv, old.cap_v);
+        nw.cap_c = cap(nc, old.cap_c);
+        nw.cap_g = cap(std::max<size_t>(ng, 1), old.cap_g);
+        nw.cap_b = cap(nb, old.cap_b);
+        nw.cap_p = cap(np, old.cap_p);
+        nw.rounds = old.rounds || rounds;
+        Carver c;
+        c.add(&nw.cur, nw.cap_v);
+        c.add(&nw.lst, nw.cap_v);
+        c.add(&nw.wide, nw.cap_v);
+        if (nw.rounds) {
+            c.add(&nw.rl, nw.cap_v);
+            c.add(&nw.rw, nw.cap_v);
+        }
+        for (int k = 0; k < 2; k++) c.add(&nw.list[k], nw.cap_v);
+        c.add(&nw.queue, nw.cap_v);
+        c.add(&nw.mate, nw.cap_v);
+        c.add(&nw.part, LIST_KEPT * nw.cap_c);
+        c.add(&nw.pcnt, nw.cap_c);
+        c.add(&nw.segs, nw.cap_g);
+        c.add(&nw.bmap, nw.cap_b);
+        c.add(&nw.pmap, nw.cap_p);
+        c.add(&nw.pcount, nw.cap_p);
+        c.add(&nw.grounds, nw.cap_g);
+        c.add(&nw.gmatched, nw.cap_g);
+        void* p = nullptr;
+        if (!inject) err = cudaMalloc(&p, c.total);
+        if (err != cudaSuccess) {
+            cudaGetLastError();
+            if (room && !inject) continue;
+            return fail(ctx, LM_ENOMEM, "workspace of %zu bytes: %s", c.total, cudaGetErrorString(err));
+        }
+        c.assign(p);
+        nw.block = p;
+        w = nw;
+        break;
     }
-    for (int k = 0; k < 2; k++) c.add(&nw.list[k], nw.cap_v);
-    c.add(&nw.queue, nw.cap_v);
-    c.add(&nw.mate, nw.cap_v);
-    c.add(&nw.part, LIST_KEPT * nw.cap_c);
-    c.add(&nw.pcnt, nw.cap_c);
-    c.add(&nw.segs, nw.cap_g);
-    c.add(&nw.bmap, nw.cap_b);
-    c.add(&nw.pmap, nw.cap_p);
-    c.add(&nw.pcount, nw.cap_p);
-    c.add(&nw.grounds, nw.cap_g);
-    c.add(&nw.gmatched, nw.cap_g);
-    if (w.block) {
-        cudaFree(w.block);
-        w.block = nullptr;
-    }
-    void* p = nullptr;
-    const cudaError_t err = fault_alloc(ctx) ? cudaErrorMemoryAllocation : cudaMalloc(&p, c.total);
-    if (err != cudaSuccess) {
-        cudaGetLastError();
-        e.lw = ListWs();
-        return fail(ctx, LM_ENOMEM, "workspace of %zu bytes: %s", c.total, cudaGetErrorString(err));
-    }
-    c.assign(p);
-    nw.block = p;
-    e.lw = nw;
-    LM_CK(ctx, cudaMemsetAsync(e.lw.pcnt, 0, std::max<size_t>(nw.cap_c, 1) * sizeof(uint32_t), e.stream));
+    LM_CK(ctx, cudaMemsetAsync(w.pcnt, 0, std::max<size_t>(w.cap_c, 1) * sizeof(uint32_t), e.stream));
     return LM_OK;
 }
 

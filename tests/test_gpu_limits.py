@@ -176,3 +176,27 @@ def test_injected_allocation_failures_return_enomem(monkeypatch):
         lm.lm_graph_destroy(h)
     finally:
         A.close()
+
+
+def test_scratch_that_grows_leaves_room():
+    """Growing frees a block, which waits for the whole device: slightly larger graphs must
+    not do it again and again.  The first growth leaves a quarter more."""
+    L = Lm()
+    try:
+        gs = [synth.er(n, 2 * n, seed=1) for n in (500_000, 510_000, 560_000, 630_000)]
+        hs = [L.graph(g) for g in gs]
+        free = []
+        for g, h in zip(gs, hs):
+            L.torch.cuda.empty_cache()
+            mate = L.torch.empty(g.n, dtype=L.torch.int32, device="cuda")
+            L.lm.lm_match(L.ctx, h, 1, mate)
+            del mate
+            L.torch.cuda.empty_cache()
+            free.append(L.torch.cuda.mem_get_info()[0])
+        assert free[1] < free[0]                  # grown once, by more than it needed,
+        assert free[1] == free[2] == free[3]      # so that these fit
+        for g, h in zip(gs, hs):
+            _exact(L, g, 7, handle=h)
+            L.lm.lm_graph_destroy(h)
+    finally:
+        L.close()
