@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(CT) k_c_keys(const uint32_t* __restrict__ eu, 
 // ---- partitions --------------------------------------------------------------
 // The crossing edges go to 2^pb partitions by the top bits of their hash, as (hash, edge)
 // items in no particular order, each partition in a room of cap items of its own
-// (gcur: its items; more than cap: the count goes on, the items are not kept).  A block
+// (gcur: its items; more than cap: counts[4] is set, the items are not kept).  A block
 // maps and keys a tile of PT_TILE edges, counts them by partition in shared memory
 // (each item's rank is what the count returned), takes a run of every partition's room with
 // one atomic, and writes the tile out in partition order, so that runs of 8 items and
@@ -309,7 +309,11 @@ __global__ void __launch_bounds__(PT_T, 2)
     }
 #pragma unroll
     for (uint32_t i = 0; i < D; i++) {
-        if (c[i]) S.gofs[D * tid + i] = atomicAdd(&gcur[D * tid + i], c[i]) - start;
+        if (c[i]) {
+            const uint32_t had = atomicAdd(&gcur[D * tid + i], c[i]);
+            if (had + c[i] > cap) atomicOr(&counts[4], 1u);
+            S.gofs[D * tid + i] = had - start;
+        }
         S.cnt[D * tid + i] = start;
         start += c[i];
     }
@@ -698,7 +702,7 @@ __global__ void __launch_bounds__(BK_T, 2)
 // over all; scale 22, 62K items: 2150 and 1424).  R-MAT scale 21: 154 us, of which both
 // passes over the items 120 (a bitmap in L2 instead, by atomics of the keys' kernel, cost
 // it 240 us: 130 G atomics/s).
-// counts[4]: a partition outgrew its room (nothing of this is used then).
+// counts[4]: a partition outgrew its room, and the list is sorted instead.
 constexpr uint32_t GP_J = 12;
 template <int B>  // 512 << B threads
 struct GpSmem {
@@ -726,11 +730,10 @@ __global__ void __launch_bounds__(512 << B, 2 >> B)
     extern __shared__ __align__(16) unsigned char gp_raw[];
     SM& S = *reinterpret_cast<SM*>(gp_raw);
     const uint32_t tid = threadIdx.x, lane = tid & 31;
+    // (few pairs with many edges each, 4M edges among 64 vertices: all blocks' work for
+    // nothing took 1.1 ms before the sort's 2.4)
+    if (counts[4]) return;
     const uint32_t total = gcur[blockIdx.x];
-    if (total > cap) {
-        if (tid == 0) atomicOr(&counts[4], 1u);
-        return;
-    }
     const uint2* it = items + (size_t)blockIdx.x * cap;
     for (uint32_t i = tid; i < 1u << (gb - 5); i += GP_T) S.seen[i] = S.rep[i] = 0;
     __syncthreads();

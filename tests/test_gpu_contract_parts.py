@@ -56,6 +56,16 @@ def test_groups_beyond_a_partition(lmc, kind):
     _same(_contract(lmc, n, eu, ev, w, mate), oracle.contract(n, eu, ev, w, mate))
 
 
+@pytest.mark.parametrize("n,m", [(64, 4_000_000), (12, 400_000)])
+def test_few_pairs_outgrow_their_partitions(lmc, n, m):
+    # 2016 and 66 pairs over 512 and 64 partitions: some get more than twice the average of 4
+    # and 1, so the list is sorted
+    rng = np.random.default_rng(n)
+    eu, ev, w = _edges(rng, n, m)
+    for mate in (np.full(n, NIL, np.uint32), oracle.greedy(n, eu, ev, w, 7)):
+        _same(_contract(lmc, n, eu, ev, w, mate), oracle.contract(n, eu, ev, w, mate))
+
+
 @pytest.mark.parametrize("m", [66_000_001, 70_000_000, 135_000_003])
 def test_many_partitions(lmc, m):
     # 1024, 2048 and 4096 partitions, against the sort (which the smaller sizes tie to the
