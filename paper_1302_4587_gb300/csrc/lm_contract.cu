@@ -350,7 +350,7 @@ __global__ void __launch_bounds__(PT_T, 2)
 // and any run that does not fit the walk, is flagged in ofl (a bit per edge) for the
 // general path below: taken out in order with its pair as the key and sorted by the pair
 // (which clears the same bits again).
-constexpr uint32_t GR_MAX = 64, GR_PAIRS = 4;
+constexpr uint32_t GR_MAX = 64, GR_PAIRS = 4, GR_SHORT = 8;
 constexpr uint32_t BK_T = 512, BK_J = 12, BK_W = BK_T * BK_J, BK_C = 4096, BK_TS = 8192, BK_TS_BITS = 13;
 constexpr uint32_t BK_AVG = 2048;  // the sort takes as few bytes as leave at most this many items to a bucket
 constexpr uint32_t BK_EMPTY = 0xFFFFFFFFu;
@@ -364,10 +364,11 @@ struct BkSmem {
         uint32_t dl[BK_W];      // items of runs, slot << 16 | window index, grouped by slot
     };
     uint32_t cnt[BK_TS / 2];    // a 16-bit field per slot: its items, then where its run goes in dl
-    uint32_t dupb[BK_TS / 32];  // slots whose key repeats
+    uint32_t dupb[BK_TS / 32];  // slots whose key repeats,
+    uint32_t longb[BK_TS / 32]; // and those of more than GR_MAX items
     uint32_t hand[BK_J * (BK_T / 32) + 1];  // each warp's last keys, and the key before the window
     uint32_t wsum[BK_T / 32];
-    uint32_t first, lastp1, end, ndup;
+    uint32_t first, lastp1, end, ndup, nmid;
 };
 
 template <uint32_t TSB>
@@ -414,7 +415,7 @@ __device__ __forceinline__ void bk_table(SM& S, const uint32_t (&k)[J], uint32_t
     // slots 16 t .. 16 t + 15, cnt words 8 t .. 8 t + 7)
     {
         uint4* cq = reinterpret_cast<uint4*>(S.cnt) + 2 * tid;
-        uint32_t tot = 0, bits = 0;
+        uint32_t tot = 0, bits = 0, lng = 0;
 #pragma unroll
         for (int v = 0; v < 2; v++) {
             const uint4 x = cq[v];
@@ -425,6 +426,7 @@ __device__ __forceinline__ void bk_table(SM& S, const uint32_t (&k)[J], uint32_t
                 if (c >= 2) {
                     tot += c;
                     bits |= 1u << (8 * v + h);
+                    if (c > GR_MAX) lng |= 1u << (8 * v + h);
                 }
             }
         }
@@ -454,7 +456,11 @@ __device__ __forceinline__ void bk_table(SM& S, const uint32_t (&k)[J], uint32_t
             cq[v] = make_uint4(wv[0], wv[1], wv[2], wv[3]);
         }
         reinterpret_cast<uint16_t*>(S.dupb)[tid] = (uint16_t)bits;  // bit 16 t + h: slot 16 t + h
-        if (tid == T - 1) S.ndup = run;
+        reinterpret_cast<uint16_t*>(S.longb)[tid] = (uint16_t)lng;
+        if (tid == T - 1) {
+            S.ndup = run;
+            S.nmid = 0;
+        }
     }
     __syncthreads();
     // the items of repeated keys into dl, grouped by slot
@@ -471,22 +477,19 @@ __device__ __forceinline__ void bk_table(SM& S, const uint32_t (&k)[J], uint32_t
         }
     }
     __syncthreads();
-    // each run by the thread that holds its first entry: back in input order
-    // (insertion sort on the window index, or on the edge; its entries share their slot
-    // bits, which is all that other threads read of them); a long one is flagged
+    // each run back in input order, by the window index or by the edge: short ones by the
+    // thread that holds their first entry (an insertion sort; its entries share their slot
+    // bits, which is all that other threads read of them), those of more than GR_SHORT
+    // by a warp; long ones are flagged below.  (Slots' cnt: where their runs end.)
     const uint32_t nd = S.ndup;
+    uint32_t* mid = S.tab + T * J;   // their first entries and lengths, behind dl
+    static_assert(T * J / (GR_SHORT + 1) <= TS - T * J && GR_MAX <= 64, "room for them, two items a lane");
     for (uint32_t i = tid; i < nd; i += T) {
         const uint32_t sl = S.dl[i] >> 16;
-        if (i > 0 && (S.dl[i - 1] >> 16) == sl) continue;
-        uint32_t len = 1;
-        while (i + len < nd && (S.dl[i + len] >> 16) == sl) len++;
-        if (len > GR_MAX) {
-            for (uint32_t a = 0; a < len; a++) {
-                const uint32_t p = val[S.dl[i + a] & 0xFFFFu];
-                atomicOr(&ofl[p >> 5], 1u << (p & 31));
-                S.dl[i + a] |= 0xFFFFu;  // (no window index)
-            }
-            atomicAdd(&counts[1], len);
+        if ((i > 0 && (S.dl[i - 1] >> 16) == sl) || ((S.longb[sl >> 5] >> (sl & 31)) & 1u)) continue;
+        const uint32_t len = ((S.cnt[sl >> 1] >> (16 * (sl & 1))) & 0xFFFFu) - i;
+        if (len > GR_SHORT) {
+            mid[atomicAdd(&S.nmid, 1u)] = len << 16 | i;
             continue;
         }
         for (uint32_t a = 1; a < len; a++) {
@@ -502,12 +505,59 @@ __device__ __forceinline__ void bk_table(SM& S, const uint32_t (&k)[J], uint32_t
     }
     if (tid == 0 && nd) S.wsum[0] = atomicAdd(&counts[5], nd);
     __syncthreads();
-    const uint32_t lbase = S.wsum[0];
-    for (uint32_t i = tid; i < nd; i += T) {
-        const uint32_t x = S.dl[i];
-        const bool start = i == 0 || (S.dl[i - 1] >> 16) != (x >> 16);
-        list[lbase + i] = (x & 0xFFFFu) == 0xFFFFu ? RUN_NONE : val[x & 0xFFFFu] | (start ? RUN_START : 0u);
+    const uint32_t nmid = S.nmid;
+    for (uint32_t k = warp; k < nmid; k += T / 32) {
+        const uint32_t i = mid[k] & 0xFFFFu, len = mid[k] >> 16;
+        // items lane and lane + 32, in order by a bitonic network (no item: above all)
+        uint32_t x[2], v[2];
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            const uint32_t q = lane + 32 * h;
+            x[h] = q < len ? S.dl[i + q] : 0u;
+            v[h] = q >= len ? 0xFFFFFFFFu : BYVAL ? val[x[h] & 0xFFFFu] : x[h];
+        }
+#pragma unroll
+        for (uint32_t w = 2; w <= 64; w *= 2)
+#pragma unroll
+            for (uint32_t d = w / 2; d > 0; d /= 2) {
+                if (d == 32) {
+                    if (v[0] > v[1]) {
+                        const uint32_t tv = v[0], tx = x[0];
+                        v[0] = v[1]; x[0] = x[1];
+                        v[1] = tv; x[1] = tx;
+                    }
+                    continue;
+                }
+#pragma unroll
+                for (int h = 0; h < 2; h++) {
+                    const uint32_t ov = __shfl_xor_sync(0xFFFFFFFFu, v[h], d), ox = __shfl_xor_sync(0xFFFFFFFFu, x[h], d);
+                    const bool up = ((lane + 32 * h) & w) == 0, low = (lane & d) == 0;
+                    if ((ov < v[h]) == (up == low) && ov != v[h]) {
+                        v[h] = ov;
+                        x[h] = ox;
+                    }
+                }
+            }
+#pragma unroll
+        for (int h = 0; h < 2; h++)
+            if (lane + 32 * h < len) S.dl[i + lane + 32 * h] = x[h];
     }
+    if (nmid) __syncthreads();
+    const uint32_t lbase = S.wsum[0];
+    uint32_t lng = 0;
+    for (uint32_t i = tid; i < nd; i += T) {
+        const uint32_t x = S.dl[i], sl = x >> 16, e = val[x & 0xFFFFu];
+        const bool start = i == 0 || (S.dl[i - 1] >> 16) != sl;
+        if ((S.longb[sl >> 5] >> (sl & 31)) & 1u) {   // to the general path
+            list[lbase + i] = RUN_NONE;
+            atomicOr(&ofl[e >> 5], 1u << (e & 31));
+            lng++;
+        } else {
+            list[lbase + i] = e | (start ? RUN_START : 0u);
+        }
+    }
+    lng = __reduce_add_sync(0xFFFFFFFFu, lng);
+    if (lane == 0 && lng) atomicAdd(&counts[1], lng);
 }
 
 // The runs of list (counts[5] entries: edges in input order, RUN_START on a run's first; runs
@@ -716,9 +766,9 @@ struct GpSmem {
     };
     uint32_t cnt[1u << (GP_TSB - 1)];
     uint32_t vall[GP_CAP];
-    uint32_t dupb[(1u << GP_TSB) / 32];
+    uint32_t dupb[(1u << GP_TSB) / 32], longb[(1u << GP_TSB) / 32];
     uint32_t wsum[GP_T / 32];
-    uint32_t ndup, nc;
+    uint32_t ndup, nmid, nc;
 };
 
 template <int B>

@@ -66,6 +66,34 @@ def test_few_pairs_outgrow_their_partitions(lmc, n, m):
         _same(_contract(lmc, n, eu, ev, w, mate), oracle.contract(n, eu, ev, w, mate))
 
 
+@pytest.mark.parametrize("bits", [0, 8], ids=["partitions", "sort"])
+@pytest.mark.parametrize("length", [2, 8, 9, 31, 32, 33, 63, 64, 65, 200])
+def test_runs_of_every_length(lmc, length, bits):
+    # runs put in order by a thread (up to 8), by a warp (up to 64), or left to the pair sort;
+    # a few longer and shorter ones among them, all shuffled, orientations mixed
+    lm, rng = lmc.lm, np.random.default_rng(length)
+    n = 5000
+    pairs = 12_000 // length
+    times = np.full(pairs, length)
+    times[::7] = rng.integers(1, 2 * length + 2, times[::7].size)
+    u = rng.integers(0, n, pairs, dtype=np.uint32)
+    v = ((u + rng.integers(1, n, pairs, dtype=np.uint32)) % n).astype(np.uint32)
+    eu, ev = np.repeat(u, times), np.repeat(v, times)
+    p = rng.permutation(eu.size)
+    eu, ev = eu[p], ev[p]
+    flip = rng.random(eu.size) < 0.5
+    eu, ev = np.where(flip, ev, eu), np.where(flip, eu, ev)
+    w = rng.standard_normal(eu.size).astype(np.float32)
+    mate = np.full(n, NIL, np.uint32)
+    keep = lm.lm_get_tuning(lmc.ctx)
+    tune = {x: keep[x] for x in ("rmax", "chunk", "sweep_ctas_per_sm", "vertex_ctas_per_sm", "batch")}
+    try:
+        lm.lm_set_tuning(lmc.ctx, **tune, contract_bits=bits)
+        _same(_contract(lmc, n, eu, ev, w, mate), oracle.contract(n, eu, ev, w, mate))
+    finally:
+        lm.lm_set_tuning(lmc.ctx, **tune, contract_bits=keep["contract_bits"])
+
+
 @pytest.mark.parametrize("m", [66_000_001, 70_000_000, 135_000_003])
 def test_many_partitions(lmc, m):
     # 1024, 2048 and 4096 partitions, against the sort (which the smaller sizes tie to the
