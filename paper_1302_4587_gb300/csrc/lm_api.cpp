@@ -1225,6 +1225,7 @@ int lm_graph_create(lm_ctx* ctx, uint32_t n, uint32_t m, const uint32_t* eu, con
         tc.add(&t_w, m);
     }
     tc.add(&bt.deg, nn);
+    if (build_apart(n, m)) tc.add(&bt.degu, nn);
     tc.add(&flags, nn);
     tc.add(&rowidx, nn);
     tc.add(&scan_tmp, scan_words);
@@ -1264,6 +1265,7 @@ int lm_graph_create(lm_ctx* ctx, uint32_t n, uint32_t m, const uint32_t* eu, con
     bt.edges = g->edges;
     bt.eword = g->eword;
     LM_CK(ctx, cudaMemsetAsync(bt.deg, 0, nn * 4, s));
+    if (bt.degu) LM_CK(ctx, cudaMemsetAsync(bt.degu, 0, nn * 4, s));
     LM_CK(ctx, cudaMemsetAsync(bt.err, 0, 48, s));
     // validation rides on the passes: endpoint < n and no self loop on the degree count, no NaN on
     // the fill
@@ -1304,7 +1306,7 @@ int lm_graph_create(lm_ctx* ctx, uint32_t n, uint32_t m, const uint32_t* eu, con
     int rc = ensure_pinned(ctx, e, 64);  // 16 words
     if (rc) return rc;
     uint32_t* hp = static_cast<uint32_t*>(e.pinned);
-    LM_CK(ctx, launch_nonzero_flags(s, bt.deg, n + 1, flags, bt.err + 4));
+    LM_CK(ctx, launch_nonzero_flags(s, bt, n + 1, flags, bt.err + 4));
     LM_CK(ctx, launch_exclusive_scan(s, flags, rowidx, n + 1, scan_tmp, scan_words));
     LM_CK(ctx, launch_build_counts(s, bt.err, rowidx + n, hp));
     LM_CK(ctx, cudaStreamSynchronize(s));
@@ -1328,7 +1330,7 @@ int lm_graph_create(lm_ctx* ctx, uint32_t n, uint32_t m, const uint32_t* eu, con
     gc.assign(g->block[1]);
     g->bytes = ec.total + gc.total;
     LM_CK(ctx, launch_exclusive_scan(s, bt.deg, g->off, n + 1, scan_tmp, scan_words));
-    LM_CK(ctx, launch_build_rows(s, bt.deg, rowidx, g->off, n, g->nrows, g->nent, g->vid, g->rdeg, g->roff, g->task,
+    LM_CK(ctx, launch_build_rows(s, bt, rowidx, g->off, n, g->nrows, g->nent, g->vid, g->rdeg, g->roff, g->task,
                                  g->ntask[3], bt.err + 8));
     if (g->nrows) {
         LM_CK(ctx, cudaMemsetAsync(g->rbits, 0, ((size_t)g->ntiles * (TILE0 / 32) + 8) * 4, s));

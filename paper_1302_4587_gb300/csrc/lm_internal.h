@@ -398,16 +398,20 @@ int launch_edge_round(void* stream, const EdgeArgs* dargs, int phase);  // phase
 void destroy_job_graph(void* exec);
 
 // graph construction
-// scratch and outputs of the build's passes (see k_build_degrees): deg is zero before them
+// scratch and outputs of the build's passes (see k_build_degrees): deg and degu are zero before them
 struct BuildTmp {
     uint32_t* deg;            // [n + 1] degrees
+    // NULL, or the ends apart: deg is the second ends of each vertex, then (launch_nonzero_flags) its
+    // degree; [n + 1] first ends, then (launch_build_rows) the place of its first second end
+    uint32_t* degu;
     uint32_t* err;            // bit 0: invalid input, 1: a place outside 2m
-    uint2* rank;              // [m] rank of either end among its vertex's entries
+    uint2* rank;              // [m] rank of either end among its vertex's entries (apart: of its kind)
     uint32_t *hist, *offs;    // [build_scan_count(m)] second ends per bucket and tile, their prefix
     uint4* vrec;              // [m] second-end records in bucket order
     uint64_t* edges;          // [m] edge records (the graph's own)
     uint32_t* eword;          // [m] ord(weight) (the graph's own)
 };
+bool build_apart(uint32_t n, uint32_t m);
 uint32_t build_scan_count(uint32_t m);
 uint32_t build_step(uint32_t m, uint32_t chunks);  // edges a chunk of the degree pass (whole tiles)
 // degrees, ranks, records and bucket counts of edges first .. first + count - 1 (first: whole tiles)
@@ -425,13 +429,13 @@ size_t exclusive_scan_tmp_words(uint32_t count);
 // (err[4..7]), written straight to pinned memory, and their cursors to err[8..11]
 int launch_build_counts(void* stream, uint32_t* err, const uint32_t* nrows, uint32_t* host);
 // cursors: the next place in task of each kind
-int launch_build_rows(void* stream, const uint32_t* deg, const uint32_t* rowidx_excl, const uint32_t* off,
+int launch_build_rows(void* stream, const BuildTmp& t, const uint32_t* rowidx_excl, const uint32_t* off,
                       uint32_t n, uint32_t nrows, uint32_t nent, uint32_t* vid0, uint32_t* rdeg0, uint32_t* roff,
                       uint4* task, uint32_t ntask, uint32_t* cursors);
 int launch_build_tilemap(void* stream, const uint32_t* roff, uint32_t nrows, uint32_t nent, uint32_t* tmap,
                          uint32_t* rbits, uint4* tdesc);
-// flags[v] = deg[v] != 0; counts[0 .. 3] += the tasks of each kind (see ListSeg::ntask)
-int launch_nonzero_flags(void* stream, const uint32_t* deg, uint32_t n, uint32_t* flags, uint32_t* counts);
+// t.deg[v] += t.degu[v] (if any); flags[v] = t.deg[v] != 0; counts[0 .. 3] += the tasks of each kind (see ListSeg::ntask)
+int launch_nonzero_flags(void* stream, const BuildTmp& t, uint32_t n, uint32_t* flags, uint32_t* counts);
 // union set-up of a batch: for every graph g (vertices [gvbase[g], gvbase[g+1])):
 // start[v] = ebase[g] + off_g[v - gvbase[g]], gid[v] = g, len0[v] = degree
 int launch_union_setup(void* stream, const uint32_t* gvbase, const uint32_t* ebase, const uint32_t* const* offs,

@@ -1395,7 +1395,7 @@ static_assert(BF_TILE % (BF_T * BF_U) == 0 && BF_T == BF_NB, "whole steps, a thr
 
 __global__ void __launch_bounds__(BF_T) k_build_degrees(const uint32_t* __restrict__ eu, const uint32_t* __restrict__ ev,
                                                         uint32_t n, uint32_t m, uint32_t first, uint32_t shift,
-                                                        uint32_t tiles, uint32_t* deg, uint32_t* err,
+                                                        uint32_t tiles, uint32_t* degu, uint32_t* degv, uint32_t* err,
                                                         uint2* __restrict__ rank, uint64_t* __restrict__ edges,
                                                         uint32_t* __restrict__ hist) {
     __shared__ uint32_t h[BF_NB];
@@ -1428,8 +1428,8 @@ __global__ void __launch_bounds__(BF_T) k_build_degrees(const uint32_t* __restri
         uint32_t ru[BF_U], rv[BF_U];
 #pragma unroll
         for (uint32_t q = 0; q < BF_U; q++) {
-            ru[q] = warp_add(&deg[ok[q] ? u[q] : 0], u[q], ok[q], lane);
-            rv[q] = warp_add(&deg[ok[q] ? v[q] : 0], v[q], ok[q], lane);
+            ru[q] = warp_add(&degu[ok[q] ? u[q] : 0], u[q], ok[q], lane);
+            rv[q] = warp_add(&degv[ok[q] ? v[q] : 0], v[q], ok[q], lane);
         }
 #pragma unroll
         for (uint32_t q = 0; q < BF_U; q++) {
@@ -1444,7 +1444,7 @@ __global__ void __launch_bounds__(BF_T) k_build_degrees(const uint32_t* __restri
 __global__ void __launch_bounds__(BF_T) k_build_fill_u(const uint64_t* __restrict__ edges,
                                                        const float* __restrict__ w, uint32_t* __restrict__ eword,
                                                        const uint2* __restrict__ rank, const uint32_t* __restrict__ off,
-                                                       uint32_t first, uint32_t m_all, uint32_t m, uint32_t shift,
+                                                       const uint32_t* __restrict__ offv, uint32_t first, uint32_t m_all, uint32_t m, uint32_t shift,
                                                        uint32_t tiles, const uint32_t* __restrict__ offs,
                                                        uint32_t* __restrict__ eid,
                                                        uint64_t* __restrict__ ent, uint4* __restrict__ vrec,
@@ -1469,7 +1469,7 @@ __global__ void __launch_bounds__(BF_T) k_build_fill_u(const uint64_t* __restric
 #pragma unroll
         for (uint32_t q = 0; q < BF_U; q++) {
             pu[q] = __ldg(off + (uint32_t)rec[q]) + r[q].x;
-            pv[q] = __ldg(off + (uint32_t)(rec[q] >> 32)) + r[q].y;
+            pv[q] = __ldg(offv + (uint32_t)(rec[q] >> 32)) + r[q].y;
         }
 #pragma unroll
         for (uint32_t q = 0; q < BF_U; q++) {
@@ -1511,14 +1511,16 @@ __global__ void __launch_bounds__(BF_T) k_build_fill_v(const uint4* __restrict__
 __device__ __forceinline__ uint32_t task_kind(uint32_t d) {
     return d > LIST_CHUNK ? 0u : d > LIST_WARP ? 1u : d > LIST_GROUP ? 2u : d > LIST_SHORT ? 3u : 4u;
 }
-__global__ void k_nonzero_flags(const uint32_t* deg, uint32_t n, uint32_t* flags, uint32_t* counts) {
+__global__ void k_nonzero_flags(uint32_t* deg, const uint32_t* degu, uint32_t n, uint32_t* flags, uint32_t* counts) {
     __shared__ uint32_t s[4];
     if (threadIdx.x < 4) s[threadIdx.x] = 0;
     __syncthreads();
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     uint32_t c[4] = {0, 0, 0, 0};
     for (uint64_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
-        const uint32_t d = deg[v], k = task_kind(d);
+        uint32_t d = deg[v];
+        if (degu) deg[v] = d += degu[v];
+        const uint32_t k = task_kind(d);
         flags[v] = d ? 1u : 0u;
 #pragma unroll
         for (uint32_t q = 0; q < 4; q++)
@@ -1549,8 +1551,9 @@ __global__ void k_build_counts(uint32_t* err, const uint32_t* nrows, uint32_t* h
 }
 
 // The compact row arrays, and the list path's tasks, each kind from its cursor on; a
-// block reserves its 256 vertices' places with one atomic per kind.
-__global__ void __launch_bounds__(256) k_build_rows(const uint32_t* deg, const uint32_t* rowidx, const uint32_t* off,
+// block reserves its 256 vertices' places with one atomic per kind.  degu (or NULL): first
+// ends, then where the second ends of a row start.
+__global__ void __launch_bounds__(256) k_build_rows(const uint32_t* deg, uint32_t* degu, const uint32_t* rowidx, const uint32_t* off,
                                                     uint32_t n, uint32_t nrows, uint32_t nent, uint32_t* vid0,
                                                     uint32_t* rdeg0, uint32_t* roff, uint4* task, uint32_t ntask,
                                                     uint32_t* cursors) {
@@ -1563,6 +1566,7 @@ __global__ void __launch_bounds__(256) k_build_rows(const uint32_t* deg, const u
         if (d) {
             const uint32_t i = rowidx[v];
             o = off[v];
+            if (degu) degu[v] += o;
             vid0[i] = (uint32_t)v;
             rdeg0[i] = d;
             roff[i] = o;
@@ -1893,6 +1897,14 @@ static uint32_t build_shift(uint32_t n) {  // bucket = v >> shift, below 256
     while (((uint64_t)(n - 1) >> shift) > BF_NB - 1) shift++;
     return shift;
 }
+// Rows of first ends, then second ends, from an average degree of 48 on: each half of a row is
+// then written from one end to the other by its pass, whose open sectors L2 holds; with
+// the ends mixed a pass leaves half of every sector to the other one.  Shorter rows are a few
+// sectors in all, and counts of their own cost more than that.  Uniform graphs of 8M edges, apart and
+// mixed: degree 512 781 and 990 us, 64 879 and 1008, 32 1007 and 1053, 4 1247 and 1178;
+// 32M edges: 64 3.98 and 4.14 ms, 32 4.35 and 4.31, 4 6.49 and 5.40; 100M: 128 12.5 and 13.1,
+// 64 13.7 and 13.7, 16 18.4 and 15.7.
+bool build_apart(uint32_t n, uint32_t m) { return m / 24 >= n; }
 static uint32_t build_tiles(uint32_t m) { return (uint32_t)(((uint64_t)m + BF_TILE - 1) / BF_TILE); }
 uint32_t build_scan_count(uint32_t m) { return BF_NB * build_tiles(m); }
 uint32_t build_step(uint32_t m, uint32_t chunks) {
@@ -1904,7 +1916,7 @@ int launch_build_degrees(void* stream, const uint32_t* eu, const uint32_t* ev, u
     if (first % BF_TILE) return (int)cudaErrorInvalidValue;
     // (the arrays are those of the whole list; edges first .. first + count - 1 are there)
     k_build_degrees<<<build_tiles(count), BF_T, 0, (cudaStream_t)stream>>>(
-        eu, ev, n, first + count, first, build_shift(n), build_tiles(m), t.deg, t.err, t.rank, t.edges, t.hist);
+        eu, ev, n, first + count, first, build_shift(n), build_tiles(m), t.degu ? t.degu : t.deg, t.deg, t.err, t.rank, t.edges, t.hist);
     return (int)cudaGetLastError();
 }
 int launch_build_fill_u(void* stream, const float* w, uint32_t n, uint32_t m, uint32_t first, uint32_t count,
@@ -1912,7 +1924,7 @@ int launch_build_fill_u(void* stream, const float* w, uint32_t n, uint32_t m, ui
     if (count == 0) return 0;
     if (first % BF_TILE) return (int)cudaErrorInvalidValue;
     k_build_fill_u<<<build_tiles(count), BF_T, 0, (cudaStream_t)stream>>>(
-        t.edges, w, t.eword, t.rank, off, first, m, first + count, build_shift(n), build_tiles(m), t.offs, eid, ent,
+        t.edges, w, t.eword, t.rank, off, t.degu ? t.degu : off, first, m, first + count, build_shift(n), build_tiles(m), t.offs, eid, ent,
         t.vrec, t.err);
     return (int)cudaGetLastError();
 }
@@ -1920,18 +1932,18 @@ int launch_build_fill_v(void* stream, uint32_t m, uint32_t* eid, uint64_t* ent, 
     k_build_fill_v<<<(uint32_t)(((uint64_t)m + BF_T - 1) / BF_T), BF_T, 0, (cudaStream_t)stream>>>(t.vrec, m, eid, ent);
     return (int)cudaGetLastError();
 }
-int launch_nonzero_flags(void* stream, const uint32_t* deg, uint32_t n, uint32_t* flags, uint32_t* counts) {
-    k_nonzero_flags<<<grid_for(n, 256), 256, 0, (cudaStream_t)stream>>>(deg, n, flags, counts);
+int launch_nonzero_flags(void* stream, const BuildTmp& t, uint32_t n, uint32_t* flags, uint32_t* counts) {
+    k_nonzero_flags<<<grid_for(n, 256), 256, 0, (cudaStream_t)stream>>>(t.deg, t.degu, n, flags, counts);
     return (int)cudaGetLastError();
 }
 int launch_build_counts(void* stream, uint32_t* err, const uint32_t* nrows, uint32_t* host) {
     k_build_counts<<<1, 1, 0, (cudaStream_t)stream>>>(err, nrows, host);
     return (int)cudaGetLastError();
 }
-int launch_build_rows(void* stream, const uint32_t* deg, const uint32_t* rowidx_excl, const uint32_t* off,
+int launch_build_rows(void* stream, const BuildTmp& t, const uint32_t* rowidx_excl, const uint32_t* off,
                       uint32_t n, uint32_t nrows, uint32_t nent, uint32_t* vid0, uint32_t* rdeg0, uint32_t* roff,
                       uint4* task, uint32_t ntask, uint32_t* cursors) {
-    k_build_rows<<<grid_for(n, 256), 256, 0, (cudaStream_t)stream>>>(deg, rowidx_excl, off, n, nrows, nent, vid0,
+    k_build_rows<<<grid_for(n, 256), 256, 0, (cudaStream_t)stream>>>(t.deg, t.degu, rowidx_excl, off, n, nrows, nent, vid0,
                                                                      rdeg0, roff, task, ntask, cursors);
     return (int)cudaGetLastError();
 }
