@@ -1270,7 +1270,8 @@ int lm_graph_create(lm_ctx* ctx, uint32_t n, uint32_t m, const uint32_t* eu, con
     // validation rides on the passes: endpoint < n and no self loop on the degree count, no NaN on
     // the fill
     const bool upload = mem == LM_HOST && m > 0;
-    const uint32_t step = upload ? build_step(m, lm_ctx::UP_CHUNKS) : m;
+    const uint32_t chunks = std::max(1u, std::min(m / lm_ctx::UP_EDGES, lm_ctx::UP_CHUNKS));
+    const uint32_t step = upload ? build_step(m, chunks) : m;
     // no return before the uploads have read the caller's arrays and left the staging
     struct UpWait {
         cudaStream_t s;

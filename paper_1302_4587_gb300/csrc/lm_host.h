@@ -117,7 +117,11 @@ struct lm_ctx {
     // upload of a host edge list in chunks on its own stream, each chunk's degree
     // count on the context's stream while the next chunk is in flight
     cudaStream_t up = nullptr;
-    static constexpr uint32_t UP_CHUNKS = 8;  // chunks of an uploaded edge list
+    // chunks of an uploaded edge list, of at least UP_EDGES edges: a chunk is nine calls, about
+    // 25 us of the host's time, in which the link moves 5 MB (creation from pinned arrays, eight
+    // chunks always, chunks of 256K, 1M, 2M edges: 50,000 edges 338, 151, 155, 155 us, 1M 432, 266, 235,
+    // 234, 4M 705, 702, 695, 700; from pageable ones 4M 991, 1005, 848, 739)
+    static constexpr uint32_t UP_CHUNKS = 8, UP_EDGES = 1u << 21;
     cudaEvent_t up_ev = nullptr, up_w[UP_CHUNKS] = {};
     // limits of every match (lm_set_limits): a round cap (0 = none beyond m + 2)
     // and a time limit in ns (0 = LOOP_LIMIT_NS)

@@ -86,8 +86,8 @@ def test_host_and_device_outputs_agree(lmctx):
 
 @pytest.mark.parametrize("m", [1, 31, 33, 255, 257, 4099])
 def test_host_upload_in_chunks(lmctx, m):
-    # graphs from host arrays go up in eight chunks of a multiple of 32 edges,
-    # each chunk's degrees counted as it lands: sizes around that rounding
+    # graphs from small host arrays go up in one chunk (several: see below), in whole tiles:
+    # sizes around a warp, a block and a tile
     g = synth.pairs(max(4, m // 3), m, m, "uniform")
     h = lmctx.graph(g, device=False)
     try:
@@ -311,3 +311,30 @@ def test_rmat_scale23_full_parity(lmgraph):
     assert bad.size == 0, f"{bad.size} vertices differ"
     assert st["matched"] == int((want != NIL).sum()) // 2
     assert st["rounds"] <= 3 * math.ceil(math.log2(g.m + 1)) + 4
+
+
+@pytest.mark.parametrize("m", [(1 << 22) - 1, 1 << 22, (1 << 22) + 4097, 3 << 21])
+def test_host_lists_in_one_and_several_chunks(lmctx, m):
+    # chunks of at least 2^21 edges: one, two, two of uneven size, three; as from device memory,
+    # and what the first and last chunk hold wrong is found
+    import paper_1302_4587_gb300 as lm
+    rng = np.random.default_rng(m)
+    n = 300_000
+    eu = rng.integers(0, n, m, dtype=np.uint32)
+    ev = ((eu + rng.integers(1, n, m, dtype=np.uint32)) % n).astype(np.uint32)
+    g = synth.Graph(n, eu, ev, rng.random(m, dtype=np.float32), f"chunks{m}")
+    got = []
+    for device in (True, False):
+        h = lmctx.graph(g, device=device)
+        got.append(lmctx.match(g, 5, handle=h)[0])
+        lm.lm_graph_destroy(h)
+    assert np.array_equal(*got)
+    assert np.array_equal(got[0], oracle.greedy(n, g.eu, g.ev, g.w, 5))
+    for at in (7, m - 1):
+        for a, bad in ((g.eu, n), (g.ev, int(g.eu[at])), (g.w, np.nan)):
+            keep = a[at]
+            a[at] = bad
+            with pytest.raises(lm.LmError) as ei:
+                lmctx.graph(g, device=False)
+            assert ei.value.code == lm.LM_EINVAL
+            a[at] = keep
