@@ -687,7 +687,7 @@ static ListSeg list_seg(const lm_graph* g, uint64_t seed, uint32_t* dst) {
     d.m = g->m;
     d.nrows = g->nrows;
     memcpy(d.ntask, g->ntask, sizeof d.ntask);
-    d.nblk = list_blocks(g->ntask, g->nrows);
+    d.nblk = list_blocks(g->ntask, g->nrows, g->n);
     d.k0 = (uint32_t)z;
     d.k1 = (uint32_t)(z >> 32);
     d.seed = seed;
@@ -877,7 +877,7 @@ int list_batch_start(lm_ctx* ctx, Engine& e, const lm_graph* const* gs, uint32_t
     for (uint32_t i = 0; i < count; i++) {
         nv += gs[i]->n;
         nc += gs[i]->ntask[0];
-        nb += list_blocks(gs[i]->ntask, gs[i]->nrows);
+        nb += list_blocks(gs[i]->ntask, gs[i]->nrows, gs[i]->n);
         np += list_parts(ctx, gs[i], nr, ne);
     }
     R.rounds = want || ctx->lim_rounds;

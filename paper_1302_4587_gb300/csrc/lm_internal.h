@@ -383,7 +383,7 @@ int launch_job_graph(void* exec, void* stream);
 // list path (lm_list.cu): blocks of k_top for one graph, the maps for several, and the launches
 // (rounds: 64-bit words)
 uint32_t list_live_blocks(int device);  // blocks of k_live that run at once
-uint32_t list_blocks(const uint32_t task[4], uint32_t nrows);
+uint32_t list_blocks(const uint32_t task[4], uint32_t nrows, uint32_t n);
 int launch_list_map(void* stream, const ListArgs& a, uint32_t nsegs, uint32_t* bmap, uint32_t* pmap);
 int launch_top(void* stream, const ListArgs& a, uint32_t blocks, bool rounds);
 int launch_live(void* stream, const ListArgs& a, uint32_t nparts, bool rounds);

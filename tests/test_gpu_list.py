@@ -148,3 +148,33 @@ def test_batches_queued_matches_and_host_results(L):
         lm.lm_destroy(actx)
         for h in hs:
             lm.lm_graph_destroy(h)
+
+
+@pytest.mark.parametrize("n", [4095, 4096, 4097, 100_000, 5_000_001])
+def test_few_edges_among_many_vertices(n):
+    # the vertices without edges have blocks of their own that clear their results; alone, in a
+    # batch between others, and with rounds wanted
+    import paper_1302_4587_gb300 as lm
+    L = Lm()
+    torch = L.torch
+    try:
+        rng = np.random.default_rng(n)
+        eu = rng.permutation(n)[:120].astype(np.uint32)
+        ev = np.concatenate([eu[1:], eu[:1]])
+        g = synth.Graph(n, eu, ev, rng.random(120, dtype=np.float32), f"sparse{n}")
+        want = oracle.greedy(n, g.eu, g.ev, g.w, 3)
+        other = synth.er(500, 2000, seed=4)
+        h, ho = L.graph(g), L.graph(other)
+        for stats in (False, True):
+            mate = torch.full((n,), 7, dtype=torch.int32, device="cuda")
+            lm.lm_match(L.ctx, h, 3, mate, stats=stats)
+            assert np.array_equal(mate.cpu().numpy().view(np.uint32), want)
+            mates = [torch.full((k,), 7, dtype=torch.int32, device="cuda") for k in (500, n, 500)]
+            lm.lm_batch_match(L.ctx, [ho, h, ho], [3, 3, 3], mates, stats=stats)
+            assert np.array_equal(mates[1].cpu().numpy().view(np.uint32), want)
+            assert np.array_equal(mates[2].cpu().numpy().view(np.uint32),
+                                  oracle.greedy(500, other.eu, other.ev, other.w, 3))
+        lm.lm_graph_destroy(h)
+        lm.lm_graph_destroy(ho)
+    finally:
+        L.close()
