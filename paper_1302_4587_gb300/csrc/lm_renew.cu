@@ -30,6 +30,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "../../include/lm.h"
 #include "lm_device.cuh"
 #include "lm_internal.h"
@@ -488,14 +490,16 @@ __global__ void __launch_bounds__(RT, RMINB) k_renew(const __grid_constant__ Ren
 
 }  // namespace
 
-// (every block resident, and no more than have a warp's work)
+// (every block resident, and no more than have work)
 int launch_renew(void* stream, const RenewArgs& a, bool counts) {
     int dev = 0;
     cudaGetDevice(&dev);
     const uint32_t* t = a.g.ntask;
     const uint64_t warps = (uint64_t)t[2] + (t[3] - t[2] + 7) / 8 + (a.g.nrows + 31) / 32;
     const uint64_t most = (uint64_t)device_sm_count(dev) * RMINB;
-    const uint64_t want = (warps + RW - 1) / RW;
+    // (a graph with few edges: blocks that clear its result, 64 vertices a thread; by its rows'
+    // block alone 5M vertices and 100 edges took 749 us)
+    const uint64_t want = std::max((warps + RW - 1) / RW, (uint64_t)a.g.n / (64 * RT));
     const uint32_t grid = (uint32_t)(want < 1 ? 1 : want < most ? want : most);
     static_assert(BAR < RENEW_CTRS, "counters");
     const cudaError_t e = cudaMemsetAsync(a.ctr, 0, RENEW_CTRS * sizeof(uint32_t), (cudaStream_t)stream);

@@ -82,3 +82,13 @@ def test_queued(rn):
             lm.lm_graph_destroy(h)
     finally:
         lm.lm_destroy(ctx)
+
+
+@pytest.mark.parametrize("n", [16_383, 16_384, 40_000, 5_000_001])
+def test_few_edges_among_many_vertices(rn, n):
+    # blocks beyond those that the rows need clear the result
+    rng = np.random.default_rng(n)
+    eu = rng.permutation(n)[:300].astype(np.uint32)
+    ev = np.concatenate([eu[1:], eu[:1]])
+    w = rng.integers(1, 3, 300).astype(np.float32)
+    _check(rn, synth.Graph(n, eu, ev, w, f"sparse{n}"), 5)
