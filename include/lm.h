@@ -252,6 +252,8 @@ int  lm_set_tuning(lm_ctx* ctx, const lm_tuning* t);
  * own workload -- lm_match of g[0] when count == 1, lm_batch_match of the
  * `count` graphs otherwise (one warm-up call and three timed calls each) --
  * keeps the fastest in the context and returns it in *best (best may be NULL).
+ * A workload whose path does not use the parameters (see lm_tuning) is timed with the
+ * current ones only, which stay and are returned with its time.
  * mates receive the results as in lm_batch_match.  Errors: as lm_batch_match. */
 int  lm_autotune(lm_ctx* ctx, const lm_graph* const* g, uint32_t count, const uint64_t* seeds,
                  uint32_t* const* mates, lm_tuning* best);

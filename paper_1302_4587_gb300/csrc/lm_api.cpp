@@ -1572,6 +1572,14 @@ void tuning_of(const LaunchCfg& c, lm_tuning* t) {
     t->contract_bits = c.contract_bits;
     t->ms = 0.0;
 }
+// whether a match of these graphs takes the round-by-round path, which the task sizes and
+// CTAs shape (see match_one, match_batch)
+bool reads_tuning(const lm_ctx* ctx, const lm_graph* const* g, uint32_t count) {
+    if (count == 1) return !(ctx->flags & LM_F_EDGE_CENTRIC) && g[0]->nent && g[0]->n >= 0x80000000u;
+    for (uint32_t i = 0; i < count; i++)
+        if (!list_path(ctx->eng, g[i])) return true;
+    return false;
+}
 }  // namespace
 
 int lm_set_limits(lm_ctx* ctx, uint32_t max_rounds, uint32_t time_limit_ms) {
@@ -1602,32 +1610,44 @@ int lm_autotune(lm_ctx* ctx, const lm_graph* const* g, uint32_t count, const uin
                 uint32_t* const* mates, lm_tuning* best) {
     if (!ctx) return LM_EINVAL;
     if (count == 0 || !g || !seeds || !mates) return fail(ctx, LM_EINVAL, "nothing to tune on");
+    for (uint32_t i = 0; i < count; i++)
+        if (!g[i]) return fail(ctx, LM_EINVAL, "null graph at %u", i);
+    lm_tuning keep;
+    lm_get_tuning(ctx, &keep);
+    // median time of three calls after one
+    const auto timed = [&](double* out) -> int {
+        std::vector<double> ms;
+        for (int it = 0; it < 4; it++) {
+            const auto t0 = std::chrono::steady_clock::now();
+            const int rc = count == 1 ? lm_match(ctx, g[0], seeds[0], mates[0], nullptr)
+                                      : lm_batch_match(ctx, g, count, seeds, mates, nullptr);
+            if (rc) return rc;
+            if (it > 0) ms.push_back(std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count());
+        }
+        std::sort(ms.begin(), ms.end());
+        *out = ms[ms.size() / 2];
+        return LM_OK;
+    };
+    if (!reads_tuning(ctx, g, count)) {   // nothing to choose: the parameters stay
+        const int rc = timed(&keep.ms);
+        if (rc == LM_OK && best) *best = keep;
+        return rc;
+    }
     // candidates (rmax, chunk, batch): task sizes from many short tasks to few long
     // ones, sweep at full or three-quarter occupancy
     static const uint32_t sizes[][3] = {{256, 1024, 256}, {512, 1024, 256}, {1024, 1024, 512}, {2048, 4096, 1024}};
     static const uint32_t sweeps[] = {0, 3};
-    lm_tuning keep;
-    lm_get_tuning(ctx, &keep);
     lm_tuning top = keep;
     top.ms = -1.0;
     for (const auto& sz : sizes) {
         for (uint32_t sw : sweeps) {
             lm_tuning t = {sz[0], sz[1], sw, keep.vertex_ctas_per_sm, sz[2], keep.contract_bits, 0.0};
             int rc = lm_set_tuning(ctx, &t);
-            if (rc) return rc;
-            std::vector<double> ms;
-            for (int it = 0; it < 4; it++) {
-                const auto t0 = std::chrono::steady_clock::now();
-                rc = count == 1 ? lm_match(ctx, g[0], seeds[0], mates[0], nullptr)
-                                : lm_batch_match(ctx, g, count, seeds, mates, nullptr);
-                if (rc) {
-                    lm_set_tuning(ctx, &keep);
-                    return rc;
-                }
-                if (it > 0) ms.push_back(std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count());
+            if (!rc) rc = timed(&t.ms);
+            if (rc) {
+                lm_set_tuning(ctx, &keep);
+                return rc;
             }
-            std::sort(ms.begin(), ms.end());
-            t.ms = ms[ms.size() / 2];
             if (top.ms < 0 || t.ms < top.ms) top = t;
         }
     }

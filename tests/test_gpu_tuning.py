@@ -113,3 +113,33 @@ def test_autotune_keeps_a_candidate_and_results_stay_exact():
             lm.lm_graph_destroy(h)
     finally:
         L.close()
+
+
+def test_autotune_chooses_only_where_the_parameters_are_read():
+    # the row lists and the renewed order's kernel read none of them: the context keeps its own;
+    # batches under a renewed order do
+    import torch
+    import paper_1302_4587_gb300 as lm
+    mine = dict(rmax=77, chunk=2048, sweep_ctas_per_sm=2, vertex_ctas_per_sm=1, batch=128)
+    for renew in (False, True):
+        L = Lm(renew=renew)
+        try:
+            gs = synth.batch(5, seed=9, n_lo=64, n_hi=4096)
+            seeds = [100 + i for i in range(len(gs))]
+            hs = [L.graph(g) for g in gs]
+            mates = [torch.empty(max(g.n, 1), dtype=torch.int32, device="cuda")[:g.n] for g in gs]
+            for count in (1, len(gs)):
+                lm.lm_set_tuning(L.ctx, **mine)
+                best = lm.lm_autotune(L.ctx, hs[:count], seeds[:count], mates[:count])
+                now = lm.lm_get_tuning(L.ctx)
+                assert best["ms"] > 0
+                for t in (best, now):
+                    if renew and count > 1:
+                        assert (t["rmax"], t["chunk"], t["batch"]) in [(256, 1024, 256), (512, 1024, 256),
+                                                                       (1024, 1024, 512), (2048, 4096, 1024)]
+                    else:
+                        assert {k: t[k] for k in mine} == mine
+            for h in hs:
+                lm.lm_graph_destroy(h)
+        finally:
+            L.close()
