@@ -209,7 +209,10 @@ int  lm_set_limits(lm_ctx* ctx, uint32_t max_rounds, uint32_t time_limit_ms);
  * environment; nothing on the GPU is made to fail):
  *   LM_FAULT=alloc      every device allocation the new context makes after
  *                       lm_create fails as out of memory (calls return LM_ENOMEM)
- *   LM_FAULT=alloc:N    only the next N of them fail. */
+ *   LM_FAULT=alloc:N    only the next N of them fail.
+ * Likewise LM_PATH=rounds: lm_match, lm_batch_match and served requests of the new context
+ * take the round-by-round path for every graph, as graphs of 2^31 vertices and more do
+ * (same results; for tests of that path, which is the slower one for smaller graphs). */
 
 /* Launch parameters of a context's matching and contraction paths (the paper
  * has no counterpart; they only affect speed, never the result):

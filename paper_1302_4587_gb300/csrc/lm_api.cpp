@@ -648,7 +648,9 @@ static int ensure_list(lm_ctx* ctx, Engine& e, size_t nv, size_t nc, size_t ng, 
 
 // The list path needs the top bit of a vertex id and an order that holds for the
 // whole job; a renewed order keys every round anew (match_renewed, or run_job for batches).
-bool list_path(const Engine& e, const lm_graph* g) { return !e.cfg.renew && g->n < 0x80000000u; }
+bool list_path(const Engine& e, const lm_graph* g) {
+    return !e.cfg.renew && !e.cfg.by_round && g->n < 0x80000000u;
+}
 
 // Parts of a graph in a job of `rows` rows and `ents` entries in all: one for every block of
 // the live pass that runs at once, within the limits.  A graph's own never exceed those
@@ -831,7 +833,7 @@ int match_one(lm_ctx* ctx, Engine& e, const lm_graph* g, uint64_t seed, uint32_t
     if (rc) return rc;
     if (g->nent && list_path(e, g))
         return match_list(ctx, e, g, seed, mate, dev_out, prof, async && dev_out && !prof.on, rounds, counts);
-    if (g->nent && g->n < 0x80000000u)
+    if (g->nent && g->n < 0x80000000u && !e.cfg.by_round)
         return match_renewed(ctx, e, g, seed, mate, dev_out, prof, async && dev_out && !prof.on, counts);
     rc = ensure_ws(ctx, e, g->n, g->nent, 1);
     if (rc) return rc;
@@ -1141,6 +1143,7 @@ int lm_create(const lm_config* cfg, lm_ctx** out) {
             ctx->fault_alloc = k;
         }
     }
+    if (const char* p = getenv("LM_PATH")) ctx->eng.cfg.by_round = !strcmp(p, "rounds");
     {
         cudaMemPoolProps pp;
         memset(&pp, 0, sizeof pp);
@@ -1575,7 +1578,8 @@ void tuning_of(const LaunchCfg& c, lm_tuning* t) {
 // whether a match of these graphs takes the round-by-round path, which the task sizes and
 // CTAs shape (see match_one, match_batch)
 bool reads_tuning(const lm_ctx* ctx, const lm_graph* const* g, uint32_t count) {
-    if (count == 1) return !(ctx->flags & LM_F_EDGE_CENTRIC) && g[0]->nent && g[0]->n >= 0x80000000u;
+    if (count == 1)
+        return !(ctx->flags & LM_F_EDGE_CENTRIC) && g[0]->nent && (g[0]->n >= 0x80000000u || ctx->eng.cfg.by_round);
     for (uint32_t i = 0; i < count; i++)
         if (!list_path(ctx->eng, g[i])) return true;
     return false;
@@ -1601,7 +1605,8 @@ int lm_set_tuning(lm_ctx* ctx, const lm_tuning* t) {
     LaunchCfg c;
     if (!cfg_from(t, &c)) return fail(ctx, LM_EINVAL, "tuning out of range");
     std::lock_guard<std::mutex> lk(ctx->call_mu);
-    c.renew = ctx->eng.cfg.renew;  // the order is the context's, not a tuning knob
+    c.renew = ctx->eng.cfg.renew;  // the order and the path are the context's, not tuning knobs
+    c.by_round = ctx->eng.cfg.by_round;
     ctx->eng.cfg = c;
     return LM_OK;
 }

@@ -136,6 +136,7 @@ struct LaunchCfg {
     uint32_t vertex_ctas_per_sm = 4;
     uint32_t batch_shift = LM_BATCH_SHIFT;  // 32: batches of 32 rows only
     bool renew = false;  // sweeps renew the order every round (LM_F_RENEW)
+    bool by_round = false;  // every graph by the round-by-round path (LM_PATH=rounds)
     uint32_t contract_bits = 0;  // bits of the contraction's hash sort (0: by size); no match graph uses it
     LaunchCfg() {
         while ((1u << chunk_shift) < CHUNK) chunk_shift++;

@@ -16,12 +16,14 @@ from gpu_util import to_u32
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def actx():
+@pytest.fixture(scope="module", params=["lists", "rounds"])   # the default path, and round by round
+def actx(request):
     import torch
     import paper_1302_4587_gb300 as lm
     torch.cuda.init()
-    c = lm.lm_create(0, None, flags=lm.LM_F_ASYNC)
+    with pytest.MonkeyPatch.context() as mp:
+        mp.setenv("LM_PATH", request.param)
+        c = lm.lm_create(0, None, flags=lm.LM_F_ASYNC)
     yield lm, torch, c
     lm.lm_destroy(c)
 

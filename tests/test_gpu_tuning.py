@@ -1,6 +1,6 @@
 """Launch parameters (lm_set_tuning / lm_autotune) change speed, never results:
-under every setting the CUDA path's mate[] and per-round counts must equal the
-oracle's, through the C ABI, on both launch paths."""
+under every setting the mate[] and per-round counts of the round-by-round path, which
+they shape, must equal the oracle's, through the C ABI, on both launch paths."""
 from __future__ import annotations
 
 import numpy as np
@@ -55,19 +55,71 @@ def _check(L, g, seed):
     k = min(r, 64)
     assert st["round_m"][:k] == [int(x) for x in rm[:k]]
     assert st["round_n"][:k] == [int(x) for x in rn[:k]]
+    return st
 
 
 @pytest.mark.parametrize("profile", [False, True], ids=["graph", "stream"])
 @pytest.mark.parametrize("setting", SETTINGS, ids=lambda s: f"r{s[0]}_c{s[1]}_s{s[2]}_v{s[3]}_b{s[4]}")
-def test_parity_under_every_setting(profile, setting):
+def test_parity_under_every_setting(profile, setting, monkeypatch):
     import paper_1302_4587_gb300 as lm
+    monkeypatch.setenv("LM_PATH", "rounds")   # the path whose kernels the settings shape
     L = Lm(profile=profile)
     try:
         lm.lm_set_tuning(L.ctx, *setting)
         got = lm.lm_get_tuning(L.ctx)
         assert (got["rmax"], got["chunk"], got["sweep_ctas_per_sm"], got["vertex_ctas_per_sm"], got["batch"]) == setting
         for g, seed in _graphs():
-            _check(L, g, seed)
+            st = _check(L, g, seed)
+            assert st["kernel_launches"][lm.LM_K_VERTEX] > 0   # (the row lists have no vertex pass)
+    finally:
+        L.close()
+
+
+@pytest.mark.parametrize("setting", SETTINGS, ids=lambda s: f"r{s[0]}_c{s[1]}_s{s[2]}_v{s[3]}_b{s[4]}")
+def test_renewed_batches_under_every_setting(setting):
+    import torch
+    import paper_1302_4587_gb300 as lm
+    L = Lm(renew=True)
+    try:
+        lm.lm_set_tuning(L.ctx, *setting)
+        gs = _graphs()
+        hs = [L.graph(g) for g, _ in gs]
+        mates = [torch.empty(g.n, dtype=torch.int32, device="cuda") for g, _ in gs]
+        _, st = lm.lm_batch_match(L.ctx, hs, [s for _, s in gs], mates, stats=True)
+        for (g, seed), m, s in zip(gs, mates, st):
+            want, r, _, _ = oracle.seq_local_max(g.n, g.eu, g.ev, g.w, seed, renew=True)
+            assert np.array_equal(to_u32(m), want) and s["rounds"] == r, g.name
+        for h in hs:
+            lm.lm_graph_destroy(h)
+    finally:
+        L.close()
+
+
+def test_batched_and_served_round_by_round(monkeypatch):
+    # the forms around that path: batches, host results, groups of served requests
+    import paper_1302_4587_gb300 as lm
+    monkeypatch.setenv("LM_PATH", "rounds")
+    L = Lm()
+    try:
+        gs = _graphs() + [(synth.er(300 + 50 * i, 900, seed=30 + i), i) for i in range(6)]
+        hs = [L.graph(g) for g, _ in gs]
+        want = [oracle.greedy(g.n, g.eu, g.ev, g.w, s) for g, s in gs]
+        new = lambda: [L.torch.empty(g.n, dtype=L.torch.int32, device="cuda") if i % 2 else np.empty(g.n, np.uint32)
+                       for i, (g, _) in enumerate(gs)]
+        mates = new()
+        _, st = lm.lm_batch_match(L.ctx, hs, [s for _, s in gs], mates, stats=True)
+        assert st[0]["kernel_launches"][lm.LM_K_VERTEX] > 0
+        for m, x in zip(mates, want):
+            assert np.array_equal(to_u32(m), x)
+        mates = new()
+        tickets = [lm.lm_submit(L.ctx, h, s, m) for h, (_, s), m in zip(hs, gs, mates)]
+        for t, m, x in zip(tickets, mates, want):
+            assert lm.lm_wait(L.ctx, t, 60_000)
+            done, st = lm.lm_poll(L.ctx, t)
+            assert done and st["matched"] == int((x != 0xFFFFFFFF).sum()) // 2
+            assert np.array_equal(to_u32(m), x)
+        for h in hs:
+            lm.lm_graph_destroy(h)
     finally:
         L.close()
 
