@@ -224,9 +224,6 @@ def run_lm(args, ws, rank, local):
     graph_bytes = lm.lm_graph_info(h)[2]
     del eu, ev, w
     mate = torch.empty(g.n, dtype=torch.int32, device=dev)
-    # launch parameters picked by the library's autotuner on this graph (untimed; the
-    # edge-centric path has none)
-    tuning = None if edge else lm.lm_autotune(ctx, [h], [seed], [mate])
     for _ in range(max(args.warmup, 3)):
         _, st = lm.lm_match(ctx, h, seed, mate, stats=True)
     torch.cuda.synchronize()
@@ -247,9 +244,6 @@ def run_lm(args, ws, rank, local):
 
     # per-kernel device times (CUDA events recorded by the library on its stream)
     pctx = lm.lm_create(local, stream, flags=lm.LM_F_PROFILE | (lm.LM_F_EDGE_CENTRIC if edge else 0) | order)
-    if tuning:
-        lm.lm_set_tuning(pctx, tuning["rmax"], tuning["chunk"], tuning["sweep_ctas_per_sm"],
-                         tuning["vertex_ctas_per_sm"], tuning["batch"])
     kms = {k: [] for k in range(lm.LM_K_COUNT)}
     total_ms = []
     for i in range(max(args.warmup, 3) + args.steps):
@@ -276,9 +270,10 @@ def run_lm(args, ws, rank, local):
         names = {lm.LM_K_SWEEP: "k_renew"}
         models = {"k_renew": (lm.LM_K_SWEEP, renew_model_bytes(pst))}
     else:
-        # (the profiled matches want the rounds' counts: k_live with 64-bit words, and
-        # k_round_bytes + k_round_counts, which the timed matches do not run)
-        names = {lm.LM_K_CAND: "k_top", lm.LM_K_SWEEP: "k_live",
+        # the profiled matches want the rounds' counts: k_live with 64-bit words, and
+        # k_round_bytes + k_round_counts, which the timed matches do not run.  So the timed
+        # matches' k_live is their time less k_top's (the same kernel but for the word that it writes)
+        names = {lm.LM_K_CAND: "k_top", lm.LM_K_SWEEP: "k_live (64-bit words: matches with statistics)",
                  lm.LM_K_OTHER: "k_round_bytes + k_round_counts (statistics only)"}
         models = {"k_top": (lm.LM_K_CAND, top_model_bytes(pst, g.n)),
                   "k_live": (lm.LM_K_SWEEP, live_model_bytes(pst))}
@@ -288,6 +283,10 @@ def run_lm(args, ws, rank, local):
     per_kernel = {name: {"bytes_per_match": by, "ms_per_match": med[kind],
                          "launches_per_match": pst["kernel_launches"][kind]}
                   for name, (kind, by) in models.items()}
+    if "k_live" in per_kernel:
+        per_kernel["k_live"].update(ms_per_match=ms_max - med[lm.LM_K_CAND], launches_per_match=1,
+                                    time="the timed match (32-bit words) less k_top's time: with the launch and the "
+                                         "host's wait; rows given back would be another launch")
     for kname, d in per_kernel.items():
         d["achieved"] = gbs(d["bytes_per_match"], d["ms_per_match"])
         d["frac"] = d["achieved"] / peak
@@ -351,7 +350,7 @@ def run_lm(args, ws, rank, local):
         "config": {"workload": args.workload, "desc": desc, "n": g.n, "m": g.m, "seed": seed,
                    "rounds": pst["rounds"], "graph_bytes": graph_bytes,
                    "l2": f"inputs larger than L2 (graph arrays {graph_bytes / 1e9:.1f} GB, L2 0.13 GB)",
-                   "tuning": tuning, "algorithm": "edge-centric" if edge else "segmented",
+                   "algorithm": "edge-centric" if edge else "segmented",
                    "order": args.order,
                    "parallelism": f"replicas x{ws}" if ws > 1 else "single GPU"},
         "roofline": ({"bound": "hbm", "kernel": "k_ec_offer + k_ec_match + k_ec_compact (all launches)",
@@ -412,7 +411,6 @@ def batched_form(args, local, steps: int):
     mates = [torch.empty(max(g.n, 1), dtype=torch.int32, device=dev)[:g.n] for g in gs]
     m_tot = sum(g.m for g in gs)
     job = lm.BatchArgs(hs, seeds, mates)  # marshalled once, reused by every step
-    tuning = lm.lm_autotune(ctx, job)     # launch parameters picked on this batch (untimed)
     for _ in range(3):
         lm.lm_batch_match(ctx, job)
     torch.cuda.synchronize()
@@ -470,7 +468,7 @@ def batched_form(args, local, steps: int):
         "graphs": len(gs), "sum_m": m_tot, "sum_n": sum(g.n for g in gs),
         "desc": "4096 graphs, n log-uniform [64,65536], degree U[4,16], ER/grid/R-MAT mixed, w~U[0,1), gen seed 4, "
                 "match seeds 1000+i",
-        "graph_bytes": graph_bytes, "tuning": tuning, "steps": steps, "ms_per_call": ms,
+        "graph_bytes": graph_bytes, "steps": steps, "ms_per_call": ms,
         "graphs_per_s": len(gs) / (ms * 1e-3), "edges_per_s": m_tot / (ms * 1e-3),
         "offered_together": {
             "latency": "all 4096 graphs offered at t=0; a graph's latency = time until its mate is complete",
