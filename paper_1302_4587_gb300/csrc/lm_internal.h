@@ -1,20 +1,26 @@
-// Internal declarations shared by the kernels (lm_kernels.cu, lm_contract.cu) and
-// the host code (lm_api.cpp, lm_serve.cpp).  Not part of the public ABI (include/lm.h is).
+// Internal declarations shared by the kernels (*.cu) and the host code (lm_api.cpp,
+// lm_serve.cpp).  Not part of the public ABI (include/lm.h is).
 //
-// Layout of one matching job (one graph, or the disjoint union of a batch):
-//   * vertices live in a union id space [0, N); graph g owns [vbase_g, vbase_g + n_g)
-//   * adjacency entries live in a union entry space; vertex v's row occupies
-//     [start[v], start[v] + deg(v)) -- the graph's own CSR range, shifted by the
-//     graph's entry base.  The row never moves: in every round its surviving
-//     entries are compacted to the front of the same range of the other
-//     ping-pong buffer, and len[round & 1][v] says how many there are.
-//   * a round works from two task lists built by the vertex pass:
-//       R  rows with 1..RMAX live entries (a warp takes 32 rows and walks
-//          their entries as one flattened sequence)
-//       C  chunks of up to CHUNK entries of longer rows (one warp per chunk)
-//   * a row keeps only the heaviest surviving key; the neighbour over that
-//     edge is recovered from the key itself: its low half is perm_seed(e),
-//     which is inverted to the edge index e, whose record holds both ends.
+// A graph's adjacency entries lie row by row (off, ent, eid) and never move.  Three paths match:
+//   * row lists (lm_list.cu; the default): a word and the heaviest neighbours of every
+//     vertex, live rows in parts; see ListSeg, ListArgs
+//   * one graph under a renewed order (lm_renew.cu): a candidate and a matched bit of every
+//     vertex; see RenewArgs
+//   * round by round (lm_kernels.cu; batches under a renewed order, graphs of 2^31 vertices
+//     and more), over the disjoint union of a job's graphs:
+//       - vertices live in a union id space [0, N); graph g owns [vbase_g, vbase_g + n_g)
+//       - adjacency entries live in a union entry space; vertex v's row occupies
+//         [start[v], start[v] + deg(v)) -- the graph's own CSR range, shifted by the
+//         graph's entry base.  In every round a row's surviving entries are compacted
+//         to the front of the same range of the other ping-pong buffer, and
+//         len[round & 1][v] says how many there are.
+//       - a round works from two task lists built by the vertex pass:
+//           R  rows with 1..RMAX live entries (a warp takes 32 rows and walks
+//              their entries as one flattened sequence)
+//           C  chunks of up to CHUNK entries of longer rows (one warp per chunk)
+//       - a row keeps only the heaviest surviving key; the neighbour over that
+//         edge is recovered from the key itself: its low half is perm_seed(e),
+//         which is inverted to the edge index e, whose record holds both ends.
 #pragma once
 #include <stdint.h>
 #include <stddef.h>

@@ -769,8 +769,9 @@ __device__ __forceinline__ void refill_put(W* cur, const RowLists& R, uint32_t v
 
 // ---------------------------------------------------------------- k_live
 constexpr int LT = 128, LW = LT / 32;
-// blocks an SM: rounds' words apart, 8 need no spills but 10 cover more latency (R-MAT scale 23
-// 1.32 and 1.28 ms, 4096 graphs 3.88 and 3.80; 12: 1.30, 3.72, but coarsening 9.9 ms for 9.5)
+// blocks an SM, chosen on 32-bit words: 8 need no spills but 10 cover more latency (R-MAT scale 23
+// 1.32 and 1.28 ms, 4096 graphs 3.88 and 3.80; 12: 1.30, 3.72, but coarsening 9.9 ms for 9.5).
+// 64-bit words take the same 48 registers and spill 426 bytes of stores there.
 constexpr int LMINB = 10;
 constexpr uint32_t BLOCK_ROW = 1024;  // longer rows are refilled by the whole block
 constexpr uint32_t IDLE_MAX = 48;     // passes without a change before a block gives its rows back

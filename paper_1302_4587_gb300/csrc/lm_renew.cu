@@ -24,8 +24,8 @@
 // unit grid of 1M vertices 195 us (317), 5,000 edges 75 us (167).
 //
 // Bound by the passes over the entries in the first three rounds (R-MAT scale 20, unit
-// weights, 15.7M edges, 8 rounds: 541 us; rounds as launches with the
-// entries compacted after each one, 915 us, which read and wrote 16 bytes an entry
+// weights, 15.7M edges, 8 rounds: 524 us; rounds as launches with the
+// entries compacted after each one, 919 us, which read and wrote 16 bytes an entry
 // and gathered every neighbour's state).
 #include <cuda_runtime.h>
 #include <stdint.h>

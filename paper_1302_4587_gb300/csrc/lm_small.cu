@@ -14,8 +14,9 @@
 // of edge ids in the static scratch.
 //
 // 10,000 vertices and 50,000 edges, 7 rounds: 314 us with one block and 64-bit offers in
-// global memory (every phase waiting on L2), 92 us with sixteen blocks here, 122 us
-// with eight; 512 threads a block with twice the edges each: 99 us.
+// global memory (every phase waiting on L2), 75 us with sixteen blocks here.  Waited for
+// call by call: 92 us with sixteen blocks, 122 with eight, 99 with 512 threads a block and
+// twice the edges each.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
